@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -36,9 +37,18 @@ struct Block {
   long long ebase = -1;   // offset of its gather map in d_emap (blocks with a non-periodic face)
 };
 
+// The blocks that one line-filter launch covers: along the pass axis they have the same number of
+// sub-domains and equally long longest lines (the length sizes the shared-memory tiles).
+struct FilterGroup {
+  int Lt = 0, nblk = 0;
+  unsigned ctas = 0;
+  cfs::FilterBlk* d_blks = nullptr;
+};
+
 struct cfs_ctx {
   cfs_params p{};
   std::vector<Block> blocks;
+  std::vector<FilterGroup> fgroups[3];  // per pass axis
   cudaStream_t stream = nullptr;
   cfs_alloc_fn alloc = nullptr;
   cfs_free_fn freef = nullptr;
@@ -72,6 +82,7 @@ struct cfs_ctx {
   int max_pad = 0, max_own = 0, max_flux = 0;
   double* d_thomas = nullptr;
   float* d_thomas32 = nullptr;
+  double* d_thomas_k = nullptr;  // FP64 line filter: the factors, 1 / m_i times the filter's scale
   int Lmax = 0;
   double filt_h[6] = {0};
   double* d_partial = nullptr;
@@ -734,10 +745,11 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   c->d_partial = (double*)dev_alloc(c, sizeof(double) * DIAG_NQ * c->diag_blocks * c->blocks.size());
   c->d_thomas = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   c->d_thomas32 = (float*)dev_alloc(c, sizeof(float) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
+  c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   for (void* q : c->owned)
     if (!q) return fail(c, CFS_ENOMEM, "device allocation failed");
   if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && (!c->Wp || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
-      !c->d_partial || !c->d_out || !c->d_thomas || !c->d_thomas32)
+      !c->d_partial || !c->d_out || !c->d_thomas || !c->d_thomas32 || !c->d_thomas_k)
     return fail(c, CFS_ENOMEM, "device allocation failed");
   for (const Block& b : c->blocks)
     for (int a = 0; a < 3; ++a)
@@ -842,7 +854,22 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       im[i] = 1.0 / m;
     }
   }
+  // the factors of the FP64 line filter, 1 / m_i times (1 - 2 alpha) / 1024, eliminated in long
+  // double (alpha near 1/2 makes the system nearly singular at the shortest wave)
+  std::vector<double> thk(th.size(), 0.0);
+  for (int len = 1; len <= c->Lmax; ++len) {
+    double* cp = thk.data() + (size_t)len * 2 * c->Lmax;
+    double* im = cp + c->Lmax;
+    long double ci = 0.0L;
+    for (int i = 0; i < len; ++i) {
+      const long double m = 1.0L - (long double)al * ci;
+      ci = (long double)al / m;
+      cp[i] = (double)ci;
+      im[i] = (double)((1.0L - 2.0L * (long double)al) / 1024.0L / m);
+    }
+  }
   cudaStream_t st = c->stream;
+  CUDA_TRY(c, cudaMemcpyAsync(c->d_thomas_k, thk.data(), sizeof(double) * thk.size(), cudaMemcpyHostToDevice, st), "upload filter");
   CUDA_TRY(c, cudaMemcpyAsync(c->d_subs, c->subs.data(), sizeof(SubDev) * nsub, cudaMemcpyHostToDevice, st), "upload sub-domains");
   CUDA_TRY(c, cudaMemcpyAsync(c->d_W, W.data(), sizeof(double) * nW, cudaMemcpyHostToDevice, st), "upload weights");
   CUDA_TRY(c, cudaMemcpyAsync(c->d_Wf, Wf.data(), sizeof(double) * nWf, cudaMemcpyHostToDevice, st), "upload weights");
@@ -866,6 +893,52 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       CUDA_TRY(c, cudaMemcpyAsync(b.d_owner[a], keep[k0].data(), sizeof(int) * n3[a], cudaMemcpyHostToDevice, st), "upload tables");
       CUDA_TRY(c, cudaMemcpyAsync(b.d_axis_off[a], keep[k0 + 1].data(), sizeof(int) * b.P[a], cudaMemcpyHostToDevice, st), "upload tables");
       CUDA_TRY(c, cudaMemcpyAsync(b.d_axis_len[a], keep[k0 + 2].data(), sizeof(int) * b.P[a], cudaMemcpyHostToDevice, st), "upload tables");
+    }
+  }
+  // line filter: per pass axis the blocks by the length of their longest line and their split
+  std::vector<std::vector<cfs::FilterBlk>> fkeep;  // (alive until the stream is synchronised below)
+  if (c->p.filter) {
+    for (int ax = 0; ax < c->ndim; ++ax) {
+      std::map<std::pair<int, int>, std::vector<const Block*>> by_len;
+      for (const Block& b : c->blocks) {
+        const int n3[3] = {b.nx, b.ny, b.nz};
+        by_len[{(n3[ax] + b.P[ax] - 1) / b.P[ax], b.P[ax]}].push_back(&b);
+      }
+      for (const auto& kv : by_len) {
+        FilterGroup fg;
+        fg.Lt = kv.first.first;
+        std::vector<cfs::FilterBlk> v;
+        for (const Block* b : kv.second) {
+          cfs::FilterBlk e{};
+          e.ebase = b->ebase;
+          e.gmx = b->nx + 2 * c->geo.GE;
+          e.gmy = b->ny + 2 * c->geo.GE;
+          for (int q = 0; q < 6; ++q) {
+            if (b->face[q].type >= cfs::FACE_WALL) e.phys |= 1 << q;
+            if (b->face[q].type == cfs::FACE_WALL) e.wall |= 1 << q;
+          }
+          e.n[0] = b->nx; e.n[1] = b->ny; e.n[2] = b->nz;
+          e.bN = b->N;
+          e.bbase = b->base;
+          e.sid0 = b->sid0;
+          for (int a = 0; a < 3; ++a) {
+            e.P[a] = b->P[a];
+            e.owner[a] = b->d_owner[a];
+            e.axis_off[a] = b->d_axis_off[a];
+            e.axis_len[a] = b->d_axis_len[a];
+          }
+          e.cta0 = fg.ctas;
+          fg.ctas += cfs::filter_ctas(e.n, e.P, ax, fg.Lt);
+          v.push_back(e);
+        }
+        fg.nblk = (int)v.size();
+        fg.d_blks = (cfs::FilterBlk*)dev_alloc(c, sizeof(cfs::FilterBlk) * v.size());
+        if (!fg.d_blks) return fail(c, CFS_ENOMEM, "device allocation failed");
+        fkeep.push_back(std::move(v));
+        CUDA_TRY(c, cudaMemcpyAsync(fg.d_blks, fkeep.back().data(), sizeof(cfs::FilterBlk) * fkeep.back().size(),
+                                    cudaMemcpyHostToDevice, st), "upload filter blocks");
+        c->fgroups[ax].push_back(fg);
+      }
     }
   }
   CUDA_TRY(c, cudaMemsetAsync(c->ring, 0, sizeof(double) * 5 * N * c->R, st), "clear ring");
@@ -1096,35 +1169,18 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       // graph mode: the sub-domain filter (returns on synchronous steps) before the per-pass
       // kernels (which then return on asynchronous steps)
       if (op == c->s && c->fblock_n && graph) rc = launch_fblock(c, g, sc, src, nullptr, true);
-      for (const Block& b : c->blocks) {
+      for (const FilterGroup& fg : c->fgroups[op - c->s]) {
         if (rc != 0) break;
         cfs::FilterLaunch f{};
         f.Uin = src; f.Uout = dst; f.ring = c->ring;
         f.in_ring = in_ring; f.out_ring = out_ring;
-        f.nx = b.nx; f.ny = b.ny; f.nz = b.nz; f.bN = b.N; f.bbase = b.base; f.sid0 = b.sid0;
-        f.ebase = b.ebase;
-        f.gmx = b.nx + 2 * c->geo.GE;
-        f.gmy = b.ny + 2 * c->geo.GE;
-        f.wall = f.phys = 0;
-        for (int q = 0; q < 6; ++q) {
-          if (b.face[q].type >= cfs::FACE_WALL) f.phys |= 1 << q;
-          if (b.face[q].type == cfs::FACE_WALL) f.wall |= 1 << q;
-        }
-        for (int a = 0; a < 3; ++a) {
-          f.owner[a] = b.d_owner[a]; f.axis_off[a] = b.d_axis_off[a]; f.axis_len[a] = b.d_axis_len[a];
-          f.P[a] = b.P[a];
-        }
-        f.thomas = c->d_thomas; f.thomas32 = c->d_thomas32; f.Lmax = c->Lmax; f.alpha = c->p.alpha_f;
-        {
-          const int ax = op - c->s, n3[3] = {b.nx, b.ny, b.nz};
-          f.Lt = (n3[ax] + b.P[ax] - 1) / b.P[ax];
-        }
+        f.blks = fg.d_blks; f.nblk = fg.nblk; f.ctas = fg.ctas; f.Lt = fg.Lt;
+        f.thomas_k = c->d_thomas_k; f.thomas32 = c->d_thomas32; f.Lmax = c->Lmax; f.alpha = c->p.alpha_f;
         for (int m = 0; m < 6; ++m) f.h[m] = c->filt_h[m];
         f.b1 = c->filt_h[1] - c->p.alpha_f;
         f.only_sync = graph && c->fblock_n;
         f.subs = c->part_n > 1 ? c->d_subs : nullptr;
         rc = cfs::launch_filter(g, sc, f, op - c->s, c->p.precision, c->stream, &c->launches, tm);
-        if (rc != 0) break;
       }
     }
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");

@@ -219,26 +219,35 @@ struct Timer {
 int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a,
                  int precision, void* stream, long long* launches, const Timer* tm);
 
-struct FilterLaunch {
+// One block as the line filter sees it (device table, one entry per block of a launch).
+struct FilterBlk {
   long long ebase;         // the block's gather map (SubDev::ebase), or -1
   int gmx, gmy;
   int wall;                // bit f: face f of the block is a no-slip wall (momentum held at zero)
   int phys;                // bit f: face f of the block is a physical boundary
-  const double* Uin;
-  double* Uout;
-  const double* ring;
-  int nx, ny, nz;          // the block being filtered
+  int n[3];                // the block's size
+  int P[3];                // sub-domains per axis
   long long bN, bbase;     // its points and the offset of its state in a state array
   int sid0;                // index of its first sub-domain
-  int in_ring, out_ring;   // graph mode: input is ring level n / output is ring level n + 1
+  unsigned cta0;           // first CTA of the launch that works on it
   const int* owner[3];     // device: sub-domain index along each axis for every global coordinate
   const int* axis_off[3];  // device: per sub-domain index along the axis, its origin
   const int* axis_len[3];  // device: ... and its length
-  const double* thomas;    // device: [Lmax+1 rows][2][Lmax] Thomas factors per line length
-  const float* thomas32;   // device: the same table rounded to FP32 (d2f_fast), for the FP32 form
+};
+
+struct FilterLaunch {
+  const double* Uin;
+  double* Uout;
+  const double* ring;
+  int in_ring, out_ring;   // graph mode: input is ring level n / output is ring level n + 1
+  const FilterBlk* blks;   // device: the blocks of this launch (their longest lines along the pass
+  int nblk;                // axis are all Lt points, which sizes the tiles)
+  unsigned ctas;
+  const double* thomas_k;  // device: FP64 form: [Lmax+1 rows][2][Lmax] per line length: c_i, and 1 / m_i
+                           // times the filter's scale (1 - 2 alpha)/1024
+  const float* thomas32;   // device: FP32 form: c_i and 1 / m_i rounded to FP32 (d2f_fast)
   int Lmax;
-  int Lt;                  // longest sub-domain line of this block along the pass axis (sizes the tiles)
-  int P[3];                // sub-domains per axis
+  int Lt;                  // longest sub-domain line of these blocks along the pass axis
   double alpha;
   double h[6];             // filter right side: a_0, a_1/2, ..., a_5/2
   double b1;               // a_1/2 - alpha: weight of the first second difference (increment form)
@@ -246,6 +255,8 @@ struct FilterLaunch {
   const SubDev* subs;      // partitioned context: the sub-domain table (lines of foreign sub-domains are
                            // skipped); null when every sub-domain is computed here
 };
+// CTAs of a launch that one block of size n, split P, takes along `axis` with lines of Lt points
+unsigned filter_ctas(const int* n, const int* P, int axis, int Lt);
 
 // FP32-intermediate filter of asynchronous steps, all three passes per (sub-domain, variable)
 // (filter_block.cu); cubic sub-domains of n points per axis, n in {16, 32}.
@@ -269,8 +280,8 @@ bool filter_block_supported(int n);
 int launch_filter_block(const Geometry& g, const StepSched& sc, const FilterBlockLaunch& f, int n, void* stream,
                         long long* launches, const Timer* tm);
 
-int filter_prepare(int Lmax, int precision);
-int launch_round_table(const double* x, float* y, long long n, void* stream);  // y = d2f_fast(x)  // shared-memory attribute of the filter kernels; nonzero if too long
+int filter_prepare(int Lmax, int precision);  // shared-memory attribute of the filter kernels; nonzero if too long
+int launch_round_table(const double* x, float* y, long long n, void* stream);  // y = d2f_fast(x)
 int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f, int axis, int precision,
                   void* stream, long long* launches, const Timer* tm);
 

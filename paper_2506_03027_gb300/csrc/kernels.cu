@@ -19,6 +19,7 @@
 // boxes of all sub-domains.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <type_traits>
@@ -811,14 +812,28 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 
 // ------------------------------------------------------------------------------- k_filter
 
-// One CTA per (variable, line segment of one sub-domain, group of LN lines); one thread per line
-// in the solve.  Lines along `axis`; the two other axes are f1 (x unless axis is x) and f2.  The
-// CTA first stages the 11-point windows of all its lines -- own values, and halo values by the
-// schedule (SA: live neighbour; AT: extrapolation to t_{n+1} with the weights c(k+1) in FP64;
-// AS: the latest delayed level) -- in shared memory with coalesced loads (consecutive threads
-// along the line for the x pass, across lines for y and z), solves each line from there, and
-// stores the result with the same pattern.  Right side: sum_n (a_n/2)(f_{i+n} + f_{i-n});
-// Dirichlet closure f^_{-1} = f_{-1}, f^_L = f_L; Thomas factors precomputed per line length.
+// One CTA per (variable, line segment of one sub-domain, group of LN lines) of the launch's blocks;
+// one thread per line in the solve.  Lines along `axis`; the two other axes are f1 (x unless axis
+// is x) and f2.  The CTA first stages the 11-point windows of all its lines -- own values, and halo
+// values by the schedule (SA: live neighbour; AT: extrapolation to t_{n+1} with the weights c(k+1)
+// in FP64; AS: the latest delayed level) -- in shared memory with coalesced loads (consecutive
+// threads along the line for the x pass, across lines for y and z), solves each line from there,
+// and stores the result with the same pattern.  Blocks with the same split and line length
+// along the axis share a launch: the twelve blocks of an airfoil grid take seven launches per step
+// instead of 36 that each fill a part of the chip.
+//
+// Both forms solve for the increment d = f^ - f, with d = 0 at the first halo point (the Dirichlet
+// closure f^_{-1} = f_{-1}, f^_L = f_L).  The conditions that fix the coefficients -- T = 1 +
+// O(w^10), T(pi) = 0 -- make the right side minus (alpha, 1, alpha) f equal to
+// (1 - 2 alpha)/1024 delta^10 f, so the FP64 form needs ten differences per point:
+//   (alpha, 1, alpha) d = (1 - 2 alpha)/1024 delta^10 f.
+// It is bound by the FP64 pipe when it differences in FP64 (2 FMA per clock and SM), so the
+// differences are 64-bit integers instead: every value of the line's window as a fixed-point number
+// with the last place of its largest value as the quantum (2^(E-52), smaller values rounded down;
+// the mean of that rounding drops out of the differences), ten integer subtractions give delta^10
+// exactly, and the two sweeps and the final sum f + d are four FP64 operations per point.  What the
+// rounding leaves passes through 1 - T <= 1, which is small everywhere but next to the shortest
+// wave, so it adds less than the rounding of the final sum.
 struct FilterTile {
   int LN;  // lines per CTA
   int TW;  // row stride in doubles (odd: 64-bit accesses of a warp's rows hit distinct banks)
@@ -842,6 +857,26 @@ __host__ __device__ inline size_t filter_smem_bytes(int Lmax, int precision) {
   return (filter_tile_doubles(t, precision) + t.TW) * 8;
 }
 
+// x in units of 2^(E-52), rounded down, E + 1023 = ex the exponent field of a number no smaller
+__device__ __forceinline__ long long fixed_point(double x, int ex) {
+  const int hi = __double2hiint(x);
+  const int sh = min(ex - ((hi >> 20) & 0x7ff), 63);
+  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x));
+  const long long sg = hi >> 31;
+  return ((m ^ sg) - sg) >> sh;
+}
+
+// g 2^(q20 >> 20) in FP64 (|g| < 2^63), truncated to 53 bits, on the integer pipe
+__device__ __forceinline__ double from_fixed_point(long long g, int q20) {
+  const long long sg = g >> 63;
+  const unsigned long long m = (unsigned long long)((g ^ sg) - sg);
+  const int lz = __clzll((long long)m);
+  const unsigned long long t = (m << lz) >> 11;  // the leading one at bit 52
+  // (adding the leading one to the exponent field raises it by one)
+  const int hi = (int)(t >> 32) + ((1023 + 62 - lz) << 20) + q20;
+  return m ? __hiloint2double(hi | ((int)sg & (int)0x80000000), (int)t) : 0.0;
+}
+
 template <typename T, int axis>
 __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
   pdl_enter();
@@ -852,8 +887,16 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
   double* __restrict__ Uout = const_cast<double*>(ring_or(f.Uout, f.out_ring, f.ring, sc, 1));
   constexpr int f1 = (axis == 0) ? 1 : 0;
   constexpr int f2 = (axis == 2) ? 1 : 2;
-  const int n[3] = {f.nx, f.ny, f.nz};
-  const long long strides[3] = {1, f.nx, (long long)f.nx * f.ny};
+  // the block of this CTA: the last one that starts at or before it
+  int bi = 0;
+  for (int hi = f.nblk; hi - bi > 1;) {
+    const int mid = (bi + hi) >> 1;
+    if (f.blks[mid].cta0 <= blockIdx.x) bi = mid;
+    else hi = mid;
+  }
+  const FilterBlk& B = f.blks[bi];
+  const int n[3] = {B.n[0], B.n[1], B.n[2]};
+  const long long strides[3] = {1, n[0], (long long)n[0] * n[1]};
   const FilterTile tl = filter_tile(f.Lt);
   const int LN = tl.LN, TW = tl.TW;
   extern __shared__ __align__(16) double fsm[];
@@ -865,12 +908,12 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
 
   const long long nl = (long long)n[f1] * n[f2];
   const int groups = (int)((nl + LN - 1) / LN);
-  int b = blockIdx.x;
+  int b = (int)(blockIdx.x - B.cta0);
   const int grp = b % groups;
   b /= groups;
-  const int seg = b % f.P[axis];
-  const int var = b / f.P[axis];
-  const int off = f.axis_off[axis][seg], len = f.axis_len[axis][seg];
+  const int seg = b % B.P[axis];
+  const int var = b / B.P[axis];
+  const int off = B.axis_off[axis][seg], len = B.axis_len[axis][seg];
   const int W = len + 10;
   const long long l0 = (long long)grp * LN;
   const int nlines = (int)min((long long)LN, nl - l0);
@@ -884,29 +927,29 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
   __shared__ int sSid[128], sT1[128], sT2[128];  // blocks with a gather map: the line's sub-domain and position
   __shared__ double sRef[128];                   // FP32 form: the line's first own value
   __shared__ unsigned char sOk[128];             // the line belongs to a sub-domain computed here
-  const bool gmap = f.ebase >= 0;
+  const bool gmap = B.ebase >= 0;
   for (int t = threadIdx.x; t < nlines; t += blockDim.x) {
     const long long t12 = l0 + t;
     const int t1 = (int)(t12 % n[f1]), t2 = (int)(t12 / n[f1]);
-    sBase[t] = f.bbase + (long long)var * f.bN + (long long)t1 * strides[f1] + (long long)t2 * strides[f2];
+    sBase[t] = B.bbase + (long long)var * B.bN + (long long)t1 * strides[f1] + (long long)t2 * strides[f2];
     sOk[t] = 1;
     if (f.subs) {  // partitioned context: skip the lines of another process's sub-domains
       int sidx[3];
       sidx[axis] = seg;
-      sidx[f1] = f.owner[f1][t1];
-      sidx[f2] = f.owner[f2][t2];
-      sOk[t] = (unsigned char)f.subs[f.sid0 + sidx[0] + f.P[0] * (sidx[1] + f.P[1] * sidx[2])].own;
+      sidx[f1] = B.owner[f1][t1];
+      sidx[f2] = B.owner[f2][t2];
+      sOk[t] = (unsigned char)f.subs[B.sid0 + sidx[0] + B.P[0] * (sidx[1] + B.P[1] * sidx[2])].own;
     }
     int kl = 0, kr = 0;
     if (sc.mode != 0 || gmap) {
       int sidx[3];
       sidx[axis] = seg;
-      sidx[f1] = f.owner[f1][t1];
-      sidx[f2] = f.owner[f2][t2];
-      const int sid = f.sid0 + sidx[0] + f.P[0] * (sidx[1] + f.P[1] * sidx[2]);
+      sidx[f1] = B.owner[f1][t1];
+      sidx[f2] = B.owner[f2][t2];
+      const int sid = B.sid0 + sidx[0] + B.P[0] * (sidx[1] + B.P[1] * sidx[2]);
       // a sub-domain face on a physical block boundary has no neighbouring PE and no delay
-      const bool pl = seg == 0 && ((f.phys >> (2 * axis)) & 1);
-      const bool pr = seg == f.P[axis] - 1 && ((f.phys >> (2 * axis + 1)) & 1);
+      const bool pl = seg == 0 && ((B.phys >> (2 * axis)) & 1);
+      const bool pr = seg == B.P[axis] - 1 && ((B.phys >> (2 * axis + 1)) & 1);
       if (sc.mode != 0) {
         kl = pl ? 0 : face_delay(sc, sid, 2 * axis);
         kr = pr ? 0 : face_delay(sc, sid, 2 * axis + 1);
@@ -937,7 +980,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
     cc[axis] = u;
     cc[f1] = sT1[line];
     cc[f2] = sT2[line];
-    const int ei = g.emap[f.ebase + (cc[0] + g.GE) + (long long)f.gmx * ((cc[1] + g.GE) + (long long)f.gmy * cc[2])];
+    const int ei = g.emap[B.ebase + (cc[0] + g.GE) + (long long)B.gmx * ((cc[1] + g.GE) + (long long)B.gmy * cc[2])];
     const GatherEntry& E = g.gent[ei];
     const int kd = sKd[pos < 0 ? 0 : 1][line];
     double v = E.cst[var];
@@ -959,12 +1002,17 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
     return v;
   };
   // halo slot inside the block: SA the neighbour's value, AS the latest visible level, AT the
-  // extrapolation to t_{n+1} with the weights c(k+1), in FP64
+  // extrapolation to t_{n+1} with the weights c(k+1), in FP64 (the levels' loads before the sum)
   auto halo_value = [&](int line, int pos, long long gi) -> double {
     const int kd = sKd[pos < 0 ? 0 : 1][line];
     if (sc.mode == 2) return f.ring[sLev[kd * sc.C] + gi];
+    double r[CFS_MAX_LEVELS];
+#pragma unroll
+    for (int l = 0; l < CFS_MAX_LEVELS; ++l) r[l] = l < sc.C ? f.ring[sLev[kd * sc.C + l] + gi] : 0.0;
     double v = 0.0;
-    for (int l = 0; l < sc.C; ++l) v = fma(__ldg(sc.Wf + kd * sc.C + l), f.ring[sLev[kd * sc.C + l] + gi], v);
+#pragma unroll
+    for (int l = 0; l < CFS_MAX_LEVELS; ++l)
+      if (l < sc.C) v = fma(__ldg(sc.Wf + kd * sc.C + l), r[l], v);
     return v;
   };
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -981,18 +1029,22 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       else *dst = halo_value(line, pos, gi);
     };
     if (axis == 0) {
-      // own points: a warp per line, lanes along it (contiguous in memory); the 10 window points
-      // outside the segment: a thread per line, so that no warp mixes copies with extrapolations
+      // own points: a warp per line, lanes along it (contiguous in memory); then the 10 window
+      // points outside the segment, consecutive threads on consecutive points of a line's end, so
+      // that no warp mixes copies with extrapolations
       for (int line = warp; line < nlines; line += nwarp)
         if (sOk[line])
           for (int i = 5 + lane; i < 5 + len; i += 32) cp_async8(tile + line * TW + i, Uin + sBase[line] + sPos[i]);
-      for (int line = threadIdx.x; line < nlines; line += blockDim.x)
-        if (sOk[line])
-          for (int h = 0; h < 10; ++h) stage(line, h < 5 ? h : len + h);
+      for (int e = threadIdx.x; e < 10 * nlines; e += blockDim.x) {
+        const int line = e / 10, h = e - 10 * line;
+        if (sOk[line]) stage(line, h < 5 ? h : len + h);
+      }
     } else {  // threads across lines (consecutive x)
       for (int line = threadIdx.x; line < nlines; line += blockDim.x)
-        if (sOk[line])
-          for (int i = 0; i < W; ++i) stage(line, i);
+        if (sOk[line]) {
+          for (int i = 5; i < 5 + len; ++i) cp_async8(tile + line * TW + i, Uin + sBase[line] + sPos[i]);
+          for (int h = 0; h < 10; ++h) stage(line, h < 5 ? h : len + h);
+        }
     }
   } else {
     // FP32 form: every value converted on arrival to its offset from the line's first own value
@@ -1014,16 +1066,20 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       for (int line = warp; line < nlines; line += nwarp)
         if (sOk[line])
           for (int i = 5 + lane; i < 5 + len; i += 32) put(line, i, Uin[sBase[line] + sPos[i]]);
+      for (int e = threadIdx.x; e < 10 * nlines; e += blockDim.x) {
+        const int line = e / 10, h = e - 10 * line, i = h < 5 ? h : len + h;
+        if (sOk[line]) put(line, i, value(line, i));
+      }
+    } else {
       for (int line = threadIdx.x; line < nlines; line += blockDim.x)
-        if (sOk[line])
+        if (sOk[line]) {
+#pragma unroll 4
+          for (int i = 5; i < 5 + len; ++i) put(line, i, Uin[sBase[line] + sPos[i]]);
           for (int h = 0; h < 10; ++h) {
             const int i = h < 5 ? h : len + h;
             put(line, i, value(line, i));
           }
-    } else {
-      for (int line = threadIdx.x; line < nlines; line += blockDim.x)
-        if (sOk[line])
-          for (int i = 0; i < W; ++i) put(line, i, value(line, i));
+        }
     }
   }
   cp_async_commit();
@@ -1033,47 +1089,60 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
   // ---- one line per thread
   const int line = threadIdx.x;
   if (line < nlines && sOk[line]) {
-    double* row = tile + line * TW;
-    const double* cp = f.thomas + (long long)len * 2 * f.Lmax;
-    const double* im = cp + f.Lmax;
     if (!F32) {
-      // FP64: the system as written, alpha f^_{i-1} + f^_i + alpha f^_{i+1} = rhs_i; the forward
-      // sweep parks d_i in slot i (position i - 5, no longer read), back substitution overwrites
-      const double al = f.alpha;
-      double win[11];
+      // FP64 form: the line's largest exponent (the window with its halo), the fixed-point values,
+      // their tenth differences, and the sweeps z_i = g_i - c_{i-1} z_{i-1}, d_i = z_i / m_i -
+      // c_i d_{i+1}, the filter's scale in the 1 / m_i.  The forward sweep parks z_i in slot i
+      // (position i - 5, no longer read); back substitution leaves d_i there.
+      double* row = tile + line * TW;
+      int top = 0;
+#pragma unroll 8
+      for (int i = 0; i < W; ++i) top = max(top, __double2hiint(row[i]) & 0x7fffffff);
+      int ex = top >> 20;
+      // a NaN or an infinity anywhere in the window (or a value of 2^1009 and more) reaches every
+      // point of the line: d = NaN
+      const bool bad = ex >= 0x7f0;
+      // a line of nothing but values below 2^-822 stays as it is: d = 0
+      const bool tiny = ex < 200;
+      ex = max(ex, 200);
+      const int q20 = (ex - 1023 - 52) * (1 << 20);
+      const double* __restrict__ cp = f.thomas_k + (long long)len * 2 * f.Lmax;
+      const double* __restrict__ im = cp + f.Lmax;
+      long long s[10];
+      auto diff10 = [&](int i) {
+        long long t = fixed_point(row[i], ex);
 #pragma unroll
-      for (int m = 0; m < 11; ++m) win[m] = row[m];
-      const double hm1 = row[4], hpl = row[len + 5];
-      double dprev = 0.0;
-      #pragma unroll 4
+        for (int j = 0; j < 10; ++j) {
+          const long long nt = t - s[j];
+          s[j] = t;
+          t = nt;
+        }
+        return t;
+      };
+#pragma unroll
+      for (int j = 0; j < 10; ++j) s[j] = 0;
+#pragma unroll
+      for (int i = 0; i < 10; ++i) diff10(i);
+      double z = 0.0, c = 0.0;
+#pragma unroll 4
       for (int i = 0; i < len; ++i) {
-        double rhs = f.h[0] * win[5];
-#pragma unroll
-        for (int m = 1; m <= 5; ++m) rhs = fma(f.h[m], win[5 + m] + win[5 - m], rhs);
-        if (i == 0) rhs -= al * hm1;
-        if (i == len - 1) rhs -= al * hpl;
-        const double dcur = (i == 0 ? rhs : rhs - al * dprev) * __ldg(im + i);
-        row[i] = dcur;
-        dprev = dcur;
-#pragma unroll
-        for (int m = 0; m < 10; ++m) win[m] = win[m + 1];
-        if (i + 11 < W) win[10] = row[i + 11];
+        z = fma(-c, z, from_fixed_point(diff10(i + 10), q20));
+        row[i] = z;
+        c = __ldg(cp + i);
       }
-      double xnext = dprev;
-      #pragma unroll 4
-      for (int i = len - 2; i >= 0; --i) {
-        const double x = row[i] - __ldg(cp + i) * xnext;
-        row[i] = x;
-        xnext = x;
+      double x = bad ? __longlong_as_double(0x7ff8000000000000LL) : 0.0;
+#pragma unroll 4
+      for (int i = len - 1; i >= 0; --i) {
+        x = fma(-__ldg(cp + i), x, row[i] * __ldg(im + i));
+        row[i] = tiny ? 0.0 : x;
       }
     } else {
-      // FP32 form: solve for the increment d = f^ - f.  Its right side is
-      // (a_1/2 - alpha) D_1 + sum_{n>=2} (a_n/2) D_n with D_n = f_{i+n} + f_{i-n} - 2 f_i (exact
-      // algebra, using sum a_n = 1 + 2 alpha), the Dirichlet closure becomes d = 0 at the first
-      // halo point, and the values enter as the FP32 offsets staged from an FP64 reference of the
-      // line, so FP32 rounding never acts on the full magnitude of the state.  The forward sweep
-      // parks its d_i in slot i (no longer read), back substitution leaves the increment of point
-      // i there; the store adds it to the FP64 value.
+      // FP32 form: the right side is (a_1/2 - alpha) D_1 + sum_{n>=2} (a_n/2) D_n with
+      // D_n = f_{i+n} + f_{i-n} - 2 f_i (exact algebra, using sum a_n = 1 + 2 alpha), and the values
+      // enter as the FP32 offsets staged from an FP64 reference of the line, so FP32 rounding never
+      // acts on the full magnitude of the state.  The forward sweep parks its d_i in slot i (no
+      // longer read), back substitution leaves the increment of point i there; the store adds it
+      // to the FP64 value.
       float* frow = ftile + line * TW;
       const float* cp32 = f.thomas32 + (long long)len * 2 * f.Lmax;  // the factors in FP32
       const float* im32 = cp32 + f.Lmax;
@@ -1110,18 +1179,19 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
   __syncthreads();
 
   // ---- store the own points; no-slip wall points keep zero momentum
-  const bool wz = f.wall && var >= 1 && var <= 3;
+  const bool wz = B.wall && var >= 1 && var <= 3;
   auto wall_pt = [&](int ln, int i) {
     const int u = off + i, a1 = sT1[ln], a2 = sT2[ln];
-    return (((f.wall >> (2 * axis)) & 1) && u == 0) || (((f.wall >> (2 * axis + 1)) & 1) && u == n[axis] - 1) ||
-           (((f.wall >> (2 * f1)) & 1) && a1 == 0) || (((f.wall >> (2 * f1 + 1)) & 1) && a1 == n[f1] - 1) ||
-           (((f.wall >> (2 * f2)) & 1) && a2 == 0) || (((f.wall >> (2 * f2 + 1)) & 1) && a2 == n[f2] - 1);
+    return (((B.wall >> (2 * axis)) & 1) && u == 0) || (((B.wall >> (2 * axis + 1)) & 1) && u == n[axis] - 1) ||
+           (((B.wall >> (2 * f1)) & 1) && a1 == 0) || (((B.wall >> (2 * f1 + 1)) & 1) && a1 == n[f1] - 1) ||
+           (((B.wall >> (2 * f2)) & 1) && a2 == 0) || (((B.wall >> (2 * f2 + 1)) & 1) && a2 == n[f2] - 1);
   };
-  // the filtered value of point i: slot i (FP64), or the FP64 value plus the FP32 increment
+  // the filtered value of point i: the FP64 value plus the increment of slot i
   auto result = [&](int ln, int i, long long gi) -> double {
     if (wz && wall_pt(ln, i)) return 0.0;
-    if (F32) return Uin[gi] + f2d_fast(ftile[ln * TW + i]);
-    return tile[ln * TW + i];
+    const double u = Uin[gi];
+    if (F32) return u + f2d_fast(ftile[ln * TW + i]);
+    return u + tile[ln * TW + i];
   };
   if (axis == 0) {
     for (int ln = warp; ln < nlines; ln += nwarp)
@@ -1132,11 +1202,13 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
         }
   } else {
     for (int ln = threadIdx.x; ln < nlines; ln += blockDim.x)
-      if (sOk[ln])
+      if (sOk[ln]) {
+#pragma unroll 4
         for (int i = 0; i < len; ++i) {
           const long long gi = sBase[ln] + sPos[i + 5];
           Uout[gi] = result(ln, i, gi);
         }
+      }
   }
 }
 
@@ -1154,7 +1226,9 @@ int launch_round_table(const double* x, float* y, long long n, void* stream) {
 // context of the process: it only ever rises (to the largest size a context on the device has
 // needed), so a context with shorter lines cannot lower it under another one still stepping.
 int filter_prepare(int Lmax, int precision) {
-  const size_t sm = filter_smem_bytes(Lmax, precision);
+  // (not monotonic in the line length: longer lines take fewer lines per CTA)
+  size_t sm = 0;
+  for (int L = 1; L <= Lmax; ++L) sm = std::max(sm, filter_smem_bytes(L, precision));
   if (sm > 227 * 1024) return (int)cudaErrorInvalidValue;
   static std::mutex mu;
   static int set_to[64][2] = {};
@@ -1179,14 +1253,17 @@ int filter_prepare(int Lmax, int precision) {
   return (int)e;
 }
 
-int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f, int axis, int precision,
-                  void* stream, long long* launches, const Timer* tm) {
-  const int n[3] = {f.nx, f.ny, f.nz};
+unsigned filter_ctas(const int* n, const int* P, int axis, int Lt) {
   const int f1 = (axis == 0) ? 1 : 0;
   const int f2 = (axis == 2) ? 1 : 2;
-  const FilterTile tl = filter_tile(f.Lt);
+  const FilterTile tl = filter_tile(Lt);
   const long long nl = (long long)n[f1] * n[f2];
-  const unsigned nb = (unsigned)(5LL * f.P[axis] * ((nl + tl.LN - 1) / tl.LN));
+  return (unsigned)(5LL * P[axis] * ((nl + tl.LN - 1) / tl.LN));
+}
+
+int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f, int axis, int precision,
+                  void* stream, long long* launches, const Timer* tm) {
+  const unsigned nb = f.ctas;
   const size_t sm = filter_smem_bytes(f.Lt, precision);
   cudaStream_t st = (cudaStream_t)stream;
   if (tm) tm->rec(tm->self, 3, 1);
