@@ -121,6 +121,12 @@ struct cfs_ctx {
   int* d_work = nullptr;
   float* Wh = nullptr;
 
+  // FP64 form on pairs of floats (3-D Navier-Stokes)
+  bool pairs = false;
+  cfs::PairPhysics pphys{};
+  void* d_hpair = nullptr;       // AT halo states of every stage, [2 s][nhalo] float4 then [s][nhalo] float2
+  float2* d_metric_p = nullptr;  // metric planes as pairs
+
   Geometry geo{};
   Physics phys{};
 
@@ -237,6 +243,11 @@ static void dev_free(cfs_ctx* c, void* p) {
       c->freef(p, c->user);
       return;
     }
+}
+
+static float2 pair_of(long double x) {
+  const float hi = (float)x;
+  return float2{hi, (float)(x - (long double)hi)};
 }
 
 static void split_axis(int n, int p, int idx, int* off, int* len) {
@@ -513,7 +524,9 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
             const double h = b.mbase >= 0 ? 1.0 : b.h[a];  // curvilinear: index space
             d.c1[a] = (a_cd / 2.0) / h;
             d.c2[a] = (b_cd / 4.0) / h;
+            d.cg[a] = pair_of(c->p.order == 4 ? d.c2[a] : d.c1[a]);
           }
+          d.iso = d.c1[0] == d.c1[1] && d.c1[0] == d.c1[2] && d.c2[0] == d.c2[1] && d.c2[0] == d.c2[2];
           const long long npad = (long long)d.ex * d.ey * d.ez;
           pbase += npad;
           const long long nown = (long long)d.sx * d.sy * d.sz;
@@ -564,10 +577,34 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     ph.c1[a] = (a_cd / 2.0) / b0.h[a];
     ph.c2[a] = (b_cd / 4.0) / b0.h[a];
   }
+  // The FP64 form of 3-D Navier-Stokes runs its right-hand side on pairs of floats (stage_pairs.cu)
+  // when its constants, and with them a flow's nondimensional values (p about 1/(gamma M^2), rho and
+  // u about 1), lie well inside the FP32 range; the FP64 kernels take what is left, 2-D and
+  // inviscid runs (whose few operations per point leave the FP64 pipe less to do) and the compact
+  // scheme.  Runs without the filter keep the FP64 kernels too: there a step's error against 64-bit
+  // arithmetic is the 5e-17 of the final rounding, which the pairs would raise to 2e-16 at CFL 0.5.
+  c->pairs = c->p.precision == 0 && c->ndim == 3 && c->p.viscous && c->p.filter && !c->p.compact;
+  {
+    auto in_range = [](double x) { const double a = std::fabs(x); return a == 0.0 || (a > 1e-12 && a < 1e12); };
+    c->pairs = c->pairs && in_range(ph.p_ref) && in_range(ph.kappa) && in_range(ph.kgM2) && in_range(ph.ire) && in_range(ph.ivT);
+    for (const SubDev& d : c->subs)
+      for (int a = 0; a < 3; ++a) c->pairs = c->pairs && in_range(d.c1[a]) && in_range(d.c2[a]);
+    cfs::PairPhysics& pp = c->pphys;
+    pp.Eref = (float)ph.E_ref;
+    pp.gm1 = pair_of(ph.gm1);
+    pp.kgM2 = pair_of(ph.kgM2);
+    pp.kT0 = pair_of((long double)ph.kgM2 * ph.gm1 * pp.Eref);
+    pp.H = pair_of((long double)ph.gamma * pp.Eref);
+    pp.ivT = pair_of(ph.ivT);
+    pp.visc_law = ph.visc_law;
+    pp.visc_exp = ph.visc_exp;
+  }
   // tables of the FP64 power (power-law viscosity)
   if (c->p.viscous && c->p.visc_law == 1) {
     const int rc = cfs::pow_tables_init();
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "power tables");
+    c->pphys.powtab = cfs::pow_table_address();
+    if (!c->pphys.powtab) return fail(c, CFS_ECUDA, "power tables");
   }
   // device memory
   c->ring = (double*)dev_alloc(c, sizeof(double) * 5 * N * c->R);
@@ -584,7 +621,12 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   if (curv) {
     c->d_metric = (double*)dev_alloc(c, sizeof(double) * mtot);
     if (!c->d_metric) return fail(c, CFS_ENOMEM, "device allocation failed");
+    if (c->pairs) {
+      c->d_metric_p = (float2*)dev_alloc(c, sizeof(float2) * mtot);
+      if (!c->d_metric_p) return fail(c, CFS_ENOMEM, "device allocation failed");
+    }
     std::vector<double> M;
+    std::vector<float2> Mp;
     for (size_t bi = 0; bi < c->blocks.size(); ++bi) {
       const Block& b = c->blocks[bi];
       if (b.mbase < 0) continue;
@@ -599,9 +641,16 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       c->volume += vb * b.nz;
       CUDA_TRY(c, cudaMemcpy(c->d_metric + b.mbase, M.data(), sizeof(double) * M.size(), cudaMemcpyHostToDevice),
                "upload metrics");
+      if (c->pairs) {
+        Mp.resize(M.size());
+        for (size_t q = 0; q < M.size(); ++q) Mp[q] = pair_of(M[q]);
+        CUDA_TRY(c, cudaMemcpy(c->d_metric_p + b.mbase, Mp.data(), sizeof(float2) * Mp.size(), cudaMemcpyHostToDevice),
+                 "upload metrics");
+      }
     }
   }
   g.metric = c->d_metric;
+  g.metric_p = c->d_metric_p;
   // gather maps: every point of a non-periodic block's (x, y) range extended by `need` (faces to
   // that depth, corners to r x r), all z; entries for the points outside the block
   g.GE = need;
@@ -781,6 +830,10 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       if (!c->d_halo) return fail(c, CFS_ENOMEM, "device allocation failed");
       CUDA_TRY(c, cudaMemcpy(c->d_halo, hl.data(), sizeof(int) * hl.size(), cudaMemcpyHostToDevice), "upload halo list");
     }
+  }
+  if (c->pairs && c->nhalo > 0) {
+    c->d_hpair = dev_alloc(c, (2 * sizeof(float4) + sizeof(float2)) * (size_t)c->s * (size_t)c->nhalo);
+    if (!c->d_hpair) return fail(c, CFS_ENOMEM, "device allocation failed");
   }
   // exchange plan of a partitioned context: state offsets and block sizes of the strips sent to /
   // received from every peer, and the packed buffers (5 values per point)
@@ -1128,6 +1181,11 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
                                           &c->launches, tm);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
   }
+  if (c->pairs && (graph || sc.mode != 0)) {
+    const int rc = cfs::launch_at_halo(g, c->pphys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->d_hpair, c->s, c->stream,
+                                       &c->launches, tm);
+    if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
+  }
   for (int op = 0; op < nops; ++op) {
     const bool last_op = op == nops - 1;
     double* dst = last_op ? (graph ? nullptr : level_ptr(c, n + 1)) : c->buf[pp];
@@ -1158,7 +1216,8 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       a.max_pad = c->max_pad; a.max_own = c->max_own; a.max_flux = c->max_flux;
       a.halo = c->d_halo; a.nhalo = c->nhalo;
       a.compact = c->p.compact; a.R = c->Rbuf; a.cthomas = c->d_cthomas; a.Lmax = c->Lmax;
-      rc = cfs::launch_stage(g, c->phys, sc, a, c->p.precision, c->stream, &c->launches, tm);
+      rc = c->pairs ? cfs::launch_stage_pairs(g, c->pphys, sc, a, c->d_hpair, c->stream, &c->launches, tm)
+                    : cfs::launch_stage(g, c->phys, sc, a, c->p.precision, c->stream, &c->launches, tm);
     } else if (op == c->s && c->fblock_n && !graph && sc.mode != 0) {
       // asynchronous step, FP32 form: the three passes in one launch, straight into level n + 1
       rc = launch_fblock(c, g, sc, src, level_ptr(c, n + 1), false);

@@ -2,6 +2,8 @@
 // the CUDA translation units of libcfs.  Not part of the public C ABI (include/cfs.h).
 #pragma once
 
+#include <vector_types.h>
+
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -42,6 +44,10 @@ struct SubDev {
   long long bN;       // block points
   long long bbase;    // offset of the block's state [5][bnz][bny][bnx] in a state array (doubles)
   double c1[3], c2[3];  // CD coefficients of the block's spacing: c1 = (a/2)/h, c2 = (b/4)/h
+  // FP64 form on pairs of floats: the coefficient of its unscaled differences (c2 for CD4, c1 for
+  // CD2) per axis as a pair (hi, lo), and whether the three are equal
+  float2 cg[3];
+  int iso;
   // curvilinear block: offset of its metric plane in Geometry::metric, -1 for a uniform Cartesian
   // block (c1, c2 are then the index-space coefficients, h = 1).  The plane covers the block's
   // (x, y) points extended by G on every side, row length mx, component stride mpl; it is the
@@ -92,6 +98,7 @@ struct Geometry {
   // metric planes of the curvilinear blocks, [NMETRIC][mpl] per block (device), or null:
   // xi^_x, xi^_y, eta^_x, eta^_y, zeta^_z (= J^-1 d(xi,eta,zeta)/dx of App. A), J^-1, J
   const double* metric;
+  const float2* metric_p;  // the same planes as pairs of floats (FP64 form on pairs), or null
   // gather maps and entries of the blocks with non-periodic faces (device), or null
   const int* emap;
   const GatherEntry* gent;
@@ -115,6 +122,17 @@ struct Physics {
   // and H_ref = E_ref + p_ref; primitives carry p - p_ref and rho E - E_ref so that FP32 rounding
   // acts on O(1) deviations instead of p ~ 1/(gamma M^2)
   double p_ref, E_ref, H_ref;
+};
+
+// Constants of the FP64 form on pairs of floats (stage_pairs.cu), each a pair (hi, lo).  Pressure and
+// total energy are deviations from E_ref (p_ref / (gamma - 1) rounded to FP32) and p_ref =
+// (gamma - 1) E_ref: kT = (kgM2 p' + kT0) / rho with kT0 = kgM2 p_ref, H = E_ref + p_ref.
+struct PairPhysics {
+  float2 gm1, kgM2, kT0, H, ivT;
+  float Eref;
+  int visc_law;
+  double visc_exp;
+  const double* powtab;    // device: tables of the FP64 power
 };
 
 // Delay schedule as seen by the kernels of one step.
@@ -218,6 +236,13 @@ struct Timer {
 
 int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a,
                  int precision, void* stream, long long* launches, const Timer* tm);
+
+// The stage of the FP64 form for 3-D Navier-Stokes on pairs of floats (stage_pairs.cu), and the AT
+// halo states of all s stages once per asynchronous step: H [2 s][nhalo] float4, [s][nhalo] float2.
+int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const StageLaunch& a, const void* H,
+                       void* stream, long long* launches, const Timer* tm);
+int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
+                   const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm);
 
 // One block as the line filter sees it (device table, one entry per block of a launch).
 struct FilterBlk {
@@ -378,6 +403,7 @@ struct StripPlan {
 };
 const char* strip_plan(const TopoBlock* B, int nb, int nsub, const int* starts, int nranks, int rank, int depth,
                        int depth_z, int r, bool viscous, int ndim, StripPlan* out);
+const double* pow_table_address();  // its device address on the current device, or null
 int pow_tables_init();  // tables of the FP64 power on the current device, once per device; nonzero on a CUDA error
 
 }  // namespace cfs

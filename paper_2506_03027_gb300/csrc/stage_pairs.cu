@@ -1,0 +1,566 @@
+// stage_pairs.cu -- the Runge-Kutta stage of the FP64 form for 3-D Navier-Stokes: FP64 state, FP64
+// low-storage update, and the right-hand side between them on pairs of floats (pairs.cuh).
+//
+// In FP64 the stage is bound by the FP64 pipe: about 215 FP64 operations per point and stage at 2
+// per clock and SM, while the FP32 pipe (64 times as fast) and memory idle.  dt R is a small
+// correction of the state (the time step keeps it below about 1e-2 of it), so a right-hand side that
+// is good to a few 2^-48 leaves the error of U + B Q where it was, at the FP64 rounding of the sum.
+// Pressure and total energy are carried as deviations from the reference state (p_ref =
+// 1/(gamma M^2) is 70 times the dynamic pressure at M = 0.1), which makes the pressure gradient
+// more accurate than the FP64 sums over the full pressure were.
+//
+// The kernels are those of kernels.cu (view, flux, update) with pairs in the scratch arrays, two
+// values interleaved where the same operation acts on both, so that one 16-byte load and the
+// packed FP32 instructions serve (u, v) and (w, kappa T) together:
+//   W    A (u, v), B (w, kappa T), C (rho, p - p_ref): float4 {h, h, l, l}; D (rho E + p - H_ref): float2
+//   Phi  per direction a: M (x, y momentum), E (z momentum, energy): float4; N (mass): float2
+// and one more, once per asynchronous step: k_at_halo forms the AT halo values of all stages from
+// one read of the delayed levels (they would be read once per stage otherwise).
+#include <cuda_runtime.h>
+
+#include "cfs_internal.h"
+#include "device_common.cuh"
+#include "launch_common.cuh"
+#include "pairs.cuh"
+
+namespace cfs {
+
+namespace {
+
+struct WView {
+  float4 *A, *B, *C;
+  float2* D;
+};
+__device__ __forceinline__ WView w_view(void* W, long long P) {
+  float4* a = (float4*)W;
+  return {a, a + P, a + 2 * P, (float2*)(a + 3 * P)};
+}
+
+__device__ __forceinline__ P1 cst(float2 c) { return {c.x, c.y}; }
+
+// Primitives of the conserved state at scratch index o: u = (rho, rho u, rho v, rho w, rho E - E_ref).
+__device__ __forceinline__ void store_prims_p(const PairPhysics& ph, const WView& W, long long o, P1 rho, P2 mxy, P1 mz,
+                                              P1 rE) {
+  const P1 ir = p_recip(rho);
+  const P2 uv = p_norm(p_mul(mxy, p_bc(ir)));
+  const P1 w = p_norm(p_mul(mz, ir));
+  const P2 k2 = p_mul(mxy, uv);
+  const P1 ke = p_scale(p_fma(mz, w, p_add(p_x(k2), p_y(k2))), 0.5f);
+  const P1 p = p_norm(p_mul(cst(ph.gm1), p_norm(p_sub(rE, ke))));
+  const P1 kT = p_norm(p_mul(p_norm(p_fma(cst(ph.kgM2), p, cst(ph.kT0))), ir));
+  W.A[o] = p_store(uv);
+  W.B[o] = p_store(p_pair(w, kT));
+  W.C[o] = p_store(p_pair(rho, p));
+  W.D[o] = p_store(p_norm(p_add(rE, p)));
+}
+
+__device__ __forceinline__ void store_state_p(const PairPhysics& ph, const WView& W, long long o, const double* u) {
+  store_prims_p(ph, W, o, p_split(u[0]), p_pair(p_split(u[1]), p_split(u[2])), p_split(u[3]),
+                p_norm(p_add(p_split(u[4]), P1{-ph.Eref, 0.f})));
+}
+
+// Delay of a halo point: the largest of the faces it lies beyond; faces on a physical boundary of
+// the block carry none for points beyond the block.
+__device__ __forceinline__ int point_delay(const StepSched& sc, const SubDev& d, int sid, int ci, int cj, int ck, bool beyond) {
+  int kd = 0;
+  if ((ci < 0 || ci >= d.sx) && !(beyond && ((d.phys >> (ci < 0 ? 0 : 1)) & 1))) kd = max(kd, face_delay(sc, sid, ci < 0 ? 0 : 1));
+  if ((cj < 0 || cj >= d.sy) && !(beyond && ((d.phys >> (cj < 0 ? 2 : 3)) & 1))) kd = max(kd, face_delay(sc, sid, cj < 0 ? 2 : 3));
+  if ((ck < 0 || ck >= d.sz) && !(beyond && ((d.phys >> (ck < 0 ? 4 : 5)) & 1))) kd = max(kd, face_delay(sc, sid, ck < 0 ? 4 : 5));
+  return kd;
+}
+
+struct HaloPoint {
+  int sid, q, ci, cj, ck;
+  long long gi;   // state offset of the wrapped point
+  bool beyond;    // beyond a non-periodic block face: ent is its gather entry
+  const GatherEntry* ent;
+};
+
+__device__ __forceinline__ HaloPoint halo_point(const Geometry& g, const SubDev& d, int2 e) {
+  HaloPoint h;
+  h.sid = e.x;
+  h.q = e.y;
+  const int exy = d.ex * d.ey;
+  const int k = h.q / exy, r2 = h.q - k * exy, j = r2 / d.ex, i = r2 - j * d.ex;
+  h.ci = i - g.G;
+  h.cj = j - g.G;
+  h.ck = k - g.Gz;
+  auto wrap1 = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+  const int ux = d.ox + h.ci, uy = d.oy + h.cj;
+  const int gx = wrap1(ux, d.bnx), gy = wrap1(uy, d.bny), gz = wrap1(d.oz + h.ck, d.bnz);
+  h.gi = d.bbase + (long long)gx + (long long)d.bnx * ((long long)gy + (long long)d.bny * gz);
+  h.beyond = d.ebase >= 0 && (ux < 0 || ux >= d.bnx || uy < 0 || uy >= d.bny);
+  h.ent = nullptr;
+  if (h.beyond) h.ent = &g.gent[g.emap[d.ebase + (ux + g.GE) + (long long)d.gmx * ((uy + g.GE) + (long long)d.gmy * gz)]];
+  return h;
+}
+
+// Whether source t of the entry is the sub-domain's own current value (a wall mirror or an outflow
+// copy, for points inside the sub-domain in z; beyond a z face the source is a neighbouring PE's)
+__device__ __forceinline__ bool own_source(const HaloPoint& h, const SubDev& d, int t) {
+  return h.ck >= 0 && h.ck < d.sz && !(h.ent->flags[t] & 2) && h.ent->sid[t] == h.sid;
+}
+__device__ __forceinline__ bool any_own_source(const HaloPoint& h, const SubDev& d) {
+  bool own = false;
+  for (int t = 0; t < h.ent->nt; ++t) own = own || own_source(h, d, t);
+  return own;
+}
+
+// The value of a gather entry at stage `stage`: own sources from the stage input, a neighbouring
+// PE's by the mode (live, latest delayed level, or the AT weights), far-field constants; FP64.
+__device__ __forceinline__ void gather_value(const Geometry& g, const StepSched& sc, const HaloPoint& h, const SubDev& d, int kd,
+                                             const double* __restrict__ Uin, const double* __restrict__ ring, int stage,
+                                             int s, double* u) {
+  const GatherEntry& E = *h.ent;
+  const int nR = (int)(sc.n % sc.R);
+  const long long lvN = 5 * g.N;
+  auto slot = [&](int l) { const int q = nR - kd - l; return (long long)(q < 0 ? q + sc.R : q) * lvN; };
+#pragma unroll
+  for (int v = 0; v < 5; ++v) u[v] = E.cst[v];
+  for (int t = 0; t < E.nt; ++t) {
+    const double wt = E.w[t], wf = (E.flags[t] & 1) ? -wt : wt;
+    const long long o = E.off[t], bN = E.bN[t];
+    double x[5];
+    if (sc.mode == 0 || (Uin && own_source(h, d, t))) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) x[v] = Uin[o + v * bN];
+    } else if (sc.mode == 2) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) x[v] = ring[slot(0) + o + v * bN];
+    } else {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) x[v] = 0.0;
+      for (int l = 0; l < sc.C; ++l) {
+        const double wl = __ldg(sc.W + (kd * s + stage) * sc.C + l);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) x[v] = fma(wl, ring[slot(l) + o + v * bN], x[v]);
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) u[v] = fma((v >= 1 && v <= 3) ? wf : wt, x[v], u[v]);
+  }
+}
+
+}  // namespace
+
+// ------------------------------------------------------------------------------- k_at_halo
+
+// Once per asynchronous step: for every entry of the halo list the conserved state of all S stages,
+// U^(m) = sum_l W^(m)_l(k) U^{n-k-l} (Eq. 14-15 and the buffer updates of Eq. 8 collapsed into
+// weights), as U_0 + (S_m - 1) U_0 + sum_{l>=1} W^(m)_l (U_l - U_0) with U_l = U^{n-k-l} and S_m the
+// sum of the weights: the levels differ by a step's change, so the products of pairs keep the sum
+// at the accuracy of the FP64 one.  With the learned halo, face points start from the network's
+// stage-0 value and add the sums with W^(m) - W^(0).  Stored [stage][entry]: (rho, rho u), (rho v,
+// rho w) and rho E - E_ref.  Bound by its reads: C x 40 bytes per entry at the sub-domains' faces.
+template <int S>
+__global__ void __launch_bounds__(256) k_at_halo(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ ring,
+                                                 const SubDev* __restrict__ subs, const int2* __restrict__ halo,
+                                                 long long nhalo, float4* __restrict__ H4, float2* __restrict__ H2) {
+  pdl_enter();
+  sc = resolve(sc);
+  if (sc.mode == 0) return;
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nhalo) return;
+  const int2 hv = halo[e];
+  const SubDev d = subs[hv.x];
+  const HaloPoint h = halo_point(g, d, hv);
+  const int kd = point_delay(sc, d, h.sid, h.ci, h.cj, h.ck, h.beyond);
+  auto put = [&](int m, P2 a, P2 b, P1 c) {
+    H4[(long long)(2 * m) * nhalo + e] = p_store(a);
+    H4[(long long)(2 * m + 1) * nhalo + e] = p_store(b);
+    H2[(long long)m * nhalo + e] = p_store(c);
+  };
+  auto put64 = [&](int m, const double* u) {
+    put(m, p_pair(p_split(u[0]), p_split(u[1])), p_pair(p_split(u[2]), p_split(u[3])),
+        p_norm(p_add(p_split(u[4]), P1{-ph.Eref, 0.f})));
+  };
+  if (h.beyond) {
+    // (entries with an own source are formed from the live stage input by k_view_p)
+    if (any_own_source(h, d)) return;
+    for (int m = 0; m < (sc.mode == 2 ? 1 : S); ++m) {
+      double u[5];
+      gather_value(g, sc, h, d, kd, nullptr, ring, m, S, u);
+      put64(m, u);
+    }
+    return;
+  }
+  const long long lvN = 5 * g.N;
+  const int nR = (int)(sc.n % sc.R);
+  auto slot = [&](int l) { const int q = nR - kd - l; return (long long)(q < 0 ? q + sc.R : q) * lvN; };
+  const int C = sc.mode == 2 ? 1 : sc.C;
+  double r[CFS_MAX_LEVELS][5];
+#pragma unroll
+  for (int l = 0; l < CFS_MAX_LEVELS; ++l)
+    if (l < C) {
+      const double* src = ring + slot(l) + h.gi;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) r[l][v] = src[v * d.bN];
+    }
+  if (sc.mode == 2) {  // AS: the latest visible level, the same for every stage
+    put64(0, r[0]);
+    return;
+  }
+  const bool learned = sc.LH && ((int)(h.ci < 0 || h.ci >= d.sx) + (int)(h.cj < 0 || h.cj >= d.sy) + (int)(h.ck < 0 || h.ck >= d.sz) == 1);
+  auto split5 = [&](const double* u, P2& a, P2& b, P1& c) {
+    a = p_pair(p_split(u[0]), p_split(u[1]));
+    b = p_pair(p_split(u[2]), p_split(u[3]));
+    c = p_split(u[4]);
+  };
+  P2 a0, b0, aa[S], ab[S];
+  P1 c0, ac[S];
+  split5(r[0], a0, b0, c0);
+  const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * C;
+  {
+    // what the sums are added to: U_0, or the network's stage-0 value
+    P2 sa = a0, sb = b0;
+    P1 se = c0;
+    if (learned) {
+      double u[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) u[v] = sc.LH[(long long)v * g.Ptot + d.pbase + h.q];
+      split5(u, sa, sb, se);
+    }
+    se = p_norm(p_add(se, P1{-ph.Eref, 0.f}));
+#pragma unroll
+    for (int m = 0; m < S; ++m) {
+      // (with the network, stage 0 is its value: the weights W^(0) - W^(0) are zero)
+      const float2 cm = __ldg(wt + m * C);
+      const P1 c = {cm.x, cm.y};
+      aa[m] = p_fma(p_bc(c), a0, sa);
+      ab[m] = p_fma(p_bc(c), b0, sb);
+      ac[m] = p_fma(c, c0, se);
+    }
+  }
+#pragma unroll
+  for (int l = 1; l < CFS_MAX_LEVELS; ++l)
+    if (l < C) {
+      P2 a, b;
+      P1 c;
+      split5(r[l], a, b, c);
+      a = p_norm(p_sub(a, a0));
+      b = p_norm(p_sub(b, b0));
+      c = p_norm(p_sub(c, c0));
+#pragma unroll
+      for (int m = 0; m < S; ++m) {
+        const float2 wm = __ldg(wt + m * C + l);
+        const P1 w = {wm.x, wm.y};
+        aa[m] = p_fma(p_bc(w), a, aa[m]);
+        ab[m] = p_fma(p_bc(w), b, ab[m]);
+        ac[m] = p_fma(w, c, ac[m]);
+      }
+    }
+#pragma unroll
+  for (int m = 0; m < S; ++m) put(m, p_norm(aa[m]), p_norm(ab[m]), p_norm(ac[m]));
+}
+
+// ------------------------------------------------------------------------------- k_view_p
+
+// The stage input as primitives, own points and halo points in one launch (as k_view).
+__global__ void __launch_bounds__(512) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
+                                                const double* __restrict__ ring, int in_ring, const SubDev* __restrict__ subs,
+                                                const int2* __restrict__ halo, long long nhalo, const float4* __restrict__ H4,
+                                                const float2* __restrict__ H2, void* Wp, int stage, int s, int own_blocks) {
+  pdl_enter();
+  sc = resolve(sc);
+  const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
+  const WView W = w_view(Wp, g.Ptot);
+  const long long b = blockIdx.x, nown = (long long)own_blocks * g.nsub;
+  if (b < nown) {
+    const int sid = (int)(b / own_blocks);
+    const SubDev& d = subs[sid];
+    if (!d.own) return;  // another process's sub-domain
+    const int t = (int)(b - (long long)sid * own_blocks) * blockDim.x + threadIdx.x;
+    if (t >= d.sx * d.sy * d.sz) return;
+    const int sxy = d.sx * d.sy, ck = t / sxy, r2 = t - ck * sxy, cj = r2 / d.sx, ci = r2 - cj * d.sx;
+    const long long gi = (long long)(d.ox + ci) + (long long)d.bnx * ((long long)(d.oy + cj) + (long long)d.bny * (d.oz + ck));
+    const long long q = (long long)(ci + g.G) + (long long)d.ex * ((long long)(cj + g.G) + (long long)d.ey * (ck + g.Gz));
+    double u[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) u[v] = Uin[d.bbase + v * d.bN + gi];
+    store_state_p(ph, W, d.pbase + q, u);
+    return;
+  }
+  const long long e = (b - nown) * blockDim.x + threadIdx.x;
+  if (e >= nhalo) return;
+  const int2 hv = halo[e];
+  const SubDev& d = subs[hv.x];
+  const long long o = d.pbase + hv.y;
+  if (sc.mode == 0 || d.ebase >= 0) {
+    const HaloPoint h = halo_point(g, d, hv);
+    if (sc.mode == 0 || (h.beyond && any_own_source(h, d))) {
+      double u[5];
+      if (h.beyond) {
+        const int kd = sc.mode == 0 ? 0 : point_delay(sc, d, h.sid, h.ci, h.cj, h.ck, true);
+        gather_value(g, sc, h, d, kd, Uin, ring, stage, s, u);
+      } else {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) u[v] = Uin[v * d.bN + h.gi];
+      }
+      store_state_p(ph, W, o, u);
+      return;
+    }
+  }
+  const int m = sc.mode == 2 ? 0 : stage;
+  const P2 a = p_of(H4[(long long)(2 * m) * nhalo + e]), c = p_of(H4[(long long)(2 * m + 1) * nhalo + e]);
+  store_prims_p(ph, W, o, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e]));
+}
+
+// ------------------------------------------------------------------------------- k_flux_p
+
+namespace {
+
+// Central difference without its factor (times c2 for CD4, c1 for CD2), of two values
+template <int R>
+__device__ __forceinline__ P2 diff2(const float4* __restrict__ f, long long q, long long st) {
+  const P2 c = p_of(f[q + st]), d = p_of(f[q - st]);
+  if (R == 1) return p_norm(p_sub(c, d));
+  const P2 a = p_of(f[q + 2 * st]), b = p_of(f[q - 2 * st]);
+  const float2 m8 = make_float2(-8.f, -8.f);
+  const P2 x = p_2diff(a.h, b.h), y = p_2diff(c.h, d.h);
+  const P2 s = p_2sum(x.h, v_mul(m8, y.h));
+  const float2 lo = v_add(v_fma(m8, y.l, x.l), v_fma(m8, v_sub(c.l, d.l), v_sub(a.l, b.l)));
+  return p_norm(P2{s.h, v_add(s.l, lo)});
+}
+template <int R>
+__device__ __forceinline__ P1 diff1(const float2* __restrict__ f, long long q, long long st) {
+  const P1 c = p_of(f[q + st]), d = p_of(f[q - st]);
+  if (R == 1) return p_norm(p_sub(c, d));
+  const P1 a = p_of(f[q + 2 * st]), b = p_of(f[q - 2 * st]);
+  const P1 x = p_2diff(a.h, b.h), y = p_2diff(c.h, d.h);
+  const P1 s = p_2sum(x.h, v_mul(-8.f, y.h));
+  const float lo = v_add(v_fma(-8.f, y.l, x.l), v_fma(-8.f, v_sub(c.l, d.l), v_sub(a.l, b.l)));
+  return p_norm(P1{s.h, v_add(s.l, lo)});
+}
+
+}  // namespace
+
+// Combined fluxes at the owned points and the strips of r points beyond each face (the flux along
+// that face's axis only), thread by thread as in k_flux.  CURV: the context has curvilinear
+// blocks.  R: stencil radius (CD4: 2).
+template <int R, bool CURV>
+__global__ void __launch_bounds__(256) k_flux_p(Geometry g, PairPhysics ph, const SubDev* __restrict__ subs,
+                                                const void* __restrict__ Wp, void* __restrict__ Phi) {
+  pdl_enter();
+  const int sid = blockIdx.y;
+  const SubDev& d = subs[sid];
+  if (!d.own) return;  // another process's sub-domain
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int ci, cj, ck, kind;
+  if (!flux_point<3>(d, R, t, ci, cj, ck, kind)) return;
+  const int as = kind - 1;  // strip axis (-1: owned point, every axis)
+  const long long P = g.Ptot;
+  const long long st[3] = {1, d.ex, (long long)d.ex * d.ey};
+  const long long q = d.pbase + (long long)(ci + g.G) + st[1] * (cj + g.G) + st[2] * (ck + g.Gz);
+  const float4* __restrict__ A = (const float4*)Wp;
+  const float4* __restrict__ B = A + P;
+  const float4* __restrict__ Cc = A + 2 * P;
+  const float2* __restrict__ D = (const float2*)(A + 3 * P);
+  float4* __restrict__ F4 = (float4*)Phi;
+  float2* __restrict__ F2 = (float2*)(F4 + 6 * P);
+
+  const P2 uv = p_of(A[q]), wT = p_of(B[q]), rp = p_of(Cc[q]);
+  const P1 w = p_x(wT), rho = p_x(rp), pr = p_y(rp);
+  const P1 netH = p_neg(p_norm(p_add(p_of(D[q]), cst(ph.H))));  // -(rho E + p)
+  P1 iv = cst(ph.ivT);  // the factor of the viscous terms: 1/Re x (units of the differences) x mu
+  // differences of (u, v) and (w, kappa T) along each axis
+  P2 Gx = diff2<R>(A, q, st[0]), Gy = diff2<R>(A, q, st[1]), Gz = diff2<R>(A, q, st[2]);
+  P2 Hz = diff2<R>(B, q, st[2]);
+  P2 Hx = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, Hy = Hx;
+  if (as != 1) Hx = diff2<R>(B, q, st[0]);
+  if (as != 0) Hy = diff2<R>(B, q, st[1]);
+  const bool curv = CURV && d.mbase >= 0;
+  P2 xi = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, et = xi;  // metric rows (xi_x, xi_y), (eta_x, eta_y)
+  P1 zz = {0.f, 0.f};
+  if (curv) {
+    // index-space differences to physical gradients / J: x: xi_x, eta_x; y: xi_y, eta_y; z: zeta_z
+    const float2* M = g.metric_p + d.mbase + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
+    const long long pl = d.mpl;
+    xi = p_pair(p_of(M[0]), p_of(M[pl]));
+    et = p_pair(p_of(M[2 * pl]), p_of(M[3 * pl]));
+    zz = p_of(M[4 * pl]);
+    if (as == 1) Hx = diff2<R>(B, q, st[0]);  // (the rows mix the two in-plane differences)
+    if (as == 0) Hy = diff2<R>(B, q, st[1]);
+    const P2 g0 = Gx, h0 = Hx;
+    Gx = p_norm(p_fma(p_bc(p_x(et)), Gy, p_mul(p_bc(p_x(xi)), g0)));
+    Hx = p_norm(p_fma(p_bc(p_x(et)), Hy, p_mul(p_bc(p_x(xi)), h0)));
+    Gy = p_norm(p_fma(p_bc(p_y(et)), Gy, p_mul(p_bc(p_y(xi)), g0)));
+    Hy = p_norm(p_fma(p_bc(p_y(et)), Hy, p_mul(p_bc(p_y(xi)), h0)));
+    Gz = p_norm(p_mul(p_bc(zz), Gz));
+    Hz = p_norm(p_mul(p_bc(zz), Hz));
+    iv = p_norm(p_mul(iv, p_norm(p_mul(cst(d.cg[0]), p_of(M[6 * pl])))));
+  } else if (d.iso) {
+    iv = p_norm(p_mul(iv, cst(d.cg[0])));
+  } else {
+    const P2 kx = p_bc(cst(d.cg[0])), ky = p_bc(cst(d.cg[1])), kz = p_bc(cst(d.cg[2]));
+    Gx = p_norm(p_mul(kx, Gx));
+    Hx = p_norm(p_mul(kx, Hx));
+    Gy = p_norm(p_mul(ky, Gy));
+    Hy = p_norm(p_mul(ky, Hy));
+    Gz = p_norm(p_mul(kz, Gz));
+    Hz = p_norm(p_mul(kz, Hz));
+  }
+  if (ph.visc_law == 1) iv = p_norm(p_mul(iv, p_split(pow_tab(p_double(p_y(wT)), ph.visc_exp, ph.powtab))));
+  // tau / (mu gs): diagonal (t00, t11), t22, t01, and (t02, t12)
+  const P2 dia = p_pair(p_x(Gx), p_y(Gy));
+  const P1 div = p_norm(p_mul(P1{-0.6666667f, 1.9868216e-08f}, p_norm(p_add(p_add(p_x(dia), p_y(dia)), p_x(Hz)))));
+  const P2 td = p_norm(p_add(p_scale(dia, 2.f), p_bc(div)));
+  const P1 t22 = p_norm(p_add(p_scale(p_x(Hz), 2.f), div));
+  const P1 t01 = p_norm(p_add(p_x(Gy), p_y(Gx)));
+  const P2 t2 = p_norm(p_add(Gz, p_pair(p_x(Hx), p_x(Hy))));
+  // b_a = u_i tau_ai + kappa mu dT/dx_a of row (ra, rc) = ((tau_a0, tau_a1), tau_a2)
+  auto heat = [&](P2 ra, P1 rc, P1 dT) {
+    const P2 x = p_mul(uv, ra);
+    return p_norm(p_fma(w, rc, p_add(p_add(p_x(x), p_y(x)), dT)));
+  };
+  auto put = [&](int a, P1 n, P2 m, P2 e) {
+    F2[(long long)a * P + q] = p_store(n);
+    F4[(long long)(2 * a) * P + q] = p_store(p_norm(m));
+    F4[(long long)(2 * a + 1) * P + q] = p_store(p_norm(e));
+  };
+  const P1 zero = {0.f, 0.f};
+  if (curv) {
+    const P1 b0 = heat(p_pair(p_x(td), t01), p_x(t2), p_y(Hx)), b1 = heat(p_pair(t01, p_y(td)), p_y(t2), p_y(Hy)),
+             b2 = heat(t2, t22, p_y(Hz));
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      if (as >= 0 && as != a) continue;
+      const P2 row = a == 0 ? xi : et;
+      const P2 x = p_mul(row, uv);
+      const P1 Uc = p_norm(p_add(p_x(x), p_y(x)));  // contravariant velocity
+      const P1 n = p_norm(p_neg(p_mul(rho, Uc)));
+      const P2 r0 = p_bc(p_x(row)), r1 = p_bc(p_y(row));
+      P2 m = p_sub(p_mul(p_bc(n), uv), p_mul(p_bc(pr), row));
+      m = p_fma(p_bc(iv), p_norm(p_fma(r0, p_pair(p_x(td), t01), p_mul(r1, p_pair(t01, p_y(td))))), m);
+      P2 e = p_mul(p_pair(n, netH), p_pair(w, Uc));
+      e = p_fma(p_bc(iv), p_norm(p_fma(r0, p_pair(p_x(t2), b0), p_mul(r1, p_pair(p_y(t2), b1)))), e);
+      put(a, n, m, e);
+    }
+    if (as < 0 || as == 2) {
+      const P1 Uc = p_norm(p_mul(zz, w)), n = p_norm(p_neg(p_mul(rho, Uc)));
+      const P2 iz = p_bc(p_norm(p_mul(iv, zz)));
+      const P2 m = p_fma(iz, t2, p_mul(p_bc(n), uv));
+      P2 e = p_mul(p_pair(n, netH), p_pair(w, Uc));
+      e = p_sub(e, p_pair(p_mul(zz, pr), zero));
+      put(2, n, m, p_fma(iz, p_pair(t22, b2), e));
+    }
+    return;
+  }
+  const P2 nuv = p_norm(p_neg(p_mul(p_bc(rho), uv)));  // -rho u, -rho v
+  if (as < 0 || as == 0) {
+    const P2 ra = p_pair(p_x(td), t01);
+    P2 m = p_sub(p_mul(p_bc(p_x(nuv)), uv), p_pair(pr, zero));
+    P2 e = p_mul(p_pair(p_x(nuv), netH), p_pair(w, p_x(uv)));
+    put(0, p_x(nuv), p_fma(p_bc(iv), ra, m), p_fma(p_bc(iv), p_pair(p_x(t2), heat(ra, p_x(t2), p_y(Hx))), e));
+  }
+  if (as < 0 || as == 1) {
+    const P2 ra = p_pair(t01, p_y(td));
+    P2 m = p_sub(p_mul(p_bc(p_y(nuv)), uv), p_pair(zero, pr));
+    P2 e = p_mul(p_pair(p_y(nuv), netH), p_pair(w, p_y(uv)));
+    put(1, p_y(nuv), p_fma(p_bc(iv), ra, m), p_fma(p_bc(iv), p_pair(p_y(t2), heat(ra, p_y(t2), p_y(Hy))), e));
+  }
+  if (as < 0 || as == 2) {
+    const P1 n = p_norm(p_neg(p_mul(rho, w)));
+    const P2 m = p_mul(p_bc(n), uv);
+    P2 e = p_sub(p_mul(p_pair(n, netH), p_pair(w, w)), p_pair(pr, zero));
+    put(2, n, p_fma(p_bc(iv), t2, m), p_fma(p_bc(iv), p_pair(t22, heat(t2, t22, p_y(Hz))), e));
+  }
+}
+
+// ------------------------------------------------------------------------------- k_rk_p
+
+// dt R = sum_a dt D_a Phi_a (times J on a curvilinear block) in pairs, then the low-storage update
+// Q = A Q + dt R, U^(m) = U^(m-1) + B Q in FP64.
+template <int R>
+__global__ void __launch_bounds__(256) k_rk_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
+                                              const void* __restrict__ Phi, const double* __restrict__ Uin0,
+                                              double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
+                                              int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
+                                              int last) {
+  pdl_enter();
+  sc = resolve(sc);
+  const double* Uin = ring_or(Uin0, in_ring, ring, sc, 0);
+  double* Uout = const_cast<double*>(ring_or(Uout0, out_ring, ring, sc, 1));
+  const int sid = blockIdx.y;
+  const SubDev& d = subs[sid];
+  if (!d.own) return;  // another process's sub-domain
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= d.sx * d.sy * d.sz) return;
+  const int sxy = d.sx * d.sy, ck = t / sxy, r2 = t - ck * sxy, cj = r2 / d.sx, ci = r2 - cj * d.sx;
+  const long long st[3] = {1, d.ex, (long long)d.ex * d.ey};
+  const long long q = d.pbase + (long long)(ci + g.G) + st[1] * (cj + g.G) + st[2] * (ck + g.Gz);
+  const long long gi = d.bbase + (long long)(d.ox + ci) + (long long)d.bnx * ((long long)(d.oy + cj) + (long long)d.bny * (d.oz + ck));
+  const long long P = g.Ptot;
+  const float4* __restrict__ F4 = (const float4*)Phi;
+  const float2* __restrict__ F2 = (const float2*)(F4 + 6 * P);
+  double qv[5], uv[5];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    qv[c] = first ? 0.0 : Q[c * d.bN + gi];
+    uv[c] = Uin[c * d.bN + gi];
+  }
+  P2 m = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, e = m;
+  P1 n = {0.f, 0.f};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const P1 k = p_norm(p_mul(cst(dt), cst(d.cg[a])));
+    m = p_fma(p_bc(k), diff2<R>(F4 + (long long)(2 * a) * P, q, st[a]), m);
+    e = p_fma(p_bc(k), diff2<R>(F4 + (long long)(2 * a + 1) * P, q, st[a]), e);
+    n = p_fma(k, diff1<R>(F2 + (long long)a * P, q, st[a]), n);
+  }
+  if (d.mbase >= 0) {
+    const P1 J = p_of(g.metric_p[d.mbase + 6 * d.mpl + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G)]);
+    m = p_mul(p_bc(J), p_norm(m));
+    e = p_mul(p_bc(J), p_norm(e));
+    n = p_mul(J, p_norm(n));
+  }
+  m = p_norm(m);
+  e = p_norm(e);
+  const double dtR[5] = {p_double(p_norm(n)), p_double(p_x(m)), p_double(p_y(m)), p_double(p_x(e)), p_double(p_y(e))};
+  const bool wallpt = d.wall && ((((d.wall >> 0) & 1) && ci == 0) || (((d.wall >> 1) & 1) && ci == d.sx - 1) ||
+                                 (((d.wall >> 2) & 1) && cj == 0) || (((d.wall >> 3) & 1) && cj == d.sy - 1));
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    double qn = first ? dtR[c] : fma(A, qv[c], dtR[c]);
+    double un = fma(B, qn, uv[c]);
+    if (wallpt && c >= 1 && c <= 3) qn = un = 0.0;  // no-slip wall points keep zero momentum
+    if (!last) Q[c * d.bN + gi] = qn;
+    Uout[c * d.bN + gi] = un;
+  }
+}
+
+// ------------------------------------------------------------------------------- launchers
+
+int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
+                   const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm) {
+  if (nhalo <= 0) return 0;
+  float4* H4 = (float4*)H;
+  float2* H2 = (float2*)(H4 + 2LL * s * nhalo);
+  TIMED(tm, 0, (launch_pdl(s == 2 ? k_at_halo<2> : k_at_halo<5>, dim3(nblk(nhalo, 256)), dim3(256), 0, (cudaStream_t)stream, g,
+                           ph, sc, ring, subs, (const int2*)halo, nhalo, H4, H2)));
+  if (launches) *launches += 1;
+  return (int)cudaGetLastError();
+}
+
+int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const StageLaunch& a, const void* H,
+                       void* stream, long long* launches, const Timer* tm) {
+  const cudaStream_t st = (cudaStream_t)stream;
+  const int B = a.threads == 128 ? 128 : 256;
+  const float4* H4 = (const float4*)H;
+  const float2* H2 = (const float2*)(H4 + 2LL * a.s * a.nhalo);
+  const unsigned own_blocks = nblk(a.max_own, B);
+  const unsigned nb = own_blocks * (unsigned)g.nsub + nblk(a.nhalo, B);
+  const dim3 gf(nblk(a.max_flux, B), g.nsub), gr(nblk(a.max_own, B), g.nsub);
+  const float dth = (float)a.dt;
+  const float2 dt = make_float2(dth, (float)(a.dt - (double)dth));
+  TIMED(tm, 0, (launch_pdl(k_view_p, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring, a.in_ring, a.subs, (const int2*)a.halo,
+                           a.nhalo, H4, H2, a.Wp, a.stage, a.s, (int)own_blocks)));
+  auto flux = g.r == 2 ? (g.metric ? k_flux_p<2, true> : k_flux_p<2, false>) : (g.metric ? k_flux_p<1, true> : k_flux_p<1, false>);
+  TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi)));
+  auto rk = g.r == 2 ? k_rk_p<2> : k_rk_p<1>;
+  TIMED(tm, 2, (launch_pdl(rk, gr, dim3(B), 0, st, g, sc, a.subs, (const void*)a.Phi, a.Uin, a.Uout, a.ring, a.in_ring,
+                           a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last)));
+  if (launches) *launches += 3;
+  return (int)cudaGetLastError();
+}
+
+}  // namespace cfs

@@ -1,0 +1,65 @@
+"""The arithmetic on pairs of floats (pairs.cuh) against extended precision, element by element."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(HERE, "..", "paper_2506_03027_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("pairs") / "libpairs.so")
+    subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
+                    "-I", CSRC, os.path.join(HERE, "cuda", "pairs_check.cu"), "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    lib.pairs_check.argtypes = [ctypes.c_void_p] * 5 + [ctypes.c_int]
+    return lib
+
+
+# values near 1, over many magnitudes, and sums that cancel almost entirely
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["unit", "wide", "cancel"])
+def test_pair_operations(lib, kind):
+    import torch
+    rng = np.random.default_rng(11)
+    n = 1 << 18
+    a, b, c = (rng.choice([-1.0, 1.0], n) * rng.uniform(0.5, 2.0, n) for _ in range(3))
+    if kind == "wide":
+        a, b, c = (x * 10.0 ** rng.uniform(-9, 9, n) for x in (a, b, c))
+    if kind == "cancel":
+        b = a * (1.0 + 10.0 ** rng.uniform(-14, -3, n))
+        c = -a * b * (1.0 + 10.0 ** rng.uniform(-14, -3, n))
+    t = [torch.tensor(x, device="cuda") for x in (a, b, c)]
+    out = torch.empty((7, n, 2), dtype=torch.float32, device="cuda")
+    dbl = torch.empty(n, dtype=torch.float64, device="cuda")
+    assert lib.pairs_check(*(x.data_ptr() for x in t), out.data_ptr(), dbl.data_ptr(), n) == 0
+    got = out.cpu().numpy().astype(np.longdouble).sum(axis=-1)
+    a, b, c = (x.astype(np.longdouble) for x in (a, b, c))
+    u = np.longdouble(2.0) ** -48
+    # h to 24 bits and l to 24 bits of what is left; the other operations on split operands (each off by
+    # u/2) with a handful of roundings of low words, u/2 of the operands' magnitudes each
+    exact = [(a, u / 2 * abs(a)), (a + b, 3 * u * (abs(a) + abs(b))), (a - b, 3 * u * (abs(a) + abs(b))),
+             (a * b, 4 * u * abs(a * b)), (a * b + c, 6 * u * (abs(a * b) + abs(c))), (1 / a, 4 * u / abs(a)),
+             (a * b + c, 6 * u * (abs(a * b) + abs(c)))]
+    for k, (ref, tol) in enumerate(exact):
+        assert np.all(abs(got[k] - ref) <= tol), (k, float(np.max(abs(got[k] - ref) / tol)))
+    assert np.all(dbl.cpu().numpy().astype(np.longdouble) == got[0])  # 48 bits and a sign: exact in FP64
+
+
+@pytest.mark.gpu
+def test_split_outside_the_fp32_range(lib):
+    """Nonfinite values and values beyond FP32 give NaN, values below it zero."""
+    import torch
+    x = np.array([np.nan, np.inf, -np.inf, 1e39, -1e200, 1e-39, -1e-300, 0.0, -0.0, 1e38, 2.0 ** -126])
+    t = torch.tensor(x, device="cuda")
+    one = torch.ones_like(t)
+    out = torch.empty((7, len(x), 2), dtype=torch.float32, device="cuda")
+    dbl = torch.empty(len(x), dtype=torch.float64, device="cuda")
+    assert lib.pairs_check(t.data_ptr(), one.data_ptr(), one.data_ptr(), out.data_ptr(), dbl.data_ptr(), len(x)) == 0
+    d = dbl.cpu().numpy()
+    assert np.all(np.isnan(d[:5])) and np.all(d[5:9] == 0.0)
+    assert abs(d[9] - 1e38) <= 2.0 ** -49 * 1e38 and d[10] == 2.0 ** -126
