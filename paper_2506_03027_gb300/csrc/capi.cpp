@@ -597,14 +597,12 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     pp.H = pair_of((long double)ph.gamma * pp.Eref);
     pp.ivT = pair_of(ph.ivT);
     pp.visc_law = ph.visc_law;
-    pp.visc_exp = ph.visc_exp;
+    pp.visc_exp = pair_of(ph.visc_exp);
   }
   // tables of the FP64 power (power-law viscosity)
   if (c->p.viscous && c->p.visc_law == 1) {
-    const int rc = cfs::pow_tables_init();
+    const int rc = c->pairs ? cfs::pow_pair_tables_init() : cfs::pow_tables_init();
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "power tables");
-    c->pphys.powtab = cfs::pow_table_address();
-    if (!c->pphys.powtab) return fail(c, CFS_ECUDA, "power tables");
   }
   // device memory
   c->ring = (double*)dev_alloc(c, sizeof(double) * 5 * N * c->R);

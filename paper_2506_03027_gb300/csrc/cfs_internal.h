@@ -131,8 +131,7 @@ struct PairPhysics {
   float2 gm1, kgM2, kT0, H, ivT;
   float Eref;
   int visc_law;
-  double visc_exp;
-  const double* powtab;    // device: tables of the FP64 power
+  float2 visc_exp;
 };
 
 // Delay schedule as seen by the kernels of one step.
@@ -403,7 +402,7 @@ struct StripPlan {
 };
 const char* strip_plan(const TopoBlock* B, int nb, int nsub, const int* starts, int nranks, int rank, int depth,
                        int depth_z, int r, bool viscous, int ndim, StripPlan* out);
-const double* pow_table_address();  // its device address on the current device, or null
+int pow_pair_tables_init();  // the same for the pairs' power (stage_pairs.cu)
 int pow_tables_init();  // tables of the FP64 power on the current device, once per device; nonzero on a CUDA error
 
 }  // namespace cfs

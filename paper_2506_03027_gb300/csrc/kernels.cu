@@ -218,7 +218,51 @@ __global__ void __launch_bounds__(512) k_view(Geometry g, Physics ph, StepSched 
 
 // ------------------------------------------------------------------------------- k_flux
 
-__device__ double g_pow_tab[3 * 64];  // tables of pow_tab: 1/c_j, ln c_j, 2^(j/64)
+// x^a = exp(a ln x) in FP64 for positive normal x (the viscosity law mu = T^a), table-driven
+// after Tang (ACM TOMS 1989, 1990), about 20 FP64 operations.  ln x: x = m 2^e with m in [1, 2)
+// from the bit fields; the top six mantissa bits pick c_j = 1 + (j + 1/2)/64, u = m / c_j - 1
+// (|u| <= 1/129) from a table of 1/c_j, ln m = ln c_j + log1p(u) with the series of log1p to u^7.
+// exp y: y = (64 k' + j') ln2/64 + r with |r| <= ln2/128 (ln 2 / 64 split into a 32-bit head and
+// its tail: k ln2_head is exact), exp r by its Taylor series to r^5/5!, times the tabulated
+// 2^(j'/64), and 2^k' added to the exponent field.  Tables: 1/c_j rounded from the exact
+// quotient, ln c_j and 2^(j/64) rounded from long-double log1p and exp2 (pow_tables_init).
+// Relative error below 6e-16 (1 + |a ln x|).  Any other x, or |a ln x| >= 700, goes to the
+// library's pow.
+__device__ double g_pow_tab[3 * 64];  // 1/c_j, ln c_j, 2^(j/64)
+
+__device__ __forceinline__ double pow_tab(double x, double a) {
+  if (!(x >= 2.2250738585072014e-308) || !(x <= 1.7976931348623157e308)) return pow(x, a);
+  const int hi = __double2hiint(x);
+  const int e = ((hi >> 20) & 0x7ff) - 1023;
+  const int j = (hi >> 14) & 63;
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));  // [1, 2)
+  const double u = fma(m, __ldg(g_pow_tab + j), -1.0);
+  double p = 1.0 / 7.0;
+  p = fma(p, u, -1.0 / 6.0);
+  p = fma(p, u, 1.0 / 5.0);
+  p = fma(p, u, -1.0 / 4.0);
+  p = fma(p, u, 1.0 / 3.0);
+  p = fma(p, u, -0.5);
+  p = fma(p, u, 1.0);
+  const double l1p = p * u;
+  const double LN2_HEAD = 0.6931471803691238, LN2_TAIL = 1.9082149292705877e-10;
+  const double ed = (double)e;
+  // (e ln2_head + ln c_j) is exact where it cancels (x just below 1: Sterbenz), then the tails
+  const double y = a * (fma(ed, LN2_HEAD, __ldg(g_pow_tab + 64 + j)) + fma(ed, LN2_TAIL, l1p));
+  if (!(fabs(y) < 700.0)) return pow(x, a);
+  const double kd = rint(y * (64.0 / 0.6931471805599453));
+  double r = fma(-kd, LN2_HEAD / 64.0, y);
+  r = fma(-kd, LN2_TAIL / 64.0, r);
+  double q = 1.0 / 120.0;
+  q = fma(q, r, 1.0 / 24.0);
+  q = fma(q, r, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  q = fma(q, r, 1.0);
+  q = fma(q, r, 1.0);
+  const int k = (int)kd;
+  q *= __ldg(g_pow_tab + 128 + (k & 63));
+  return __hiloint2double(__double2hiint(q) + ((k >> 6) << 20), __double2loint(q));
+}
 
 // Viscosity law: mu = 1, or the power law mu = T^visc_exp -- in the intermediate precision (the
 // FP32 form evaluates it in FP32 with the hardware log2 / exp2 pair, a few ulp: a power in FP64
@@ -228,7 +272,7 @@ template <typename T>
 __device__ __forceinline__ T visc_mu(const Physics& ph, T temp) {
   if (ph.visc_law != 1) return (T)1;
   if (std::is_same<T, float>::value) return (T)__powf((float)temp, (float)ph.visc_exp);
-  return (T)pow_tab((double)temp, ph.visc_exp, g_pow_tab);
+  return (T)pow_tab((double)temp, ph.visc_exp);
 }
 
 template <typename T>
@@ -1264,7 +1308,7 @@ __global__ void k_advance_step(long long* dn) {
 
 __global__ void k_eval_power(const double* __restrict__ x, double a, double* __restrict__ y, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = pow_tab(x[i], a, g_pow_tab);
+  if (i < n) y[i] = pow_tab(x[i], a);
 }
 
 // The tables of pow_tab in the current device's copy of the __device__ array, once per device
@@ -1290,11 +1334,6 @@ int pow_tables_init() {
   if (e != cudaSuccess) return (int)e;
   done[dev] = true;
   return 0;
-}
-
-const double* pow_table_address() {
-  void* p = nullptr;
-  return cudaGetSymbolAddress(&p, g_pow_tab) == cudaSuccess ? (const double*)p : nullptr;
 }
 
 int launch_eval_power(const double* x, double a, double* y, long long n, void* stream) {

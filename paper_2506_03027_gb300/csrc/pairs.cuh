@@ -11,6 +11,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "device_common.cuh"
 
 namespace cfs {
@@ -132,5 +134,72 @@ __device__ __forceinline__ P1 p_split(double x) {
 }
 // pair -> FP64: one FP64 addition
 __device__ __forceinline__ double p_double(P1 a) { return f2d_fast(a.h) + f2d_fast(a.l); }
+
+// x^a = exp(a ln x) for positive x, table-driven after Tang (ACM TOMS 1989, 1990) as the FP64 power
+// of kernels.cu, on pairs.  ln x: x = m 2^e with m in [1, 2); the top six mantissa bits pick a
+// float rc_j near 1 / c_j, c_j = 1 + (j + 1/2)/64; u = m rc_j - 1 (|u| < 1/128, the product split
+// exactly), ln m = -ln rc_j + log1p(u): u, u^2/2 and u^3/3 as pairs, u^4 to u^7 in FP32.  exp y: y =
+// (64 k' + j') ln2/64 + r, |r| <= ln2/128, exp r with r and r^2/2 as pairs and r^3 to r^5 in FP32,
+// times the tabulated 2^(j'/64), times 2^k'.  Relative error below 2^-44 (1 + |a ln x|).  About 120
+// FP32 operations, where the FP64 power's 20 take the time of 1,280.  Other x, or |a ln x| >= 60, go to
+// the library's pow.  tab: [5][64]: rc_j, -ln rc_j (h, l), 2^(j/64) (h, l).
+#define POW_PAIR_TAB (5 * 64)
+__device__ __forceinline__ P1 p_pow(P1 x, P1 a, const float* __restrict__ tab) {
+  const unsigned b = __float_as_uint(x.h);
+  if (b - 0x08000000u < 0x6f000000u) {  // 2^-111 <= x.h < 2^111
+    const int e = (int)(b >> 23) - 127;
+    const int j = (int)(b >> 17) & 63;
+    const float m = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
+    const float ml = __fmul_rn(x.l, __uint_as_float((unsigned)(127 - e) << 23));
+    const float rc = __ldg(tab + j);
+    const float p = __fmul_rn(m, rc);
+    const P1 u = p_fast2sum(__fsub_rn(p, 1.f), __fmaf_rn(ml, rc, __fmaf_rn(m, rc, -p)));
+    const P1 u2 = p_norm(p_mul(u, u));
+    const P1 u3 = p_mul(p_norm(p_mul(u2, u)), P1{0.33333334f, -9.934108e-09f});
+    float t = 1.f / 7.f;
+    t = __fmaf_rn(t, u.h, -1.f / 6.f);
+    t = __fmaf_rn(t, u.h, 1.f / 5.f);
+    t = __fmaf_rn(t, u.h, -1.f / 4.f);
+    t = __fmul_rn(t, __fmul_rn(u2.h, u2.h));
+    // ln 2 = 0.693145751953125 (16 bits, e times it is exact) + the rest as a pair
+    const float ef = (float)e;
+    P1 L = p_add(P1{__fmul_rn(ef, 0.693145751953125f), 0.f}, P1{__ldg(tab + 64 + j), __ldg(tab + 128 + j)});
+    L = p_add(L, p_mul(P1{ef, 0.f}, P1{1.4286068e-06f, 5.497923e-14f}));
+    P1 s = p_add(p_add(u, p_scale(u2, -0.5f)), u3);
+    s.l = __fadd_rn(s.l, t);
+    const P1 y = p_norm(p_mul(p_norm(p_add(L, s)), a));
+    if (fabsf(y.h) < 60.f) {
+      const float kf = rintf(__fmul_rn(y.h, 92.332482f));  // 64 / ln 2
+      // ln2/64 = 0.01082611083984375 (11 bits, k times it is exact) + the rest as a pair
+      P1 r = p_add(y, P1{__fmul_rn(kf, -0.01082611083984375f), 0.f});
+      r = p_norm(p_add(r, p_mul(P1{kf, 0.f}, P1{-4.3138566e-06f, 2.0164563e-13f})));
+      const P1 r2 = p_mul(r, r);
+      float q = 1.f / 120.f;
+      q = __fmaf_rn(q, r.h, 1.f / 24.f);
+      q = __fmaf_rn(q, r.h, 1.f / 6.f);
+      q = __fmul_rn(q, __fmul_rn(r2.h, r.h));
+      P1 w = p_add(r, p_scale(r2, 0.5f));
+      w.l = __fadd_rn(w.l, q);
+      w = p_norm(p_add(P1{1.f, 0.f}, w));
+      const int k = (int)kf;
+      w = p_norm(p_mul(w, P1{__ldg(tab + 192 + (k & 63)), __ldg(tab + 256 + (k & 63))}));
+      return p_scale(w, __uint_as_float((unsigned)((k >> 6) + 127) << 23));
+    }
+  }
+  return p_split(pow((double)x.h + (double)x.l, (double)a.h + (double)a.l));
+}
+
+// The tables of p_pow (host).
+inline void pow_pair_table(float* t) {
+  auto put = [&](int at, int j, long double x) {
+    t[at + j] = (float)x;
+    t[at + 64 + j] = (float)(x - (long double)t[at + j]);
+  };
+  for (int j = 0; j < 64; ++j) {
+    t[j] = (float)(128.0 / (129.0 + 2.0 * j));
+    put(64, j, -logl((long double)t[j]));
+    put(192, j, exp2l((long double)j / 64.0L));
+  }
+}
 
 }  // namespace cfs

@@ -18,6 +18,9 @@
 // one read of the delayed levels (they would be read once per stage otherwise).
 #include <cuda_runtime.h>
 
+#include <mutex>
+#include <type_traits>
+
 #include "cfs_internal.h"
 #include "device_common.cuh"
 #include "launch_common.cuh"
@@ -106,8 +109,8 @@ __device__ __forceinline__ bool any_own_source(const HaloPoint& h, const SubDev&
   return own;
 }
 
-// The value of a gather entry at stage `stage`: own sources from the stage input, a neighbouring
-// PE's by the mode (live, latest delayed level, or the AT weights), far-field constants; FP64.
+// The value of a gather entry with an own source at stage `stage`: own sources from the stage input, a
+// neighbouring PE's by the mode (live, latest delayed level, or the AT weights), far-field constants; FP64.
 __device__ __forceinline__ void gather_value(const Geometry& g, const StepSched& sc, const HaloPoint& h, const SubDev& d, int kd,
                                              const double* __restrict__ Uin, const double* __restrict__ ring, int stage,
                                              int s, double* u) {
@@ -121,7 +124,7 @@ __device__ __forceinline__ void gather_value(const Geometry& g, const StepSched&
     const double wt = E.w[t], wf = (E.flags[t] & 1) ? -wt : wt;
     const long long o = E.off[t], bN = E.bN[t];
     double x[5];
-    if (sc.mode == 0 || (Uin && own_source(h, d, t))) {
+    if (sc.mode == 0 || own_source(h, d, t)) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) x[v] = Uin[o + v * bN];
     } else if (sc.mode == 2) {
@@ -153,7 +156,7 @@ __device__ __forceinline__ void gather_value(const Geometry& g, const StepSched&
 // stage-0 value and add the sums with W^(m) - W^(0).  Stored [stage][entry]: (rho, rho u), (rho v,
 // rho w) and rho E - E_ref.  Bound by its reads: C x 40 bytes per entry at the sub-domains' faces.
 template <int S>
-__global__ void __launch_bounds__(256) k_at_halo(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ ring,
+__global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ ring,
                                                  const SubDev* __restrict__ subs, const int2* __restrict__ halo,
                                                  long long nhalo, float4* __restrict__ H4, float2* __restrict__ H2) {
   pdl_enter();
@@ -165,92 +168,88 @@ __global__ void __launch_bounds__(256) k_at_halo(Geometry g, PairPhysics ph, Ste
   const SubDev d = subs[hv.x];
   const HaloPoint h = halo_point(g, d, hv);
   const int kd = point_delay(sc, d, h.sid, h.ci, h.cj, h.ck, h.beyond);
-  auto put = [&](int m, P2 a, P2 b, P1 c) {
-    H4[(long long)(2 * m) * nhalo + e] = p_store(a);
-    H4[(long long)(2 * m + 1) * nhalo + e] = p_store(b);
-    H2[(long long)m * nhalo + e] = p_store(c);
-  };
-  auto put64 = [&](int m, const double* u) {
-    put(m, p_pair(p_split(u[0]), p_split(u[1])), p_pair(p_split(u[2]), p_split(u[3])),
-        p_norm(p_add(p_split(u[4]), P1{-ph.Eref, 0.f})));
-  };
-  if (h.beyond) {
-    // (entries with an own source are formed from the live stage input by k_view_p)
-    if (any_own_source(h, d)) return;
-    for (int m = 0; m < (sc.mode == 2 ? 1 : S); ++m) {
-      double u[5];
-      gather_value(g, sc, h, d, kd, nullptr, ring, m, S, u);
-      put64(m, u);
-    }
-    return;
-  }
+  // (entries with an own source are formed from the live stage input by k_view_p)
+  if (h.beyond && any_own_source(h, d)) return;
   const long long lvN = 5 * g.N;
   const int nR = (int)(sc.n % sc.R);
   auto slot = [&](int l) { const int q = nR - kd - l; return (long long)(q < 0 ? q + sc.R : q) * lvN; };
   const int C = sc.mode == 2 ? 1 : sc.C;
-  double r[CFS_MAX_LEVELS][5];
+  long long lev[CFS_MAX_LEVELS];
 #pragma unroll
-  for (int l = 0; l < CFS_MAX_LEVELS; ++l)
-    if (l < C) {
-      const double* src = ring + slot(l) + h.gi;
+  for (int l = 0; l < CFS_MAX_LEVELS; ++l) lev[l] = l < C ? slot(l) : 0;
+  const bool learned = sc.LH && sc.mode == 1 && ((int)(h.ci < 0 || h.ci >= d.sx) + (int)(h.cj < 0 || h.cj >= d.sy) + (int)(h.ck < 0 || h.ck >= d.sz) == 1);
+  // (AS, mode 2: the latest visible level, the same for every stage -- stage 0 alone is stored)
+  const int ns = sc.mode == 2 ? 1 : S;
+  const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * sc.C;
+  const long long lh = d.pbase + h.q;
+  // two components at a time (rho and rho u, rho v and rho w, rho E alone): few registers, so that
+  // several warps per scheduler keep the levels' loads in flight
 #pragma unroll
-      for (int v = 0; v < 5; ++v) r[l][v] = src[v * d.bN];
+  for (int grp = 0; grp < 3; ++grp) {
+    const int v0 = 2 * grp, v1 = grp < 2 ? v0 + 1 : v0;
+    double x[CFS_MAX_LEVELS], y[CFS_MAX_LEVELS];
+    if (!h.beyond) {
+#pragma unroll
+      for (int l = 0; l < CFS_MAX_LEVELS; ++l)
+        if (l < C) {
+          x[l] = ring[lev[l] + h.gi + v0 * d.bN];
+          if (grp < 2) y[l] = ring[lev[l] + h.gi + v1 * d.bN];
+        }
+    } else {
+      // beyond a non-periodic block face: the weighted sources of the gather entry and the far-field
+      // constant, level by level (FP64)
+      const GatherEntry& E = *h.ent;
+#pragma unroll
+      for (int l = 0; l < CFS_MAX_LEVELS; ++l) {
+        x[l] = E.cst[v0];
+        y[l] = E.cst[v1];
+      }
+      for (int t = 0; t < E.nt; ++t) {
+        const double w = E.w[t], wf = (E.flags[t] & 1) ? -w : w;
+        const double w0 = grp == 1 ? wf : w, w1 = wf;  // (components 0, 1 | 2, 3 | 4)
+        const double* src = ring + E.off[t];
+        const long long sN = E.bN[t];
+#pragma unroll
+        for (int l = 0; l < CFS_MAX_LEVELS; ++l)
+          if (l < C) {
+            x[l] = fma(w0, src[lev[l] + v0 * sN], x[l]);
+            if (grp < 2) y[l] = fma(w1, src[lev[l] + v1 * sN], y[l]);
+          }
+      }
     }
-  if (sc.mode == 2) {  // AS: the latest visible level, the same for every stage
-    put64(0, r[0]);
-    return;
-  }
-  const bool learned = sc.LH && ((int)(h.ci < 0 || h.ci >= d.sx) + (int)(h.cj < 0 || h.cj >= d.sy) + (int)(h.ck < 0 || h.ck >= d.sz) == 1);
-  auto split5 = [&](const double* u, P2& a, P2& b, P1& c) {
-    a = p_pair(p_split(u[0]), p_split(u[1]));
-    b = p_pair(p_split(u[2]), p_split(u[3]));
-    c = p_split(u[4]);
-  };
-  P2 a0, b0, aa[S], ab[S];
-  P1 c0, ac[S];
-  split5(r[0], a0, b0, c0);
-  const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * C;
-  {
     // what the sums are added to: U_0, or the network's stage-0 value
-    P2 sa = a0, sb = b0;
-    P1 se = c0;
+    P1 bx = p_split(x[0]), by = grp < 2 ? p_split(y[0]) : P1{0.f, 0.f};
+    const P2 u0 = p_pair(bx, by);
     if (learned) {
-      double u[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) u[v] = sc.LH[(long long)v * g.Ptot + d.pbase + h.q];
-      split5(u, sa, sb, se);
+      bx = p_split(sc.LH[(long long)v0 * g.Ptot + lh]);
+      if (grp < 2) by = p_split(sc.LH[(long long)v1 * g.Ptot + lh]);
     }
-    se = p_norm(p_add(se, P1{-ph.Eref, 0.f}));
+    if (grp == 2) bx = p_norm(p_add(bx, P1{-ph.Eref, 0.f}));
+    P2 acc[S];
 #pragma unroll
     for (int m = 0; m < S; ++m) {
       // (with the network, stage 0 is its value: the weights W^(0) - W^(0) are zero)
-      const float2 cm = __ldg(wt + m * C);
-      const P1 c = {cm.x, cm.y};
-      aa[m] = p_fma(p_bc(c), a0, sa);
-      ab[m] = p_fma(p_bc(c), b0, sb);
-      ac[m] = p_fma(c, c0, se);
+      const float2 c = sc.mode == 2 ? make_float2(0.f, 0.f) : __ldg(wt + m * C);
+      acc[m] = p_fma(p_bc(P1{c.x, c.y}), u0, p_pair(bx, by));
+    }
+#pragma unroll
+    for (int l = 1; l < CFS_MAX_LEVELS; ++l)
+      if (l < C) {
+        const P2 dl = p_norm(p_sub(p_pair(p_split(x[l]), grp < 2 ? p_split(y[l]) : P1{0.f, 0.f}), u0));
+#pragma unroll
+        for (int m = 0; m < S; ++m) {
+          const float2 w = __ldg(wt + m * C + l);
+          acc[m] = p_fma(p_bc(P1{w.x, w.y}), dl, acc[m]);
+        }
+      }
+#pragma unroll
+    for (int m = 0; m < S; ++m) {
+      if (m >= ns) break;
+      const P2 a = p_norm(acc[m]);
+      if (grp < 2) H4[(long long)(2 * m + grp) * nhalo + e] = p_store(a);
+      else H2[(long long)m * nhalo + e] = p_store(p_x(a));
     }
   }
-#pragma unroll
-  for (int l = 1; l < CFS_MAX_LEVELS; ++l)
-    if (l < C) {
-      P2 a, b;
-      P1 c;
-      split5(r[l], a, b, c);
-      a = p_norm(p_sub(a, a0));
-      b = p_norm(p_sub(b, b0));
-      c = p_norm(p_sub(c, c0));
-#pragma unroll
-      for (int m = 0; m < S; ++m) {
-        const float2 wm = __ldg(wt + m * C + l);
-        const P1 w = {wm.x, wm.y};
-        aa[m] = p_fma(p_bc(w), a, aa[m]);
-        ab[m] = p_fma(p_bc(w), b, ab[m]);
-        ac[m] = p_fma(w, c, ac[m]);
-      }
-    }
-#pragma unroll
-  for (int m = 0; m < S; ++m) put(m, p_norm(aa[m]), p_norm(ab[m]), p_norm(ac[m]));
 }
 
 // ------------------------------------------------------------------------------- k_view_p
@@ -334,11 +333,13 @@ __device__ __forceinline__ P1 diff1(const float2* __restrict__ f, long long q, l
 
 }  // namespace
 
+__device__ float g_pow_pair[POW_PAIR_TAB];  // tables of p_pow
+
 // Combined fluxes at the owned points and the strips of r points beyond each face (the flux along
 // that face's axis only), thread by thread as in k_flux.  CURV: the context has curvilinear
-// blocks.  R: stencil radius (CD4: 2).
-template <int R, bool CURV>
-__global__ void __launch_bounds__(256) k_flux_p(Geometry g, PairPhysics ph, const SubDev* __restrict__ subs,
+// blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.
+template <int R, bool CURV, bool LAW>
+__global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPhysics ph, const SubDev* __restrict__ subs,
                                                 const void* __restrict__ Wp, void* __restrict__ Phi) {
   pdl_enter();
   const int sid = blockIdx.y;
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(256) k_flux_p(Geometry g, PairPhysics ph, cons
     Gz = p_norm(p_mul(kz, Gz));
     Hz = p_norm(p_mul(kz, Hz));
   }
-  if (ph.visc_law == 1) iv = p_norm(p_mul(iv, p_split(pow_tab(p_double(p_y(wT)), ph.visc_exp, ph.powtab))));
+  if (LAW) iv = p_norm(p_mul(iv, p_pow(p_y(wT), cst(ph.visc_exp), g_pow_pair)));
   // tau / (mu gs): diagonal (t00, t11), t22, t01, and (t02, t12)
   const P2 dia = p_pair(p_x(Gx), p_y(Gy));
   const P1 div = p_norm(p_mul(P1{-0.6666667f, 1.9868216e-08f}, p_norm(p_add(p_add(p_x(dia), p_y(dia)), p_x(Hz)))));
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(256) k_flux_p(Geometry g, PairPhysics ph, cons
 // dt R = sum_a dt D_a Phi_a (times J on a curvilinear block) in pairs, then the low-storage update
 // Q = A Q + dt R, U^(m) = U^(m-1) + B Q in FP64.
 template <int R>
-__global__ void __launch_bounds__(256) k_rk_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
+__global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
                                               const void* __restrict__ Phi, const double* __restrict__ Uin0,
                                               double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
                                               int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
@@ -530,6 +531,26 @@ __global__ void __launch_bounds__(256) k_rk_p(Geometry g, StepSched sc, const Su
 
 // ------------------------------------------------------------------------------- launchers
 
+// The tables of p_pow in the current device's copy of the array, once per device (as
+// pow_tables_init).
+int pow_pair_tables_init() {
+  constexpr int kMaxDev = 64;
+  static std::mutex mu;
+  static bool done[kMaxDev] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return (int)e;
+  if (dev < 0 || dev >= kMaxDev) return (int)cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(mu);
+  if (done[dev]) return 0;
+  float t[POW_PAIR_TAB];
+  pow_pair_table(t);
+  e = cudaMemcpyToSymbol(g_pow_pair, t, sizeof(t));
+  if (e != cudaSuccess) return (int)e;
+  done[dev] = true;
+  return 0;
+}
+
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
                    const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm) {
   if (nhalo <= 0) return 0;
@@ -554,7 +575,12 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   const float2 dt = make_float2(dth, (float)(a.dt - (double)dth));
   TIMED(tm, 0, (launch_pdl(k_view_p, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring, a.in_ring, a.subs, (const int2*)a.halo,
                            a.nhalo, H4, H2, a.Wp, a.stage, a.s, (int)own_blocks)));
-  auto flux = g.r == 2 ? (g.metric ? k_flux_p<2, true> : k_flux_p<2, false>) : (g.metric ? k_flux_p<1, true> : k_flux_p<1, false>);
+  auto pick = [&](auto r) {
+    constexpr int R = decltype(r)::value;
+    if (ph.visc_law == 1) return g.metric ? k_flux_p<R, true, true> : k_flux_p<R, false, true>;
+    return g.metric ? k_flux_p<R, true, false> : k_flux_p<R, false, false>;
+  };
+  const auto flux = g.r == 2 ? pick(std::integral_constant<int, 2>{}) : pick(std::integral_constant<int, 1>{});
   TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi)));
   auto rk = g.r == 2 ? k_rk_p<2> : k_rk_p<1>;
   TIMED(tm, 2, (launch_pdl(rk, gr, dim3(B), 0, st, g, sc, a.subs, (const void*)a.Phi, a.Uin, a.Uout, a.ring, a.in_ring,

@@ -19,3 +19,19 @@ extern "C" int pairs_check(const double* a, const double* b, const double* c, fl
   k_pairs<<<(n + 255) / 256, 256>>>(a, b, c, out, dbl, n);
   return (int)cudaDeviceSynchronize();
 }
+
+__global__ void k_pairs_pow(const double* x, double a, const float* tab, float2* out, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = p_store(p_pow(p_split(x[i]), p_split(a), tab));
+}
+
+extern "C" int pairs_pow(const double* x, double a, float2* out, int n) {
+  float t[POW_PAIR_TAB], *d = nullptr;
+  pow_pair_table(t);
+  if (cudaMalloc(&d, sizeof(t)) != cudaSuccess) return 1;
+  cudaMemcpy(d, t, sizeof(t), cudaMemcpyHostToDevice);
+  k_pairs_pow<<<(n + 255) / 256, 256>>>(x, a, d, out, n);
+  const int rc = (int)cudaDeviceSynchronize();
+  cudaFree(d);
+  return rc;
+}

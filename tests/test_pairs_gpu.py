@@ -17,6 +17,7 @@ def lib(tmp_path_factory):
                     "-I", CSRC, os.path.join(HERE, "cuda", "pairs_check.cu"), "-o", out], check=True)
     lib = ctypes.CDLL(out)
     lib.pairs_check.argtypes = [ctypes.c_void_p] * 5 + [ctypes.c_int]
+    lib.pairs_pow.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p, ctypes.c_int]
     return lib
 
 
@@ -63,3 +64,35 @@ def test_split_outside_the_fp32_range(lib):
     d = dbl.cpu().numpy()
     assert np.all(np.isnan(d[:5])) and np.all(d[5:9] == 0.0)
     assert abs(d[9] - 1e38) <= 2.0 ** -49 * 1e38 and d[10] == 2.0 ** -126
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("a", [0.76, -0.76, 1.5, 0.001])
+def test_power(lib, a):
+    """x^a near 1 (every table entry, both sides of 1), over the FP32 range, and where it falls back."""
+    import torch
+    rng = np.random.default_rng(13)
+    x = np.concatenate([1.0 + rng.uniform(-0.05, 0.05, 1 << 16), rng.uniform(0.2, 4.0, 1 << 16), 300.0 * rng.uniform(0.5, 2.0, 1 << 16),
+                        10.0 ** rng.uniform(-30, 30, 1 << 16), 1.0 + np.array([0.0, 2.0 ** -30, -2.0 ** -30, 1e-13])])
+    t = torch.tensor(x, device="cuda")
+    out = torch.empty((len(x), 2), dtype=torch.float32, device="cuda")
+    assert lib.pairs_pow(t.data_ptr(), a, out.data_ptr(), len(x)) == 0
+    got = out.cpu().numpy().astype(np.longdouble).sum(axis=-1)
+    pairs = torch.empty((7, len(x), 2), dtype=torch.float32, device="cuda")  # (the power of the pair, which below 2^-97 is h alone)
+    dbl = torch.empty(len(x), dtype=torch.float64, device="cuda")
+    assert lib.pairs_check(t.data_ptr(), t.data_ptr(), t.data_ptr(), pairs.data_ptr(), dbl.data_ptr(), len(x)) == 0
+    X, A = pairs[0].cpu().numpy().astype(np.longdouble).sum(axis=-1), np.longdouble(a)
+    ref = X ** A
+    ok = (ref > 1e-25) & (ref < 1e25)
+    tol = np.longdouble(2.0) ** -44 * (1 + abs(A * np.log(X))) * ref
+    assert np.all(abs(got - ref)[ok] <= tol[ok]), float(np.max((abs(got - ref) / tol)[ok]))
+
+
+@pytest.mark.gpu
+def test_power_of_bad_values(lib):
+    import torch
+    x = np.array([-1.0, np.nan, np.inf])
+    t = torch.tensor(x, device="cuda")
+    out = torch.empty((3, 2), dtype=torch.float32, device="cuda")
+    assert lib.pairs_pow(t.data_ptr(), 0.76, out.data_ptr(), 3) == 0
+    assert bool(torch.isnan(out.sum(dim=-1)).all())
