@@ -87,7 +87,7 @@ struct cfs_ctx {
   double filt_h[6] = {0};
   double* d_partial = nullptr;
   double* d_out = nullptr;
-  int diag_blocks = 0;
+  long long diag_total = 0;  // rows of partial sums of all blocks
 
   // compact list of the halo points of every sub-domain: (sub-domain, padded index)
   int* d_halo = nullptr;
@@ -243,11 +243,6 @@ static void dev_free(cfs_ctx* c, void* p) {
       c->freef(p, c->user);
       return;
     }
-}
-
-static float2 pair_of(long double x) {
-  const float hi = (float)x;
-  return float2{hi, (float)(x - (long double)hi)};
 }
 
 static void split_axis(int n, int p, int idx, int* off, int* len) {
@@ -524,7 +519,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
             const double h = b.mbase >= 0 ? 1.0 : b.h[a];  // curvilinear: index space
             d.c1[a] = (a_cd / 2.0) / h;
             d.c2[a] = (b_cd / 4.0) / h;
-            d.cg[a] = pair_of(c->p.order == 4 ? d.c2[a] : d.c1[a]);
+            d.cg[a] = cfs::pair_of(c->p.order == 4 ? d.c2[a] : d.c1[a]);
           }
           d.iso = d.c1[0] == d.c1[1] && d.c1[0] == d.c1[2] && d.c2[0] == d.c2[1] && d.c2[0] == d.c2[2];
           const long long npad = (long long)d.ex * d.ey * d.ez;
@@ -591,13 +586,13 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       for (int a = 0; a < 3; ++a) c->pairs = c->pairs && in_range(d.c1[a]) && in_range(d.c2[a]);
     cfs::PairPhysics& pp = c->pphys;
     pp.Eref = (float)ph.E_ref;
-    pp.gm1 = pair_of(ph.gm1);
-    pp.kgM2 = pair_of(ph.kgM2);
-    pp.kT0 = pair_of((long double)ph.kgM2 * ph.gm1 * pp.Eref);
-    pp.H = pair_of((long double)ph.gamma * pp.Eref);
-    pp.ivT = pair_of(ph.ivT);
+    pp.gm1 = cfs::pair_of(ph.gm1);
+    pp.kgM2 = cfs::pair_of(ph.kgM2);
+    pp.kT0 = cfs::pair_of((long double)ph.kgM2 * ph.gm1 * pp.Eref);
+    pp.H = cfs::pair_of((long double)ph.gamma * pp.Eref);
+    pp.ivT = cfs::pair_of(ph.ivT);
     pp.visc_law = ph.visc_law;
-    pp.visc_exp = pair_of(ph.visc_exp);
+    pp.visc_exp = cfs::pair_of(ph.visc_exp);
   }
   // tables of the FP64 power (power-law viscosity)
   if (c->p.viscous && c->p.visc_law == 1) {
@@ -641,7 +636,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
                "upload metrics");
       if (c->pairs) {
         Mp.resize(M.size());
-        for (size_t q = 0; q < M.size(); ++q) Mp[q] = pair_of(M[q]);
+        for (size_t q = 0; q < M.size(); ++q) Mp[q] = cfs::pair_of(M[q]);
         CUDA_TRY(c, cudaMemcpy(c->d_metric_p + b.mbase, Mp.data(), sizeof(float2) * Mp.size(), cudaMemcpyHostToDevice),
                  "upload metrics");
       }
@@ -788,8 +783,9 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   if (c->p.filter && cfs::filter_prepare(c->Lmax, c->p.precision) != 0)
     return fail(c, CFS_EINVAL, "filter: a sub-domain is too long along an axis for the shared-memory line tiles "
                                "(at most about 700 points)");
-  c->diag_blocks = 2 * 152;
-  c->d_partial = (double*)dev_alloc(c, sizeof(double) * DIAG_NQ * c->diag_blocks * c->blocks.size());
+  c->diag_total = 0;
+  for (const Block& b : c->blocks) c->diag_total += cfs::diag_rows(b.nx, b.ny, b.nz, 1 << 16);
+  c->d_partial = (double*)dev_alloc(c, sizeof(double) * DIAG_NQ * (size_t)c->diag_total);
   c->d_thomas = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   c->d_thomas32 = (float*)dev_alloc(c, sizeof(float) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
@@ -1395,9 +1391,11 @@ cfs_status cfs_diagnostics(cfs_ctx* c, double* out) {
       }
       db.sid0 = b.sid0;
     }
-    int rc = cfs::launch_diagnostics_block(c->geo, db, U, c->d_partial, row, c->diag_blocks, c->stream);
+    for (int a = 0; a < 3; ++a) db.cg[a] = cfs::pair_of(c->r == 2 ? db.c2[a] : db.c1[a]);
+    const int rows = cfs::diag_rows(b.nx, b.ny, b.nz, 1 << 16);
+    int rc = cfs::launch_diagnostics_block(db, U, c->d_partial, row, rows, c->stream);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "diagnostics launch");
-    row += c->diag_blocks;
+    row += rows;
   }
   {
     int rc = cfs::launch_diagnostics_final(c->d_partial, row, c->d_out, c->volume, c->stream);

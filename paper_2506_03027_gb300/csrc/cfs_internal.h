@@ -167,6 +167,11 @@ bool buffer_dudt_weights(int order, int e, int k, long double* d);
 int at_weight_table(int order, int kmax, double* W);
 int filter_extrap_table(int order, int kmax, double* Wf);
 bool pade10_coeffs(double alpha, double* a);
+// x as a pair of floats (hi, lo)
+inline float2 pair_of(long double x) {
+  const float hi = (float)x;
+  return float2{hi, (float)(x - (long double)hi)};
+}
 // Block topology (host): faces of the connected multi-block grid.
 enum { FACE_PERIODIC = 0, FACE_INTERFACE = 1, FACE_WALL = 2, FACE_FARFIELD = 3, FACE_OUTFLOW = 4 };
 struct FaceSpec {
@@ -363,6 +368,7 @@ struct DiagBlock {
   int nx, ny, nz;
   long long bN, bbase;
   double c1[3], c2[3], dV;
+  float2 cg[3];     // the coefficient of the unscaled difference (c2 for CD4, c1 for CD2) as a pair
   const double* M;  // the block's metric plane (curvilinear), or null
   int mx, G;        // its row length and extension
   long long mpl;    // its component stride
@@ -376,8 +382,10 @@ struct DiagBlock {
   int P[3], sid0;
 };
 #define DIAG_NQ 9   // per block row: K, enstrophy, 5 totals, non-finite flag, enstrophy volume
-int launch_diagnostics_block(const Geometry& g, const DiagBlock& b, const double* U, double* partial, int row0,
-                             int nblocks, void* stream);
+// Rows of partial sums a block takes (at most `most` unless the fixed general grid needs more), for
+// launch_diagnostics_block's `rows`.
+int diag_rows(int nx, int ny, int nz, int most);
+int launch_diagnostics_block(const DiagBlock& b, const double* U, double* partial, int row0, int rows, void* stream);
 int launch_diagnostics_final(const double* partial, int nrows, double* out, double volume, void* stream);
 int launch_advance_step(long long* dn, void* stream);
 int launch_eval_power(const double* x, double a, double* y, long long n, void* stream);

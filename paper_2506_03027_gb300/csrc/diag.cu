@@ -1,0 +1,323 @@
+// diag.cu -- diagnostics of a state: kinetic energy, enstrophy, totals and the non-finite flag.
+//
+// Per block of points one CTA (a tile of 32 x 8 columns marching through a chunk of z planes) writes
+// one row of partial sums; a last CTA adds the rows in a fixed order.  In FP64 the sums are bound by
+// the FP64 pipe: a reciprocal of the density and six differences per point are about 110 FP64
+// operations at 2 per clock and SM.  Only the five totals need FP64 accumulation point by point; the
+// velocities, their differences and the two squares are formed on pairs of floats (pairs.cuh), a
+// column's few values per chunk added as pairs and the columns in FP64.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "cfs_internal.h"
+#include "device_common.cuh"
+#include "pairs.cuh"
+
+namespace cfs {
+
+namespace {
+
+constexpr int DTX = 32, DTY = 8;
+
+// The five totals, the kinetic energy (x 2) and the enstrophy (x 2, and the volume it covers) of one
+// point in FP64: any block (curvilinear, two-dimensional, not periodic, partitioned), any finite or
+// non-finite value.
+__device__ __noinline__ void diag_point(const DiagBlock& b, const double* __restrict__ U, int x, int y, int z, double* acc) {
+  const int ndim = b.nz > 1 ? 3 : 2;
+  const long long i = (long long)x + (long long)b.nx * ((long long)y + (long long)b.ny * z);
+  const long long mq = (long long)(x + b.G) + (long long)b.mx * (y + b.G);  // metric plane index
+  const double dV = b.M ? b.M[5 * b.mpl + mq] : b.dV;  // cell volume (J^-1 on a curvilinear grid)
+  double u[5];
+  for (int v = 0; v < 5; ++v) {
+    u[v] = U[b.bbase + v * b.bN + i];
+    if (!isfinite(u[v])) acc[7] = 1.0;
+    acc[2 + v] += u[v] * dV;
+  }
+  const double rho = u[0], ir = 1.0 / rho;
+  acc[0] += 0.5 * ir * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * dV;
+  // enstrophy only where the CD stencils stay in the block or cross periodic faces
+  if (b.nonper) {
+    const int c3[3] = {x, y, z}, n3[3] = {b.nx, b.ny, b.nz};
+    for (int a = 0; a < ndim; ++a) {
+      if (((b.nonper >> (2 * a)) & 1) && c3[a] < b.rs) return;
+      if (((b.nonper >> (2 * a + 1)) & 1) && c3[a] > n3[a] - 1 - b.rs) return;
+    }
+  }
+  acc[8] += dV;
+  // velocity differences by the CD scheme, one reciprocal of the density per stencil point
+  double dv[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  for (int a = 0; a < ndim; ++a)
+    for (int o = 1; o <= (b.c2[a] != 0.0 ? 2 : 1); ++o)
+      for (int sd = -1; sd <= 1; sd += 2) {
+        const int xs = x + (a == 0 ? sd * o : 0), ys = y + (a == 1 ? sd * o : 0), zs = z + (a == 2 ? sd * o : 0);
+        const long long gi = b.bbase + (long long)wrapc(xs, b.nx) +
+                             (long long)b.nx * ((long long)wrapc(ys, b.ny) + (long long)b.ny * wrapc(zs, b.nz));
+        const double w = sd * (o == 1 ? b.c1[a] : b.c2[a]) / U[gi];
+        for (int c = 0; c < 3; ++c) dv[c][a] = fma(w, U[(1 + c) * b.bN + gi], dv[c][a]);
+      }
+  if (b.M) {  // index-space derivatives -> physical: d/dx_j = J sum_k (metric row k)_j d/dxi_k
+    const double J = b.M[6 * b.mpl + mq];
+    const double m[3][3] = {{b.M[mq], b.M[b.mpl + mq], 0.0}, {b.M[2 * b.mpl + mq], b.M[3 * b.mpl + mq], 0.0},
+                            {0.0, 0.0, b.M[4 * b.mpl + mq]}};
+    double dp[3][3];
+    for (int c = 0; c < 3; ++c)
+      for (int j = 0; j < 3; ++j) dp[c][j] = J * (m[0][j] * dv[c][0] + m[1][j] * dv[c][1] + m[2][j] * dv[c][2]);
+    for (int c = 0; c < 3; ++c)
+      for (int j = 0; j < 3; ++j) dv[c][j] = dp[c][j];
+  }
+  const double wx = dv[2][1] - dv[1][2], wy = dv[0][2] - dv[2][0], wz = dv[1][0] - dv[0][1];
+  acc[1] += 0.5 * rho * (wx * wx + wy * wy + wz * wz) * dV;
+}
+
+// acc of 256 threads -> one row: warp shuffles, then one thread per quantity over the warp sums.
+__device__ __forceinline__ void diag_row(const double* acc, double* __restrict__ row) {
+  __shared__ double sh[DIAG_NQ][8];
+  const int tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+  for (int c = 0; c < DIAG_NQ; ++c) {
+    double v = acc[c];
+    for (int o = 16; o > 0; o >>= 1) {
+      const double other = __shfl_down_sync(0xffffffffu, v, o);
+      v = (c == 7) ? fmax(v, other) : v + other;
+    }
+    if (lane == 0) sh[c][wid] = v;
+  }
+  __syncthreads();
+  if (tid < DIAG_NQ) {
+    double v = 0.0;
+    for (int w = 0; w < 8; ++w) v = (tid == 7) ? fmax(v, sh[tid][w]) : v + sh[tid][w];
+    row[tid] = v;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_diag(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial) {
+  double acc[DIAG_NQ] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < b.bN; i += (long long)gridDim.x * blockDim.x) {
+    const int x = (int)(i % b.nx), y = (int)((i / b.nx) % b.ny), z = (int)(i / ((long long)b.nx * b.ny));
+    if (b.subs && !b.subs[b.sid0 + b.owner[0][x] + b.P[0] * (b.owner[1][y] + b.P[1] * b.owner[2][z])].own) continue;
+    diag_point(b, U, x, y, z, acc);
+  }
+  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ);
+}
+
+// One differenced pair of values from points -2, -1, 1, 2 (or -1, 1), without its factor.
+template <int R, class V>
+__device__ __forceinline__ Pr<V> diff_pts(Pr<V> m2, Pr<V> m1, Pr<V> p1, Pr<V> p2) {
+  if (R == 1) return p_norm(p_sub(p1, m1));
+  const V m8 = v_bc<V>(-8.f);
+  const Pr<V> x = p_2diff(p2.h, m2.h), y = p_2diff(p1.h, m1.h);
+  const Pr<V> s = p_2sum(x.h, v_mul(m8, y.h));
+  const V lo = v_add(v_fma(m8, y.l, x.l), v_fma(m8, v_sub(p1.l, m1.l), v_sub(p2.l, m2.l)));
+  return p_norm(Pr<V>{s.h, v_add(s.l, lo)});
+}
+
+// Cartesian 3-D block: a CTA marches its tile of columns through planes [z0, z1).  Per plane the
+// velocities of the tile and of R points beyond it in x and y go to one of four shared-memory planes
+// (one barrier per plane), the column's own (u, v) stay in registers for the z differences; plane
+// L - R is finished when plane L has arrived.  A CTA that meets a value outside the pairs' range
+// (a density, a momentum; also NaN and infinity) takes its points in FP64 instead.
+template <int R>
+__global__ void __launch_bounds__(DTX * DTY) k_diag_tile(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial,
+                                                         int tiles_x, int tiles, int zc, int rows) {
+  if ((int)blockIdx.x >= rows) {  // beyond the block's work: a row of zeros
+    const int t = threadIdx.x + DTX * threadIdx.y;
+    if (t < DIAG_NQ) partial[(long long)blockIdx.x * DIAG_NQ + t] = 0.0;
+    return;
+  }
+  constexpr int BX = DTX + 2 * R, BY = DTY + 2 * R, XS = BX + 1;
+  __shared__ float4 sUV[4][BY * XS];
+  __shared__ float2 sW[4][BY * XS];
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + DTX * ty;
+  const int tile = blockIdx.x % tiles, chunk = blockIdx.x / tiles;
+  const int x0 = (tile % tiles_x) * DTX, y0 = (tile / tiles_x) * DTY, z0 = chunk * zc, z1 = min(b.nz, z0 + zc);
+  const int x = x0 + tx, y = y0 + ty;
+  const bool own = x < b.nx && y < b.ny;
+  const long long plane = (long long)b.nx * b.ny;
+  const double* __restrict__ base = U + b.bbase;
+  const long long col = (long long)wrapc(x, b.nx) + (long long)b.nx * wrapc(y, b.ny);
+  // a second point: the R columns beyond the tile in x, the R rows beyond it in y
+  constexpr int NX = 2 * R * DTY, NXY = NX + 2 * R * DTX;
+  int hx = 0, hy = 0;
+  if (tid < NX) {
+    const int c = tid % (2 * R);
+    hx = c < R ? c - R : DTX + c - R;
+    hy = tid / (2 * R);
+  } else if (tid < NXY) {
+    const int r = (tid - NX) / DTX;
+    hx = (tid - NX) % DTX;
+    hy = r < R ? r - R : DTY + r - R;
+  }
+  const long long hcol = (long long)wrapc(x0 + hx, b.nx) + (long long)b.nx * wrapc(y0 + hy, b.ny);
+  const int so = (ty + R) * XS + tx + R, sh = (hy + R) * XS + hx + R;
+  bool bad = false;
+  auto outside = [](double v, int lo) {  // |v| >= 2^60, or below 2^(lo - 1023) (lo > 0)
+    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    return e >= 1023 + 60 || e < lo;
+  };
+  double acc[DIAG_NQ] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  P2 uv[2 * R + 1];     // (u, v) of the column, planes L - 2R .. L
+  P1 rh[R + 1];         // density, planes L - R .. L
+  P1 kin = {0.f, 0.f}, ens = {0.f, 0.f};
+  const P1 cx = {b.cg[0].x, b.cg[0].y}, cy = {b.cg[1].x, b.cg[1].y}, cz = {b.cg[2].x, b.cg[2].y};
+#pragma unroll
+  for (int k = 0; k <= 2 * R; ++k) uv[k] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int k = 0; k <= R; ++k) rh[k] = {0.f, 0.f};
+  int nens = 0;
+  for (int L = z0 - R; L < z1 + R; ++L) {
+    const bool inner = L >= z0 && L < z1;
+    const double* __restrict__ pl = base + plane * wrapc(L, b.nz);
+    double u[5], hu[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) u[v] = pl[v * b.bN + col];
+    if (inner) {
+      u[4] = pl[4 * b.bN + col];
+      if (tid < NXY) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) hu[v] = pl[v * b.bN + hcol];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * R; ++k) uv[k] = uv[k + 1];
+#pragma unroll
+    for (int k = 0; k < R; ++k) rh[k] = rh[k + 1];
+    bad = bad || outside(u[0], 1023 - 60) || outside(u[1], 0) || outside(u[2], 0) || outside(u[3], 0);
+    const P1 rho = p_split(u[0]), ir = p_recip(rho);
+    const P2 mxy = p_pair(p_split(u[1]), p_split(u[2]));
+    uv[2 * R] = p_norm(p_mul(mxy, p_bc(ir)));
+    rh[R] = rho;
+    if (inner) {
+      const P1 mz = p_split(u[3]), w = p_norm(p_mul(mz, ir));
+      sUV[L & 3][so] = p_store(uv[2 * R]);
+      sW[L & 3][so] = p_store(w);
+      if (tid < NXY) {
+        bad = bad || outside(hu[0], 1023 - 60) || outside(hu[1], 0) || outside(hu[2], 0) || outside(hu[3], 0);
+        const P1 hi = p_recip(p_split(hu[0]));
+        sUV[L & 3][sh] = p_store(p_norm(p_mul(p_pair(p_split(hu[1]), p_split(hu[2])), p_bc(hi))));
+        sW[L & 3][sh] = p_store(p_norm(p_mul(p_split(hu[3]), hi)));
+      }
+      if (own) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) acc[2 + v] += u[v];
+        bad = bad || outside(u[4], 0);
+        const P2 k2 = p_mul(mxy, uv[2 * R]);
+        kin = p_norm(p_add(kin, p_norm(p_fma(mz, w, p_add(p_x(k2), p_y(k2))))));
+      }
+    }
+    __syncthreads();
+    const int z = L - R;
+    if (z < z0 || !own) continue;
+    if (b.nonper) {
+      const int c3[3] = {x, y, z}, n3[3] = {b.nx, b.ny, b.nz};
+      bool in = true;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        in = in && !(((b.nonper >> (2 * a)) & 1) && c3[a] < R) && !(((b.nonper >> (2 * a + 1)) & 1) && c3[a] > n3[a] - 1 - R);
+      if (!in) continue;
+    }
+    ++nens;
+    const float4* A = sUV[z & 3] + so;
+    const float2* W = sW[z & 3] + so;
+    auto vw = [&](int o) { const float4 t = A[o]; const float2 w = W[o]; return P2{make_float2(t.y, w.x), make_float2(t.w, w.y)}; };
+    auto uw = [&](int o) { const float4 t = A[o]; const float2 w = W[o]; return P2{make_float2(t.x, w.x), make_float2(t.z, w.y)}; };
+    constexpr int T = R == 2 ? 2 : 1;
+    const P2 dx = p_mul(p_bc(cx), diff_pts<R>(vw(-T), vw(-1), vw(1), vw(T)));                          // d(v, w)/dx
+    const P2 dy = p_mul(p_bc(cy), diff_pts<R>(uw(-T * XS), uw(-XS), uw(XS), uw(T * XS)));              // d(u, w)/dy
+    const P2 dz = p_mul(p_bc(cz), diff_pts<R>(uv[0], uv[R - 1], uv[R + 1], uv[2 * R]));                // d(u, v)/dz
+    const P2 a = p_norm(p_sub(p_pair(p_y(dy), p_x(dz)), p_pair(p_y(dz), p_y(dx))));                    // w_x, w_y
+    const P1 c = p_norm(p_sub(p_x(dx), p_x(dy)));                                                      // w_z
+    const P2 a2 = p_mul(a, a);
+    const P1 w2 = p_norm(p_fma(c, c, p_add(p_x(a2), p_y(a2))));
+    ens = p_norm(p_add(ens, p_norm(p_mul(rh[0], w2))));
+  }
+  if (__syncthreads_or(bad)) {
+    for (int c = 0; c < DIAG_NQ; ++c) acc[c] = 0.0;
+    if (own)
+      for (int z = z0; z < z1; ++z) diag_point(b, U, x, y, z, acc);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) acc[2 + v] *= b.dV;
+    acc[0] = 0.5 * b.dV * ((double)kin.h + (double)kin.l);
+    acc[1] = 0.5 * b.dV * ((double)ens.h + (double)ens.l);
+    acc[8] = nens * b.dV;
+  }
+  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ);
+}
+
+// The rows in a fixed order, a warp per quantity: lane l adds rows l, l + 32, ..., the lanes combine
+// in a fixed tree.  K is a volume average (sum of value x cell volume over the total volume), the
+// enstrophy an average over the volume of the points it covers.
+__global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double* __restrict__ partial, int nrows,
+                                                            double* __restrict__ out, double volume) {
+  __shared__ double tot[DIAG_NQ];
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+#pragma unroll 8
+  for (int r = lane; r < nrows; r += 32) {
+    const double x = partial[(long long)r * DIAG_NQ + c];
+    v = (c == 7) ? fmax(v, x) : v + x;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double other = __shfl_down_sync(0xffffffffu, v, o);
+    v = (c == 7) ? fmax(v, other) : v + other;
+  }
+  if (lane == 0) tot[c] = v;
+  __syncthreads();
+  if (threadIdx.x >= 8) return;
+  const int q = threadIdx.x;
+  double r = tot[q];
+  if (q == 0) r /= volume;
+  if (q == 1) r = tot[8] > 0.0 ? r / tot[8] : 0.0;
+  out[q] = r;
+}
+
+struct TileShape {
+  int tiles_x, tiles, zc;
+  long long rows;
+};
+
+// Planes per CTA: 8 (a quarter of a CTA's plane work is then the 2R planes beyond its chunk) until
+// the rows pass a few thousand, which the last kernel adds in a few microseconds.
+TileShape tile_shape(int nx, int ny, int nz) {
+  TileShape s;
+  s.tiles_x = (nx + DTX - 1) / DTX;
+  const long long t = (long long)s.tiles_x * ((ny + DTY - 1) / DTY);
+  s.tiles = (int)std::min<long long>(t, 1 << 30);
+  s.zc = 8;
+  while (s.zc < nz && t * ((nz + s.zc - 1) / s.zc) > 4096) s.zc *= 2;
+  s.rows = t * ((nz + s.zc - 1) / s.zc);
+  return s;
+}
+
+constexpr int kGeneralRows = 2 * 152;
+
+// the marching kernel: 3-D Cartesian blocks computed here as a whole
+bool tiled(const DiagBlock& b) { return b.nz > 1 && !b.M && !b.subs; }
+
+}  // namespace
+
+int diag_rows(int nx, int ny, int nz, int most) {
+  const TileShape s = tile_shape(nx, ny, nz);
+  return (int)std::max<long long>(kGeneralRows, s.rows <= most ? s.rows : kGeneralRows);
+}
+
+int launch_diagnostics_block(const DiagBlock& b, const double* U, double* partial, int row0, int rows, void* stream) {
+  cudaStream_t st = (cudaStream_t)stream;
+  double* p = partial + (long long)row0 * DIAG_NQ;
+  const TileShape s = tile_shape(b.nx, b.ny, b.nz);
+  if (tiled(b) && s.rows <= rows) {
+    if (b.rs == 2) k_diag_tile<2><<<rows, dim3(DTX, DTY), 0, st>>>(b, U, p, s.tiles_x, s.tiles, s.zc, (int)s.rows);
+    else k_diag_tile<1><<<rows, dim3(DTX, DTY), 0, st>>>(b, U, p, s.tiles_x, s.tiles, s.zc, (int)s.rows);
+  } else {
+    k_diag<<<rows, 256, 0, st>>>(b, U, p);
+  }
+  return (int)cudaGetLastError();
+}
+
+int launch_diagnostics_final(const double* partial, int nrows, double* out, double volume, void* stream) {
+  k_diag_final<<<1, 32 * DIAG_NQ, 0, (cudaStream_t)stream>>>(partial, nrows, out, volume);
+  return (int)cudaGetLastError();
+}
+
+}  // namespace cfs

@@ -1198,109 +1198,6 @@ int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f,
   return (int)cudaGetLastError();
 }
 
-// ------------------------------------------------------------------------------- diagnostics
-
-// Velocity component c at (x, y, z) of a block with periodic wrap.
-__device__ __forceinline__ double vel_at(const double* U, const DiagBlock& b, int x, int y, int z, int c) {
-  const long long gi = b.bbase + (long long)wrapc(x, b.nx) + (long long)b.nx * ((long long)wrapc(y, b.ny) + (long long)b.ny * wrapc(z, b.nz));
-  return U[(1 + c) * b.bN + gi] / U[gi];
-}
-
-__global__ void __launch_bounds__(256) k_diag(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial) {
-  double acc[DIAG_NQ] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  const int ndim = b.nz > 1 ? 3 : 2;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < b.bN; i += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % b.nx), y = (int)((i / b.nx) % b.ny), z = (int)(i / ((long long)b.nx * b.ny));
-    if (b.subs && !b.subs[b.sid0 + b.owner[0][x] + b.P[0] * (b.owner[1][y] + b.P[1] * b.owner[2][z])].own) continue;
-    const long long mq = (long long)(x + b.G) + (long long)b.mx * (y + b.G);  // metric plane index
-    const double dV = b.M ? b.M[5 * b.mpl + mq] : b.dV;  // cell volume (J^-1 on a curvilinear grid)
-    double u[5];
-    for (int v = 0; v < 5; ++v) {
-      u[v] = U[b.bbase + v * b.bN + i];
-      if (!isfinite(u[v])) acc[7] = 1.0;
-      acc[2 + v] += u[v] * dV;
-    }
-    const double rho = u[0];
-    const double vx = u[1] / rho, vy = u[2] / rho, vz = u[3] / rho;
-    acc[0] += 0.5 * rho * (vx * vx + vy * vy + vz * vz) * dV;
-    // enstrophy only where the CD stencils stay in the block or cross periodic faces
-    if (b.nonper) {
-      const int c3[3] = {x, y, z}, n3[3] = {b.nx, b.ny, b.nz};
-      bool inner = true;
-      for (int a = 0; a < ndim; ++a) {
-        if (((b.nonper >> (2 * a)) & 1) && c3[a] < b.rs) inner = false;
-        if (((b.nonper >> (2 * a + 1)) & 1) && c3[a] > n3[a] - 1 - b.rs) inner = false;
-      }
-      if (!inner) continue;
-    }
-    acc[8] += dV;
-    // vorticity by the CD scheme
-    double dv[3][3];
-    for (int c = 0; c < 3; ++c)
-      for (int a = 0; a < 3; ++a) {
-        if (a >= ndim) { dv[c][a] = 0.0; continue; }
-        const int ex = a == 0, ey = a == 1, ez = a == 2;
-        double dd = b.c1[a] * (vel_at(U, b, x + ex, y + ey, z + ez, c) - vel_at(U, b, x - ex, y - ey, z - ez, c));
-        if (b.c2[a] != 0.0)
-          dd += b.c2[a] * (vel_at(U, b, x + 2 * ex, y + 2 * ey, z + 2 * ez, c) -
-                           vel_at(U, b, x - 2 * ex, y - 2 * ey, z - 2 * ez, c));
-        dv[c][a] = dd;
-      }
-    if (b.M) {  // index-space derivatives -> physical: d/dx_j = J sum_k (metric row k)_j d/dxi_k
-      const double J = b.M[6 * b.mpl + mq];
-      const double m[3][3] = {{b.M[mq], b.M[b.mpl + mq], 0.0}, {b.M[2 * b.mpl + mq], b.M[3 * b.mpl + mq], 0.0},
-                              {0.0, 0.0, b.M[4 * b.mpl + mq]}};
-      double dp[3][3];
-      for (int c = 0; c < 3; ++c)
-        for (int j = 0; j < 3; ++j) dp[c][j] = J * (m[0][j] * dv[c][0] + m[1][j] * dv[c][1] + m[2][j] * dv[c][2]);
-      for (int c = 0; c < 3; ++c)
-        for (int j = 0; j < 3; ++j) dv[c][j] = dp[c][j];
-    }
-    const double wx = dv[2][1] - dv[1][2], wy = dv[0][2] - dv[2][0], wz = dv[1][0] - dv[0][1];
-    acc[1] += 0.5 * rho * (wx * wx + wy * wy + wz * wz) * dV;
-  }
-  // block reduction: warp shuffles, then one warp over the warp sums
-  __shared__ double sh[DIAG_NQ][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int c = 0; c < DIAG_NQ; ++c) {
-    double v = acc[c];
-    for (int o = 16; o > 0; o >>= 1) {
-      const double other = __shfl_down_sync(0xffffffffu, v, o);
-      v = (c == 7) ? fmax(v, other) : v + other;
-    }
-    if (lane == 0) sh[c][wid] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < DIAG_NQ) {
-    const int c = threadIdx.x;
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = (c == 7) ? fmax(v, sh[c][w]) : v + sh[c][w];
-    partial[(long long)blockIdx.x * DIAG_NQ + c] = v;
-  }
-}
-
-// Deterministic second pass: one thread per quantity sums the block partials in block order.
-// K is a volume average (sum of value x cell volume over the total volume), the enstrophy an
-// average over the volume of the points it covers.
-__global__ void k_diag_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out, double volume) {
-  const int c = threadIdx.x;
-  if (c >= 8) return;
-  double v = 0.0, ve = 0.0;
-  for (int b = 0; b < nblocks; ++b) {
-    v = (c == 7) ? fmax(v, partial[(long long)b * DIAG_NQ + c]) : v + partial[(long long)b * DIAG_NQ + c];
-    ve += partial[(long long)b * DIAG_NQ + 8];
-  }
-  if (c == 0) v /= volume;
-  if (c == 1) v = ve > 0.0 ? v / ve : 0.0;
-  out[c] = v;
-}
-
-int launch_diagnostics_block(const Geometry& g, const DiagBlock& b, const double* U, double* partial, int row0,
-                             int nblocks, void* stream) {
-  k_diag<<<nblocks, 256, 0, (cudaStream_t)stream>>>(b, U, partial + (long long)row0 * DIAG_NQ);
-  return (int)cudaGetLastError();
-}
-
 __global__ void k_advance_step(long long* dn) {
   pdl_enter();
   if (threadIdx.x == 0 && blockIdx.x == 0) *dn += 1;
@@ -1417,11 +1314,6 @@ int launch_strip_unpack(double* U, const long long* off, const int* bN, long lon
 
 int launch_advance_step(long long* dn, void* stream) {
   launch_pdl(k_advance_step, dim3(1), dim3(32), 0, (cudaStream_t)stream, dn);
-  return (int)cudaGetLastError();
-}
-
-int launch_diagnostics_final(const double* partial, int nrows, double* out, double volume, void* stream) {
-  k_diag_final<<<1, 32, 0, (cudaStream_t)stream>>>(partial, nrows, out, volume);
   return (int)cudaGetLastError();
 }
 
