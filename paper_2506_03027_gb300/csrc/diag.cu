@@ -70,24 +70,27 @@ __device__ __noinline__ void diag_point(const DiagBlock& b, const double* __rest
   acc[1] += 0.5 * rho * (wx * wx + wy * wy + wz * wz) * dV;
 }
 
-// acc of 256 threads -> one row: warp shuffles, then one thread per quantity over the warp sums.
-__device__ __forceinline__ void diag_row(const double* acc, double* __restrict__ row) {
-  __shared__ double sh[DIAG_NQ][8];
+// acc of 256 threads -> one row: through shared memory, a warp per quantity (each lane eight threads'
+// values, then a shuffle tree): a third of the FP64 additions of a tree per warp and quantity.
+// buf: DIAG_NQ x 256 doubles.
+__device__ __forceinline__ void diag_row(const double* acc, double* __restrict__ row, double* buf) {
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31, wid = tid >> 5;
+  __syncthreads();  // (buf may hold what the march read)
 #pragma unroll
-  for (int c = 0; c < DIAG_NQ; ++c) {
-    double v = acc[c];
+  for (int c = 0; c < DIAG_NQ; ++c) buf[c * 256 + tid] = acc[c];
+  __syncthreads();
+  for (int c = wid; c < DIAG_NQ; c += 8) {
+    double v = buf[c * 256 + lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+      const double o = buf[c * 256 + lane + 32 * k];
+      v = (c == 7) ? fmax(v, o) : v + o;
+    }
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_down_sync(0xffffffffu, v, o);
       v = (c == 7) ? fmax(v, other) : v + other;
     }
-    if (lane == 0) sh[c][wid] = v;
-  }
-  __syncthreads();
-  if (tid < DIAG_NQ) {
-    double v = 0.0;
-    for (int w = 0; w < 8; ++w) v = (tid == 7) ? fmax(v, sh[tid][w]) : v + sh[tid][w];
-    row[tid] = v;
+    if (lane == 0) row[c] = v;
   }
 }
 
@@ -98,7 +101,8 @@ __global__ void __launch_bounds__(256) k_diag(DiagBlock b, const double* __restr
     if (b.subs && !b.subs[b.sid0 + b.owner[0][x] + b.P[0] * (b.owner[1][y] + b.P[1] * b.owner[2][z])].own) continue;
     diag_point(b, U, x, y, z, acc);
   }
-  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ);
+  __shared__ double buf[DIAG_NQ * 256];
+  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ, buf);
 }
 
 // One differenced pair of values from points -2, -1, 1, 2 (or -1, 1), without its factor.
@@ -118,7 +122,7 @@ __device__ __forceinline__ Pr<V> diff_pts(Pr<V> m2, Pr<V> m1, Pr<V> p1, Pr<V> p2
 // L - R is finished when plane L has arrived.  A CTA that meets a value outside the pairs' range
 // (a density, a momentum; also NaN and infinity) takes its points in FP64 instead.
 template <int R>
-__global__ void __launch_bounds__(DTX * DTY) k_diag_tile(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial,
+__global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial,
                                                          int tiles_x, int tiles, int zc, int rows) {
   if ((int)blockIdx.x >= rows) {  // beyond the block's work: a row of zeros
     const int t = threadIdx.x + DTX * threadIdx.y;
@@ -242,7 +246,8 @@ __global__ void __launch_bounds__(DTX * DTY) k_diag_tile(DiagBlock b, const doub
     acc[1] = 0.5 * b.dV * ((double)ens.h + (double)ens.l);
     acc[8] = nens * b.dV;
   }
-  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ);
+  static_assert(sizeof(sUV) >= sizeof(double) * DIAG_NQ * 256, "the reduction reuses the planes");
+  diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ, reinterpret_cast<double*>(&sUV[0][0]));
 }
 
 // The rows in a fixed order, a warp per quantity: lane l adds rows l, l + 32, ..., the lanes combine
@@ -277,15 +282,23 @@ struct TileShape {
   long long rows;
 };
 
-// Planes per CTA: 8 (a quarter of a CTA's plane work is then the 2R planes beyond its chunk) until
-// the rows pass a few thousand, which the last kernel adds in a few microseconds.
+// Planes per CTA: the chunk count that takes the least time, waves of 3 CTAs on 152 SMs times the
+// planes a CTA marches (its own and four beyond), a last wave that is nearly empty included.
 TileShape tile_shape(int nx, int ny, int nz) {
   TileShape s;
   s.tiles_x = (nx + DTX - 1) / DTX;
   const long long t = (long long)s.tiles_x * ((ny + DTY - 1) / DTY);
   s.tiles = (int)std::min<long long>(t, 1 << 30);
-  s.zc = 8;
-  while (s.zc < nz && t * ((nz + s.zc - 1) / s.zc) > 4096) s.zc *= 2;
+  s.zc = nz;
+  long long best = -1;
+  for (int c = 1; c <= std::min(nz, 64); ++c) {
+    const int zc = (nz + c - 1) / c;
+    const long long rows = t * ((nz + zc - 1) / zc), cost = ((rows + 455) / 456) * (zc + 4);
+    if (best < 0 || cost < best) {
+      best = cost;
+      s.zc = zc;
+    }
+  }
   s.rows = t * ((nz + s.zc - 1) / s.zc);
   return s;
 }

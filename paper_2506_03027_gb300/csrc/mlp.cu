@@ -15,6 +15,7 @@
 
 #include "cfs_internal.h"
 #include "device_common.cuh"
+#include "launch_common.cuh"
 
 namespace cfs {
 
@@ -22,59 +23,155 @@ namespace {
 
 constexpr int S = 32;  // samples per CTA
 constexpr int NT = 256;
+constexpr int LD = 68;  // row stride in shared memory: 16-byte rows on distinct banks, 65 inputs zero-padded
 
-__device__ __forceinline__ float gelu(float z) {
+// GELU in tanh form and its derivative from one tanh
+__device__ __forceinline__ float gelu(float z, float* grad) {
   const float k0 = 0.7978845608028654f, k1 = 0.044715f;  // sqrt(2/pi)
-  return 0.5f * z * (1.f + tanhf(k0 * (z + k1 * z * z * z)));
+  const float t = tanhf(k0 * (z + k1 * z * z * z));
+  *grad = 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * k0 * (1.f + 3.f * k1 * z * z);
+  return 0.5f * z * (1.f + t);
+}
+__device__ __forceinline__ float gelu(float z) {
+  float g;
+  return gelu(z, &g);
 }
 
-__device__ __forceinline__ float gelu_grad(float z) {
-  const float k0 = 0.7978845608028654f, k1 = 0.044715f;
-  const float u = k0 * (z + k1 * z * z * z);
-  const float t = tanhf(u);
-  return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * k0 * (1.f + 3.f * k1 * z * z);
-}
-
+// The network's weights and a chunk of S samples.  Every product runs from 16-byte shared-memory reads
+// on register tiles (a warp's FMA takes a third of a shared-memory wavefront; one output per thread
+// took two and was bound by them), each output still summed in input order.
 struct Smem {
-  float w[MLP_NPARAM];
-  float x[S][MLP_NIN + 1];
-  float z1[S][MLP_NH], h1[S][MLP_NH], z2[S][MLP_NH], h2[S][MLP_NH], y[S][MLP_NOUT];
+  float w1[MLP_NH * LD], w2[MLP_NH * LD], w3[MLP_NOUT * LD];
+  float b1[MLP_NH], b2[MLP_NH], b3[MLP_NOUT];
+  float x[S * LD];
+  float h1[S * LD], g1[S * LD], h2[S * LD], g2[S * LD];  // activations; derivatives, later the deltas
+  float yt[MLP_NOUT * (S + 4)];                         // outputs, later their deltas: [output][sample]
+  float red[NT / 32];
 };
 
-// dst[s][o] = act(b[o] + sum_i W[o][i] src[s][i]) for s < ns, with z (pre-activation) stored too
-__device__ __forceinline__ void layer(const float* W, const float* b, const float* src, int ld_src, int nin, int nout,
-                                      float* z, float* h, int ld_dst, int ns, bool act) {
-  for (int e = threadIdx.x; e < ns * nout; e += NT) {
-    const int s = e / nout, o = e % nout;
-    float acc = b[o];
-    const float* wr = W + o * nin;
-    const float* xr = src + s * ld_src;
-    for (int i = 0; i < nin; ++i) acc = fmaf(wr[i], xr[i], acc);
-    if (z) z[s * ld_dst + o] = acc;
-    h[s * ld_dst + o] = act ? gelu(acc) : acc;
+// The weights by asynchronous copies, all in flight at once (completed by load_done).
+__device__ __forceinline__ void load_weights(Smem& sm, const float* __restrict__ params) {
+  for (int e = threadIdx.x; e < MLP_NH * MLP_NIN; e += NT) {
+    const int o = e / MLP_NIN, i = e - o * MLP_NIN;
+    cp_async4(sm.w1 + o * LD + i, params + MLP_OFF_W1 + e);
   }
+  for (int e = threadIdx.x; e < MLP_NH * MLP_NH; e += NT) cp_async4(sm.w2 + (e >> 6) * LD + (e & 63), params + MLP_OFF_W2 + e);
+  for (int e = threadIdx.x; e < MLP_NOUT * MLP_NH; e += NT) cp_async4(sm.w3 + (e >> 6) * LD + (e & 63), params + MLP_OFF_W3 + e);
+  if (threadIdx.x < MLP_NH) {
+    cp_async4(sm.b1 + threadIdx.x, params + MLP_OFF_B1 + threadIdx.x);
+    cp_async4(sm.b2 + threadIdx.x, params + MLP_OFF_B2 + threadIdx.x);
+    for (int i = MLP_NIN; i < LD; ++i) sm.w1[threadIdx.x * LD + i] = 0.f;
+  }
+  if (threadIdx.x < MLP_NOUT) cp_async4(sm.b3 + threadIdx.x, params + MLP_OFF_B3 + threadIdx.x);
+  cp_async_commit();
 }
-
-__device__ void load_chunk(Smem& sm, const float* __restrict__ params, const __nv_bfloat16* __restrict__ x, long long base,
-                           int ns) {
-  for (int p = threadIdx.x; p < MLP_NPARAM; p += NT) sm.w[p] = params[p];
-  for (int e = threadIdx.x; e < ns * MLP_NIN; e += NT) {
-    const int s = e / MLP_NIN, i = e % MLP_NIN;
-    sm.x[s][i] = __bfloat162float(x[(base + s) * MLP_NIN + i]);
-  }
+__device__ __forceinline__ void load_done() {
+  cp_async_wait_all();
   __syncthreads();
 }
 
-__device__ void forward_chunk(Smem& sm, int ns) {
-  const float* W1 = sm.w + MLP_OFF_W1;
-  const float* W2 = sm.w + MLP_OFF_W2;
-  const float* W3 = sm.w + MLP_OFF_W3;
-  layer(W1, sm.w + MLP_OFF_B1, &sm.x[0][0], MLP_NIN + 1, MLP_NIN, MLP_NH, &sm.z1[0][0], &sm.h1[0][0], MLP_NH, ns, true);
+// Samples base .. base + ns - 1; the rest of the chunk zero.
+__device__ __forceinline__ void load_samples(Smem& sm, const __nv_bfloat16* __restrict__ x, long long base, int ns) {
+  const __nv_bfloat16* __restrict__ src = x + base * MLP_NIN;
+  constexpr int K = (S * MLP_NIN + NT - 1) / NT;
+  float v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int e = threadIdx.x + k * NT;
+    v[k] = e < ns * MLP_NIN ? __bfloat162float(src[e]) : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int e = threadIdx.x + k * NT, s = e / MLP_NIN, i = e - s * MLP_NIN;
+    if (e < S * MLP_NIN) sm.x[s * LD + i] = v[k];
+  }
+  if (threadIdx.x < S)
+    for (int i = MLP_NIN; i < LD; ++i) sm.x[threadIdx.x * LD + i] = 0.f;
+}
+
+__device__ __forceinline__ float fma4(float4 a, float4 b, float c) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+}
+
+// h[s][o] = GELU(b[o] + sum_i W[o][i] src[s][i]) for 64 outputs, NQ groups of 4 inputs; a thread takes
+// outputs og + 16 k and two samples.  g: the derivative of the activation.
+template <int NQ>
+__device__ __forceinline__ void hidden(const float* W, const float* b, const float* src, float* h, float* g) {
+  const int og = threadIdx.x & 15, s0 = (threadIdx.x >> 4) * 2;
+  float acc[2][4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[0][k] = acc[1][k] = b[og + 16 * k];
+#pragma unroll 4
+  for (int i = 0; i < NQ; ++i) {
+    const float4 x0 = *(const float4*)(src + s0 * LD + 4 * i), x1 = *(const float4*)(src + (s0 + 1) * LD + 4 * i);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 w = *(const float4*)(W + (og + 16 * k) * LD + 4 * i);
+      acc[0][k] = fma4(w, x0, acc[0][k]);
+      acc[1][k] = fma4(w, x1, acc[1][k]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float d;
+      h[(s0 + j) * LD + og + 16 * k] = gelu(acc[j][k], &d);
+      if (g) g[(s0 + j) * LD + og + 16 * k] = d;
+    }
+}
+
+// outputs (transposed) from h2
+__device__ __forceinline__ void outputs(Smem& sm) {
+  if (threadIdx.x < MLP_NOUT * 8) {  // output o, four samples
+    const int o = threadIdx.x % MLP_NOUT, s0 = (threadIdx.x / MLP_NOUT) * 4;
+    float acc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = sm.b3[o];
+#pragma unroll 4
+    for (int i = 0; i < MLP_NH / 4; ++i) {
+      const float4 w = *(const float4*)(sm.w3 + o * LD + 4 * i);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j] = fma4(w, *(const float4*)(sm.h2 + (s0 + j) * LD + 4 * i), acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sm.yt[o * (S + 4) + s0 + j] = acc[j];
+  }
+}
+
+template <bool GRAD>
+__device__ __forceinline__ void forward_chunk(Smem& sm) {
+  hidden<(MLP_NIN + 3) / 4>(sm.w1, sm.b1, sm.x, sm.h1, GRAD ? sm.g1 : nullptr);
   __syncthreads();
-  layer(W2, sm.w + MLP_OFF_B2, &sm.h1[0][0], MLP_NH, MLP_NH, MLP_NH, &sm.z2[0][0], &sm.h2[0][0], MLP_NH, ns, true);
+  hidden<MLP_NH / 4>(sm.w2, sm.b2, sm.h1, sm.h2, GRAD ? sm.g2 : nullptr);
   __syncthreads();
-  layer(W3, sm.w + MLP_OFF_B3, &sm.h2[0][0], MLP_NH, MLP_NH, MLP_NOUT, nullptr, &sm.y[0][0], MLP_NOUT, ns, false);
+  outputs(sm);
   __syncthreads();
+}
+
+// Weight gradient of a layer with NO_ x 64 weights: out[o][i] = sum_s d[s][o] a[s][i], samples in
+// order; a thread takes 4 x 4.  vec: rows of out are 16-byte aligned.
+template <int LDO>
+__device__ __forceinline__ void weight_grad(const float* d, const float* a, float* __restrict__ out, bool vec) {
+  const int i0 = (threadIdx.x & 15) * 4, o0 = (threadIdx.x >> 4) * 4;
+  float g[4][4] = {};
+#pragma unroll 4
+  for (int s = 0; s < S; ++s) {
+    const float4 dv = *(const float4*)(d + s * LD + o0), av = *(const float4*)(a + s * LD + i0);
+    const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, aa[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g[p][q] = fmaf(dd[p], aa[q], g[p][q]);
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    float* r = out + (o0 + p) * LDO + i0;
+    if (LDO % 4 == 0 && vec) *(float4*)r = make_float4(g[p][0], g[p][1], g[p][2], g[p][3]);
+    else
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = g[p][q];
+  }
 }
 
 }  // namespace
@@ -83,11 +180,14 @@ __global__ void __launch_bounds__(NT) k_mlp_fwd(const float* __restrict__ params
                                                  float* __restrict__ y, long long nsamp) {
   extern __shared__ __align__(16) unsigned char raw[];
   Smem& sm = *reinterpret_cast<Smem*>(raw);
+  pdl_enter();
+  load_weights(sm, params);
   for (long long base = (long long)blockIdx.x * S; base < nsamp; base += (long long)gridDim.x * S) {
     const int ns = (int)min((long long)S, nsamp - base);
-    load_chunk(sm, params, x, base, ns);
-    forward_chunk(sm, ns);
-    for (int e = threadIdx.x; e < ns * MLP_NOUT; e += NT) y[base * MLP_NOUT + e] = sm.y[e / MLP_NOUT][e % MLP_NOUT];
+    load_samples(sm, x, base, ns);
+    load_done();
+    forward_chunk<false>(sm);
+    for (int e = threadIdx.x; e < ns * MLP_NOUT; e += NT) y[base * MLP_NOUT + e] = sm.yt[(e % MLP_NOUT) * (S + 4) + e / MLP_NOUT];
     __syncthreads();
   }
 }
@@ -101,92 +201,149 @@ __global__ void __launch_bounds__(NT) k_mlp_bwd(const float* __restrict__ params
   Smem& sm = *reinterpret_cast<Smem*>(raw);
   const long long chunk = blockIdx.x;
   const long long base = chunk * S;
-  if (base >= nsamp) return;
   const int ns = (int)min((long long)S, nsamp - base);
-  load_chunk(sm, params, x, base, ns);
-  forward_chunk(sm, ns);
+  const int tid = threadIdx.x;
+  pdl_enter();
+  load_weights(sm, params);
+  load_samples(sm, x, base, ns);
+  load_done();
+  forward_chunk<true>(sm);
   const float scale = 2.f / ((float)nsamp * MLP_NOUT);
-  // dy (stored over y), loss
-  __shared__ float red[NT];
+  // dy (over the outputs; samples beyond the batch get zero and add nothing below), loss
   float lsum = 0.f;
-  for (int e = threadIdx.x; e < ns * MLP_NOUT; e += NT) {
+  for (int e = tid; e < S * MLP_NOUT; e += NT) {
     const int s = e / MLP_NOUT, o = e % MLP_NOUT;
-    const float d = sm.y[s][o] - target[(base + s) * MLP_NOUT + o];
+    float* y = sm.yt + o * (S + 4) + s;
+    const float d = s < ns ? *y - target[base * MLP_NOUT + e] : 0.f;
     lsum += d * d;
-    sm.y[s][o] = scale * d;
+    *y = scale * d;
   }
-  red[threadIdx.x] = lsum;
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+  if ((tid & 31) == 0) sm.red[tid >> 5] = lsum;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     float t = 0.f;
-    for (int i = 0; i < NT; ++i) t += red[i];
+    for (int i = 0; i < NT / 32; ++i) t += sm.red[i];
     loss_partial[chunk] = t;
   }
-  const float* W2 = sm.w + MLP_OFF_W2;
-  const float* W3 = sm.w + MLP_OFF_W3;
-  // dz2 = (W3^T dy) * gelu'(z2), stored over h2's slot after it is used for dW3 below: keep h2,
-  // write dz2 into z2
-  for (int e = threadIdx.x; e < ns * MLP_NH; e += NT) {
-    const int s = e / MLP_NH, i = e % MLP_NH;
-    float acc = 0.f;
-    for (int o = 0; o < MLP_NOUT; ++o) acc = fmaf(W3[o * MLP_NH + i], sm.y[s][o], acc);
-    sm.z2[s][i] = acc * gelu_grad(sm.z2[s][i]);
+  // dz2 = (W3^T dy) * gelu'(z2), in place of the derivatives; a thread takes input i, eight samples
+  {
+    const int i = tid & 63, s0 = (tid >> 6) * 8;
+    float acc[8] = {};
+#pragma unroll 4
+    for (int o = 0; o < MLP_NOUT; ++o) {
+      const float w = sm.w3[o * LD + i];
+      const float4 a = *(const float4*)(sm.yt + o * (S + 4) + s0), b = *(const float4*)(sm.yt + o * (S + 4) + s0 + 4);
+      const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] = fmaf(w, v[j], acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sm.g2[(s0 + j) * LD + i] *= acc[j];
   }
   __syncthreads();
-  // dz1 = (W2^T dz2) * gelu'(z1), written into z1
-  for (int e = threadIdx.x; e < ns * MLP_NH; e += NT) {
-    const int s = e / MLP_NH, i = e % MLP_NH;
-    float acc = 0.f;
-    for (int o = 0; o < MLP_NH; ++o) acc = fmaf(W2[o * MLP_NH + i], sm.z2[s][o], acc);
-    sm.z1[s][i] = acc * gelu_grad(sm.z1[s][i]);
+  // dz1 = (W2^T dz2) * gelu'(z1), in place; a thread takes four inputs, two samples
+  {
+    const int i0 = (tid & 15) * 4, s0 = (tid >> 4) * 2;
+    float acc[2][4] = {};
+#pragma unroll 4
+    for (int o = 0; o < MLP_NH; o += 4) {
+      const float4 d0 = *(const float4*)(sm.g2 + s0 * LD + o), d1 = *(const float4*)(sm.g2 + (s0 + 1) * LD + o);
+      const float e0[4] = {d0.x, d0.y, d0.z, d0.w}, e1[4] = {d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 w = *(const float4*)(sm.w2 + (o + k) * LD + i0);
+        const float ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc[0][q] = fmaf(ww[q], e0[k], acc[0][q]);
+          acc[1][q] = fmaf(ww[q], e1[k], acc[1][q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sm.g1[(s0 + j) * LD + i0 + q] *= acc[j][q];
   }
   __syncthreads();
   // parameter gradients of this chunk, summed over its samples in order
   float* out = partial + chunk * MLP_NPARAM;
-  for (int p = threadIdx.x; p < MLP_NPARAM; p += NT) {
-    float g = 0.f;
-    if (p < MLP_OFF_B1) {  // W1[o][i]
-      const int o = p / MLP_NIN, i = p % MLP_NIN;
-      for (int s = 0; s < ns; ++s) g = fmaf(sm.z1[s][o], sm.x[s][i], g);
-    } else if (p < MLP_OFF_W2) {
-      const int o = p - MLP_OFF_B1;
-      for (int s = 0; s < ns; ++s) g += sm.z1[s][o];
-    } else if (p < MLP_OFF_B2) {
-      const int q = p - MLP_OFF_W2, o = q / MLP_NH, i = q % MLP_NH;
-      for (int s = 0; s < ns; ++s) g = fmaf(sm.z2[s][o], sm.h1[s][i], g);
-    } else if (p < MLP_OFF_W3) {
-      const int o = p - MLP_OFF_B2;
-      for (int s = 0; s < ns; ++s) g += sm.z2[s][o];
-    } else if (p < MLP_OFF_B3) {
-      const int q = p - MLP_OFF_W3, o = q / MLP_NH, i = q % MLP_NH;
-      for (int s = 0; s < ns; ++s) g = fmaf(sm.y[s][o], sm.h2[s][i], g);
-    } else {
-      const int o = p - MLP_OFF_B3;
-      for (int s = 0; s < ns; ++s) g += sm.y[s][o];
+  // (the caller's workspace may start at any float)
+  const bool vec = ((unsigned long long)partial & 15) == 0 && MLP_NPARAM % 4 == 0 && MLP_OFF_W2 % 4 == 0 && MLP_OFF_W3 % 4 == 0;
+  weight_grad<MLP_NIN>(sm.g1, sm.x, out + MLP_OFF_W1, false);
+  weight_grad<MLP_NH>(sm.g2, sm.h1, out + MLP_OFF_W2, vec);
+  for (int o = tid >> 4; o < MLP_NOUT; o += NT / 16) {  // W3: output o, four inputs
+    const int i0 = (tid & 15) * 4;
+    float g[4] = {};
+#pragma unroll 4
+    for (int s = 0; s < S; ++s) {
+      const float d = sm.yt[o * (S + 4) + s];
+      const float4 a = *(const float4*)(sm.h2 + s * LD + i0);
+      g[0] = fmaf(d, a.x, g[0]);
+      g[1] = fmaf(d, a.y, g[1]);
+      g[2] = fmaf(d, a.z, g[2]);
+      g[3] = fmaf(d, a.w, g[3]);
     }
-    out[p] = g;
+    float* r = out + MLP_OFF_W3 + o * MLP_NH + i0;
+    if (vec) *(float4*)r = make_float4(g[0], g[1], g[2], g[3]);
+    else
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = g[q];
+  }
+  // the last input of W1 and the biases
+  float g = 0.f;
+  if (tid < MLP_NH) {
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) g = fmaf(sm.g1[s * LD + tid], sm.x[s * LD + MLP_NIN - 1], g);
+    out[MLP_OFF_W1 + tid * MLP_NIN + MLP_NIN - 1] = g;
+  } else if (tid < 2 * MLP_NH) {
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) g += sm.g1[s * LD + tid - MLP_NH];
+    out[MLP_OFF_B1 + tid - MLP_NH] = g;
+  } else if (tid < 3 * MLP_NH) {
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) g += sm.g2[s * LD + tid - 2 * MLP_NH];
+    out[MLP_OFF_B2 + tid - 2 * MLP_NH] = g;
+  } else if (tid < 3 * MLP_NH + MLP_NOUT) {
+#pragma unroll 8
+    for (int s = 0; s < S; ++s) g += sm.yt[(tid - 3 * MLP_NH) * (S + 4) + s];
+    out[MLP_OFF_B3 + tid - 3 * MLP_NH] = g;
   }
 }
 
-// grad[p] = sum over chunks (in chunk order); loss = sum of loss partials / (nsamp * NOUT)
-__global__ void k_mlp_reduce(const float* __restrict__ partial, long long nchunk, float* __restrict__ grad,
-                             const float* __restrict__ loss_partial, float* __restrict__ loss, long long nsamp) {
+// grad[p] = sum over chunks (in chunk order, 32 loads in flight); loss = sum of loss partials /
+// (nsamp * NOUT) by the last CTA's first warp (a lane's partials in order, then a fixed tree)
+__global__ void __launch_bounds__(64) k_mlp_reduce(const float* __restrict__ partial, long long nchunk, float* __restrict__ grad,
+                                                   const float* __restrict__ loss_partial, float* __restrict__ loss,
+                                                   long long nsamp) {
+  pdl_enter();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < MLP_NPARAM) {
     float g = 0.f;
-    for (long long c = 0; c < nchunk; ++c) g += partial[c * MLP_NPARAM + p];
+    long long c = 0;
+    for (; c + 32 <= nchunk; c += 32) {
+      float v[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) v[k] = partial[(c + k) * MLP_NPARAM + p];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) g += v[k];
+    }
+    for (; c < nchunk; ++c) g += partial[c * MLP_NPARAM + p];
     grad[p] = g;
   }
-  if (p == 0 && loss) {
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32 && loss) {
     float t = 0.f;
-    for (long long c = 0; c < nchunk; ++c) t += loss_partial[c];
-    *loss = t / ((float)nsamp * MLP_NOUT);
+    for (long long c = threadIdx.x; c < nchunk; c += 32) t += loss_partial[c];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) *loss = t / ((float)nsamp * MLP_NOUT);
   }
 }
 
 // AdamW (Loshchilov & Hutter): decoupled weight decay, bias-corrected moments; step >= 1
 __global__ void k_adamw(float* __restrict__ params, const float* __restrict__ grad, float* __restrict__ m,
                         float* __restrict__ v, int n, int step, float lr, float b1, float b2, float eps, float wd) {
+  pdl_enter();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const float g = grad[p];
@@ -228,7 +385,7 @@ int launch_mlp_forward(const float* params, const void* x_bf16, float* y, long l
   if (int e = set_attr()) return e;
   const long long nchunk = (nsamp + S - 1) / S;
   const unsigned grid = (unsigned)std::min<long long>(nchunk, 152LL * 2);
-  k_mlp_fwd<<<grid, NT, sizeof(Smem), (cudaStream_t)stream>>>(params, (const __nv_bfloat16*)x_bf16, y, nsamp);
+  launch_pdl(k_mlp_fwd, dim3(grid), dim3(NT), sizeof(Smem), (cudaStream_t)stream, params, (const __nv_bfloat16*)x_bf16, y, nsamp);
   return (int)cudaGetLastError();
 }
 
@@ -239,14 +396,16 @@ int launch_mlp_grad(const float* params, const void* x_bf16, const float* target
   float* partial = workspace;
   float* lpart = workspace + nchunk * MLP_NPARAM;
   cudaStream_t st = (cudaStream_t)stream;
-  k_mlp_bwd<<<(unsigned)nchunk, NT, sizeof(Smem), st>>>(params, (const __nv_bfloat16*)x_bf16, target, nsamp, partial, lpart);
-  k_mlp_reduce<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(partial, nchunk, grad, lpart, loss, nsamp);
+  launch_pdl(k_mlp_bwd, dim3((unsigned)nchunk), dim3(NT), sizeof(Smem), st, params, (const __nv_bfloat16*)x_bf16, target, nsamp,
+             partial, lpart);
+  launch_pdl(k_mlp_reduce, dim3((MLP_NPARAM + 63) / 64), dim3(64), 0, st, (const float*)partial, nchunk, grad, (const float*)lpart,
+             loss, nsamp);
   return (int)cudaGetLastError();
 }
 
 int launch_adamw(float* params, const float* grad, float* m, float* v, int n, int step, float lr, float b1, float b2,
                  float eps, float wd, void* stream) {
-  k_adamw<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(params, grad, m, v, n, step, lr, b1, b2, eps, wd);
+  launch_pdl(k_adamw, dim3((n + 63) / 64), dim3(64), 0, (cudaStream_t)stream, params, grad, m, v, n, step, lr, b1, b2, eps, wd);
   return (int)cudaGetLastError();
 }
 
