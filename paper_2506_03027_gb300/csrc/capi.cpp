@@ -121,6 +121,7 @@ struct cfs_ctx {
   int* d_work = nullptr;
   float* Wh = nullptr;
 
+  cfs::Euler2dShape euler2d{0, 0};  // tiles > 0: the stage runs in one launch (euler2d.cu)
   // FP64 form on pairs of floats (3-D Navier-Stokes)
   bool pairs = false;
   cfs::PairPhysics pphys{};
@@ -594,6 +595,10 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     pp.visc_law = ph.visc_law;
     pp.visc_exp = cfs::pair_of(ph.visc_exp);
   }
+  // 2-D inviscid FP64 runs on periodic Cartesian blocks: one launch per stage
+  c->euler2d = {0, 0};
+  if (c->p.precision == 0 && c->ndim == 2 && !c->p.viscous && !c->p.compact && c->all_periodic && mtot == 0)
+    c->euler2d = cfs::euler2d_shape(c->subs.data(), nsub);
   // tables of the FP64 power (power-law viscosity)
   if (c->p.viscous && c->p.visc_law == 1) {
     const int rc = c->pairs ? cfs::pow_pair_tables_init() : cfs::pow_tables_init();
@@ -732,7 +737,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     if (cfs::fused_blocks_per_sm(c->fused_fy, curv ? 1 : 0, &per_sm) != 0 || per_sm < 1)
       return fail(c, CFS_ECUDA, "fused stage kernel does not fit on this device");
     c->fused_grid = std::max(1, std::min(c->nwork, per_sm * std::max(1, sms)));
-  } else {
+  } else if (c->euler2d.tiles == 0) {
     c->Wp = dev_alloc(c, tsz * 7 * (size_t)pbase);
     c->Phi = dev_alloc(c, tsz * 15 * (size_t)pbase);
   }
@@ -791,7 +796,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   for (void* q : c->owned)
     if (!q) return fail(c, CFS_ENOMEM, "device allocation failed");
-  if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && (!c->Wp || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
+  if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && !c->euler2d.tiles && (!c->Wp || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
       !c->d_partial || !c->d_out || !c->d_thomas || !c->d_thomas32 || !c->d_thomas_k)
     return fail(c, CFS_ENOMEM, "device allocation failed");
   for (const Block& b : c->blocks)
@@ -1211,6 +1216,7 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       a.halo = c->d_halo; a.nhalo = c->nhalo;
       a.compact = c->p.compact; a.R = c->Rbuf; a.cthomas = c->d_cthomas; a.Lmax = c->Lmax;
       rc = c->pairs ? cfs::launch_stage_pairs(g, c->pphys, sc, a, c->d_hpair, c->stream, &c->launches, tm)
+           : c->euler2d.tiles ? cfs::launch_euler2d(g, c->phys, sc, a, c->euler2d, c->stream, &c->launches, tm)
                     : cfs::launch_stage(g, c->phys, sc, a, c->p.precision, c->stream, &c->launches, tm);
     } else if (op == c->s && c->fblock_n && !graph && sc.mode != 0) {
       // asynchronous step, FP32 form: the three passes in one launch, straight into level n + 1

@@ -248,6 +248,15 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
                    const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm);
 
+// The stage of 2-D inviscid runs on periodic Cartesian blocks in one launch (euler2d.cu): small or
+// large tiles, and the most tiles a sub-domain has.
+struct Euler2dShape {
+  int small, tiles;
+};
+Euler2dShape euler2d_shape(const SubDev* subs, int nsub);
+int launch_euler2d(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a, Euler2dShape e,
+                   void* stream, long long* launches, const Timer* tm);
+
 // One block as the line filter sees it (device table, one entry per block of a launch).
 struct FilterBlk {
   long long ebase;         // the block's gather map (SubDev::ebase), or -1

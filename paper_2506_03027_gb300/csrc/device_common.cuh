@@ -12,15 +12,14 @@ __device__ __forceinline__ int wrapc(int i, int n) {
   return r < 0 ? r + n : r;
 }
 
-// 1/x for FP64: hardware approximation refined by two Newton-Raphson steps r <- r + r (1 - x r)
-// (Newton's method for the reciprocal; each step squares the relative error).  Within one ulp of
+// 1/x for FP64: the hardware approximation r (20 bits and more) refined by r (1 + e + e^2), e = 1 - x r
+// (the next term of the series, e^3, is below 2^-60): three FP64 operations.  Within one ulp of
 // the correctly rounded quotient for the positive normal densities it is used on.
 __device__ __forceinline__ double recip(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
   return fma(r, e, r);
 }
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
@@ -119,10 +118,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(const unsigned long long* bar,
   }
 }
 
+// n mod R for n >= 0 (a 64-bit remainder takes a hundred instructions more)
+__device__ __forceinline__ int mod_ring(long long n, int R) {
+  return (n >> 31) == 0 ? (int)((unsigned)n % (unsigned)R) : (int)(n % R);
+}
+
 // Delay of face f (0..5) of sub-domain sid at this step, clamped so every level exists.
 __device__ __forceinline__ int face_delay(const StepSched& sc, int sid, int f) {
   int k = 0;
-  if (sc.algo == 1) k = (int)((sc.n - sc.C) % sc.L);
+  if (sc.algo == 1) k = sc.n >= sc.C ? mod_ring(sc.n - sc.C, sc.L) : 0;
   else if (sc.algo == 2) k = sc.table[sid * 6 + f];
   if (k > sc.cap) k = (int)sc.cap;
   if (k < 0) k = 0;
@@ -144,7 +148,7 @@ __device__ __forceinline__ StepSched resolve(StepSched sc) {
 // Ring level n (plus = 0) or n + 1 (plus = 1) when flagged, otherwise the given buffer.
 __device__ __forceinline__ const double* ring_or(const double* p, int flag, const double* ring, const StepSched& sc,
                                                  int plus) {
-  return flag ? ring + (long long)((sc.n + plus) % sc.R) * 5 * sc.Ntot : p;
+  return flag ? ring + (long long)mod_ring(sc.n + plus, sc.R) * 5 * sc.Ntot : p;
 }
 
 }  // namespace cfs

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_filter_block_halo(Geometry g, StepSched
   // wrapped once) and their weights c(k + 1)
   long long lev[2][CFS_MAX_LEVELS];
   double wf[2][CFS_MAX_LEVELS];
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
 #pragma unroll
   for (int sd = 0; sd < 2; ++sd) {
     const int kd = face_delay(sc, sid, 2 * axis + sd);

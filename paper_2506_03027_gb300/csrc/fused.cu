@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
   if ((cj < 0 || cj >= d.sy) && !(gather && ((d.phys >> (cj < 0 ? 2 : 3)) & 1))) kd = max(kd, face_delay(sc, sid, cj < 0 ? 2 : 3));
   if (ck < 0 || ck >= d.sz) kd = max(kd, face_delay(sc, sid, ck < 0 ? 4 : 5));
   // ring slot of level n - kd - l: (n mod R) - kd - l, wrapped once (kd + l < R)
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
   auto slot = [&](int l) { const int q = nR - kd - l; return q < 0 ? q + sc.R : q; };
   if (gather) {
     // beyond a non-periodic block face (a connected grid): the gather entry's sources.  Entries

@@ -98,7 +98,7 @@ __device__ __forceinline__ void view_halo(const Geometry& g, const Physics& ph, 
   const int gx = wrap1(d.ox + ci, d.bnx), gy = wrap1(d.oy + cj, d.bny), gz = wrap1(d.oz + ck, d.bnz);
   const long long gi = d.bbase + (long long)gx + (long long)d.bnx * ((long long)gy + (long long)d.bny * gz);
   // ring slot of level n - kd - l: (n mod R) - kd - l, wrapped once (kd + l < R)
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
   double u[5];
   const int ux = d.ox + ci, uy = d.oy + cj;
   if (d.ebase >= 0 && (ux < 0 || ux >= d.bnx || uy < 0 || uy >= d.bny)) {
@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
     const int nk = (int)min((long long)CFS_MAX_DELAY + 1, max(sc.cap, 0LL) + 1);
     for (int t = threadIdx.x; t < nk * sc.C; t += blockDim.x) {
       const int kd = t / sc.C, l = t % sc.C;
-      sLev[t] = (long long)((sc.n - kd - l) % sc.R) * lvN;
+      sLev[t] = (long long)mod_ring(sc.n - kd - l, sc.R) * lvN;
     }
   }
   __syncthreads();

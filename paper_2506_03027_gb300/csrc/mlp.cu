@@ -452,7 +452,7 @@ __device__ __forceinline__ void column_depth(const Geometry& g, const StepSched&
   column_point(d, f, t1, t2, j, false, c);
   const long long go = global_index(g, d, c);
   // ring slots of levels n, n-k, n-k-1, n-k-2 (k + 2 < R)
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
   auto slot = [&](int back) { const int q = nR - back; return q < 0 ? q + sc.R : q; };
   const double* Lk0 = ring + (long long)slot(k) * lvN;
   const double* Lk1 = ring + (long long)slot(k + 1) * lvN;
@@ -495,7 +495,7 @@ __global__ void k_halo_samples(Geometry g, StepSched sc, const double* __restric
   for (int e = 0; e < MLP_NOUT; ++e) target[i * MLP_NOUT + e] = (float)((truth[e] - at3[e]) * ms.out[e % 5]);
   if (at4) {
     const long long lvN = 5 * g.N;
-    const int nR = (int)(sc.n % sc.R);
+    const int nR = mod_ring(sc.n, sc.R);
     const double* w = sc.W + (long long)k * s * sc.C;  // stage 0: c(k)
     for (int j = 1; j <= MLP_HDEPTH; ++j) {
       int c[3];

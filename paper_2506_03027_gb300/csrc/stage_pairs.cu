@@ -115,7 +115,7 @@ __device__ __forceinline__ void gather_value(const Geometry& g, const StepSched&
                                              const double* __restrict__ Uin, const double* __restrict__ ring, int stage,
                                              int s, double* u) {
   const GatherEntry& E = *h.ent;
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
   const long long lvN = 5 * g.N;
   auto slot = [&](int l) { const int q = nR - kd - l; return (long long)(q < 0 ? q + sc.R : q) * lvN; };
 #pragma unroll
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
   // (entries with an own source are formed from the live stage input by k_view_p)
   if (h.beyond && any_own_source(h, d)) return;
   const long long lvN = 5 * g.N;
-  const int nR = (int)(sc.n % sc.R);
+  const int nR = mod_ring(sc.n, sc.R);
   auto slot = [&](int l) { const int q = nR - kd - l; return (long long)(q < 0 ? q + sc.R : q) * lvN; };
   const int C = sc.mode == 2 ? 1 : sc.C;
   long long lev[CFS_MAX_LEVELS];
