@@ -164,7 +164,7 @@ struct cfs_ctx {
 
   // compact scheme: the flux divergence [5][N] and the Thomas factors of its line systems
   double* Rbuf = nullptr;
-  double* d_cthomas = nullptr;
+  void* d_cthomas = nullptr;  // double, or float2 pairs when `pairs`
 
   // per-kernel event timing
   bool timing = false;
@@ -573,13 +573,13 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     ph.c1[a] = (a_cd / 2.0) / b0.h[a];
     ph.c2[a] = (b_cd / 4.0) / b0.h[a];
   }
-  // The FP64 form of 3-D Navier-Stokes runs its right-hand side on pairs of floats (stage_pairs.cu)
+  // The FP64 form of filtered 3-D runs computes its right-hand side on pairs of floats (stage_pairs.cu)
   // when its constants, and with them a flow's nondimensional values (p about 1/(gamma M^2), rho and
-  // u about 1), lie well inside the FP32 range; the FP64 kernels take what is left, 2-D and
-  // inviscid runs (whose few operations per point leave the FP64 pipe less to do) and the compact
-  // scheme.  Runs without the filter keep the FP64 kernels too: there a step's error against 64-bit
-  // arithmetic is the 5e-17 of the final rounding, which the pairs would raise to 2e-16 at CFL 0.5.
-  c->pairs = c->p.precision == 0 && c->ndim == 3 && c->p.viscous && c->p.filter && !c->p.compact;
+  // u about 1), lie well inside the FP32 range.  Runs without the filter keep the FP64 kernels: there
+  // a step's error against 64-bit arithmetic is the 5e-17 of the final rounding, which the pairs
+  // would raise to 2e-16 at CFL 0.5.  The compact passes hold their lines in shared memory as pairs
+  // of two components (210 points; the scheme itself takes 128).
+  c->pairs = c->p.precision == 0 && c->ndim == 3 && c->p.filter;
   {
     auto in_range = [](double x) { const double a = std::fabs(x); return a == 0.0 || (a > 1e-12 && a < 1e12); };
     c->pairs = c->pairs && in_range(ph.p_ref) && in_range(ph.kappa) && in_range(ph.kgM2) && in_range(ph.ire) && in_range(ph.ivT);
@@ -738,7 +738,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       return fail(c, CFS_ECUDA, "fused stage kernel does not fit on this device");
     c->fused_grid = std::max(1, std::min(c->nwork, per_sm * std::max(1, sms)));
   } else if (c->euler2d.tiles == 0) {
-    c->Wp = dev_alloc(c, tsz * 7 * (size_t)pbase);
+    if (!c->pairs || c->p.viscous) c->Wp = dev_alloc(c, tsz * 7 * (size_t)pbase);
     c->Phi = dev_alloc(c, tsz * 15 * (size_t)pbase);
   }
   c->d_subs = (SubDev*)dev_alloc(c, sizeof(SubDev) * nsub);
@@ -766,7 +766,8 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     if (!c->all_periodic) return fail(c, CFS_EINVAL, "the compact scheme needs blocks periodic on every face");
     if (c->Lmax > CFS_MAX_LINE) return fail(c, CFS_EINVAL, "the compact scheme's sub-domain lines are limited to 128 points");
     c->Rbuf = (double*)dev_alloc(c, sizeof(double) * 5 * (size_t)N);
-    c->d_cthomas = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
+    c->d_cthomas = dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
+    if (c->pairs && cfs::compact_pairs_prepare(c->Lmax) != 0) return fail(c, CFS_ECUDA, "compact passes do not fit this device");
     if (!c->Rbuf || !c->d_cthomas) return fail(c, CFS_ENOMEM, "device allocation failed");
     // Thomas factors of the compact system (unit diagonal, off-diagonals 1/3) per line length
     std::vector<double> ct((size_t)(c->Lmax + 1) * 2 * c->Lmax, 0.0);
@@ -783,6 +784,21 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
         im[i] = 1.0 / m;
       }
     }
+    if (c->pairs) {
+      // the same factors as pairs of floats, eliminated in long double, in the same number of bytes
+      float2* t = (float2*)ct.data();
+      for (int len = 1; len <= c->Lmax; ++len) {
+        float2* cp = t + (size_t)len * 2 * c->Lmax;
+        float2* im = cp + c->Lmax;
+        long double ci = 0.0L;
+        for (int i = 0; i < len; ++i) {
+          const long double m = 1.0L - ci / 3.0L;
+          ci = 1.0L / 3.0L / m;
+          cp[i] = cfs::pair_of(ci);
+          im[i] = cfs::pair_of(1.0L / m);
+        }
+      }
+    }
     CUDA_TRY(c, cudaMemcpy(c->d_cthomas, ct.data(), sizeof(double) * ct.size(), cudaMemcpyHostToDevice), "upload compact factors");
   }
   if (c->p.filter && cfs::filter_prepare(c->Lmax, c->p.precision) != 0)
@@ -796,7 +812,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
   for (void* q : c->owned)
     if (!q) return fail(c, CFS_ENOMEM, "device allocation failed");
-  if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && !c->euler2d.tiles && (!c->Wp || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
+  if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && !c->euler2d.tiles && ((!c->Wp && !(c->pairs && !c->p.viscous)) || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
       !c->d_partial || !c->d_out || !c->d_thomas || !c->d_thomas32 || !c->d_thomas_k)
     return fail(c, CFS_ENOMEM, "device allocation failed");
   for (const Block& b : c->blocks)

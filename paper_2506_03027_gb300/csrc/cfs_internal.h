@@ -227,7 +227,7 @@ struct StageLaunch {
   // length (forward factor c'_i, reciprocal pivot 1 / m_i)
   int compact;
   double* R;
-  const double* cthomas;
+  const void* cthomas;   // double, or float2 on pairs
   int Lmax;
 };
 
@@ -245,6 +245,8 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 // halo states of all s stages once per asynchronous step: H [2 s][nhalo] float4, [s][nhalo] float2.
 int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const StageLaunch& a, const void* H,
                        void* stream, long long* launches, const Timer* tm);
+// (compact scheme: StageLaunch::R holds N float4, N float4, N float2; cthomas the factors as pairs)
+int compact_pairs_prepare(int Lmax);
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
                    const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm);
 

@@ -694,13 +694,13 @@ static int stage_impl(const Geometry& g, const Physics& ph, const StepSched& sc,
     const dim3 gl(nblk(nl, 128), g.nsub);
     if (g.ndim == 3) {
       TIMED(tm, 1, ((g.metric ? k_flux<T, 3, true> : k_flux<T, 3, false>)<<<gf, B, 0, st>>>(g, ph, a.subs, (const T*)a.Wp, (T*)a.Phi)));
-      TIMED(tm, 2, (k_compact_div<T, 0><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, a.cthomas, a.Lmax)));
-      TIMED(tm, 2, (k_compact_div<T, 1><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, a.cthomas, a.Lmax)));
-      TIMED(tm, 2, (k_compact_div<T, 2><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, a.cthomas, a.Lmax)));
+      TIMED(tm, 2, (k_compact_div<T, 0><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, (const double*)a.cthomas, a.Lmax)));
+      TIMED(tm, 2, (k_compact_div<T, 1><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, (const double*)a.cthomas, a.Lmax)));
+      TIMED(tm, 2, (k_compact_div<T, 2><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, (const double*)a.cthomas, a.Lmax)));
     } else {
       TIMED(tm, 1, ((g.metric ? k_flux<T, 2, true> : k_flux<T, 2, false>)<<<gf, B, 0, st>>>(g, ph, a.subs, (const T*)a.Wp, (T*)a.Phi)));
-      TIMED(tm, 2, (k_compact_div<T, 0><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, a.cthomas, a.Lmax)));
-      TIMED(tm, 2, (k_compact_div<T, 1><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, a.cthomas, a.Lmax)));
+      TIMED(tm, 2, (k_compact_div<T, 0><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, (const double*)a.cthomas, a.Lmax)));
+      TIMED(tm, 2, (k_compact_div<T, 1><<<gl, 128, 0, st>>>(g, a.subs, (const T*)a.Phi, a.R, (const double*)a.cthomas, a.Lmax)));
     }
     TIMED(tm, 2, (k_rk_from_R<<<gr, B, 0, st>>>(sc, a.subs, a.R, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A,
                                                 a.B, a.dt, a.first, a.last)));

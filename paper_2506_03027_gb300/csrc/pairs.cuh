@@ -113,24 +113,48 @@ __device__ __forceinline__ P1 p_recip(P1 a) {
   return p_fast2sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
 }
 
-// FP64 -> pair on the integer pipe: x is the exact sum of three floats, its FP32 truncation t and
-// the remaining 29 mantissa bits as 23 + 6 (split_fast's construction); h = t + q1 rounded, l the
-// rest, rounded once (2^-49 |x|).  |x| < 2^-126 gives zero, |x| >= 2^128, infinities and NaN give
-// NaN; below 2^-97 the remaining bits are dropped.
-__device__ __forceinline__ P1 p_split(double x) {
+// FP64 -> the exact sum of three floats on the integer pipe: the FP32 truncation t and the remaining 29
+// mantissa bits as 23 + 6, q1 and q2 (split_fast's construction).  |x| < 2^-126 gives zero, |x| >=
+// 2^128, infinities and NaN give NaN; below 2^-97 the remaining bits are dropped.
+struct Triple {
+  float t, q1, q2;
+};
+__device__ __forceinline__ Triple p_split3(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned ahi = hi & 0x7fffffffu, e = ahi >> 20, sg = hi & 0x80000000u;
   unsigned t = (__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u;
   t = (ahi < 0x38100000u) ? 0u : t;
   t = (ahi >= 0x47f00000u) ? 0x7fc00000u : t;
   const unsigned m = lo & 0x1fffffffu;
-  const unsigned eb1 = (e - 919u) << 23, eb2 = (e - 925u) << 23;  // 2^(E-1046), 2^(E-1052)
+  const unsigned eb1 = ((e - 919u) << 23) | sg, eb2 = ((e - 925u) << 23) | sg;  // +-2^(E-1046), 2^(E-1052)
   const float q1 = __uint_as_float(eb1 | (m >> 6)) - __uint_as_float(eb1);
   const float q2 = __uint_as_float(eb2 | (m & 63u)) - __uint_as_float(eb2);
   const bool ok = e >= 926u;
-  const P1 s = p_fast2sum(__uint_as_float(t), ok ? q1 : 0.f);
-  const float l = __fadd_rn(s.l, ok ? q2 : 0.f);
-  return {__uint_as_float(__float_as_uint(s.h) ^ sg), __uint_as_float(__float_as_uint(l) ^ sg)};
+  return {__uint_as_float(t | sg), ok ? q1 : 0.f, ok ? q2 : 0.f};
+}
+// FP64 -> pair: h = t + q1 rounded, l the rest, rounded once (2^-49 |x|)
+__device__ __forceinline__ P1 p_pair_of(Triple x) {
+  const P1 s = p_fast2sum(x.t, x.q1);
+  return {s.h, __fadd_rn(s.l, x.q2)};
+}
+__device__ __forceinline__ P1 p_split(double x) { return p_pair_of(p_split3(x)); }
+// Two FP64 values as triples, and the difference of two such as pairs: exact but for the last rounding
+// (2^-48 of the difference, however small it is against the values)
+struct Triple2 {
+  float2 t, q1, q2;
+};
+__device__ __forceinline__ Triple2 p_triples(double a, double b) {
+  const Triple x = p_split3(a), y = p_split3(b);
+  return {make_float2(x.t, y.t), make_float2(x.q1, y.q1), make_float2(x.q2, y.q2)};
+}
+__device__ __forceinline__ P2 p_pair_of(Triple2 x) {
+  const P2 s = p_fast2sum(x.t, x.q1);
+  return {s.h, v_add(s.l, x.q2)};
+}
+__device__ __forceinline__ P2 p_diff(Triple2 a, Triple2 b) {
+  const P2 s = p_2diff(a.t, b.t);
+  const P2 r = p_2sum(s.h, v_sub(a.q1, b.q1));
+  return p_norm(P2{r.h, v_add(r.l, v_add(s.l, v_sub(a.q2, b.q2)))});
 }
 // pair -> FP64: one FP64 addition
 __device__ __forceinline__ double p_double(P1 a) { return f2d_fast(a.h) + f2d_fast(a.l); }

@@ -41,25 +41,69 @@ __device__ __forceinline__ WView w_view(void* W, long long P) {
 
 __device__ __forceinline__ P1 cst(float2 c) { return {c.x, c.y}; }
 
-// Primitives of the conserved state at scratch index o: u = (rho, rho u, rho v, rho w, rho E - E_ref).
-__device__ __forceinline__ void store_prims_p(const PairPhysics& ph, const WView& W, long long o, P1 rho, P2 mxy, P1 mz,
-                                              P1 rE) {
+// Primitives of a conserved state (rho E as its deviation from E_ref): velocities, p - p_ref, kappa T and
+// rho E + p - H_ref.
+struct PrimsP {
+  P1 rho, mz, w, p, kT, et;
+  P2 mxy, uv;
+};
+__device__ __forceinline__ PrimsP prims_p(const PairPhysics& ph, P1 rho, P2 mxy, P1 mz, P1 rE) {
+  PrimsP r;
   const P1 ir = p_recip(rho);
-  const P2 uv = p_norm(p_mul(mxy, p_bc(ir)));
-  const P1 w = p_norm(p_mul(mz, ir));
-  const P2 k2 = p_mul(mxy, uv);
-  const P1 ke = p_scale(p_fma(mz, w, p_add(p_x(k2), p_y(k2))), 0.5f);
-  const P1 p = p_norm(p_mul(cst(ph.gm1), p_norm(p_sub(rE, ke))));
-  const P1 kT = p_norm(p_mul(p_norm(p_fma(cst(ph.kgM2), p, cst(ph.kT0))), ir));
-  W.A[o] = p_store(uv);
-  W.B[o] = p_store(p_pair(w, kT));
-  W.C[o] = p_store(p_pair(rho, p));
-  W.D[o] = p_store(p_norm(p_add(rE, p)));
+  r.rho = rho;
+  r.mxy = mxy;
+  r.mz = mz;
+  r.uv = p_norm(p_mul(mxy, p_bc(ir)));
+  r.w = p_norm(p_mul(mz, ir));
+  const P2 k2 = p_mul(mxy, r.uv);
+  const P1 ke = p_scale(p_fma(mz, r.w, p_add(p_x(k2), p_y(k2))), 0.5f);
+  r.p = p_norm(p_mul(cst(ph.gm1), p_norm(p_sub(rE, ke))));
+  r.kT = p_norm(p_mul(p_norm(p_fma(cst(ph.kgM2), r.p, cst(ph.kT0))), ir));
+  r.et = p_norm(p_add(rE, r.p));
+  return r;
+}
+__device__ __forceinline__ PrimsP prims_of(const PairPhysics& ph, const double* u) {
+  return prims_p(ph, p_split(u[0]), p_pair(p_split(u[1]), p_split(u[2])), p_split(u[3]),
+                 p_norm(p_add(p_split(u[4]), P1{-ph.Eref, 0.f})));
+}
+__device__ __forceinline__ void store_prims(const WView& W, long long o, const PrimsP& r) {
+  W.A[o] = p_store(r.uv);
+  W.B[o] = p_store(p_pair(r.w, r.kT));
+  W.C[o] = p_store(p_pair(r.rho, r.p));
+  W.D[o] = p_store(r.et);
 }
 
-__device__ __forceinline__ void store_state_p(const PairPhysics& ph, const WView& W, long long o, const double* u) {
-  store_prims_p(ph, W, o, p_split(u[0]), p_pair(p_split(u[1]), p_split(u[2])), p_split(u[3]),
-                p_norm(p_add(p_split(u[4]), P1{-ph.Eref, 0.f})));
+// Inviscid combined fluxes -F_a (Eq. A2) at scratch index o, along axis `as` or (as < 0) every axis;
+// M: the metric terms of the point on a curvilinear block, or null.  The Cartesian mass flux is the
+// momentum itself.
+__device__ __forceinline__ void store_euler_flux(const PairPhysics& ph, void* Phi, long long P, long long o, const PrimsP& r,
+                                                 int as, const float2* M, long long pl) {
+  float4* __restrict__ F4 = (float4*)Phi;
+  float2* __restrict__ F2 = (float2*)(F4 + 6 * P);
+  const P1 netH = p_neg(p_norm(p_add(r.et, cst(ph.H)))), zero = {0.f, 0.f};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (as >= 0 && as != a) continue;
+    P1 U = a == 0 ? p_x(r.uv) : (a == 1 ? p_y(r.uv) : r.w);
+    P1 n = p_neg(a == 0 ? p_x(r.mxy) : (a == 1 ? p_y(r.mxy) : r.mz));
+    P2 pxy = {make_float2(a == 0 ? r.p.h : 0.f, a == 1 ? r.p.h : 0.f), make_float2(a == 0 ? r.p.l : 0.f, a == 1 ? r.p.l : 0.f)};
+    P1 pz = a == 2 ? r.p : zero;
+    if (M) {
+      if (a < 2) {
+        const P2 row = p_pair(p_of(M[2 * a * pl]), p_of(M[(2 * a + 1) * pl])), x = p_mul(row, r.uv);
+        U = p_norm(p_add(p_x(x), p_y(x)));
+        pxy = p_mul(p_bc(r.p), row);
+      } else {
+        const P1 zz = p_of(M[4 * pl]);
+        U = p_norm(p_mul(zz, r.w));
+        pz = p_mul(zz, r.p);
+      }
+      n = p_norm(p_neg(p_mul(r.rho, U)));
+    }
+    F2[(long long)a * P + o] = p_store(n);
+    F4[(long long)(2 * a) * P + o] = p_store(p_norm(p_sub(p_mul(p_bc(n), r.uv), pxy)));
+    F4[(long long)(2 * a + 1) * P + o] = p_store(p_norm(p_sub(p_mul(p_pair(n, netH), p_pair(r.w, U)), p_pair(pz, zero))));
+  }
 }
 
 // Delay of a halo point: the largest of the faces it lies beyond; faces on a physical boundary of
@@ -218,8 +262,9 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
       }
     }
     // what the sums are added to: U_0, or the network's stage-0 value
-    P1 bx = p_split(x[0]), by = grp < 2 ? p_split(y[0]) : P1{0.f, 0.f};
-    const P2 u0 = p_pair(bx, by);
+    const Triple2 t0 = p_triples(x[0], grp < 2 ? y[0] : 0.0);
+    const P2 u0 = p_pair_of(t0);
+    P1 bx = p_x(u0), by = p_y(u0);
     if (learned) {
       bx = p_split(sc.LH[(long long)v0 * g.Ptot + lh]);
       if (grp < 2) by = p_split(sc.LH[(long long)v1 * g.Ptot + lh]);
@@ -235,7 +280,9 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
 #pragma unroll
     for (int l = 1; l < CFS_MAX_LEVELS; ++l)
       if (l < C) {
-        const P2 dl = p_norm(p_sub(p_pair(p_split(x[l]), grp < 2 ? p_split(y[l]) : P1{0.f, 0.f}), u0));
+        // (the weights of long delays sum to hundreds in magnitude: the differences are taken before
+        // anything is rounded to a pair)
+        const P2 dl = p_diff(p_triples(x[l], grp < 2 ? y[l] : 0.0), t0);
 #pragma unroll
         for (int m = 0; m < S; ++m) {
           const float2 w = __ldg(wt + m * C + l);
@@ -254,15 +301,26 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
 
 // ------------------------------------------------------------------------------- k_view_p
 
-// The stage input as primitives, own points and halo points in one launch (as k_view).
-__global__ void __launch_bounds__(512) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
+// The stage input as primitives, own points and halo points in one launch (as k_view).  EULER: the
+// inviscid fluxes, which need no more than the point itself, instead of the primitives -- along
+// every axis at own points, along the axis of the face a halo point lies beyond.
+template <bool EULER>
+__global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
                                                 const double* __restrict__ ring, int in_ring, const SubDev* __restrict__ subs,
                                                 const int2* __restrict__ halo, long long nhalo, const float4* __restrict__ H4,
                                                 const float2* __restrict__ H2, void* Wp, int stage, int s, int own_blocks) {
   pdl_enter();
   sc = resolve(sc);
   const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
-  const WView W = w_view(Wp, g.Ptot);
+  auto put = [&](const SubDev& d, const PrimsP& r, long long o, int ci, int cj, int as) {
+    if (EULER) {
+      const float2* M = nullptr;
+      if (d.mbase >= 0) M = g.metric_p + d.mbase + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
+      store_euler_flux(ph, Wp, g.Ptot, o, r, as, M, d.mpl);
+    } else {
+      store_prims(w_view(Wp, g.Ptot), o, r);
+    }
+  };
   const long long b = blockIdx.x, nown = (long long)own_blocks * g.nsub;
   if (b < nown) {
     const int sid = (int)(b / own_blocks);
@@ -276,7 +334,7 @@ __global__ void __launch_bounds__(512) k_view_p(Geometry g, PairPhysics ph, Step
     double u[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) u[v] = Uin[d.bbase + v * d.bN + gi];
-    store_state_p(ph, W, d.pbase + q, u);
+    put(d, prims_of(ph, u), d.pbase + q, ci, cj, -1);
     return;
   }
   const long long e = (b - nown) * blockDim.x + threadIdx.x;
@@ -284,24 +342,25 @@ __global__ void __launch_bounds__(512) k_view_p(Geometry g, PairPhysics ph, Step
   const int2 hv = halo[e];
   const SubDev& d = subs[hv.x];
   const long long o = d.pbase + hv.y;
-  if (sc.mode == 0 || d.ebase >= 0) {
-    const HaloPoint h = halo_point(g, d, hv);
-    if (sc.mode == 0 || (h.beyond && any_own_source(h, d))) {
-      double u[5];
-      if (h.beyond) {
-        const int kd = sc.mode == 0 ? 0 : point_delay(sc, d, h.sid, h.ci, h.cj, h.ck, true);
-        gather_value(g, sc, h, d, kd, Uin, ring, stage, s, u);
-      } else {
+  HaloPoint h{};
+  int as = -1;
+  if (EULER || sc.mode == 0 || d.ebase >= 0) h = halo_point(g, d, hv);
+  if (EULER) as = h.ci < 0 || h.ci >= d.sx ? 0 : (h.cj < 0 || h.cj >= d.sy ? 1 : 2);
+  if (sc.mode == 0 || (d.ebase >= 0 && h.beyond && any_own_source(h, d))) {
+    double u[5];
+    if (h.beyond) {
+      const int kd = sc.mode == 0 ? 0 : point_delay(sc, d, h.sid, h.ci, h.cj, h.ck, true);
+      gather_value(g, sc, h, d, kd, Uin, ring, stage, s, u);
+    } else {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) u[v] = Uin[v * d.bN + h.gi];
-      }
-      store_state_p(ph, W, o, u);
-      return;
+      for (int v = 0; v < 5; ++v) u[v] = Uin[v * d.bN + h.gi];
     }
+    put(d, prims_of(ph, u), o, h.ci, h.cj, as);
+    return;
   }
   const int m = sc.mode == 2 ? 0 : stage;
   const P2 a = p_of(H4[(long long)(2 * m) * nhalo + e]), c = p_of(H4[(long long)(2 * m + 1) * nhalo + e]);
-  store_prims_p(ph, W, o, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e]));
+  put(d, prims_p(ph, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e])), o, h.ci, h.cj, as);
 }
 
 // ------------------------------------------------------------------------------- k_flux_p
@@ -529,6 +588,173 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
   }
 }
 
+// ------------------------------------------------------------------------------- compact scheme
+
+// Sixth-order compact derivative (Eq. 2, alpha = 1/3; closure as k_compact_div) of the fluxes along
+// `axis` on pairs, one thread per line and group of components: M (x, y momentum), E (z momentum,
+// energy), N (mass).  In units of b/(4h) the right side is (f_{i+2} - f_{i-2}) + 28 (f_{i+1} -
+// f_{i-1}); the sweeps z_i = rhs_i - c_{i-1} z_{i-1}, x_i = z_i / m_i - c_i x_{i+1} keep z_i in
+// shared memory ([n][LN], LN lines per CTA).  The x pass stages its lines there first (a warp along a
+// line); the y and z passes read the fluxes directly, a warp across 32 lines.  dt R gathers in the
+// pairs R over the x and y passes; the z pass adds its part and takes the low-storage update, so the
+// divergence is neither written nor read a third time.  In FP64 the three passes were bound by
+// their eight operations per value (190 us each at 128^3).
+constexpr int CL = 64;  // lines per CTA
+
+template <class V>
+struct PairMem;
+template <>
+struct PairMem<float2> {
+  using T = float4;
+};
+template <>
+struct PairMem<float> {
+  using T = float2;
+};
+
+template <int axis, class V>
+__device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d, const typename PairMem<V>::T* __restrict__ F,
+                                              typename PairMem<V>::T* __restrict__ R, const float2* __restrict__ cth, int Lmax,
+                                              float2 dt, unsigned char* raw, int grp, const double* __restrict__ Uin,
+                                              double* __restrict__ Uout, double* __restrict__ Q, double A, double B, int first,
+                                              int last) {
+  using T = typename PairMem<V>::T;
+  T* sm = reinterpret_cast<T*>(raw);
+  constexpr int LD = axis == 0 ? CL + 1 : CL;
+  constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  const int sz[3] = {d.sx, d.sy, d.sz};
+  const int n = sz[axis], nl = sz[a1] * sz[a2], tid = threadIdx.x;
+  const int l0 = blockIdx.x * CL, nlines = min(CL, nl - l0);
+  const long long st[3] = {1, d.ex, (long long)d.ex * d.ey}, gst[3] = {1, d.bnx, (long long)d.bnx * d.bny};
+  const long long q0 = d.pbase + g.G + st[1] * g.G + st[2] * g.Gz;
+  const long long r0 = d.bbase / 5 + (long long)d.ox + gst[1] * d.oy + gst[2] * d.oz;
+  // line l of the CTA: its first point in the padded box and in the state's point order
+  auto line_at = [&](int l, long long& q, long long& r) {
+    const int t = l0 + l, t1 = t % sz[a1], t2 = t / sz[a1];
+    q = q0 + t1 * st[a1] + t2 * st[a2];
+    r = r0 + t1 * gst[a1] + t2 * gst[a2];
+  };
+  if (axis == 0) {
+    const int lane = tid & 31;
+    for (int l = tid >> 5; l < nlines; l += CL / 32) {
+      long long q, r;
+      line_at(l, q, r);
+      for (int i = lane; i < n + 8; i += 32) sm[i * LD + l] = F[q + i - 4];
+    }
+    __syncthreads();
+  }
+  const bool act = tid < nlines;
+  long long q = 0, r = 0;
+  if (act) {
+    line_at(tid, q, r);
+    const float2* __restrict__ cp = cth + (long long)n * 2 * Lmax;
+    const float2* __restrict__ im = cp + Lmax;
+    auto f = [&](int i) -> Pr<V> { return p_of(axis == 0 ? sm[(i + 4) * LD + tid] : F[q + i * st[axis]]); };
+    // closures at the first halo points, 0.6 (45 (f_1 - f_-1) - 9 (f_2 - f_-2) + (f_3 - f_-3)), times alpha
+    auto cst1 = [](float h, float l) { return Pr<V>{v_bc<V>(h), v_bc<V>(l)}; };
+    auto closure = [&](Pr<V> d1, Pr<V> d2, Pr<V> d3) {
+      Pr<V> x = p_fma(cst1(45.f, 0.f), d1, d3);
+      x = p_norm(p_fma(cst1(-9.f, 0.f), d2, x));
+      return p_norm(p_mul(cst1(0.2f, -2.9802323e-09f), x));  // 0.6 / 3
+    };
+    Pr<V> w[5];  // f(i - 2) .. f(i + 2)
+    const Pr<V> m4 = f(-4), m3 = f(-3);
+    w[0] = f(-2);
+    w[1] = f(-1);
+    w[2] = f(0);
+    w[3] = f(1);
+    w[4] = f(2);
+    const Pr<V> dl = closure(p_norm(p_sub(w[2], w[0])), p_norm(p_sub(w[3], m3)), p_sub(w[4], m4));
+    Pr<V> z = {v_bc<V>(0.f), v_bc<V>(0.f)};
+    float2 cm = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      Pr<V> rhs = p_fma(cst1(28.f, 0.f), p_norm(p_sub(w[3], w[1])), p_sub(w[4], w[0]));
+      if (i == 0) rhs = p_sub(rhs, dl);
+      if (i == n - 1)
+        rhs = p_sub(rhs, closure(p_norm(p_sub(w[4], w[2])), p_norm(p_sub(f(n + 2), w[1])), p_sub(f(n + 3), w[0])));
+      z = p_norm(p_fma(cst1(-cm.x, -cm.y), z, rhs));
+      // (slot i of the staged x lines holds f(i - 4), no longer read)
+      sm[i * LD + tid] = p_store(z);
+      cm = __ldg(cp + i);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k] = w[k + 1];
+      if (i + 1 < n) w[4] = f(i + 3);
+    }
+    // k = dt b / (4h): the difference coefficient of the block is -1 / (12 h)
+    const P1 k1 = p_norm(p_mul(p_norm(p_mul(P1{dt.x, dt.y}, cst(d.cg[axis]))), P1{-0.33333334f, 9.934108e-09f}));
+    const Pr<V> kk = cst1(k1.h, k1.l);
+    Pr<V> x = {v_bc<V>(0.f), v_bc<V>(0.f)};
+#pragma unroll 4
+    for (int i = n - 1; i >= 0; --i) {
+      const float2 c = __ldg(cp + i), m = __ldg(im + i);
+      x = p_norm(p_fma(cst1(-c.x, -c.y), x, p_mul(cst1(m.x, m.y), p_of(sm[i * LD + tid]))));
+      const Pr<V> kx = p_mul(kk, x);
+      if (axis == 0) {
+        sm[i * LD + tid] = p_store(p_norm(kx));
+      } else {
+        const long long ri = r + (long long)i * gst[axis];
+        const Pr<V> sum = p_norm(p_add(kx, p_of(R[ri])));
+        if (axis == 1) {
+          R[ri] = p_store(sum);
+        } else {
+          const long long pt = ri - d.bbase / 5;
+          auto update = [&](int v, P1 dtR) {
+            const long long gi = d.bbase + (long long)v * d.bN + pt;
+            const double t = p_double(dtR);
+            const double qn = first ? t : fma(A, Q[gi], t);
+            if (!last) Q[gi] = qn;
+            Uout[gi] = fma(B, qn, Uin[gi]);
+          };
+          if constexpr (sizeof(V) == 8) {
+            update(1 + 2 * grp, p_x(sum));
+            update(2 + 2 * grp, p_y(sum));
+          } else {
+            update(0, sum);
+          }
+        }
+      }
+    }
+  }
+  if (axis == 0) {
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int l = tid >> 5; l < nlines; l += CL / 32) {
+      long long ql, rl;
+      line_at(l, ql, rl);
+      for (int i = lane; i < n; i += 32) R[rl + i] = sm[i * LD + l];
+    }
+  }
+}
+
+template <int axis>
+__global__ void __launch_bounds__(CL) k_compact_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
+                                                  const void* __restrict__ Phi, void* __restrict__ Rv,
+                                                  const float2* __restrict__ cth, int Lmax, const double* __restrict__ Uin0,
+                                                  double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
+                                                  int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
+                                                  int last) {
+  extern __shared__ __align__(16) unsigned char craw[];
+  pdl_enter();
+  const SubDev& d = subs[blockIdx.z];
+  constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  const int sz[3] = {d.sx, d.sy, d.sz};
+  if (!d.own || (int)blockIdx.x * CL >= sz[a1] * sz[a2]) return;
+  sc = resolve(sc);
+  const double* Uin = axis == 2 ? ring_or(Uin0, in_ring, ring, sc, 0) : nullptr;
+  double* Uout = axis == 2 ? const_cast<double*>(ring_or(Uout0, out_ring, ring, sc, 1)) : nullptr;
+  const int grp = blockIdx.y;  // 0: M, 1: E, 2: N
+  const long long P = g.Ptot, N = g.N;
+  const float4* F4 = (const float4*)Phi;
+  float4* R4 = (float4*)Rv;
+  if (grp < 2)
+    compact_group<axis, float2>(g, d, F4 + (2 * axis + grp) * P, R4 + grp * N, cth, Lmax, dt, craw, grp, Uin, Uout, Q, A, B,
+                                first, last);
+  else
+    compact_group<axis, float>(g, d, (const float2*)(F4 + 6 * P) + axis * P, (float2*)(R4 + 2 * N), cth, Lmax, dt, craw, grp, Uin,
+                               Uout, Q, A, B, first, last);
+}
+
 // ------------------------------------------------------------------------------- launchers
 
 // The tables of p_pow in the current device's copy of the array, once per device (as
@@ -573,20 +799,61 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   const dim3 gf(nblk(a.max_flux, B), g.nsub), gr(nblk(a.max_own, B), g.nsub);
   const float dth = (float)a.dt;
   const float2 dt = make_float2(dth, (float)(a.dt - (double)dth));
-  TIMED(tm, 0, (launch_pdl(k_view_p, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring, a.in_ring, a.subs, (const int2*)a.halo,
-                           a.nhalo, H4, H2, a.Wp, a.stage, a.s, (int)own_blocks)));
-  auto pick = [&](auto r) {
-    constexpr int R = decltype(r)::value;
-    if (ph.visc_law == 1) return g.metric ? k_flux_p<R, true, true> : k_flux_p<R, false, true>;
-    return g.metric ? k_flux_p<R, true, false> : k_flux_p<R, false, false>;
-  };
-  const auto flux = g.r == 2 ? pick(std::integral_constant<int, 2>{}) : pick(std::integral_constant<int, 1>{});
-  TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi)));
+  // (inviscid: the fluxes come straight from the view)
+  TIMED(tm, 0, (launch_pdl(g.viscous ? k_view_p<false> : k_view_p<true>, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring,
+                           a.in_ring, a.subs, (const int2*)a.halo, a.nhalo, H4, H2, g.viscous ? a.Wp : a.Phi, a.stage, a.s,
+                           (int)own_blocks)));
+  if (launches) *launches += 1;
+  if (a.compact) {
+    // x and y passes gather dt R, the z pass takes the update
+    const size_t slots = (size_t)a.Lmax * CL, staged = (size_t)(a.Lmax + 8) * (CL + 1);
+    const dim3 gc(nblk((long long)a.Lmax * a.Lmax, CL), 3, g.nsub);
+    const float2* cth = (const float2*)a.cthomas;
+    auto run = [&](auto kernel, size_t smem) {
+      TIMED(tm, 2, (launch_pdl(kernel, gc, dim3(CL), smem * sizeof(float4), st, g, sc, a.subs, (const void*)a.Phi, (void*)a.R, cth,
+                               a.Lmax, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last)));
+    };
+    run(k_compact_p<0>, staged);
+    run(k_compact_p<1>, slots);
+    run(k_compact_p<2>, slots);
+    if (launches) *launches += 3;
+    return (int)cudaGetLastError();
+  }
+  if (g.viscous) {
+    auto pick = [&](auto r) {
+      constexpr int R = decltype(r)::value;
+      if (ph.visc_law == 1) return g.metric ? k_flux_p<R, true, true> : k_flux_p<R, false, true>;
+      return g.metric ? k_flux_p<R, true, false> : k_flux_p<R, false, false>;
+    };
+    const auto flux = g.r == 2 ? pick(std::integral_constant<int, 2>{}) : pick(std::integral_constant<int, 1>{});
+    TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi)));
+    if (launches) *launches += 1;
+  }
   auto rk = g.r == 2 ? k_rk_p<2> : k_rk_p<1>;
   TIMED(tm, 2, (launch_pdl(rk, gr, dim3(B), 0, st, g, sc, a.subs, (const void*)a.Phi, a.Uin, a.Uout, a.ring, a.in_ring,
                            a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last)));
-  if (launches) *launches += 3;
+  if (launches) *launches += 1;
   return (int)cudaGetLastError();
+}
+
+// The shared-memory opt-in of the compact passes for lines of up to Lmax points: a per-device attribute
+// shared by every context, so it only ever rises (as filter_prepare).
+int compact_pairs_prepare(int Lmax) {
+  const size_t sm = (size_t)(Lmax + 8) * (CL + 1) * sizeof(float4);
+  if (sm > 227 * 1024) return (int)cudaErrorInvalidValue;
+  static std::mutex mu;
+  static int set_to[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return (int)e;
+  if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(mu);
+  if ((int)sm <= set_to[dev]) return 0;
+  e = cudaFuncSetAttribute(k_compact_p<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_compact_p<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_compact_p<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess) set_to[dev] = (int)sm;
+  return (int)e;
 }
 
 }  // namespace cfs
