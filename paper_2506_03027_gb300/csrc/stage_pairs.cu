@@ -594,12 +594,17 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
 // `axis` on pairs, one thread per line and group of components: M (x, y momentum), E (z momentum,
 // energy), N (mass).  In units of b/(4h) the right side is (f_{i+2} - f_{i-2}) + 28 (f_{i+1} -
 // f_{i-1}); the sweeps z_i = rhs_i - c_{i-1} z_{i-1}, x_i = z_i / m_i - c_i x_{i+1} keep z_i in
-// shared memory ([n][LN], LN lines per CTA).  The x pass stages its lines there first (a warp along a
-// line); the y and z passes read the fluxes directly, a warp across 32 lines.  dt R gathers in the
+// shared memory ([n][CL], CL lines per CTA), where every line is staged first with all its loads in
+// flight (x: a warp along a line, y and z: a warp across 32 lines).  dt R gathers in the
 // pairs R over the x and y passes; the z pass adds its part and takes the low-storage update, so the
 // divergence is neither written nor read a third time.  In FP64 the three passes were bound by
 // their eight operations per value (190 us each at 128^3).
 constexpr int CL = 64;  // lines per CTA
+
+__device__ __forceinline__ void cp_async_pair(float4* dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_pair(float2* dst, const float2* src) { cp_async8(dst, src); }
 
 template <class V>
 struct PairMem;
@@ -634,22 +639,26 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
     q = q0 + t1 * st[a1] + t2 * st[a2];
     r = r0 + t1 * gst[a1] + t2 * gst[a2];
   };
+  const bool act = tid < nlines;
+  long long q = 0, r = 0;
+  if (act) line_at(tid, q, r);
   if (axis == 0) {
     const int lane = tid & 31;
     for (int l = tid >> 5; l < nlines; l += CL / 32) {
-      long long q, r;
-      line_at(l, q, r);
-      for (int i = lane; i < n + 8; i += 32) sm[i * LD + l] = F[q + i - 4];
+      long long ql, rl;
+      line_at(l, ql, rl);
+      for (int i = lane; i < n + 8; i += 32) cp_async_pair(sm + i * LD + l, F + ql + i - 4);
     }
-    __syncthreads();
+  } else if (act) {
+    for (int i = 0; i < n + 8; ++i) cp_async_pair(sm + i * LD + tid, F + q + (i - 4) * st[axis]);
   }
-  const bool act = tid < nlines;
-  long long q = 0, r = 0;
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
   if (act) {
-    line_at(tid, q, r);
     const float2* __restrict__ cp = cth + (long long)n * 2 * Lmax;
     const float2* __restrict__ im = cp + Lmax;
-    auto f = [&](int i) -> Pr<V> { return p_of(axis == 0 ? sm[(i + 4) * LD + tid] : F[q + i * st[axis]]); };
+    auto f = [&](int i) -> Pr<V> { return p_of(sm[(i + 4) * LD + tid]); };
     // closures at the first halo points, 0.6 (45 (f_1 - f_-1) - 9 (f_2 - f_-2) + (f_3 - f_-3)), times alpha
     auto cst1 = [](float h, float l) { return Pr<V>{v_bc<V>(h), v_bc<V>(l)}; };
     auto closure = [&](Pr<V> d1, Pr<V> d2, Pr<V> d3) {
@@ -674,7 +683,7 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
       if (i == n - 1)
         rhs = p_sub(rhs, closure(p_norm(p_sub(w[4], w[2])), p_norm(p_sub(f(n + 2), w[1])), p_sub(f(n + 3), w[0])));
       z = p_norm(p_fma(cst1(-cm.x, -cm.y), z, rhs));
-      // (slot i of the staged x lines holds f(i - 4), no longer read)
+      // (slot i held f(i - 4), no longer read)
       sm[i * LD + tid] = p_store(z);
       cm = __ldg(cp + i);
 #pragma unroll
@@ -685,33 +694,57 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
     const P1 k1 = p_norm(p_mul(p_norm(p_mul(P1{dt.x, dt.y}, cst(d.cg[axis]))), P1{-0.33333334f, 9.934108e-09f}));
     const Pr<V> kk = cst1(k1.h, k1.l);
     Pr<V> x = {v_bc<V>(0.f), v_bc<V>(0.f)};
-#pragma unroll 4
-    for (int i = n - 1; i >= 0; --i) {
-      const float2 c = __ldg(cp + i), m = __ldg(im + i);
-      x = p_norm(p_fma(cst1(-c.x, -c.y), x, p_mul(cst1(m.x, m.y), p_of(sm[i * LD + tid]))));
-      const Pr<V> kx = p_mul(kk, x);
-      if (axis == 0) {
-        sm[i * LD + tid] = p_store(p_norm(kx));
-      } else {
+    constexpr bool two = sizeof(V) == 8;
+    // four points at a time, what they read from memory in flight before the first is solved
+    for (int i0 = n - 1; i0 >= 0; i0 -= 4) {
+      T rv[4];
+      double qv[4][2], uv[4][2];
+      if (axis > 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (i0 - k >= 0) {
+            const long long ri = r + (long long)(i0 - k) * gst[axis], pt = ri - d.bbase / 5;
+            rv[k] = R[ri];
+            if (axis == 2) {
+#pragma unroll
+              for (int v = 0; v < (two ? 2 : 1); ++v) {
+                const long long gi = d.bbase + (long long)(two ? 1 + 2 * grp + v : 0) * d.bN + pt;
+                qv[k][v] = first ? 0.0 : Q[gi];
+                uv[k][v] = Uin[gi];
+              }
+            }
+          }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 - k;
+        if (i < 0) break;
+        const float2 c = __ldg(cp + i), m = __ldg(im + i);
+        x = p_norm(p_fma(cst1(-c.x, -c.y), x, p_mul(cst1(m.x, m.y), p_of(sm[i * LD + tid]))));
+        const Pr<V> kx = p_mul(kk, x);
+        if (axis == 0) {
+          sm[i * LD + tid] = p_store(p_norm(kx));
+          continue;
+        }
         const long long ri = r + (long long)i * gst[axis];
-        const Pr<V> sum = p_norm(p_add(kx, p_of(R[ri])));
+        const Pr<V> sum = p_norm(p_add(kx, p_of(rv[k])));
         if (axis == 1) {
           R[ri] = p_store(sum);
+          continue;
+        }
+        const long long pt = ri - d.bbase / 5;
+        auto update = [&](int v, int comp, P1 dtR) {
+          const long long gi = d.bbase + (long long)comp * d.bN + pt;
+          const double t = p_double(dtR);
+          const double qn = first ? t : fma(A, qv[k][v], t);
+          if (!last) Q[gi] = qn;
+          Uout[gi] = fma(B, qn, uv[k][v]);
+        };
+        if constexpr (two) {
+          update(0, 1 + 2 * grp, p_x(sum));
+          update(1, 2 + 2 * grp, p_y(sum));
         } else {
-          const long long pt = ri - d.bbase / 5;
-          auto update = [&](int v, P1 dtR) {
-            const long long gi = d.bbase + (long long)v * d.bN + pt;
-            const double t = p_double(dtR);
-            const double qn = first ? t : fma(A, Q[gi], t);
-            if (!last) Q[gi] = qn;
-            Uout[gi] = fma(B, qn, Uin[gi]);
-          };
-          if constexpr (sizeof(V) == 8) {
-            update(1 + 2 * grp, p_x(sum));
-            update(2 + 2 * grp, p_y(sum));
-          } else {
-            update(0, sum);
-          }
+          update(0, 0, sum);
         }
       }
     }
@@ -806,7 +839,7 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   if (launches) *launches += 1;
   if (a.compact) {
     // x and y passes gather dt R, the z pass takes the update
-    const size_t slots = (size_t)a.Lmax * CL, staged = (size_t)(a.Lmax + 8) * (CL + 1);
+    const size_t slots = (size_t)(a.Lmax + 8) * CL, staged = (size_t)(a.Lmax + 8) * (CL + 1);
     const dim3 gc(nblk((long long)a.Lmax * a.Lmax, CL), 3, g.nsub);
     const float2* cth = (const float2*)a.cthomas;
     auto run = [&](auto kernel, size_t smem) {
