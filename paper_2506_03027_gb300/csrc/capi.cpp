@@ -77,6 +77,7 @@ struct cfs_ctx {
   double* d_Wf = nullptr;
   float* d_W32 = nullptr;   // pairs of W for level-difference sums, then pairs of W - W^(0)
   float* d_W32d = nullptr;
+  float* d_Wf32 = nullptr;  // pairs of Wf likewise
   SubDev* d_subs = nullptr;
   std::vector<SubDev> subs;
   int max_pad = 0, max_own = 0, max_flux = 0;
@@ -727,7 +728,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     }
     c->nwork = (int)(work.size() / 4);
     c->d_work = (int*)dev_alloc(c, sizeof(int) * work.size());
-    c->Wh = (float*)dev_alloc(c, sizeof(float) * 7 * c->s * (size_t)pbase);
+    c->Wh = (float*)dev_alloc(c, sizeof(float) * 8 * c->s * (size_t)pbase);
     if (!c->d_work || !c->Wh) return fail(c, CFS_ENOMEM, "device allocation failed");
     CUDA_TRY(c, cudaMemcpy(c->d_work, work.data(), sizeof(int) * work.size(), cudaMemcpyHostToDevice), "upload work list");
     int dev = 0, sms = 0;
@@ -745,8 +746,9 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   const int nW = (max_delay + 1) * c->s * c->C, nWf = (max_delay + 1) * c->C;
   c->d_W = (double*)dev_alloc(c, sizeof(double) * nW);
   c->d_Wf = (double*)dev_alloc(c, sizeof(double) * nWf);
-  c->d_W32 = (float*)dev_alloc(c, sizeof(float) * 4 * nW);
+  c->d_W32 = (float*)dev_alloc(c, sizeof(float) * (4 * nW + 2 * nWf));
   c->d_W32d = c->d_W32 ? c->d_W32 + 2 * (size_t)nW : nullptr;
+  c->d_Wf32 = c->d_W32 ? c->d_W32 + 4 * (size_t)nW : nullptr;
   c->d_out = (double*)dev_alloc(c, sizeof(double) * 8);
   c->d_n = (long long*)dev_alloc(c, sizeof(long long));
   c->d_status = (int*)dev_alloc(c, sizeof(int));
@@ -886,7 +888,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   // the AT weights for sums over the differences of the delayed levels from the newest one, as
   // pairs of floats (hi, lo = the rest of the FP64 value): per delay and stage S - 1 (S = sum_l W_l,
   // summed in a fixed order) and W_1 .. W_{C-1}; then the same for W^(m) - W^(0)
-  std::vector<float> W32(4 * (size_t)nW);
+  std::vector<float> W32(4 * (size_t)nW + 2 * (size_t)nWf);
   auto pair = [&](size_t i, double x) {
     W32[2 * i] = (float)x;
     W32[2 * i + 1] = (float)(x - (double)W32[2 * i]);
@@ -904,6 +906,14 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       pair(base, tab ? sum : sum - 1.0);
       for (int l = 1; l < c->C; ++l) pair(base + l, x[l]);
     }
+  for (int k = 0; k <= max_delay; ++k) {
+    const double* w = Wf.data() + (size_t)k * c->C;
+    double sum = 0.0;
+    for (int l = 0; l < c->C; ++l) sum += w[l];
+    const size_t base = 2 * (size_t)nW + (size_t)k * c->C;
+    pair(base, sum - 1.0);
+    for (int l = 1; l < c->C; ++l) pair(base + l, w[l]);
+  }
   double filt[6] = {1, 0, 0, 0, 0, 0};
   if (c->p.filter && !cfs::pade10_coeffs(c->p.alpha_f, filt)) return fail(c, CFS_EINVAL, "filter coefficients failed");
   c->filt_h[0] = filt[0];
@@ -1132,6 +1142,7 @@ static int launch_fblock(cfs_ctx* c, const Geometry& g, const StepSched& sc, con
   for (int m = 0; m < 6; ++m) f.h[m] = c->filt_h[m];
   f.b1 = c->filt_h[1] - c->p.alpha_f;
   f.halo = c->d_fbhalo;
+  f.halo_done = c->fused;
   const cfs::Timer* tm = (c->timing && !graph) ? &c->timer : nullptr;
   return cfs::launch_filter_block(g, sc, f, c->fblock_n, c->stream, &c->launches, tm);
 }
@@ -1172,6 +1183,7 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
   sc.W32 = c->d_W32;
   sc.W32d = c->d_W32d;
   sc.Wf = c->d_Wf;
+  sc.Wf32 = c->d_Wf32;
   sc.LH = nullptr;
   sc.status = c->d_status;
   sc.table = nullptr;
@@ -1192,8 +1204,11 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
     sc.LH = c->LH;
   }
   if (c->fused && (graph || sc.mode != 0)) {
-    const int rc = cfs::launch_halo_prims(g, c->phys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->Wh, c->s, c->stream,
-                                          &c->launches, tm);
+    const int rc = c->fblock_n
+                       ? cfs::launch_halo_block(g, c->phys, sc, c->ring, c->d_subs, c->fblock_n, c->Wh, c->d_fbhalo, c->stream,
+                                                &c->launches, tm)
+                       : cfs::launch_halo_prims(g, c->phys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->Wh, c->s, c->stream,
+                                                &c->launches, tm);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
   }
   if (c->pairs && (graph || sc.mode != 0)) {

@@ -148,6 +148,8 @@ struct StepSched {
   const float* W32;      // device: the same table for sums over level differences as pairs of floats
                          // (hi, lo) per entry: entry l = 0 holds sum_l W - 1, entries l >= 1 W_l
   const float* W32d;     // device: as W32 for the differences W^(m) - W^(0) (learned face halos)
+  const float* Wf32;     // device: Wf likewise as pairs for sums over level differences: entry l = 0 holds
+                         // sum_l c - 1, entries l >= 1 c_l
   const double* LH;      // device: learned stage-0 face-halo values [5][Ptot], or null (plain AT)
   const double* Wf;      // device: filter-halo extrapolation weights c(k+1) [k * C + l]
   // CUDA-graph mode: the step index lives in device memory (dn); kernels derive n, mode, cap and
@@ -312,9 +314,11 @@ struct FilterBlockLaunch {
   double alpha;
   double h[6];
   double b1;
-  // the passes' halos as FP32 deviations from the (sub-domain, variable) reference value,
-  // [nsub * 5][3 axes][10][N * N], written by k_filter_block_halo
+  // the passes' halos as FP32 deviations from the (sub-domain, variable) reference value (its first own
+  // value of level n), [nsub * 5][3 axes][10][N * N], written by k_filter_block_halo, or by k_halo_block
+  // (fused.cu) at the start of the step: halo_done
   float* halo;
+  int halo_done;
 };
 bool filter_block_supported(int n);
 int launch_filter_block(const Geometry& g, const StepSched& sc, const FilterBlockLaunch& f, int n, void* stream,
@@ -335,7 +339,7 @@ struct FusedLaunch {
   int nwork;
   int grid;             // persistent grid size
   int fy;               // tile height: 4, 8 or 16 (tile width 32)
-  const float* Wh;      // per-step AT/AS halo primitives [s][7][Ptot]
+  const float* Wh;      // per-step AT/AS halo primitives [s][Ptot][8]
   int stage;
   double A, B, dt;
   int first, last;
@@ -348,6 +352,9 @@ int fused_blocks_per_sm(int fy, int curv, int* blocks);  // sets the shared-memo
 int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
                       const int* halo, long long nhalo, float* Wh, int s, void* stream, long long* launches,
                       const Timer* tm);
+// The halo store together with the sub-domain filter's halos (cubic sub-domains of n points)
+int launch_halo_block(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs, int n,
+                      float* Wh, float* fh, void* stream, long long* launches, const Timer* tm);
 int launch_stage_fused(const Geometry& g, const Physics& ph, const StepSched& sc, const FusedLaunch& a, void* stream,
                        long long* launches, const Timer* tm);
 

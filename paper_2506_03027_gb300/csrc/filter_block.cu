@@ -39,14 +39,13 @@ __host__ __device__ inline size_t fb_smem(void) {
 // The halos of one (sub-domain, variable, pass): 5 points beyond each end of every line, from the
 // ring (wrapped in the block): AT the extrapolation to t_{n+1} with the weights c(k+1) of the C
 // delayed levels in FP64, AS the latest visible level; stored as FP32 deviations from the
-// sub-domain's reference value (its first own value of the filter input), [10][N * N] per pass.
+// sub-domain's reference value (its first own value of level n), [10][N * N] per pass.
 // Items are ordered so that consecutive threads read consecutive points: h fastest for the x pass
 // (the 5 points of an end are adjacent in x), the line (x fastest) otherwise.
 template <int N>
 __global__ void __launch_bounds__(256) k_filter_block_halo(Geometry g, StepSched sc, FilterBlockLaunch f) {
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: the per-pass kernels filter it
-  const double* __restrict__ Uin = ring_or(f.Uin, f.in_ring, f.ring, sc, 0);
   const int b = blockIdx.x;  // (sub-domain, variable, axis); the CTA loops over its 10 N^2 values
   const int sid = b / 15, var = (b / 3) % 5, axis = b % 3;
   const SubDev d = f.subs[sid];
@@ -54,7 +53,7 @@ __global__ void __launch_bounds__(256) k_filter_block_halo(Geometry g, StepSched
   const long long vbase = d.bbase + (long long)var * d.bN;
   const long long lvN = 5 * g.N;
   const long long own0 = (long long)d.ox + (long long)d.bnx * d.oy + plane * d.oz;
-  const double ref = Uin[vbase + own0];
+  const double ref = f.ring[(long long)mod_ring(sc.n, sc.R) * lvN + vbase + own0];
   const float rh = d2f_fast(ref), rl = dev_fast(ref, rh, 0.f);
   // strides along the pass axis and the two line axes (x fastest), the wrap length along the axis
   const long long sA = axis == 0 ? 1 : (axis == 1 ? (long long)d.bnx : plane);
@@ -118,7 +117,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) k_filter_block(Geometry g, Step
   const double* __restrict__ U = Uin + vbase;
   double* __restrict__ Uo = Uout + vbase;
   const long long own0 = (long long)d.ox + (long long)d.bnx * d.oy + plane * d.oz;
-  const double ref = U[own0];
+  const double ref = f.ring[(long long)mod_ring(sc.n, sc.R) * 5 * g.N + vbase + own0];
   const float rh = d2f_fast(ref), rl = dev_fast(ref, rh, 0.f);
   // Thomas factors of a line of N points (the same on every axis)
   for (int t = tid; t < 2 * N; t += FB_THREADS) {
@@ -228,14 +227,14 @@ int launch_filter_block(const Geometry& g, const StepSched& sc, const FilterBloc
   if (tm) tm->rec(tm->self, 3, 1);
   const unsigned nb = (unsigned)(5 * f.nsub);
   if (n == 32) {
-    k_filter_block_halo<32><<<(unsigned)(15 * f.nsub), 256, 0, st>>>(g, sc, f);
+    if (!f.halo_done) k_filter_block_halo<32><<<(unsigned)(15 * f.nsub), 256, 0, st>>>(g, sc, f);
     k_filter_block<32><<<nb, FB_THREADS, fb_smem<32>(), st>>>(g, sc, f);
   } else {
-    k_filter_block_halo<16><<<(unsigned)(15 * f.nsub), 256, 0, st>>>(g, sc, f);
+    if (!f.halo_done) k_filter_block_halo<16><<<(unsigned)(15 * f.nsub), 256, 0, st>>>(g, sc, f);
     k_filter_block<16><<<nb, FB_THREADS, fb_smem<16>(), st>>>(g, sc, f);
   }
   if (tm) tm->rec(tm->self, 3, 0);
-  if (launches) *launches += 2;
+  if (launches) *launches += f.halo_done ? 1 : 2;
   return (int)cudaGetLastError();
 }
 

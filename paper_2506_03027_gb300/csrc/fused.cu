@@ -28,6 +28,7 @@
 
 #include "cfs_internal.h"
 #include "device_common.cuh"
+#include "pairs.cuh"
 
 namespace cfs {
 
@@ -101,10 +102,142 @@ __device__ __forceinline__ void prims32(const double* u, const Phys32& k, float*
 
 // ------------------------------------------------------------------------------- k_halo_prims
 
+namespace {
+
+// The halo store: per stage and padded point eight floats {u, v, w, T, rho, p - p_ref, rho E + p -
+// H_ref, -}: one 32-byte sector per point, whatever the shape of the strip
+// (arrays of one primitive each leave half of the sectors of a 4-wide x strip unused, and take seven
+// 4-byte copies per point in the stage where this takes four of 8 bytes).
+__device__ __forceinline__ void store_halo(float4* __restrict__ Wh, long long P, int m, long long o, const float* w) {
+  float4* q = Wh + 2 * ((long long)m * P + o);
+  q[0] = make_float4(w[1], w[2], w[3], w[5]);
+  q[1] = make_float4(w[0], w[4], w[6], 0.f);
+}
+
+// The delayed levels of one point as the AT sums take them: U_0 = h0 + l0 (to 48 bits) and the exact
+// differences U_l - U_0 = ah + al; rho and rho u, rho v and rho w as packed pairs, rho E alone.
+struct LevelDiffs {
+  float2 h0[2], l0[2], ah[CFS_MAX_LEVELS][2], al[CFS_MAX_LEVELS][2];
+  float h4, l4, ah4[CFS_MAX_LEVELS], al4[CFS_MAX_LEVELS];
+};
+__device__ __forceinline__ void level_diffs(const double (*r)[5], int C, LevelDiffs& d) {
+  float h0[5], l0[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    h0[v] = d2f_fast(r[0][v]);
+    l0[v] = dev_fast(r[0][v], h0[v], 0.f);
+  }
+  d.h0[0] = make_float2(h0[0], h0[1]);
+  d.h0[1] = make_float2(h0[2], h0[3]);
+  d.l0[0] = make_float2(l0[0], l0[1]);
+  d.l0[1] = make_float2(l0[2], l0[3]);
+  d.h4 = h0[4];
+  d.l4 = l0[4];
+#pragma unroll
+  for (int l = 1; l < CFS_MAX_LEVELS; ++l)
+    if (l < C) {
+      float h[5], q[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) split_fast(r[l][v], h[v], q[v]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        d.ah[l][k] = v_sub(make_float2(h[2 * k], h[2 * k + 1]), d.h0[k]);
+        d.al[l][k] = v_sub(make_float2(q[2 * k], q[2 * k + 1]), d.l0[k]);
+      }
+      d.ah4[l] = v_sub(h[4], d.h4);
+      d.al4[l] = v_sub(q[4], d.l4);
+    }
+}
+
+// (S - 1) U_0 + sum_{l >= 1} W_l (U_l - U_0) with the weights c[0 .. C-1] = pairs of S - 1, W_1, ...:
+// products of the high parts split exactly with an FMA and summed with TwoSum.
+template <class V, class A, class L>
+__device__ __forceinline__ V at_sum(V h0, A ah, L al, const float2* c, int C) {
+  V sh = v_bc<V>(0.f), st = v_mul(v_bc<V>(c[0].x), h0);  // running sum and its error terms
+#pragma unroll
+  for (int l = 1; l < CFS_MAX_LEVELS; ++l)
+    if (l < C) {
+      const V wx = v_bc<V>(c[l].x), a = ah(l);
+      const V p = v_mul(wx, a);
+      const V pe = v_fma(wx, a, v_neg(p));  // exact: p + pe = c.x * ah
+      const V s2 = v_add(sh, p);            // TwoSum(sh, p)
+      const V bv = v_sub(s2, sh);
+      const V se = v_add(v_sub(sh, v_sub(s2, bv)), v_sub(p, bv));
+      sh = s2;
+      st = v_add(st, v_add(se, pe));
+      st = v_fma(wx, al(l), st);
+      st = v_fma(v_bc<V>(c[l].y), a, st);
+    }
+  return v_add(sh, st);
+}
+// the five variables' sums
+__device__ __forceinline__ void at_sums(const LevelDiffs& d, const float2* c, int C, float* out) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float2 x = at_sum(d.h0[k], [&](int l) { return d.ah[l][k]; }, [&](int l) { return d.al[l][k]; }, c, C);
+    out[2 * k] = x.x;
+    out[2 * k + 1] = x.y;
+  }
+  out[4] = at_sum(d.h4, [&](int l) { return d.ah4[l]; }, [&](int l) { return d.al4[l]; }, c, C);
+}
+
+// AT halo primitives of all S stages at padded point o: U_buf^(m) = sum_l W^(m)_l(k) U^{n-k-l}, written
+// as S_m U_0 + sum_{l>=1} W^(m)_l (U_l - U_0) with U_l = U^{n-k-l} and S_m = sum_l W^(m)_l, which is 1
+// up to the rounding of the table (the stage-0 extrapolation weights reproduce constants, the
+// derivative weights the later stages add sum to zero), and evaluated without FP64 arithmetic:
+// - each difference U_l - U_0 as an exact pair of floats: U_l = h + r (split_fast: h its FP32
+//   truncation), U_0 = h0 + l0, (h - h0) exact when the levels are within a factor of two;
+// - the weights as pairs of floats (table W32: S_m - 1, then W^(m)_1 .. W^(m)_{C-1});
+// - products of the high parts split exactly with an FMA and summed with TwoSum: the weights
+//   of large delays alternate in sign (sum |W| about 1,400 at k = 4 against 1 for the result),
+//   so plain FP32 sums would lose that factor; compensated, the sum has the accuracy of the
+//   FP64 one before its final rounding to the FP32 primitives.
+// With the learned halo, face points start from the network's stage-0 value and add the same
+// sums with W^(m) - W^(0) (table W32d).
+template <int S>
+__device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc, const Phys32& k32, const double (*r)[5],
+                                         const LevelDiffs& d, int kd, bool learned, long long o, float4* __restrict__ Wh) {
+  const int C = sc.C;
+  // the value the sums are added to: U_0, or the network's stage-0 value (rho, momenta as pairs
+  // of floats, rho E as its deviation from E_ref)
+  float bh[4], bl[4], be;
+  if (learned) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const double x = sc.LH[(long long)v * g.Ptot + o];
+      bh[v] = d2f_fast(x);
+      bl[v] = dev_fast(x, bh[v], 0.f);
+    }
+    be = dev_fast(sc.LH[4LL * g.Ptot + o], k32.Eh, k32.El);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      bh[v] = v & 1 ? d.h0[v >> 1].y : d.h0[v >> 1].x;
+      bl[v] = v & 1 ? d.l0[v >> 1].y : d.l0[v >> 1].x;
+    }
+    be = dev_fast(r[0][4], k32.Eh, k32.El);
+  }
+  const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * C;
+#pragma unroll
+  for (int m = 0; m < S; ++m) {
+    float2 c[CFS_MAX_LEVELS];
+#pragma unroll
+    for (int l = 0; l < CFS_MAX_LEVELS; ++l) c[l] = l < C ? __ldg(wt + m * C + l) : make_float2(0.f, 0.f);
+    float dl[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    if (!(learned && m == 0)) at_sums(d, c, C, dl);
+    float w[7];
+    prims32f(bh[0] + (bl[0] + dl[0]), bh[1] + (bl[1] + dl[1]), bh[2] + (bl[2] + dl[2]), bh[3] + (bl[3] + dl[3]),
+             be + dl[4], k32, w);
+    store_halo(Wh, g.Ptot, m, o, w);
+  }
+}
+
+}  // namespace
+
 template <int S>
 __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
                                                     const SubDev* __restrict__ subs, const int2* __restrict__ halo,
-                                                    long long nhalo, float* __restrict__ Wh) {
+                                                    long long nhalo, float4* __restrict__ Wh) {
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: no halo store is read
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -167,37 +300,11 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
     for (int m = 0; m < (sc.mode == 2 ? 1 : S); ++m) {
       float w[7];
       prims32(acc[m], k32, w);
-#pragma unroll
-      for (int c = 0; c < 7; ++c) Wh[(long long)(m * 7 + c) * P + o] = w[c];
+      store_halo(Wh, P, m, o, w);
     }
     return;
   }
-  if (sc.mode == 2) {  // AS: the latest visible level, the same for every stage
-    const double* src = ring + (long long)slot(0) * lvN;
-    double u[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) u[v] = src[v * d.bN + gi];
-    float w[7];
-    prims32(u, k32, w);
-#pragma unroll
-    for (int c = 0; c < 7; ++c) Wh[(long long)c * P + o] = w[c];
-    return;
-  }
-  // AT: U_buf^(m) = sum_l W^(m)_l(k) U^{n-k-l} for every stage m, written as
-  // S_m U_0 + sum_{l>=1} W^(m)_l (U_l - U_0) with U_l = U^{n-k-l} and S_m = sum_l W^(m)_l, which is 1
-  // up to the rounding of the table (the stage-0 extrapolation weights reproduce constants, the
-  // derivative weights the later stages add sum to zero), and evaluated without FP64 arithmetic:
-  // - each difference U_l - U_0 as an exact pair of floats: U_l = h + r (split_fast: h its FP32
-  //   truncation), U_0 = h0 + l0, (h - h0) exact when the levels are within a factor of two;
-  // - the weights as pairs of floats (table W32: S_m - 1, then W^(m)_1 .. W^(m)_{C-1});
-  // - products of the high parts split exactly with an FMA and summed with TwoSum: the weights
-  //   of large delays alternate in sign (sum |W| about 1,400 at k = 4 against 1 for the result),
-  //   so plain FP32 sums would lose that factor; compensated, the sum has the accuracy of the
-  //   FP64 one before its final rounding to the FP32 primitives.
-  // With the learned halo, face points start from the network's stage-0 value and add the same
-  // sums with W^(m) - W^(0) (table W32d).
-  const bool learned = sc.LH && ((int)(ci < 0 || ci >= d.sx) + (int)(cj < 0 || cj >= d.sy) + (int)(ck < 0 || ck >= d.sz) == 1);
-  const int C = sc.C;
+  const int C = sc.mode == 2 ? 1 : sc.C;
   double r[CFS_MAX_LEVELS][5];
 #pragma unroll
   for (int l = 0; l < CFS_MAX_LEVELS; ++l)
@@ -206,72 +313,109 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
 #pragma unroll
       for (int v = 0; v < 5; ++v) r[l][v] = src[v * d.bN + gi];
     }
-  float h0[5], l0[5], ah[CFS_MAX_LEVELS][5], al[CFS_MAX_LEVELS][5];  // U_l - U_0 = ah[l] + al[l]
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    h0[v] = d2f_fast(r[0][v]);
-    l0[v] = dev_fast(r[0][v], h0[v], 0.f);
+  if (sc.mode == 2) {  // AS: the latest visible level, the same for every stage
+    float w[7];
+    prims32(r[0], k32, w);
+    store_halo(Wh, P, 0, o, w);
+    return;
   }
-#pragma unroll
-  for (int l = 1; l < CFS_MAX_LEVELS; ++l)
-    if (l < C)
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        float h, q;
-        split_fast(r[l][v], h, q);
-        ah[l][v] = __fsub_rn(h, h0[v]);
-        al[l][v] = __fsub_rn(q, l0[v]);
-      }
-  // the value the sums are added to: U_0, or the network's stage-0 value (rho, momenta as pairs
-  // of floats, rho E as its deviation from E_ref)
-  float bh[4], bl[4], be;
-  if (learned) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const double x = sc.LH[(long long)v * g.Ptot + d.pbase + t];
-      bh[v] = d2f_fast(x);
-      bl[v] = dev_fast(x, bh[v], 0.f);
+  const bool learned = sc.LH && ((int)(ci < 0 || ci >= d.sx) + (int)(cj < 0 || cj >= d.sy) + (int)(ck < 0 || ck >= d.sz) == 1);
+  LevelDiffs ld;
+  level_diffs(r, C, ld);
+  at_prims<S>(g, sc, k32, r, ld, kd, learned, o, Wh);
+}
+
+// The halo store and the sub-domain filter's halos from one read of the delayed levels, for contexts
+// of cubic sub-domains of N points whose filter runs sub-domain by sub-domain (filter_block.cu): both
+// read the levels beyond every face, to depth 4 and 5, and each alone is bound by those reads.  One
+// thread per point: the six faces to depth 5 (x faces: the five points of a row fastest), then the
+// twelve r x r edges.  The filter halo is the extrapolation to t_{n+1} (weights c(k+1)) as the FP32
+// deviation from the sub-domain's reference value, [(sub-domain, variable)][axis][10][N^2].
+template <int N>
+__global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
+                                                    const SubDev* __restrict__ subs, float4* __restrict__ Wh,
+                                                    float* __restrict__ fh) {
+  constexpr int S = 5, NN = N * N, NF = 5 * NN;
+  sc = resolve(sc);
+  if (sc.mode == 0) return;  // synchronous step: neither is read
+  const int sid = blockIdx.y;
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 6 * NF + 48 * N) return;
+  const Phys32 k32 = phys32(ph);
+  const SubDev d = subs[sid];
+  int c[3], kd, face = -1, h = 0, line = 0;
+  if (t < 6 * NF) {
+    face = t / NF;
+    const int rem = t - face * NF, axis = face >> 1;
+    int dd;
+    if (axis == 0) {
+      line = rem / 5;
+      dd = rem - 5 * line;
+    } else {
+      dd = rem / NN;
+      line = rem - dd * NN;
     }
-    be = dev_fast(sc.LH[4LL * g.Ptot + d.pbase + t], k32.Eh, k32.El);
+    const int t1 = line % N, t2 = line / N, pos = (face & 1) ? N + dd : dd - 5;
+    h = (face & 1) ? 5 + dd : dd;
+    c[axis] = pos;
+    c[axis == 0 ? 1 : 0] = t1;
+    c[axis == 2 ? 1 : 2] = t2;
+    kd = face_delay(sc, sid, face);
   } else {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      bh[v] = h0[v];
-      bl[v] = l0[v];
-    }
-    be = dev_fast(r[0][4], k32.Eh, k32.El);
+    t -= 6 * NF;
+    const int e = t / (4 * N), q = t - e * 4 * N;  // edge: axes (0, 1), (0, 2), (1, 2) x four corners
+    const int pr = e >> 2, a = pr == 2 ? 1 : 0, b = pr == 0 ? 1 : 2, free = 3 - a - b;
+    const int along = q % N, ab = q / N;
+    const int sa = e & 1, sb = (e >> 1) & 1;
+    c[a] = sa ? N + (ab & 1) : -1 - (ab & 1);
+    c[b] = sb ? N + (ab >> 1) : -1 - (ab >> 1);
+    c[free] = along;
+    kd = max(face_delay(sc, sid, 2 * a + sa), face_delay(sc, sid, 2 * b + sb));
   }
-  const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * C;
+  auto wrap1 = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+  const int gx = wrap1(d.ox + c[0], d.bnx), gy = wrap1(d.oy + c[1], d.bny), gz = wrap1(d.oz + c[2], d.bnz);
+  const long long gi = d.bbase + (long long)gx + (long long)d.bnx * ((long long)gy + (long long)d.bny * gz);
+  const long long lvN = 5 * g.N;
+  const int nR = mod_ring(sc.n, sc.R), C = sc.mode == 2 ? 1 : sc.C;
+  double r[CFS_MAX_LEVELS][5];
 #pragma unroll
-  for (int m = 0; m < S; ++m) {
-    float2 c[CFS_MAX_LEVELS];
+  for (int l = 0; l < CFS_MAX_LEVELS; ++l)
+    if (l < C) {
+      const int q = nR - kd - l;
+      const double* src = ring + (long long)(q < 0 ? q + sc.R : q) * lvN + gi;
 #pragma unroll
-    for (int l = 0; l < CFS_MAX_LEVELS; ++l) c[l] = l < C ? __ldg(wt + m * C + l) : make_float2(0.f, 0.f);
-    float dl[5];
+      for (int v = 0; v < 5; ++v) r[l][v] = src[v * d.bN];
+    }
+  LevelDiffs ld;
+  level_diffs(r, C, ld);
+  if (face >= 0) {
+    // the filter's halo: deviation of U_0 from the reference, plus the weighted differences
+    const double* ref = ring + (long long)nR * lvN + d.bbase + (long long)d.ox + (long long)d.bnx * (d.oy + (long long)d.bny * d.oz);
+    const float2* __restrict__ wf = (const float2*)sc.Wf32 + (long long)kd * sc.C;
+    float2 w[CFS_MAX_LEVELS];
+#pragma unroll
+    for (int l = 0; l < CFS_MAX_LEVELS; ++l) w[l] = l < C ? __ldg(wf + l) : make_float2(0.f, 0.f);
+    float sum[5];
+    at_sums(ld, w, C, sum);
+    float* __restrict__ out = fh + ((long long)sid * 15 + (face >> 1)) * 10 * NN + h * NN + line;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      float sh = 0.f, st = __fmul_rn(c[0].x, h0[v]);  // running sum and its error terms
-#pragma unroll
-      for (int l = 1; l < CFS_MAX_LEVELS; ++l)
-        if (l < C) {
-          const float p = __fmul_rn(c[l].x, ah[l][v]);
-          const float pe = __fmaf_rn(c[l].x, ah[l][v], -p);  // exact: p + pe = c.x * ah
-          const float s2 = __fadd_rn(sh, p);                  // TwoSum(sh, p)
-          const float bv = __fsub_rn(s2, sh);
-          const float se = __fadd_rn(__fsub_rn(sh, __fsub_rn(s2, bv)), __fsub_rn(p, bv));
-          sh = s2;
-          st = __fadd_rn(st, __fadd_rn(se, pe));
-          st = __fmaf_rn(c[l].x, al[l][v], st);
-          st = __fmaf_rn(c[l].y, ah[l][v], st);
-        }
-      dl[v] = (learned && m == 0) ? 0.f : __fadd_rn(sh, st);
+      const double rv = ref[v * d.bN];
+      const float rh = d2f_fast(rv), rl = dev_fast(rv, rh, 0.f);
+      const float dv = dev_fast(r[0][v], rh, rl);
+      out[(long long)v * 30 * NN] = sc.mode == 2 ? dv : __fadd_rn(dv, sum[v]);
     }
-    float w[7];
-    prims32f(bh[0] + (bl[0] + dl[0]), bh[1] + (bl[1] + dl[1]), bh[2] + (bl[2] + dl[2]), bh[3] + (bl[3] + dl[3]),
-             be + dl[4], k32, w);
-#pragma unroll
-    for (int c7 = 0; c7 < 7; ++c7) Wh[(long long)(m * 7 + c7) * P + o] = w[c7];
+    const int depth = c[face >> 1] < 0 ? -c[face >> 1] : c[face >> 1] - N + 1;
+    if (depth > HB) return;  // the stage reads to depth 4
   }
+  const long long o = d.pbase + (c[0] + g.G) + (long long)d.ex * ((c[1] + g.G) + (long long)d.ey * (c[2] + g.Gz));
+  if (sc.mode == 2) {  // AS: the latest visible level, the same for every stage
+    float w[7];
+    prims32(r[0], k32, w);
+    store_halo(Wh, g.Ptot, 0, o, w);
+    return;
+  }
+  at_prims<S>(g, sc, k32, r, ld, kd, sc.LH && face >= 0, o, Wh);
 }
 
 // ------------------------------------------------------------------------------- k_stage_fused
@@ -349,7 +493,7 @@ __global__ void __launch_bounds__(FX* FY, (FX * FY >= 512) ? 1 : 2) k_stage_fuse
                                                         const double* __restrict__ ring, int in_ring, int out_ring,
                                                         double* __restrict__ Q, const SubDev* __restrict__ subs,
                                                         const int* __restrict__ work, int nwork,
-                                                        const float* __restrict__ Wh, int stage, double A, double B,
+                                                        const float4* __restrict__ Wh, int stage, double A, double B,
                                                         double dt, int first, int last) {
   sc = resolve(sc);
   const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
@@ -358,8 +502,8 @@ __global__ void __launch_bounds__(FX* FY, (FX * FY >= 512) ? 1 : 2) k_stage_fuse
   constexpr int BX = S::BX, NB = S::NB, WX = S::WX, NW = S::NW, NT = FX * FY;
   constexpr int FXW = FX + 4;
   extern __shared__ __align__(16) float smem[];
-  double* sStg = reinterpret_cast<double*>(smem);  // [5][NB] FP64, or FP32 pairs for halo points
-  float* sStgF = smem;
+  // [5][NB]: FP64 values, or a halo column's primitives as float2 in the first four
+  double* sStg = reinterpret_cast<double*>(smem);
   float4* sR4 = reinterpret_cast<float4*>(smem + S::STG);   // [5][NB]
   float4* sR3 = reinterpret_cast<float4*>(smem + S::STG + S::R4);  // [3][NW]
   float4* sFx4 = reinterpret_cast<float4*>(smem + S::STG + S::R4 + S::R3);  // [FY][FX + 4]
@@ -387,7 +531,7 @@ __global__ void __launch_bounds__(FX* FY, (FX * FY >= 512) ? 1 : 2) k_stage_fuse
   unsigned stg_phase = 0;  // parity of the staging barrier's next phase
   const Phys32 k32 = sPh;
   const long long P = g.Ptot;
-  const float* __restrict__ WhS = Wh + (long long)((sc.mode == 2) ? 0 : stage) * 7 * P;
+  const float4* __restrict__ WhS = Wh + 2 * (long long)((sc.mode == 2) ? 0 : stage) * P;
 
   for (int wi = blockIdx.x, par = 0; wi < nwork; wi += gridDim.x, par ^= 1) {
     const int* wk = work + 4 * wi;  // (sub-domain, x0, y0, z0 | z1 << 16)
@@ -539,9 +683,9 @@ __global__ void __launch_bounds__(FX* FY, (FX * FY >= 512) ? 1 : 2) k_stage_fuse
 #pragma unroll
           for (int v = 0; v < 5; ++v) cp_async8(sStg + v * NB + p, s0 + v * d.bN);
         } else if (src == 2) {
-          const float* s0 = WhS + pz + bc.pxy[k];
+          const double* s0 = reinterpret_cast<const double*>(WhS + 2 * (pz + bc.pxy[k]));
 #pragma unroll
-          for (int c = 0; c < 7; ++c) cp_async4(sStgF + 2 * ((c >> 1) * NB + p) + (c & 1), s0 + (long long)c * P);
+          for (int c = 0; c < 4; ++c) cp_async8(sStg + c * NB + p, s0 + c);
         }
       }
       cp_async_commit();
@@ -601,14 +745,11 @@ __global__ void __launch_bounds__(FX* FY, (FX * FY >= 512) ? 1 : 2) k_stage_fuse
             for (int v = 0; v < 5; ++v) u[v] = sStg[v * NB + p];
             prims32(u, k32, w);
           } else {
-            const float2* s2 = reinterpret_cast<const float2*>(sStgF);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const float2 t = s2[c * NB + p];
-              w[2 * c] = t.x;
-              w[2 * c + 1] = t.y;
-            }
-            w[6] = sStgF[2 * (3 * NB + p)];
+            const float2* s2 = reinterpret_cast<const float2*>(sStg) + p;
+            const float2 a0 = s2[0], a1 = s2[NB], a2 = s2[2 * NB], a3 = s2[3 * NB];
+            r4[p] = make_float4(a0.x, a0.y, a1.x, a1.y);
+            if (qw != 0xffff) r3[qw] = make_float4(a2.x, a2.y, a3.x, a3.y);
+            continue;
           }
           r4[p] = make_float4(w[1], w[2], w[3], w[5]);
           if (qw != 0xffff) r3[qw] = make_float4(w[0], w[4], w[6], 0.f);
@@ -847,8 +988,20 @@ int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc,
   if (nhalo <= 0) return 0;
   const unsigned nb = (unsigned)((nhalo + 255) / 256);
   if (tm) tm->rec(tm->self, 0, 1);
-  if (s == 2) k_halo_prims<2><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, Wh);
-  else k_halo_prims<5><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, Wh);
+  if (s == 2) k_halo_prims<2><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, (float4*)Wh);
+  else k_halo_prims<5><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, (float4*)Wh);
+  if (tm) tm->rec(tm->self, 0, 0);
+  if (launches) *launches += 1;
+  return (int)cudaGetLastError();
+}
+
+int launch_halo_block(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs, int n,
+                      float* Wh, float* fh, void* stream, long long* launches, const Timer* tm) {
+  cudaStream_t st = (cudaStream_t)stream;
+  const dim3 grid((30 * n * n + 48 * n + 255) / 256, g.nsub);
+  if (tm) tm->rec(tm->self, 0, 1);
+  if (n == 32) k_halo_block<32><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, (float4*)Wh, fh);
+  else k_halo_block<16><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, (float4*)Wh, fh);
   if (tm) tm->rec(tm->self, 0, 0);
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
@@ -891,7 +1044,7 @@ static int fused_impl(const Geometry& g, const Physics& ph, const StepSched& sc,
   const int rc = fused_prepare<FX, FY>(nullptr, a.curv);
   if (rc) return rc;
   k_stage_fused<FX, FY><<<a.grid, FX * FY, a.curv ? FusedSmem<FX, FY>::bytes_curv : FusedSmem<FX, FY>::bytes, st>>>(
-      g, ph, sc, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.subs, a.work, a.nwork, a.Wh, a.stage, a.A, a.B,
+      g, ph, sc, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.subs, a.work, a.nwork, (const float4*)a.Wh, a.stage, a.A, a.B,
       a.dt, a.first, a.last);
   return (int)cudaGetLastError();
 }

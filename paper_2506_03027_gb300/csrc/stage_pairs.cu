@@ -601,9 +601,7 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
 // their eight operations per value (190 us each at 128^3).
 constexpr int CL = 64;  // lines per CTA
 
-__device__ __forceinline__ void cp_async_pair(float4* dst, const float4* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
+__device__ __forceinline__ void cp_async_pair(float4* dst, const float4* src) { cp_async16(dst, src); }
 __device__ __forceinline__ void cp_async_pair(float2* dst, const float2* src) { cp_async8(dst, src); }
 
 template <class V>
