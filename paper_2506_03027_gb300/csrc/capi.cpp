@@ -1017,6 +1017,9 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
                                     cudaMemcpyHostToDevice, st), "upload filter blocks");
         c->fgroups[ax].push_back(fg);
       }
+      // the largest launch first: the others run beside its last CTAs
+      std::stable_sort(c->fgroups[ax].begin(), c->fgroups[ax].end(),
+                       [](const FilterGroup& a, const FilterGroup& b) { return a.ctas > b.ctas; });
     }
   }
   CUDA_TRY(c, cudaMemsetAsync(c->ring, 0, sizeof(double) * 5 * N * c->R, st), "clear ring");
@@ -1259,7 +1262,8 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       // graph mode: the sub-domain filter (returns on synchronous steps) before the per-pass
       // kernels (which then return on asynchronous steps)
       if (op == c->s && c->fblock_n && graph) rc = launch_fblock(c, g, sc, src, nullptr, true);
-      for (const FilterGroup& fg : c->fgroups[op - c->s]) {
+      const std::vector<FilterGroup>& groups = c->fgroups[op - c->s];
+      for (const FilterGroup& fg : groups) {
         if (rc != 0) break;
         cfs::FilterLaunch f{};
         f.Uin = src; f.Uout = dst; f.ring = c->ring;
@@ -1269,6 +1273,7 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
         for (int m = 0; m < 6; ++m) f.h[m] = c->filt_h[m];
         f.b1 = c->filt_h[1] - c->p.alpha_f;
         f.only_sync = graph && c->fblock_n;
+        f.chain = (&fg != &groups.back() ? 1 : 0) | (&fg != &groups.front() ? 2 : 0);
         f.subs = c->part_n > 1 ? c->d_subs : nullptr;
         rc = cfs::launch_filter(g, sc, f, op - c->s, c->p.precision, c->stream, &c->launches, tm);
       }

@@ -296,6 +296,12 @@ struct FilterLaunch {
   int only_sync;           // graph mode beside the sub-domain filter: return unless the step is synchronous
   const SubDev* subs;      // partitioned context: the sub-domain table (lines of foreign sub-domains are
                            // skipped); null when every sub-domain is computed here
+  // The launches of one pass axis read the same input and write different blocks, so they overlap: bit 0
+  // when another launch of the axis follows, bit 1 when one went before.  The first waits for its
+  // predecessor and only then lets the second start; so the later ones, which start once every CTA of
+  // the one before has started, need not wait for that input.  They wait for the launch before them
+  // at their end instead, so that the next axis, which waits for the last launch, waits for all.
+  int chain;
 };
 // CTAs of a launch that one block of size n, split P, takes along `axis` with lines of Lt points
 unsigned filter_ctas(const int* n, const int* P, int axis, int Lt);

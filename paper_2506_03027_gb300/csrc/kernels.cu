@@ -802,9 +802,17 @@ __device__ __forceinline__ double from_fixed_point(long long g, int q20) {
 
 template <typename T, int axis>
 __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
-  pdl_enter();
+  if (f.chain == 0) {
+    pdl_enter();
+  } else {  // (see FilterLaunch)
+    if (!(f.chain & 2)) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  }
   sc = resolve(sc);
-  if (f.only_sync && sc.mode != 0) return;
+  if (f.only_sync && sc.mode != 0) {
+    if (f.chain & 2) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    return;
+  }
   constexpr bool F32 = std::is_same<T, float>::value;
   const double* __restrict__ Uin = ring_or(f.Uin, f.in_ring, f.ring, sc, 0);
   double* __restrict__ Uout = const_cast<double*>(ring_or(f.Uout, f.out_ring, f.ring, sc, 1));
@@ -1172,6 +1180,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       }
     }
   }
+  if (f.chain & 2) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 __global__ void k_round_table(const double* __restrict__ x, float* __restrict__ y, long long n) {
@@ -1230,9 +1239,9 @@ int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f,
   cudaStream_t st = (cudaStream_t)stream;
   if (tm) tm->rec(tm->self, 3, 1);
   if (precision == 1) {
-    if (axis == 0) k_filter<float, 0><<<nb, 128, sm, st>>>(g, sc, f);
-    else if (axis == 1) k_filter<float, 1><<<nb, 128, sm, st>>>(g, sc, f);
-    else k_filter<float, 2><<<nb, 128, sm, st>>>(g, sc, f);
+    if (axis == 0) launch_pdl(k_filter<float, 0>, dim3(nb), dim3(128), sm, st, g, sc, f);
+    else if (axis == 1) launch_pdl(k_filter<float, 1>, dim3(nb), dim3(128), sm, st, g, sc, f);
+    else launch_pdl(k_filter<float, 2>, dim3(nb), dim3(128), sm, st, g, sc, f);
   } else {
     if (axis == 0) launch_pdl(k_filter<double, 0>, dim3(nb), dim3(128), sm, st, g, sc, f);
     else if (axis == 1) launch_pdl(k_filter<double, 1>, dim3(nb), dim3(128), sm, st, g, sc, f);
