@@ -308,7 +308,7 @@ template <bool EULER>
 __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
                                                 const double* __restrict__ ring, int in_ring, const SubDev* __restrict__ subs,
                                                 const int2* __restrict__ halo, long long nhalo, const float4* __restrict__ H4,
-                                                const float2* __restrict__ H2, void* Wp, int stage, int s, int own_blocks) {
+                                                const float2* __restrict__ H2, void* Wp, int stage, int s, int own_blocks, int rev) {
   pdl_enter();
   sc = resolve(sc);
   const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, Step
       store_prims(w_view(Wp, g.Ptot), o, r);
     }
   };
-  const long long b = blockIdx.x, nown = (long long)own_blocks * g.nsub;
+  const long long b = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x, nown = (long long)own_blocks * g.nsub;
   if (b < nown) {
     const int sid = (int)(b / own_blocks);
     const SubDev& d = subs[sid];
@@ -399,9 +399,9 @@ __device__ float g_pow_pair[POW_PAIR_TAB];  // tables of p_pow
 // blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.
 template <int R, bool CURV, bool LAW>
 __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPhysics ph, const SubDev* __restrict__ subs,
-                                                const void* __restrict__ Wp, void* __restrict__ Phi) {
+                                                const void* __restrict__ Wp, void* __restrict__ Phi, int rev) {
   pdl_enter();
-  const int sid = blockIdx.y;
+  const int sid = rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   const SubDev& d = subs[sid];
   if (!d.own) return;  // another process's sub-domain
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -529,18 +529,21 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
 // ------------------------------------------------------------------------------- k_rk_p
 
 // dt R = sum_a dt D_a Phi_a (times J on a curvilinear block) in pairs, then the low-storage update
-// Q = A Q + dt R, U^(m) = U^(m-1) + B Q in FP64.
+// Q = A Q + dt R, U^(m) = U^(m-1) + B Q in FP64.  Bound by memory latency (310 B of traffic per point
+// at half the DRAM rate, 64 registers): Q and the stage input, not read again before they
+// would be evicted anyway, pass by the caches as streaming accesses and leave the L2 to the fluxes that
+// neighbouring points share (128^3: 147 -> 122 us).
 template <int R>
 __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
                                               const void* __restrict__ Phi, const double* __restrict__ Uin0,
                                               double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
                                               int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
-                                              int last) {
+                                              int last, int rev) {
   pdl_enter();
   sc = resolve(sc);
   const double* Uin = ring_or(Uin0, in_ring, ring, sc, 0);
   double* Uout = const_cast<double*>(ring_or(Uout0, out_ring, ring, sc, 1));
-  const int sid = blockIdx.y;
+  const int sid = rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   const SubDev& d = subs[sid];
   if (!d.own) return;  // another process's sub-domain
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -555,8 +558,8 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
   double qv[5], uv[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    qv[c] = first ? 0.0 : Q[c * d.bN + gi];
-    uv[c] = Uin[c * d.bN + gi];
+    qv[c] = first ? 0.0 : __ldcs(Q + c * d.bN + gi);
+    uv[c] = __ldcs(Uin + c * d.bN + gi);
   }
   P2 m = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, e = m;
   P1 n = {0.f, 0.f};
@@ -583,7 +586,7 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
     double qn = first ? dtR[c] : fma(A, qv[c], dtR[c]);
     double un = fma(B, qn, uv[c]);
     if (wallpt && c >= 1 && c <= 3) qn = un = 0.0;  // no-slip wall points keep zero momentum
-    if (!last) Q[c * d.bN + gi] = qn;
+    if (!last) __stcs(Q + c * d.bN + gi, qn);
     Uout[c * d.bN + gi] = un;
   }
 }
@@ -707,8 +710,8 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
 #pragma unroll
               for (int v = 0; v < (two ? 2 : 1); ++v) {
                 const long long gi = d.bbase + (long long)(two ? 1 + 2 * grp + v : 0) * d.bN + pt;
-                qv[k][v] = first ? 0.0 : Q[gi];
-                uv[k][v] = Uin[gi];
+                qv[k][v] = first ? 0.0 : __ldcs(Q + gi);
+                uv[k][v] = __ldcs(Uin + gi);
               }
             }
           }
@@ -735,7 +738,7 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
           const long long gi = d.bbase + (long long)comp * d.bN + pt;
           const double t = p_double(dtR);
           const double qn = first ? t : fma(A, qv[k][v], t);
-          if (!last) Q[gi] = qn;
+          if (!last) __stcs(Q + gi, qn);
           Uout[gi] = fma(B, qn, uv[k][v]);
         };
         if constexpr (two) {
@@ -764,10 +767,10 @@ __global__ void __launch_bounds__(CL) k_compact_p(Geometry g, StepSched sc, cons
                                                   const float2* __restrict__ cth, int Lmax, const double* __restrict__ Uin0,
                                                   double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
                                                   int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
-                                                  int last) {
+                                                  int last, int rev) {
   extern __shared__ __align__(16) unsigned char craw[];
   pdl_enter();
-  const SubDev& d = subs[blockIdx.z];
+  const SubDev& d = subs[rev ? gridDim.z - 1 - blockIdx.z : blockIdx.z];
   constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
   const int sz[3] = {d.sx, d.sy, d.sz};
   if (!d.own || (int)blockIdx.x * CL >= sz[a1] * sz[a2]) return;
@@ -830,23 +833,28 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   const dim3 gf(nblk(a.max_flux, B), g.nsub), gr(nblk(a.max_own, B), g.nsub);
   const float dth = (float)a.dt;
   const float2 dt = make_float2(dth, (float)(a.dt - (double)dth));
+  // Each kernel takes the sub-domains in the opposite order of the one before it, so that it starts on
+  // what that one wrote last and the L2 still holds (a step of 128^3 in 64 sub-domains: 2450 -> 2417 us;
+  // 100^3 in 27: 1117 -> 1089)
+  const int per_stage = a.compact ? 4 : (g.viscous ? 3 : 2);
+  auto rev = [&](int k) { return (a.stage * per_stage + k) & 1; };
   // (inviscid: the fluxes come straight from the view)
   TIMED(tm, 0, (launch_pdl(g.viscous ? k_view_p<false> : k_view_p<true>, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring,
                            a.in_ring, a.subs, (const int2*)a.halo, a.nhalo, H4, H2, g.viscous ? a.Wp : a.Phi, a.stage, a.s,
-                           (int)own_blocks)));
+                           (int)own_blocks, rev(0))));
   if (launches) *launches += 1;
   if (a.compact) {
     // x and y passes gather dt R, the z pass takes the update
     const size_t slots = (size_t)(a.Lmax + 8) * CL, staged = (size_t)(a.Lmax + 8) * (CL + 1);
     const dim3 gc(nblk((long long)a.Lmax * a.Lmax, CL), 3, g.nsub);
     const float2* cth = (const float2*)a.cthomas;
-    auto run = [&](auto kernel, size_t smem) {
+    auto run = [&](auto kernel, size_t smem, int k) {
       TIMED(tm, 2, (launch_pdl(kernel, gc, dim3(CL), smem * sizeof(float4), st, g, sc, a.subs, (const void*)a.Phi, (void*)a.R, cth,
-                               a.Lmax, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last)));
+                               a.Lmax, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last, rev(k))));
     };
-    run(k_compact_p<0>, staged);
-    run(k_compact_p<1>, slots);
-    run(k_compact_p<2>, slots);
+    run(k_compact_p<0>, staged, 1);
+    run(k_compact_p<1>, slots, 2);
+    run(k_compact_p<2>, slots, 3);
     if (launches) *launches += 3;
     return (int)cudaGetLastError();
   }
@@ -857,12 +865,12 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
       return g.metric ? k_flux_p<R, true, false> : k_flux_p<R, false, false>;
     };
     const auto flux = g.r == 2 ? pick(std::integral_constant<int, 2>{}) : pick(std::integral_constant<int, 1>{});
-    TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi)));
+    TIMED(tm, 1, (launch_pdl(flux, gf, dim3(B), 0, st, g, ph, a.subs, (const void*)a.Wp, a.Phi, rev(1))));
     if (launches) *launches += 1;
   }
   auto rk = g.r == 2 ? k_rk_p<2> : k_rk_p<1>;
   TIMED(tm, 2, (launch_pdl(rk, gr, dim3(B), 0, st, g, sc, a.subs, (const void*)a.Phi, a.Uin, a.Uout, a.ring, a.in_ring,
-                           a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last)));
+                           a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last, rev(g.viscous ? 2 : 1))));
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
 }
