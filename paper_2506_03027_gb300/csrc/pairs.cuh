@@ -27,8 +27,20 @@ __device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return __ffma2_rn(
 __device__ __forceinline__ float2 v_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 v_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 v_neg(float2 a) { return make_float2(-a.x, -a.y); }
+// The same two values as plain FP32 instructions: twice as many, but the operands need not be brought
+// into register pairs
+struct F2 {
+  float x, y;
+};
+__device__ __forceinline__ F2 v_add(F2 a, F2 b) { return {__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)}; }
+__device__ __forceinline__ F2 v_sub(F2 a, F2 b) { return {__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)}; }
+__device__ __forceinline__ F2 v_mul(F2 a, F2 b) { return {__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)}; }
+__device__ __forceinline__ F2 v_fma(F2 a, F2 b, F2 c) { return {__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y)}; }
+__device__ __forceinline__ F2 v_neg(F2 a) { return {-a.x, -a.y}; }
 template <class V>
 __device__ __forceinline__ V v_bc(float a);
+template <>
+__device__ __forceinline__ F2 v_bc<F2>(float a) { return {a, a}; }
 template <>
 __device__ __forceinline__ float v_bc<float>(float a) { return a; }
 template <>
@@ -95,15 +107,22 @@ __device__ __forceinline__ Pr<V> p_scale(Pr<V> a, float f) {
   return {v_mul(a.h, v_bc<V>(f)), v_mul(a.l, v_bc<V>(f))};
 }
 
-__device__ __forceinline__ P2 p_bc(P1 a) { return {make_float2(a.h, a.h), make_float2(a.l, a.l)}; }
-__device__ __forceinline__ P2 p_pair(P1 a, P1 b) { return {make_float2(a.h, b.h), make_float2(a.l, b.l)}; }
-__device__ __forceinline__ P1 p_x(P2 a) { return {a.h.x, a.l.x}; }
-__device__ __forceinline__ P1 p_y(P2 a) { return {a.h.y, a.l.y}; }
+// (W: float2, or F2 for two values by plain instructions)
+template <class W = float2>
+__device__ __forceinline__ Pr<W> p_bc(P1 a) { return {W{a.h, a.h}, W{a.l, a.l}}; }
+template <class W = float2>
+__device__ __forceinline__ Pr<W> p_pair(P1 a, P1 b) { return {W{a.h, b.h}, W{a.l, b.l}}; }
+template <class W>
+__device__ __forceinline__ P1 p_x(Pr<W> a) { return {a.h.x, a.l.x}; }
+template <class W>
+__device__ __forceinline__ P1 p_y(Pr<W> a) { return {a.h.y, a.l.y}; }
 __device__ __forceinline__ P1 p_of(float2 a) { return {a.x, a.y}; }
 __device__ __forceinline__ float2 p_store(P1 a) { return make_float2(a.h, a.l); }
 // memory form of two pairs: (h of both, l of both)
-__device__ __forceinline__ P2 p_of(float4 a) { return {make_float2(a.x, a.y), make_float2(a.z, a.w)}; }
-__device__ __forceinline__ float4 p_store(P2 a) { return make_float4(a.h.x, a.h.y, a.l.x, a.l.y); }
+template <class W = float2>
+__device__ __forceinline__ Pr<W> p_of(float4 a) { return {W{a.x, a.y}, W{a.z, a.w}}; }
+template <class W>
+__device__ __forceinline__ float4 p_store(Pr<W> a) { return make_float4(a.h.x, a.h.y, a.l.x, a.l.y); }
 
 // 1 / a for a normalised pair: the FP32 reciprocal refined by r (1 + e + e^2), e = 1 - a r
 __device__ __forceinline__ P1 p_recip(P1 a) {

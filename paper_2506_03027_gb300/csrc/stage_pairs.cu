@@ -368,16 +368,16 @@ __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, Step
 namespace {
 
 // Central difference without its factor (times c2 for CD4, c1 for CD2), of two values
-template <int R>
-__device__ __forceinline__ P2 diff2(const float4* __restrict__ f, long long q, long long st) {
-  const P2 c = p_of(f[q + st]), d = p_of(f[q - st]);
+template <int R, class W = float2>
+__device__ __forceinline__ Pr<W> diff2(const float4* __restrict__ f, long long q, long long st) {
+  const Pr<W> c = p_of<W>(f[q + st]), d = p_of<W>(f[q - st]);
   if (R == 1) return p_norm(p_sub(c, d));
-  const P2 a = p_of(f[q + 2 * st]), b = p_of(f[q - 2 * st]);
-  const float2 m8 = make_float2(-8.f, -8.f);
-  const P2 x = p_2diff(a.h, b.h), y = p_2diff(c.h, d.h);
-  const P2 s = p_2sum(x.h, v_mul(m8, y.h));
-  const float2 lo = v_add(v_fma(m8, y.l, x.l), v_fma(m8, v_sub(c.l, d.l), v_sub(a.l, b.l)));
-  return p_norm(P2{s.h, v_add(s.l, lo)});
+  const Pr<W> a = p_of<W>(f[q + 2 * st]), b = p_of<W>(f[q - 2 * st]);
+  const W m8 = {-8.f, -8.f};
+  const Pr<W> x = p_2diff(a.h, b.h), y = p_2diff(c.h, d.h);
+  const Pr<W> s = p_2sum(x.h, v_mul(m8, y.h));
+  const W lo = v_add(v_fma(m8, y.l, x.l), v_fma(m8, v_sub(c.l, d.l), v_sub(a.l, b.l)));
+  return p_norm(Pr<W>{s.h, v_add(s.l, lo)});
 }
 template <int R>
 __device__ __forceinline__ P1 diff1(const float2* __restrict__ f, long long q, long long st) {
@@ -396,10 +396,16 @@ __device__ float g_pow_pair[POW_PAIR_TAB];  // tables of p_pow
 
 // Combined fluxes at the owned points and the strips of r points beyond each face (the flux along
 // that face's axis only), thread by thread as in k_flux.  CURV: the context has curvilinear
-// blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.
+// blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.  Bound by instruction issue
+// and memory about equally (128^3: half of each).  A Cartesian point forms most of its pairs of values from
+// components of others, and bringing those into register pairs for the packed instructions costs more than
+// they save: two plain instructions each are faster (121 -> 114 us at 128^3); on curvilinear blocks,
+// whose metric products take whole rows, the packed ones are.
 template <int R, bool CURV, bool LAW>
 __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPhysics ph, const SubDev* __restrict__ subs,
                                                 const void* __restrict__ Wp, void* __restrict__ Phi, int rev) {
+  using V2 = std::conditional_t<CURV, float2, F2>;
+  using P2 = Pr<V2>;
   pdl_enter();
   const int sid = rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
   const SubDev& d = subs[sid];
@@ -418,40 +424,40 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
   float4* __restrict__ F4 = (float4*)Phi;
   float2* __restrict__ F2 = (float2*)(F4 + 6 * P);
 
-  const P2 uv = p_of(A[q]), wT = p_of(B[q]), rp = p_of(Cc[q]);
+  const P2 uv = p_of<V2>(A[q]), wT = p_of<V2>(B[q]), rp = p_of<V2>(Cc[q]);
   const P1 w = p_x(wT), rho = p_x(rp), pr = p_y(rp);
   const P1 netH = p_neg(p_norm(p_add(p_of(D[q]), cst(ph.H))));  // -(rho E + p)
   P1 iv = cst(ph.ivT);  // the factor of the viscous terms: 1/Re x (units of the differences) x mu
   // differences of (u, v) and (w, kappa T) along each axis
-  P2 Gx = diff2<R>(A, q, st[0]), Gy = diff2<R>(A, q, st[1]), Gz = diff2<R>(A, q, st[2]);
-  P2 Hz = diff2<R>(B, q, st[2]);
-  P2 Hx = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, Hy = Hx;
-  if (as != 1) Hx = diff2<R>(B, q, st[0]);
-  if (as != 0) Hy = diff2<R>(B, q, st[1]);
+  P2 Gx = diff2<R, V2>(A, q, st[0]), Gy = diff2<R, V2>(A, q, st[1]), Gz = diff2<R, V2>(A, q, st[2]);
+  P2 Hz = diff2<R, V2>(B, q, st[2]);
+  P2 Hx = {V2{0.f, 0.f}, V2{0.f, 0.f}}, Hy = Hx;
+  if (as != 1) Hx = diff2<R, V2>(B, q, st[0]);
+  if (as != 0) Hy = diff2<R, V2>(B, q, st[1]);
   const bool curv = CURV && d.mbase >= 0;
-  P2 xi = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, et = xi;  // metric rows (xi_x, xi_y), (eta_x, eta_y)
+  P2 xi = {V2{0.f, 0.f}, V2{0.f, 0.f}}, et = xi;  // metric rows (xi_x, xi_y), (eta_x, eta_y)
   P1 zz = {0.f, 0.f};
   if (curv) {
     // index-space differences to physical gradients / J: x: xi_x, eta_x; y: xi_y, eta_y; z: zeta_z
     const float2* M = g.metric_p + d.mbase + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
     const long long pl = d.mpl;
-    xi = p_pair(p_of(M[0]), p_of(M[pl]));
-    et = p_pair(p_of(M[2 * pl]), p_of(M[3 * pl]));
+    xi = p_pair<V2>(p_of(M[0]), p_of(M[pl]));
+    et = p_pair<V2>(p_of(M[2 * pl]), p_of(M[3 * pl]));
     zz = p_of(M[4 * pl]);
-    if (as == 1) Hx = diff2<R>(B, q, st[0]);  // (the rows mix the two in-plane differences)
-    if (as == 0) Hy = diff2<R>(B, q, st[1]);
+    if (as == 1) Hx = diff2<R, V2>(B, q, st[0]);  // (the rows mix the two in-plane differences)
+    if (as == 0) Hy = diff2<R, V2>(B, q, st[1]);
     const P2 g0 = Gx, h0 = Hx;
-    Gx = p_norm(p_fma(p_bc(p_x(et)), Gy, p_mul(p_bc(p_x(xi)), g0)));
-    Hx = p_norm(p_fma(p_bc(p_x(et)), Hy, p_mul(p_bc(p_x(xi)), h0)));
-    Gy = p_norm(p_fma(p_bc(p_y(et)), Gy, p_mul(p_bc(p_y(xi)), g0)));
-    Hy = p_norm(p_fma(p_bc(p_y(et)), Hy, p_mul(p_bc(p_y(xi)), h0)));
-    Gz = p_norm(p_mul(p_bc(zz), Gz));
-    Hz = p_norm(p_mul(p_bc(zz), Hz));
+    Gx = p_norm(p_fma(p_bc<V2>(p_x(et)), Gy, p_mul(p_bc<V2>(p_x(xi)), g0)));
+    Hx = p_norm(p_fma(p_bc<V2>(p_x(et)), Hy, p_mul(p_bc<V2>(p_x(xi)), h0)));
+    Gy = p_norm(p_fma(p_bc<V2>(p_y(et)), Gy, p_mul(p_bc<V2>(p_y(xi)), g0)));
+    Hy = p_norm(p_fma(p_bc<V2>(p_y(et)), Hy, p_mul(p_bc<V2>(p_y(xi)), h0)));
+    Gz = p_norm(p_mul(p_bc<V2>(zz), Gz));
+    Hz = p_norm(p_mul(p_bc<V2>(zz), Hz));
     iv = p_norm(p_mul(iv, p_norm(p_mul(cst(d.cg[0]), p_of(M[6 * pl])))));
   } else if (d.iso) {
     iv = p_norm(p_mul(iv, cst(d.cg[0])));
   } else {
-    const P2 kx = p_bc(cst(d.cg[0])), ky = p_bc(cst(d.cg[1])), kz = p_bc(cst(d.cg[2]));
+    const P2 kx = p_bc<V2>(cst(d.cg[0])), ky = p_bc<V2>(cst(d.cg[1])), kz = p_bc<V2>(cst(d.cg[2]));
     Gx = p_norm(p_mul(kx, Gx));
     Hx = p_norm(p_mul(kx, Hx));
     Gy = p_norm(p_mul(ky, Gy));
@@ -461,12 +467,12 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
   }
   if (LAW) iv = p_norm(p_mul(iv, p_pow(p_y(wT), cst(ph.visc_exp), g_pow_pair)));
   // tau / (mu gs): diagonal (t00, t11), t22, t01, and (t02, t12)
-  const P2 dia = p_pair(p_x(Gx), p_y(Gy));
+  const P2 dia = p_pair<V2>(p_x(Gx), p_y(Gy));
   const P1 div = p_norm(p_mul(P1{-0.6666667f, 1.9868216e-08f}, p_norm(p_add(p_add(p_x(dia), p_y(dia)), p_x(Hz)))));
-  const P2 td = p_norm(p_add(p_scale(dia, 2.f), p_bc(div)));
+  const P2 td = p_norm(p_add(p_scale(dia, 2.f), p_bc<V2>(div)));
   const P1 t22 = p_norm(p_add(p_scale(p_x(Hz), 2.f), div));
   const P1 t01 = p_norm(p_add(p_x(Gy), p_y(Gx)));
-  const P2 t2 = p_norm(p_add(Gz, p_pair(p_x(Hx), p_x(Hy))));
+  const P2 t2 = p_norm(p_add(Gz, p_pair<V2>(p_x(Hx), p_x(Hy))));
   // b_a = u_i tau_ai + kappa mu dT/dx_a of row (ra, rc) = ((tau_a0, tau_a1), tau_a2)
   auto heat = [&](P2 ra, P1 rc, P1 dT) {
     const P2 x = p_mul(uv, ra);
@@ -479,7 +485,7 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
   };
   const P1 zero = {0.f, 0.f};
   if (curv) {
-    const P1 b0 = heat(p_pair(p_x(td), t01), p_x(t2), p_y(Hx)), b1 = heat(p_pair(t01, p_y(td)), p_y(t2), p_y(Hy)),
+    const P1 b0 = heat(p_pair<V2>(p_x(td), t01), p_x(t2), p_y(Hx)), b1 = heat(p_pair<V2>(t01, p_y(td)), p_y(t2), p_y(Hy)),
              b2 = heat(t2, t22, p_y(Hz));
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -488,41 +494,41 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
       const P2 x = p_mul(row, uv);
       const P1 Uc = p_norm(p_add(p_x(x), p_y(x)));  // contravariant velocity
       const P1 n = p_norm(p_neg(p_mul(rho, Uc)));
-      const P2 r0 = p_bc(p_x(row)), r1 = p_bc(p_y(row));
-      P2 m = p_sub(p_mul(p_bc(n), uv), p_mul(p_bc(pr), row));
-      m = p_fma(p_bc(iv), p_norm(p_fma(r0, p_pair(p_x(td), t01), p_mul(r1, p_pair(t01, p_y(td))))), m);
-      P2 e = p_mul(p_pair(n, netH), p_pair(w, Uc));
-      e = p_fma(p_bc(iv), p_norm(p_fma(r0, p_pair(p_x(t2), b0), p_mul(r1, p_pair(p_y(t2), b1)))), e);
+      const P2 r0 = p_bc<V2>(p_x(row)), r1 = p_bc<V2>(p_y(row));
+      P2 m = p_sub(p_mul(p_bc<V2>(n), uv), p_mul(p_bc<V2>(pr), row));
+      m = p_fma(p_bc<V2>(iv), p_norm(p_fma(r0, p_pair<V2>(p_x(td), t01), p_mul(r1, p_pair<V2>(t01, p_y(td))))), m);
+      P2 e = p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, Uc));
+      e = p_fma(p_bc<V2>(iv), p_norm(p_fma(r0, p_pair<V2>(p_x(t2), b0), p_mul(r1, p_pair<V2>(p_y(t2), b1)))), e);
       put(a, n, m, e);
     }
     if (as < 0 || as == 2) {
       const P1 Uc = p_norm(p_mul(zz, w)), n = p_norm(p_neg(p_mul(rho, Uc)));
-      const P2 iz = p_bc(p_norm(p_mul(iv, zz)));
-      const P2 m = p_fma(iz, t2, p_mul(p_bc(n), uv));
-      P2 e = p_mul(p_pair(n, netH), p_pair(w, Uc));
-      e = p_sub(e, p_pair(p_mul(zz, pr), zero));
-      put(2, n, m, p_fma(iz, p_pair(t22, b2), e));
+      const P2 iz = p_bc<V2>(p_norm(p_mul(iv, zz)));
+      const P2 m = p_fma(iz, t2, p_mul(p_bc<V2>(n), uv));
+      P2 e = p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, Uc));
+      e = p_sub(e, p_pair<V2>(p_mul(zz, pr), zero));
+      put(2, n, m, p_fma(iz, p_pair<V2>(t22, b2), e));
     }
     return;
   }
-  const P2 nuv = p_norm(p_neg(p_mul(p_bc(rho), uv)));  // -rho u, -rho v
+  const P2 nuv = p_norm(p_neg(p_mul(p_bc<V2>(rho), uv)));  // -rho u, -rho v
   if (as < 0 || as == 0) {
-    const P2 ra = p_pair(p_x(td), t01);
-    P2 m = p_sub(p_mul(p_bc(p_x(nuv)), uv), p_pair(pr, zero));
-    P2 e = p_mul(p_pair(p_x(nuv), netH), p_pair(w, p_x(uv)));
-    put(0, p_x(nuv), p_fma(p_bc(iv), ra, m), p_fma(p_bc(iv), p_pair(p_x(t2), heat(ra, p_x(t2), p_y(Hx))), e));
+    const P2 ra = p_pair<V2>(p_x(td), t01);
+    P2 m = p_sub(p_mul(p_bc<V2>(p_x(nuv)), uv), p_pair<V2>(pr, zero));
+    P2 e = p_mul(p_pair<V2>(p_x(nuv), netH), p_pair<V2>(w, p_x(uv)));
+    put(0, p_x(nuv), p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_x(t2), heat(ra, p_x(t2), p_y(Hx))), e));
   }
   if (as < 0 || as == 1) {
-    const P2 ra = p_pair(t01, p_y(td));
-    P2 m = p_sub(p_mul(p_bc(p_y(nuv)), uv), p_pair(zero, pr));
-    P2 e = p_mul(p_pair(p_y(nuv), netH), p_pair(w, p_y(uv)));
-    put(1, p_y(nuv), p_fma(p_bc(iv), ra, m), p_fma(p_bc(iv), p_pair(p_y(t2), heat(ra, p_y(t2), p_y(Hy))), e));
+    const P2 ra = p_pair<V2>(t01, p_y(td));
+    P2 m = p_sub(p_mul(p_bc<V2>(p_y(nuv)), uv), p_pair<V2>(zero, pr));
+    P2 e = p_mul(p_pair<V2>(p_y(nuv), netH), p_pair<V2>(w, p_y(uv)));
+    put(1, p_y(nuv), p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_y(t2), heat(ra, p_y(t2), p_y(Hy))), e));
   }
   if (as < 0 || as == 2) {
     const P1 n = p_norm(p_neg(p_mul(rho, w)));
-    const P2 m = p_mul(p_bc(n), uv);
-    P2 e = p_sub(p_mul(p_pair(n, netH), p_pair(w, w)), p_pair(pr, zero));
-    put(2, n, p_fma(p_bc(iv), t2, m), p_fma(p_bc(iv), p_pair(t22, heat(t2, t22, p_y(Hz))), e));
+    const P2 m = p_mul(p_bc<V2>(n), uv);
+    P2 e = p_sub(p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, w)), p_pair<V2>(pr, zero));
+    put(2, n, p_fma(p_bc<V2>(iv), t2, m), p_fma(p_bc<V2>(iv), p_pair<V2>(t22, heat(t2, t22, p_y(Hz))), e));
   }
 }
 
