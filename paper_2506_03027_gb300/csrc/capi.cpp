@@ -599,7 +599,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   // 2-D inviscid FP64 runs on periodic Cartesian blocks: one launch per stage
   c->euler2d = {0, 0};
   if (c->p.precision == 0 && c->ndim == 2 && !c->p.viscous && !c->p.compact && c->all_periodic && mtot == 0)
-    c->euler2d = cfs::euler2d_shape(c->subs.data(), nsub);
+    c->euler2d = cfs::euler2d_shape(c->subs.data(), nsub, c->r);
   // tables of the FP64 power (power-law viscosity)
   if (c->p.viscous && c->p.visc_law == 1) {
     const int rc = c->pairs ? cfs::pow_pair_tables_init() : cfs::pow_tables_init();

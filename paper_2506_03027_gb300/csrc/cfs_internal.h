@@ -257,7 +257,7 @@ int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc
 struct Euler2dShape {
   int small, tiles;
 };
-Euler2dShape euler2d_shape(const SubDev* subs, int nsub);
+Euler2dShape euler2d_shape(const SubDev* subs, int nsub, int r);
 int launch_euler2d(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a, Euler2dShape e,
                    void* stream, long long* launches, const Timer* tm);
 

@@ -224,10 +224,15 @@ namespace {
 
 // The tile shapes: large grids 32 x 16 points on 256 threads (a rim of a fifth of the tile at R = 1),
 // small ones 8 x 8 on 128 threads, half of them on the rim.  The small tile's rim costs as much as
-// the tile, but below about a thousand of them per launch the FP64 pipes of 152 SMs are idle and
-// what counts is how many SMs and warps a stage spreads over: 64 x 64 points take 64 CTAs instead
-// of 8.
-constexpr int kSmallTiles = 152 * 6;
+// the tile (at R = 2 twice as much), but on a small grid the FP64 pipes of 152 SMs are idle and what
+// counts is how many SMs and warps a stage spreads over: 64 x 64 points take 64 CTAs instead of 8.
+// A step with large / small tiles, us (square grids, sub-domains of 64 x 64):
+//          64^2         128^2        192^2        256^2         320^2        384^2        512^2
+//   R = 2  69.7 / 26.7  69.7 / 38.9  71.7 / 45.1  92.3 / 82.9  147.5 / 119   170 / 158    236 / 265
+//   R = 1  24.7 / 12.4  24.7 / 14.4  25.8 / 18.5  26.7 / 30.8  41.0 / 45.1   49.2 / 57.4  75.6 / 96.3
+// so the line lies between 384^2 and 512^2 (2304 and 4096 small tiles), and between 192^2 and 240^2
+// (576 and 1024).
+constexpr long long small_tiles(int r) { return r == 1 ? 152 * 4 : 152 * 18; }
 
 template <int R, int TX, int TY, int NT>
 int launch_tile(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a, int tiles, cudaStream_t st) {
@@ -256,7 +261,7 @@ int tiles_of(int sx, int sy, int tx, int ty) { return ((sx + tx - 1) / tx) * ((s
 
 }  // namespace
 
-Euler2dShape euler2d_shape(const SubDev* subs, int nsub) {
+Euler2dShape euler2d_shape(const SubDev* subs, int nsub, int r) {
   Euler2dShape e{0, 0};
   long long small = 0;
   int most_small = 0, most_large = 0;
@@ -266,7 +271,7 @@ Euler2dShape euler2d_shape(const SubDev* subs, int nsub) {
     most_small = std::max(most_small, t);
     most_large = std::max(most_large, tiles_of(subs[i].sx, subs[i].sy, 32, 16));
   }
-  e.small = small <= kSmallTiles;
+  e.small = small <= small_tiles(r);
   e.tiles = e.small ? most_small : most_large;
   return e;
 }
