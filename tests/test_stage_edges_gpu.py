@@ -1,0 +1,105 @@
+"""The specialised stage kernels at the edges of their tiles and forms, against the oracle: the one-launch
+stage of two-dimensional inviscid runs, the compact scheme's lines, the FP32 form's halo store with the
+latest delayed level, and the halo network's kernels at batches around their tiles."""
+import numpy as np
+import pytest
+
+from oracle import mlp as omlp
+from oracle import oracle as orc
+from paper_2506_03027_gb300 import cfs
+from paper_2506_03027_gb300 import inputs as I
+from paper_2506_03027_gb300 import learned as L
+
+from gpu_util import PARITY_TOL, ensure_built, gpu_run, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ensure_built()
+
+
+def smooth_2d(c, seed):
+    """A smooth periodic state that is not symmetric in x and y and moves in z too."""
+    rng = np.random.default_rng(seed)
+    y, x = np.meshgrid(2 * np.pi * np.arange(c.ny) / c.ny, 2 * np.pi * np.arange(c.nx) / c.nx, indexing="ij")
+    ph = rng.uniform(0, 2 * np.pi, 5)
+    rho = 1 + 0.1 * np.sin(x + 2 * y + ph[0])
+    vel = [0.3 * np.sin(2 * x - y + ph[1]), 0.2 * np.cos(x + y + ph[2]), 0.25 * np.sin(x - y + ph[3])]
+    p = (1 + 0.1 * np.cos(2 * x + y + ph[4])) / (c.gamma * c.mach ** 2)
+    U = np.zeros((5, 1, c.ny, c.nx))
+    U[0, 0] = rho
+    for k in range(3):
+        U[1 + k, 0] = rho * vel[k]
+    U[4, 0] = p / (c.gamma - 1) + 0.5 * rho * sum(v * v for v in vel)
+    return U
+
+
+# sub-domains smaller than a tile, of one tile exactly, one point more, ragged ones, and a grid
+# that takes the large tiles (more than 2736 small ones at fourth order); unequal spacings
+@pytest.mark.parametrize("n,p", [((8, 8), (1, 1)), ((9, 17), (1, 2)), ((35, 22), (3, 2)), ((64, 16), (1, 1)),
+                                 ((501, 377), (5, 4))])
+@pytest.mark.parametrize("order,algo,at", [(4, "SA", True), (2, "CAA", True), (4, "SAA", True), (4, "SAA", False)])
+def test_two_dimensional_inviscid_stage(n, p, order, algo, at):
+    c = I.vortex_case(32, 1, order=order).replace(nx=n[0], ny=n[1], px=p[0], py=p[1], lx=10.0, ly=7.0, algo=algo, at=at, kmax=2)
+    U0 = smooth_2d(c, 5)
+    c = c.replace(dt=I.cfl_dt(c, U0, 0.2))
+    nst = 10
+    d = I.saa_delays(c, nst) if algo == "SAA" else None
+    Ug, _ = gpu_run(c, U0, nst, delays=d)
+    e = rel_l2(Ug, orc.run(c, U0, nst, delays=d))
+    assert np.all(np.isfinite(Ug)) and np.all(e <= PARITY_TOL), e
+
+
+# a line per CTA slot and less, one more than the 64 of a CTA, long lines, different splits per axis
+@pytest.mark.parametrize("n,p", [((16, 8, 8), (1, 1, 1)), ((13, 21, 9), (1, 2, 1)), ((40, 33, 26), (1, 3, 2))])
+def test_compact_lines(n, p):
+    c = I.tgv_case(16, 1, "CAA", viscous=False, compact=1).replace(nx=n[0], ny=n[1], nz=n[2], px=p[0], py=p[1], pz=p[2])
+    U0 = I.tgv_state(c)
+    c = c.replace(dt=I.cfl_dt(c, U0, 0.25))
+    Ug, _ = gpu_run(c, U0, 10)
+    e = rel_l2(Ug, orc.run(c, U0, 10))
+    assert np.all(np.isfinite(Ug)) and np.all(e <= PARITY_TOL), e
+
+
+# sub-domains of 16^3 and 32^3 (the halo store and the sub-domain filter's halos in one launch)
+@pytest.mark.parametrize("n", [32, 64])
+@pytest.mark.parametrize("algo", ["CAA", "SAA"])
+def test_fp32_halo_store_latest_level(n, algo):
+    c = I.tgv_case(n, 2, algo, at=False, kmax=2)
+    U0 = I.tgv_state(c)
+    c = c.replace(dt=I.cfl_dt(c, U0, 0.1))
+    d = I.saa_delays(c, 10) if algo == "SAA" else None
+    Ug, _ = gpu_run(c, U0, 10, delays=d, precision=1)
+    e = rel_l2(Ug, orc.run(c, U0, 10, delays=d))
+    assert np.all(np.isfinite(Ug)) and np.all(e < 1e-6), e
+
+
+# one sample, odd batches, one more and one less than the tiles, inputs and workspace at an offset
+@pytest.mark.parametrize("n", [1, 3, 31, 33, 127, 129, 257, 1021])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_network_batches(n, offset):
+    import torch
+    rng = np.random.default_rng(n)
+    p = L.init_params(4)
+    x = rng.standard_normal((n + offset, omlp.NIN)).astype(np.float32)
+    bits = ((x.view(np.uint32) + 0x7FFF + ((x.view(np.uint32) >> 16) & 1)) >> 16).astype(np.uint32)
+    xb = (bits << 16).view(np.float32).astype(np.float64)[offset:]
+    T = rng.standard_normal((n, omlp.NOUT)).astype(np.float32)
+    pt = torch.from_numpy(p).cuda()
+    xt = torch.from_numpy(bits.astype(np.uint16).view(np.int16)).cuda()[offset:]
+    tt = torch.from_numpy(T).cuda()
+    g, loss = torch.zeros_like(pt), torch.zeros(1, device="cuda")
+    ws = torch.empty(cfs.cfs_mlp_workspace_bytes(n) // 4 + 1 + offset, device="cuda")[offset:]
+    cfs.cfs_mlp_grad(pt.data_ptr(), xt.data_ptr(), tt.data_ptr(), n, ws.data_ptr(), g.data_ptr(), loss.data_ptr())
+    lref, gref = omlp.loss_and_grad(p.astype(np.float64), xb, T.astype(np.float64))
+    gg = g.cpu().numpy().astype(np.float64)
+    assert abs(loss.item() - lref) <= 1e-5 * lref
+    assert np.linalg.norm(gg - gref) <= 1e-5 * np.linalg.norm(gref)
+    ref = omlp.forward(p.astype(np.float64), xb)[0]
+    y = L.predict(p, xt).cpu().numpy().astype(np.float64)
+    assert np.abs(y - ref).max() <= 2e-5 * max(1.0, np.abs(ref).max())
