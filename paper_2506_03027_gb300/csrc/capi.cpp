@@ -1006,7 +1006,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
             e.axis_len[a] = b->d_axis_len[a];
           }
           e.cta0 = fg.ctas;
-          fg.ctas += cfs::filter_ctas(e.n, e.P, ax, fg.Lt);
+          fg.ctas += cfs::filter_ctas(e.n, e.P, ax, fg.Lt, c->p.precision, c->max_delay == 0);
           v.push_back(e);
         }
         fg.nblk = (int)v.size();
@@ -1272,6 +1272,7 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
         f.thomas_k = c->d_thomas_k; f.thomas32 = c->d_thomas32; f.Lmax = c->Lmax; f.alpha = c->p.alpha_f;
         for (int m = 0; m < 6; ++m) f.h[m] = c->filt_h[m];
         f.b1 = c->filt_h[1] - c->p.alpha_f;
+        f.sync = c->max_delay == 0;
         f.only_sync = graph && c->fblock_n;
         f.chain = (&fg != &groups.back() ? 1 : 0) | (&fg != &groups.front() ? 2 : 0);
         f.subs = c->part_n > 1 ? c->d_subs : nullptr;

@@ -293,6 +293,7 @@ struct FilterLaunch {
   double alpha;
   double h[6];             // filter right side: a_0, a_1/2, ..., a_5/2
   double b1;               // a_1/2 - alpha: weight of the first second difference (increment form)
+  int sync;                // no delays in this context (max_delay 0)
   int only_sync;           // graph mode beside the sub-domain filter: return unless the step is synchronous
   const SubDev* subs;      // partitioned context: the sub-domain table (lines of foreign sub-domains are
                            // skipped); null when every sub-domain is computed here
@@ -304,7 +305,7 @@ struct FilterLaunch {
   int chain;
 };
 // CTAs of a launch that one block of size n, split P, takes along `axis` with lines of Lt points
-unsigned filter_ctas(const int* n, const int* P, int axis, int Lt);
+unsigned filter_ctas(const int* n, const int* P, int axis, int Lt, int precision, int sync);
 
 // FP32-intermediate filter of asynchronous steps, all three passes per (sub-domain, variable)
 // (filter_block.cu); cubic sub-domains of n points per axis, n in {16, 32}.

@@ -743,7 +743,8 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 // load latency per issue, DRAM at 8 to 39 %), so a thread now keeps eight of them in flight: own values in
 // groups of eight lines (x) or eight points (y, z), two halo points' levels before their sums, and the
 // eight values that a store adds its increments to.  FP32 form, 12 blocks of 9.3 M points: 2.94 -> 2.02 ms
-// per step; FP64 form, 128^3 in 64 sub-domains: 263 + 200 + 183 -> 200 + 159 + 166 us (x, y, z).
+// per step; FP64 form, 128^3 in 64 sub-domains: 263 + 200 + 183 -> 200 + 159 + 166 us (x, y, z); with the
+// tiles of filter_tile 1.71 ms and 169 + 142 + 147 us.
 //
 // Both forms solve for the increment d = f^ - f, with d = 0 at the first halo point (the Dirichlet
 // closure f^_{-1} = f_{-1}, f^_L = f_L).  The conditions that fix the coefficients -- T = 1 +
@@ -762,10 +763,17 @@ struct FilterTile {
   int TW;  // row stride in doubles (odd: 64-bit accesses of a warp's rows hit distinct banks)
 };
 
-__host__ __device__ inline FilterTile filter_tile(int Lmax) {
+// 128 lines per CTA, a thread each, while their tile leaves room for the seven CTAs per SM that the
+// registers allow; longer lines take 64, so that the threads without a line still help to stage and
+// store and more CTAs overlap staging with solving.  us per pass at 128 / 64 lines: FP64 form, L = 32:
+// 205 / 169 (x), 167 / 142 (y), 168 / 147 (z, 128^3 points); L = 16: 182 / 228 (z, 2.4 M points); FP32 form,
+// L = 48: 527 / 432 (x), 522 / 438 (y, 8.0 M points), L = 24: 397 / 498 (z).  Contexts without delays
+// (sync) read no delayed levels, so there is less to overlap: L = 34, 100^3 points, 85 / 85 (x),
+// 68 / 70 (y), 67 / 72 (z).
+__host__ __device__ inline FilterTile filter_tile(int Lmax, int precision, int sync) {
   FilterTile t;
   t.TW = (Lmax + 10) | 1;
-  t.LN = 128;
+  t.LN = sync || 128 * t.TW * (precision == 1 ? 4 : 8) <= 28 * 1024 ? 128 : 64;
   while (t.LN > 32 && (size_t)(t.LN + 1) * t.TW * 12 > 200 * 1024) t.LN /= 2;
   return t;
 }
@@ -775,8 +783,8 @@ __host__ __device__ inline FilterTile filter_tile(int Lmax) {
 __host__ __device__ inline size_t filter_tile_doubles(const FilterTile& t, int precision) {
   return precision == 1 ? ((size_t)t.LN * t.TW + 1) / 2 : (size_t)t.LN * t.TW;
 }
-__host__ __device__ inline size_t filter_smem_bytes(int Lmax, int precision) {
-  const FilterTile t = filter_tile(Lmax);
+__host__ __device__ inline size_t filter_smem_bytes(int Lmax, int precision, int sync) {
+  const FilterTile t = filter_tile(Lmax, precision, sync);
   return (filter_tile_doubles(t, precision) + t.TW) * 8;
 }
 
@@ -828,7 +836,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
   const FilterBlk& B = f.blks[bi];
   const int n[3] = {B.n[0], B.n[1], B.n[2]};
   const long long strides[3] = {1, n[0], (long long)n[0] * n[1]};
-  const FilterTile tl = filter_tile(f.Lt);
+  const FilterTile tl = filter_tile(f.Lt, F32 ? 1 : 0, f.sync);
   const int LN = tl.LN, TW = tl.TW;
   extern __shared__ __align__(16) double fsm[];
   // [LN][TW] window slots (positions -5 .. len+4): FP64 values, or in the FP32 form FP32 offsets
@@ -946,7 +954,11 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
     }
   };
   // own points: plain copies, by cp.async in the FP64 form; x pass: a warp per line, lanes along it
-  // (contiguous in memory), NB lines at a time; y and z: threads across lines (consecutive x)
+  // (contiguous in memory), NB lines at a time; y and z: threads across lines (consecutive x), NB points
+  // at a time, in the y pass the threads beyond LN further along the lines (the z pass is faster
+  // without: 147 against 154 us at 128^3)
+  const int lfirst = axis == 1 ? threadIdx.x & (LN - 1) : threadIdx.x;
+  const int ifirst = axis == 1 ? NB * (threadIdx.x / LN) : 0, istep = axis == 1 ? NB * (blockDim.x / LN) : NB;
   if (axis == 0) {
     for (int l0w = warp; l0w < nlines; l0w += NB * nwarp)
       for (int i = 5 + lane; i < 5 + len; i += 32) {
@@ -968,10 +980,10 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
           }
       }
   } else {
-    for (int line = threadIdx.x; line < nlines; line += blockDim.x) {
+    for (int line = lfirst; line < nlines; line += blockDim.x) {
       if (!sOk[line]) continue;
       const double* src = Uin + sBase[line];
-      for (int i0 = 5; i0 < 5 + len; i0 += NB) {
+      for (int i0 = 5 + ifirst; i0 < 5 + len; i0 += istep) {
         double v[NB];
 #pragma unroll
         for (int k = 0; k < NB; ++k)
@@ -1167,9 +1179,9 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
         }
       }
   } else {
-    for (int ln = threadIdx.x; ln < nlines; ln += blockDim.x) {
+    for (int ln = lfirst; ln < nlines; ln += blockDim.x) {
       if (!sOk[ln]) continue;
-      for (int i0 = 0; i0 < len; i0 += NB) {
+      for (int i0 = ifirst; i0 < len; i0 += istep) {
         double u[NB];
 #pragma unroll
         for (int k = 0; k < NB; ++k)
@@ -1199,7 +1211,7 @@ int launch_round_table(const double* x, float* y, long long n, void* stream) {
 int filter_prepare(int Lmax, int precision) {
   // (not monotonic in the line length: longer lines take fewer lines per CTA)
   size_t sm = 0;
-  for (int L = 1; L <= Lmax; ++L) sm = std::max(sm, filter_smem_bytes(L, precision));
+  for (int L = 1; L <= Lmax; ++L) sm = std::max(sm, std::max(filter_smem_bytes(L, precision, 0), filter_smem_bytes(L, precision, 1)));
   if (sm > 227 * 1024) return (int)cudaErrorInvalidValue;
   static std::mutex mu;
   static int set_to[64][2] = {};
@@ -1224,10 +1236,10 @@ int filter_prepare(int Lmax, int precision) {
   return (int)e;
 }
 
-unsigned filter_ctas(const int* n, const int* P, int axis, int Lt) {
+unsigned filter_ctas(const int* n, const int* P, int axis, int Lt, int precision, int sync) {
   const int f1 = (axis == 0) ? 1 : 0;
   const int f2 = (axis == 2) ? 1 : 2;
-  const FilterTile tl = filter_tile(Lt);
+  const FilterTile tl = filter_tile(Lt, precision, sync);
   const long long nl = (long long)n[f1] * n[f2];
   return (unsigned)(5LL * P[axis] * ((nl + tl.LN - 1) / tl.LN));
 }
@@ -1235,7 +1247,7 @@ unsigned filter_ctas(const int* n, const int* P, int axis, int Lt) {
 int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f, int axis, int precision,
                   void* stream, long long* launches, const Timer* tm) {
   const unsigned nb = f.ctas;
-  const size_t sm = filter_smem_bytes(f.Lt, precision);
+  const size_t sm = filter_smem_bytes(f.Lt, precision, f.sync);
   cudaStream_t st = (cudaStream_t)stream;
   if (tm) tm->rec(tm->self, 3, 1);
   if (precision == 1) {
