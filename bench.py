@@ -15,8 +15,10 @@ Metric: point-RK-stage updates per second (Mpoint-stage/s) = 128^3 x 5 x steps /
   e2e       the same metric through the public API with host buffers: per step the state is
             copied in from pinned host memory, stepped, and copied back out; host_link gives the
             measured bandwidth of those copies and the floor they put under an e2e step.
-  roofline  the dominant kernel's achieved FP64 rate (algorithmic flops per launch / average
-            event-timed launch duration) against the GB300 FP64 peak.
+  roofline  the dominant kernel's algorithmic bytes per launch / average event-timed launch duration
+            against the measured copy bandwidth (the stage's right-hand side runs on pairs of
+            floats, so no stage kernel is bound by the FP64 pipe); fp64_probe: the FP64 rate, which
+            the line filter and the state update use.
   cpu_baseline  the FP64 CPU oracle on the host cores on a bounded sample of the workload.
 
 forms (same metric, one GPU; each a dict in the JSON line):
@@ -59,30 +61,28 @@ FP64_FLOP_PER_CLK_SM = 4        # 2 FP64 FMA per clock per SM on GB300
 HBM_GBS_FALLBACK = 6800.0
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of each kernel kind, with the sha1 of
-# the flux kernel's source they were taken from (kernels_sha1; null once it changes); filled
-# from profiles/.
-TRAFFIC = {"source_sha1": "c488e6aad06093ada1bf5e2b117f15b1ca3752b9",
-           # k_flux<double,3>: 92.56 MB read + 81.52 MB written per launch in an ncu capture of the
-           # 96^3 case (27 sub-domains of 32^3), x 64/27 for the 64 sub-domains of 128^3
-           "bytes_per_launch": {"flux": 412.6e6}}
+# the stage's source they were taken from (kernels_sha1; null once it changes); filled from profiles/.
+TRAFFIC = {"source_sha1": "751f5b8782ee5c77e8ef08a2457c0f7557b3029e",
+           # 128^3, 64 sub-domains, read + written: k_flux_p 209.4 + 239.9 MB, k_rk_p 491.8 + 120.9 (mean of
+           # the five stages), view (k_at_halo 617.5 + 322.3 once, k_view_p 164.7 + 171.6 five times),
+           # k_filter 327.3 + 57.1 (mean of the three passes)
+           "bytes_per_launch": {"flux": 449.3e6, "stage_update": 612.7e6, "view": 436.9e6, "filter": 384.4e6}}
 
 
 def kernels_sha1(root: str = ROOT) -> str:
-    """sha1 of the source the flux kernel is built from: its section of kernels.cu (from the k_flux
-    banner to the k_rk banner), the device helpers it includes, and the descriptors it reads
-    (Geometry, Physics, SubDev); other kernels' edits leave it unchanged."""
+    """sha1 of the source the stage kernels of the FP64 form are built from: stage_pairs.cu, the
+    headers it includes, and the descriptors it reads (Geometry, SubDev); other kernels' edits leave it
+    unchanged."""
     csrc = os.path.join(root, "paper_2506_03027_gb300", "csrc")
-    with open(os.path.join(csrc, "kernels.cu")) as f:
-        k = f.read()
-    a = k.index("// " + "-" * 79 + " k_flux")
-    b = k.index("// " + "-" * 79 + " k_rk")
-    with open(os.path.join(csrc, "device_common.cuh")) as f:
-        dc = f.read()
+    src = ""
+    for name in ("stage_pairs.cu", "pairs.cuh", "launch_common.cuh", "device_common.cuh"):
+        with open(os.path.join(csrc, name)) as f:
+            src += f.read()
     with open(os.path.join(csrc, "cfs_internal.h")) as f:
         h = f.read()
     structs = "".join(h[h.index("struct " + n + " {"):h.index("};", h.index("struct " + n + " {")) + 2]
-                      for n in ("SubDev", "Geometry", "Physics"))
-    return hashlib.sha1((k[a:b] + dc + structs).encode()).hexdigest()
+                      for n in ("SubDev", "Geometry"))
+    return hashlib.sha1((src + structs).encode()).hexdigest()
 
 
 def host_link(host, nbytes: int) -> dict:
@@ -229,25 +229,24 @@ def face_points(case, depth):
     return tot
 
 
-def algorithmic_flops(case, kind):
-    """FP64 flops per launch that the method needs in each kernel (FMA = 2 flops), counted from
-    the operations of the 3-D Navier-Stokes CD4 path; see the design notes for the breakdown."""
+def algorithmic_bytes(case, kind):
+    """Bytes a launch of each kernel kind of the FP64 form has to move (scratch arrays of pairs: 56 B of
+    primitives and 40 B of fluxes per direction and point; FP64 state and Q: 40 B each per point),
+    averaged over a step's launches."""
     N = case.npts
     r = 2 if case.order == 4 else 1
+    halo, strips = face_points(case, 2 * r), face_points(case, r)
     if kind == "flux":
-        # owned points: 12 CD gradients (5 flops each) + divergence (2) + per direction 33 flops of
-        # fluxes; strip points beyond a face (depth <= r): the 8 gradients the flux along that axis
-        # needs, the divergence and one direction
-        return N * (60 + 2 + 3 * 33) + face_points(case, r) * (40 + 2 + 33)
+        return N * (56 + 120) + halo * 56 + strips * 40
     if kind == "stage_update":
-        # 15 CD derivatives (5 flops) + 3 adds per variable, then Q and U updates (5 per variable)
-        return N * (5 * (15 + 3) + 5 * 5)
+        # U in and out, Q in on every stage but the first and out on every one but the last
+        return N * (120 + 80 + 80 * (case.stages - 1) / case.stages) + strips * 40
     if kind == "view":
-        g = 2 * r
-        halo = face_points(case, g) + 0  # face halos; edges and AT weights counted in the notes
-        return (N + halo) * 16 + halo * 5 * case.levels * 2
+        # one launch for the AT halo values of all stages, one per stage for the primitives
+        at = halo * 40 * (case.levels + case.stages)
+        return (at + case.stages * (N * (40 + 56) + halo * (40 + 56))) / (1 + case.stages)
     if kind == "filter":
-        return N * 5 * 21
+        return N * 80 + face_points(case, 5) / 3 * 40 * case.levels
     return 0
 
 
@@ -457,17 +456,15 @@ def run_ours(args, rank, world, local_rank):
     kinds = {k: v for k, v in ktimes.items() if v[1] > 0 and k != "diagnostics"}
     dom = max(kinds, key=lambda k: kinds[k][0])
     dom_ms, dom_n = kinds[dom]
-    flops = algorithmic_flops(case, dom)
-    achieved_tf = flops / (dom_ms / dom_n * 1e-3) / 1e12
     if args.precision == 0:
-        probe = fp64_peak(local_rank)
-        peak_tf = probe["tflops"]
-        roof = {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
-                "frac": achieved_tf / peak_tf, "kernel": dom,
-                "peak_source": "measured FP64 pipe rate (cfs_fp64_probe: dependent-free DFMA chains, median of 5, "
-                               "on this GPU in this run)",
-                "fp64_probe": probe,
-                "nominal_peak": SM_COUNT * FP64_FLOP_PER_CLK_SM * sm_max * 1e6 / 1e12}
+        peak = peaks.get("hbm_gbs", HBM_GBS_FALLBACK)
+        bytes_ = algorithmic_bytes(case, dom)
+        achieved = bytes_ / (dom_ms / dom_n * 1e-3) / 1e9
+        roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "kernel": dom,
+                "bytes_per_launch": bytes_,
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback",
+                "fp64_probe": dict(fp64_peak(local_rank),
+                                   nominal_tflops=SM_COUNT * FP64_FLOP_PER_CLK_SM * sm_max * 1e6 / 1e12)}
     else:
         # the FP32-intermediate form's dominant kernel: the fused stage against HBM
         roof = fused_roofline(case, ktimes) or {"bound": "hbm", "achieved": None, "peak": None, "unit": "GB/s",
