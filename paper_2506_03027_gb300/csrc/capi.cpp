@@ -253,6 +253,41 @@ static void split_axis(int n, int p, int idx, int* off, int* len) {
   *off = idx * base + (idx < rem ? idx : rem);
 }
 
+// Thomas factors of the compact system (unit diagonal, off-diagonals 1/3) per line length: FP64, or pairs
+static cfs_status upload_compact_factors(cfs_ctx* c) {
+  std::vector<double> ct((size_t)(c->Lmax + 1) * 2 * c->Lmax, 0.0);
+  const double al = 1.0 / 3.0;
+  for (int len = 1; len <= c->Lmax; ++len) {
+    double* cp = ct.data() + (size_t)len * 2 * c->Lmax;
+    double* im = cp + c->Lmax;
+    double m = 1.0;
+    cp[0] = al;
+    im[0] = 1.0;
+    for (int i = 1; i < len; ++i) {
+      m = 1.0 - al * cp[i - 1];
+      cp[i] = al / m;
+      im[i] = 1.0 / m;
+    }
+  }
+  if (c->pairs) {
+    // the same factors as pairs of floats, eliminated in long double, in the same number of bytes
+    float2* t = (float2*)ct.data();
+    for (int len = 1; len <= c->Lmax; ++len) {
+      float2* cp = t + (size_t)len * 2 * c->Lmax;
+      float2* im = cp + c->Lmax;
+      long double ci = 0.0L;
+      for (int i = 0; i < len; ++i) {
+        const long double m = 1.0L - ci / 3.0L;
+        ci = 1.0L / 3.0L / m;
+        cp[i] = cfs::pair_of(ci);
+        im[i] = cfs::pair_of(1.0L / m);
+      }
+    }
+  }
+  CUDA_TRY(c, cudaMemcpy(c->d_cthomas, ct.data(), sizeof(double) * ct.size(), cudaMemcpyHostToDevice), "upload compact factors");
+  return CFS_OK;
+}
+
 extern "C" {
 
 cfs_status cfs_create(const cfs_params* p, void* cuda_stream, cfs_ctx** out) {
@@ -771,37 +806,8 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     c->d_cthomas = dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
     if (c->pairs && cfs::compact_pairs_prepare(c->Lmax) != 0) return fail(c, CFS_ECUDA, "compact passes do not fit this device");
     if (!c->Rbuf || !c->d_cthomas) return fail(c, CFS_ENOMEM, "device allocation failed");
-    // Thomas factors of the compact system (unit diagonal, off-diagonals 1/3) per line length
-    std::vector<double> ct((size_t)(c->Lmax + 1) * 2 * c->Lmax, 0.0);
-    const double al = 1.0 / 3.0;
-    for (int len = 1; len <= c->Lmax; ++len) {
-      double* cp = ct.data() + (size_t)len * 2 * c->Lmax;
-      double* im = cp + c->Lmax;
-      double m = 1.0;
-      cp[0] = al;
-      im[0] = 1.0;
-      for (int i = 1; i < len; ++i) {
-        m = 1.0 - al * cp[i - 1];
-        cp[i] = al / m;
-        im[i] = 1.0 / m;
-      }
-    }
-    if (c->pairs) {
-      // the same factors as pairs of floats, eliminated in long double, in the same number of bytes
-      float2* t = (float2*)ct.data();
-      for (int len = 1; len <= c->Lmax; ++len) {
-        float2* cp = t + (size_t)len * 2 * c->Lmax;
-        float2* im = cp + c->Lmax;
-        long double ci = 0.0L;
-        for (int i = 0; i < len; ++i) {
-          const long double m = 1.0L - ci / 3.0L;
-          ci = 1.0L / 3.0L / m;
-          cp[i] = cfs::pair_of(ci);
-          im[i] = cfs::pair_of(1.0L / m);
-        }
-      }
-    }
-    CUDA_TRY(c, cudaMemcpy(c->d_cthomas, ct.data(), sizeof(double) * ct.size(), cudaMemcpyHostToDevice), "upload compact factors");
+    const cfs_status rc = upload_compact_factors(c);
+    if (rc != CFS_OK) return rc;
   }
   if (c->p.filter && cfs::filter_prepare(c->Lmax, c->p.precision) != 0)
     return fail(c, CFS_EINVAL, "filter: a sub-domain is too long along an axis for the shared-memory line tiles "
@@ -850,7 +856,21 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   }
   if (c->pairs && c->nhalo > 0) {
     c->d_hpair = dev_alloc(c, (2 * sizeof(float4) + sizeof(float2)) * (size_t)c->s * (size_t)c->nhalo);
-    if (!c->d_hpair) return fail(c, CFS_ENOMEM, "device allocation failed");
+    if (!c->d_hpair) {
+      // no room for the halo values of all stages: the FP64 kernels, which need none
+      (void)cudaGetLastError();
+      c->pairs = false;
+      if (!c->Wp) c->Wp = dev_alloc(c, tsz * 7 * (size_t)pbase);
+      if (!c->Wp) return fail(c, CFS_ENOMEM, "device allocation failed");
+      if (c->p.viscous && c->p.visc_law == 1) {
+        const int rc = cfs::pow_tables_init();
+        if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "power tables");
+      }
+      if (c->p.compact) {
+        const cfs_status rc = upload_compact_factors(c);
+        if (rc != CFS_OK) return rc;
+      }
+    }
   }
   // exchange plan of a partitioned context: state offsets and block sizes of the strips sent to /
   // received from every peer, and the packed buffers (5 values per point)

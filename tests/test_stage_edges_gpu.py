@@ -103,3 +103,28 @@ def test_network_batches(n, offset):
     ref = omlp.forward(p.astype(np.float64), xb)[0]
     y = L.predict(p, xt).cpu().numpy().astype(np.float64)
     assert np.abs(y - ref).max() <= 2e-5 * max(1.0, np.abs(ref).max())
+
+
+# no memory for the halo values of all stages: the FP64 kernels take the run
+@pytest.mark.parametrize("kind", ["viscous", "power_law", "euler", "compact"])
+def test_run_without_room_for_the_halo_values(kind, monkeypatch):
+    kw = {"viscous": {}, "power_law": {"visc_law": 1}, "euler": {"viscous": False}, "compact": {"viscous": False, "compact": 1}}[kind]
+    c = I.tgv_case(26, 2, "CAA", **kw)
+    U0 = I.tgv_state(c)
+    c = c.replace(dt=I.cfl_dt(c, U0, 0.25))
+    G, r = (4, 2) if kind != "euler" else (2, 2)
+    w = 13
+    entries = c.nsub * 6 * w * w * G + (c.nsub * 12 * r * r * w if c.viscous else 0)
+    refused = []
+    alloc = cfs.TorchAllocator._alloc
+
+    def without(self, nbytes, user):
+        if nbytes == 40 * c.stages * entries:
+            refused.append(nbytes)
+            return None
+        return alloc(self, nbytes, user)
+    monkeypatch.setattr(cfs.TorchAllocator, "_alloc", without)
+    Ug, _ = gpu_run(c, U0, 10)
+    assert len(refused) == 1
+    e = rel_l2(Ug, orc.run(c, U0, 10))
+    assert np.all(np.isfinite(Ug)) and np.all(e <= PARITY_TOL), e
