@@ -62,7 +62,7 @@ HBM_GBS_FALLBACK = 6800.0
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of each kernel kind, with the sha1 of
 # the stage's source they were taken from (kernels_sha1; null once it changes); filled from profiles/.
-TRAFFIC = {"source_sha1": "751f5b8782ee5c77e8ef08a2457c0f7557b3029e",
+TRAFFIC = {"source_sha1": "136ec8a3bc35a787363802cd030a0add0b46a735",
            # 128^3, 64 sub-domains, read + written: k_flux_p 209.4 + 239.9 MB, k_rk_p 491.8 + 120.9 (mean of
            # the five stages), view (k_at_halo 617.5 + 322.3 once, k_view_p 164.7 + 171.6 five times),
            # k_filter 327.3 + 57.1 (mean of the three passes)

@@ -54,10 +54,13 @@ typedef struct {
   double gamma, mach, re, pr;
   int filter;        /* 1: tenth-order Pade filter (coefficient alpha_f) once per step */
   double alpha_f;
-  int precision;     /* 0: FP64 throughout; 1: FP32 derivative/flux/filter intermediates with
-                        FP64 state and RK accumulation; the AT halo values are summed to FP64
-                        accuracy (compensated FP32 sums over the delayed levels' differences,
-                        FP64 sums for the filter halos) before their rounding to FP32 */
+  int precision;     /* 0: FP64 state, RK accumulation and filter; the right-hand side in FP64, or
+                        (3-D with the filter) on unevaluated sums of two floats, 48 bits, whose
+                        error in dt R is below the rounding of the state; 1: FP32
+                        derivative/flux/filter intermediates with FP64 state and RK accumulation;
+                        the AT halo values are summed to FP64 accuracy (compensated FP32 sums over
+                        the delayed levels' differences; FP64 sums for the line filter's halos)
+                        before their rounding to FP32 */
   int compact;       /* 1: the flux divergence by the sixth-order compact scheme of Eq. 2 (alpha =
                         1/3, a = 14/9, b = 1/9), one tridiagonal solve per sub-domain line, closed by
                         the explicit sixth-order central difference at the first halo point (halo
@@ -247,8 +250,8 @@ cfs_status cfs_diagnostics(cfs_ctx* ctx, double* out);
  * a reference; EINVAL for a negative n or null buffers, ECUDA if the launch fails. */
 cfs_status cfs_eval_power(const double* x, double a, double* y, long long n, void* stream);
 
-/* Measurement aid (no counterpart in the paper): the FP64 pipe rate that the FP64 path's roofline
- * divides by.  Launches `blocks` CTAs of 256 threads, each thread running 8 independent FP64 FMA
+/* Measurement aid (no counterpart in the paper): the FP64 pipe rate, beside which the FP64
+ * path's roofline is reported.  Launches `blocks` CTAs of 256 threads, each thread running 8 independent FP64 FMA
  * chains of `iters` steps, and writes one value per thread to sink (device, blocks x 256 doubles,
  * caller-owned), asynchronously on `stream`.  FMAs executed = blocks x 256 x iters x 8 (2 flops
  * each); the caller times the launch.  EINVAL for a null sink, blocks outside 1..2^20 or

@@ -8,7 +8,9 @@
 // beyond it, halo points by the schedule), the fluxes go through shared memory, and each thread
 // updates its points.  The mass flux is the momentum itself, the off-diagonal momentum flux is
 // shared by the axes, the differences are taken without their factor where the spacings are equal,
-// and a tile without z momentum leaves that component out (it stays zero).
+// and a tile without z momentum leaves that component out (it stays zero).  Five fourth-order steps of
+// 64^2: 359 -> 171 us; a second-order step of 1024^2: 348 -> 303 us (131 us per stage, 81 of them at
+// the FP64 rate).
 #include <cuda_runtime.h>
 
 #include <algorithm>

