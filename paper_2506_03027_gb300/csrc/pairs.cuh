@@ -157,6 +157,12 @@ __device__ __forceinline__ P1 p_pair_of(Triple x) {
   return {s.h, __fadd_rn(s.l, x.q2)};
 }
 __device__ __forceinline__ P1 p_split(double x) { return p_pair_of(p_split3(x)); }
+// x - c for a float c, the difference taken before anything is rounded: 2^-48 of the difference, not of x
+__device__ __forceinline__ P1 p_less(Triple x, float c) {
+  const P1 s = p_2diff(x.t, c);
+  const P1 r = p_2sum(s.h, x.q1);
+  return p_norm(P1{r.h, __fadd_rn(r.l, __fadd_rn(s.l, x.q2))});
+}
 // Two FP64 values as triples, and the difference of two such as pairs: exact but for the last rounding
 // (2^-48 of the difference, however small it is against the values)
 struct Triple2 {
