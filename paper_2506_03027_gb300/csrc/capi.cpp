@@ -253,35 +253,27 @@ static void split_axis(int n, int p, int idx, int* off, int* len) {
   *off = idx * base + (idx < rem ? idx : rem);
 }
 
-// Thomas factors of the compact system (unit diagonal, off-diagonals 1/3) per line length: FP64, or pairs
+// Thomas factors of the compact system (unit diagonal, off-diagonals 1/3): c_i, then 1 / m_i, which
+// depend on the position i in the line alone, so that one row serves lines of every length; FP64, or pairs
+// of floats in the same number of bytes
 static cfs_status upload_compact_factors(cfs_ctx* c) {
-  std::vector<double> ct((size_t)(c->Lmax + 1) * 2 * c->Lmax, 0.0);
+  const int L = c->Lmax;
+  std::vector<double> ct(2 * (size_t)L);
+  float2* pt = (float2*)ct.data();
   const double al = 1.0 / 3.0;
-  for (int len = 1; len <= c->Lmax; ++len) {
-    double* cp = ct.data() + (size_t)len * 2 * c->Lmax;
-    double* im = cp + c->Lmax;
-    double m = 1.0;
-    cp[0] = al;
-    im[0] = 1.0;
-    for (int i = 1; i < len; ++i) {
-      m = 1.0 - al * cp[i - 1];
-      cp[i] = al / m;
-      im[i] = 1.0 / m;
-    }
-  }
-  if (c->pairs) {
-    // the same factors as pairs of floats, eliminated in long double, in the same number of bytes
-    float2* t = (float2*)ct.data();
-    for (int len = 1; len <= c->Lmax; ++len) {
-      float2* cp = t + (size_t)len * 2 * c->Lmax;
-      float2* im = cp + c->Lmax;
-      long double ci = 0.0L;
-      for (int i = 0; i < len; ++i) {
-        const long double m = 1.0L - ci / 3.0L;
-        ci = 1.0L / 3.0L / m;
-        cp[i] = cfs::pair_of(ci);
-        im[i] = cfs::pair_of(1.0L / m);
-      }
+  double cd = 0.0;
+  long double cl = 0.0L;
+  for (int i = 0; i < L; ++i) {
+    if (c->pairs) {
+      const long double m = 1.0L - cl / 3.0L;
+      cl = 1.0L / 3.0L / m;
+      pt[i] = cfs::pair_of(cl);
+      pt[L + i] = cfs::pair_of(1.0L / m);
+    } else {
+      const double m = 1.0 - al * cd;
+      cd = al / m;
+      ct[i] = cd;
+      ct[L + i] = 1.0 / m;
     }
   }
   CUDA_TRY(c, cudaMemcpy(c->d_cthomas, ct.data(), sizeof(double) * ct.size(), cudaMemcpyHostToDevice), "upload compact factors");
@@ -803,7 +795,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     if (!c->all_periodic) return fail(c, CFS_EINVAL, "the compact scheme needs blocks periodic on every face");
     if (c->Lmax > CFS_MAX_LINE) return fail(c, CFS_EINVAL, "the compact scheme's sub-domain lines are limited to 128 points");
     c->Rbuf = (double*)dev_alloc(c, sizeof(double) * 5 * (size_t)N);
-    c->d_cthomas = dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
+    c->d_cthomas = dev_alloc(c, sizeof(double) * 2 * (size_t)c->Lmax);
     if (c->pairs && cfs::compact_pairs_prepare(c->Lmax) != 0) return fail(c, CFS_ECUDA, "compact passes do not fit this device");
     if (!c->Rbuf || !c->d_cthomas) return fail(c, CFS_ENOMEM, "device allocation failed");
     const cfs_status rc = upload_compact_factors(c);
@@ -815,9 +807,9 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   c->diag_total = 0;
   for (const Block& b : c->blocks) c->diag_total += cfs::diag_rows(b.nx, b.ny, b.nz, 1 << 16);
   c->d_partial = (double*)dev_alloc(c, sizeof(double) * DIAG_NQ * (size_t)c->diag_total);
-  c->d_thomas = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
-  c->d_thomas32 = (float*)dev_alloc(c, sizeof(float) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
-  c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * (size_t)(c->Lmax + 1) * 2 * c->Lmax);
+  c->d_thomas = (double*)dev_alloc(c, sizeof(double) * 2 * (size_t)c->Lmax);
+  c->d_thomas32 = (float*)dev_alloc(c, sizeof(float) * 2 * (size_t)c->Lmax);
+  c->d_thomas_k = (double*)dev_alloc(c, sizeof(double) * 2 * (size_t)c->Lmax);
   for (void* q : c->owned)
     if (!q) return fail(c, CFS_ENOMEM, "device allocation failed");
   if (!c->d_n || !c->d_status || !c->ring || !c->buf[0] || !c->buf[1] || !c->Q || (!c->fused && !c->euler2d.tiles && ((!c->Wp && !(c->pairs && !c->p.viscous)) || !c->Phi)) || !c->d_subs || !c->d_W || !c->d_Wf || !c->d_W32 ||
@@ -938,33 +930,23 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   if (c->p.filter && !cfs::pade10_coeffs(c->p.alpha_f, filt)) return fail(c, CFS_EINVAL, "filter coefficients failed");
   c->filt_h[0] = filt[0];
   for (int m = 1; m < 6; ++m) c->filt_h[m] = 0.5 * filt[m];
-  std::vector<double> th((size_t)(c->Lmax + 1) * 2 * c->Lmax, 0.0);
+  // Thomas factors of the filter's lines, c_i and 1 / m_i; they depend on i alone, so one row serves
+  // lines of every length
   const double al = c->p.alpha_f;
-  for (int len = 1; len <= c->Lmax; ++len) {
-    double* cp = th.data() + (size_t)len * 2 * c->Lmax;
-    double* im = cp + c->Lmax;
-    double m = 1.0;
-    cp[0] = al / m;
-    im[0] = 1.0 / m;
-    for (int i = 1; i < len; ++i) {
-      m = 1.0 - al * cp[i - 1];
-      cp[i] = al / m;
-      im[i] = 1.0 / m;
-    }
+  std::vector<double> th(2 * (size_t)c->Lmax), thk(th.size());
+  for (int i = 0; i < c->Lmax; ++i) {
+    const double m = i == 0 ? 1.0 : 1.0 - al * th[i - 1];
+    th[i] = al / m;
+    th[c->Lmax + i] = 1.0 / m;
   }
   // the factors of the FP64 line filter, 1 / m_i times (1 - 2 alpha) / 1024, eliminated in long
   // double (alpha near 1/2 makes the system nearly singular at the shortest wave)
-  std::vector<double> thk(th.size(), 0.0);
-  for (int len = 1; len <= c->Lmax; ++len) {
-    double* cp = thk.data() + (size_t)len * 2 * c->Lmax;
-    double* im = cp + c->Lmax;
-    long double ci = 0.0L;
-    for (int i = 0; i < len; ++i) {
-      const long double m = 1.0L - (long double)al * ci;
-      ci = (long double)al / m;
-      cp[i] = (double)ci;
-      im[i] = (double)((1.0L - 2.0L * (long double)al) / 1024.0L / m);
-    }
+  long double ci = 0.0L;
+  for (int i = 0; i < c->Lmax && c->p.filter && c->p.precision == 0; ++i) {
+    const long double m = 1.0L - (long double)al * ci;
+    ci = (long double)al / m;
+    thk[i] = (double)ci;
+    thk[c->Lmax + i] = (double)((1.0L - 2.0L * (long double)al) / 1024.0L / m);
   }
   cudaStream_t st = c->stream;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_thomas_k, thk.data(), sizeof(double) * thk.size(), cudaMemcpyHostToDevice, st), "upload filter");

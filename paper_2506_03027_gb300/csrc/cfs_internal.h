@@ -225,8 +225,8 @@ struct StageLaunch {
   int max_own;          // largest owned box (points)
   int max_flux;         // largest flux region box (points)
   // compact scheme (Eq. 2, alpha = 1/3): the flux divergence by line solves into R ([5][N], FP64),
-  // then the stage update from R; cthomas = [Lmax + 1 rows][2][Lmax] Thomas factors per line
-  // length (forward factor c'_i, reciprocal pivot 1 / m_i)
+  // then the stage update from R; cthomas = [2][Lmax] Thomas factors (forward factor
+  // c'_i, reciprocal pivot 1 / m_i)
   int compact;
   double* R;
   const void* cthomas;   // double, or float2 on pairs
@@ -285,8 +285,8 @@ struct FilterLaunch {
   const FilterBlk* blks;   // device: the blocks of this launch (their longest lines along the pass
   int nblk;                // axis are all Lt points, which sizes the tiles)
   unsigned ctas;
-  const double* thomas_k;  // device: FP64 form: [Lmax+1 rows][2][Lmax] per line length: c_i, and 1 / m_i
-                           // times the filter's scale (1 - 2 alpha)/1024
+  const double* thomas_k;  // device: FP64 form: [2][Lmax]: c_i, and 1 / m_i times the filter's scale
+                           // (1 - 2 alpha)/1024
   const float* thomas32;   // device: FP32 form: c_i and 1 / m_i rounded to FP32 (d2f_fast)
   int Lmax;
   int Lt;                  // longest sub-domain line of these blocks along the pass axis

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) k_filter_block(Geometry g, Step
   const float rh = d2f_fast(ref), rl = dev_fast(ref, rh, 0.f);
   // Thomas factors of a line of N points (the same on every axis)
   for (int t = tid; t < 2 * N; t += FB_THREADS) {
-    const double* cp = f.thomas + (long long)N * 2 * f.Lmax;
+    const double* cp = f.thomas;
     sTh[t] = (float)(t < N ? cp[t] : cp[f.Lmax + t - N]);
   }
   // ---- load the own values as deviations (unrolled: several loads in flight per thread)

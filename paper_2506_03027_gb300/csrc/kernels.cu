@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(128) k_compact_div(Geometry g, const SubDev* _
   auto f = [&](int i) { return (double)F[(long long)i * st]; };
   const double dl = 0.6 * (45.0 * (f(0) - f(-2)) - 9.0 * (f(1) - f(-3)) + (f(2) - f(-4)));
   const double dr = 0.6 * (45.0 * (f(n + 1) - f(n - 1)) - 9.0 * (f(n + 2) - f(n - 2)) + (f(n + 3) - f(n - 3)));
-  const double* cp = cth + (long long)n * 2 * Lmax;
+  const double* cp = cth;
   const double* im = cp + Lmax;
   // forward sweep: the eliminated right sides go to a per-thread array (local memory)
   double w[CFS_MAX_LINE];
@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       const bool tiny = ex < 200;
       ex = max(ex, 200);
       const int q20 = (ex - 1023 - 52) * (1 << 20);
-      const double* __restrict__ cp = f.thomas_k + (long long)len * 2 * f.Lmax;
+      const double* __restrict__ cp = f.thomas_k;
       const double* __restrict__ im = cp + f.Lmax;
       long long s[10];
       auto diff10 = [&](int i) {
@@ -1116,7 +1116,7 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       // longer read), back substitution leaves the increment of point i there; the store adds it
       // to the FP64 value.
       float* frow = ftile + line * TW;
-      const float* cp32 = f.thomas32 + (long long)len * 2 * f.Lmax;  // the factors in FP32
+      const float* cp32 = f.thomas32;  // the factors in FP32
       const float* im32 = cp32 + f.Lmax;
       float win[11];
 #pragma unroll

@@ -668,7 +668,7 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
   cp_async_wait_all();
   __syncthreads();
   if (act) {
-    const float2* __restrict__ cp = cth + (long long)n * 2 * Lmax;
+    const float2* __restrict__ cp = cth;
     const float2* __restrict__ im = cp + Lmax;
     auto f = [&](int i) -> Pr<V> { return p_of(sm[(i + 4) * LD + tid]); };
     // closures at the first halo points, 0.6 (45 (f_1 - f_-1) - 9 (f_2 - f_-2) + (f_3 - f_-3)), times alpha

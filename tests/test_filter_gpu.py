@@ -101,3 +101,18 @@ def test_nonfinite_value_reaches_its_lines(value):
         s.diagnostics()
     s.close()
     assert np.all(np.isnan(U[2, 9, 8, :10]))
+
+
+@pytest.mark.parametrize("filt", [False, True])
+def test_memory_grows_with_the_line_not_its_square(filt, monkeypatch):
+    """A context's tables (and the time to prepare them) are proportional to the longest line."""
+    def total(n):
+        sizes = []
+        alloc = cfs.TorchAllocator._alloc
+        with monkeypatch.context() as m:
+            m.setattr(cfs.TorchAllocator, "_alloc", lambda self, b, user: (sizes.append(b), alloc(self, b, user))[1])
+            s = cfs.Solver(I.vortex_case(32, 1).replace(nx=n, ny=8, filter=filt))
+            s.close()
+        return sum(sizes)
+    a, b = total(340), total(680)
+    assert b <= 2.0 * a, (a, b)
