@@ -619,6 +619,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     pp.kgM2 = cfs::pair_of(ph.kgM2);
     pp.kT0 = cfs::pair_of((long double)ph.kgM2 * ph.gm1 * pp.Eref);
     pp.H = cfs::pair_of((long double)ph.gamma * pp.Eref);
+    pp.Hd = (double)pp.H.x + (double)pp.H.y;
     pp.ivT = cfs::pair_of(ph.ivT);
     pp.visc_law = ph.visc_law;
     pp.visc_exp = cfs::pair_of(ph.visc_exp);

@@ -129,6 +129,7 @@ struct Physics {
 // (gamma - 1) E_ref: kT = (kgM2 p' + kT0) / rho with kT0 = kgM2 p_ref, H = E_ref + p_ref.
 struct PairPhysics {
   float2 gm1, kgM2, kT0, H, ivT;
+  double Hd;  // the value of the pair H
   float Eref;
   int visc_law;
   float2 visc_exp;
@@ -247,7 +248,7 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 // halo states of all s stages once per asynchronous step: H [2 s][nhalo] float4, [s][nhalo] float2.
 int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const StageLaunch& a, const void* H,
                        void* stream, long long* launches, const Timer* tm);
-// (compact scheme: StageLaunch::R holds N float4, N float4, N float2; cthomas the factors as pairs)
+// (compact scheme: StageLaunch::R holds N float4, N float4, N doubles)
 int compact_pairs_prepare(int Lmax);
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
                    const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm);

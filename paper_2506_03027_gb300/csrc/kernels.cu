@@ -788,26 +788,6 @@ __host__ __device__ inline size_t filter_smem_bytes(int Lmax, int precision, int
   return (filter_tile_doubles(t, precision) + t.TW) * 8;
 }
 
-// x in units of 2^(E-52), rounded down, E + 1023 = ex the exponent field of a number no smaller
-__device__ __forceinline__ long long fixed_point(double x, int ex) {
-  const int hi = __double2hiint(x);
-  const int sh = min(ex - ((hi >> 20) & 0x7ff), 63);
-  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x));
-  const long long sg = hi >> 31;
-  return ((m ^ sg) - sg) >> sh;
-}
-
-// g 2^(q20 >> 20) in FP64 (|g| < 2^63), truncated to 53 bits, on the integer pipe
-__device__ __forceinline__ double from_fixed_point(long long g, int q20) {
-  const long long sg = g >> 63;
-  const unsigned long long m = (unsigned long long)((g ^ sg) - sg);
-  const int lz = __clzll((long long)m);
-  const unsigned long long t = (m << lz) >> 11;  // the leading one at bit 52
-  // (adding the leading one to the exponent field raises it by one)
-  const int hi = (int)(t >> 32) + ((1023 + 62 - lz) << 20) + q20;
-  return m ? __hiloint2double(hi | ((int)sg & (int)0x80000000), (int)t) : 0.0;
-}
-
 template <typename T, int axis>
 __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
   if (f.chain == 0) {

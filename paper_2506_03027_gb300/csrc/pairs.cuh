@@ -183,6 +183,17 @@ __device__ __forceinline__ P2 p_diff(Triple2 a, Triple2 b) {
 }
 // pair -> FP64: one FP64 addition
 __device__ __forceinline__ double p_double(P1 a) { return f2d_fast(a.h) + f2d_fast(a.l); }
+// The same of a normalised pair on the integer pipe, in a third of the issue slots of the addition: l as a
+// multiple L of the last place of h as FP64 (below a power of two, of half of it), added to the bit
+// pattern.  l is left out where |h| < 2^-66.
+__device__ __forceinline__ double p_double_int(P1 a) {
+  const unsigned hb = __float_as_uint(a.h), e = (hb >> 23) & 255u;
+  float l = __fmul_rn(a.l, __uint_as_float((306u - e) << 23));  // 2^(52 - E)
+  l = __uint_as_float(__float_as_uint(l) ^ (hb & 0x80000000u));
+  if ((hb & 0x7fffffu) == 0 && l < 0.f) l = __fadd_rn(l, l);
+  const int L = e > 60u && e < 255u ? __float2int_rn(l) : 0;
+  return __longlong_as_double(__double_as_longlong(f2d_fast(a.h)) + L);
+}
 
 // x^a = exp(a ln x) for positive x, table-driven after Tang (ACM TOMS 1989, 1990) as the FP64 power
 // of kernels.cu, on pairs.  ln x: x = m 2^e with m in [1, 2); the top six mantissa bits pick a

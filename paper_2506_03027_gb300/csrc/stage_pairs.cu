@@ -15,12 +15,18 @@
 // values interleaved where the same operation acts on both, so that one 16-byte load and the
 // packed FP32 instructions serve (u, v) and (w, kappa T) together:
 //   W    A (u, v), B (w, kappa T), C (rho, p - p_ref): float4 {h, h, l, l}; D (rho E + p - H_ref): float2
-//   Phi  per direction a: M (x, y momentum), E (z momentum, energy): float4; N (mass): float2
+//   Phi  per direction a: M (x, y momentum), E (z momentum, energy): float4; N (mass): FP64
+// The mass flux is the momentum itself: the update differences it in FP64, from the state inside a Cartesian
+// sub-domain and from N elsewhere (the strips beyond its faces; curvilinear blocks, times the metric row),
+// which the view stores.  The energy flux is H_ref times it plus a remainder, -((rho E + p -
+// H_ref) - H_ref (rho - 1)) u, which alone is a pair: pairs of the whole, 250 u at M = 0.1, would
+// raise the energy's error of a step from the 1.8e-14 of its rounding to 3.2e-14, pairs of the mass flux
+// the density's from 1.1e-16 to 1.5e-16.
 // and one more, once per asynchronous step: k_at_halo forms the AT halo values of all stages from
 // one read of the delayed levels (they would be read once per stage otherwise).
 //
-// 128^3 in 64 sub-domains, us per launch, FP64 -> pairs: view 150 -> 79 (DRAM at 52 % of its rate and
-// issue at 51 %), flux 384 -> 114 (49 %, 72 %), update 290 -> 122 (60 %, 44 %); the halo values, once per
+// 128^3 in 64 sub-domains, us per launch, FP64 -> pairs: view 150 -> 84 (DRAM at 52 % of its rate and
+// issue at 51 %), flux 384 -> 110 (49 %, 72 %), update 290 -> 135 (60 %, 44 %); the halo values, once per
 // step instead of inside the view, 223 (52 %, 55 %).
 #include <cuda_runtime.h>
 
@@ -78,14 +84,35 @@ __device__ __forceinline__ void store_prims(const WView& W, long long o, const P
   W.D[o] = p_store(r.et);
 }
 
+// What the energy flux carries beside H_ref times the mass flux, per unit velocity: -((rho E + p - H_ref) -
+// H_ref (rho - 1))
+__device__ __forceinline__ P1 rest_enthalpy(const PairPhysics& ph, P1 et, P1 rho) {
+  return p_norm(p_neg(p_fma(cst(ph.H), p_norm(p_sub(P1{1.f, 0.f}, rho)), et)));
+}
+
+// Mass fluxes rho U_a of a point from its FP64 momentum m(0 .. 2), times the metric row on a
+// curvilinear block, along axis `as` or (as < 0) every axis; stored at scratch index o.
+template <class F>
+__device__ __forceinline__ void store_mass_flux(const Geometry& g, const SubDev& d, void* Phi, long long o, F m, int ci, int cj,
+                                                int as) {
+  const double* __restrict__ M = nullptr;
+  if (d.mbase >= 0) M = g.metric + d.mbase + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
+  double* __restrict__ N = (double*)((float4*)Phi + 6 * g.Ptot) + o;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (as >= 0 && as != a) continue;
+    double f = m(a);
+    if (M) f = a < 2 ? fma(M[(2 * a + 1) * d.mpl], m(1), M[2 * a * d.mpl] * m(0)) : M[4 * d.mpl] * f;
+    N[a * g.Ptot] = f;
+  }
+}
+
 // Inviscid combined fluxes -F_a (Eq. A2) at scratch index o, along axis `as` or (as < 0) every axis;
-// M: the metric terms of the point on a curvilinear block, or null.  The Cartesian mass flux is the
-// momentum itself.
+// M: the metric terms of the point on a curvilinear block, or null.  The mass flux is stored apart.
 __device__ __forceinline__ void store_euler_flux(const PairPhysics& ph, void* Phi, long long P, long long o, const PrimsP& r,
                                                  int as, const float2* M, long long pl) {
   float4* __restrict__ F4 = (float4*)Phi;
-  float2* __restrict__ F2 = (float2*)(F4 + 6 * P);
-  const P1 netH = p_neg(p_norm(p_add(r.et, cst(ph.H)))), zero = {0.f, 0.f};
+  const P1 rest = rest_enthalpy(ph, r.et, r.rho), zero = {0.f, 0.f};
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     if (as >= 0 && as != a) continue;
@@ -105,9 +132,8 @@ __device__ __forceinline__ void store_euler_flux(const PairPhysics& ph, void* Ph
       }
       n = p_norm(p_neg(p_mul(r.rho, U)));
     }
-    F2[(long long)a * P + o] = p_store(n);
     F4[(long long)(2 * a) * P + o] = p_store(p_norm(p_sub(p_mul(p_bc(n), r.uv), pxy)));
-    F4[(long long)(2 * a + 1) * P + o] = p_store(p_norm(p_sub(p_mul(p_pair(n, netH), p_pair(r.w, U)), p_pair(pz, zero))));
+    F4[(long long)(2 * a + 1) * P + o] = p_store(p_norm(p_sub(p_mul(p_pair(n, rest), p_pair(r.w, U)), p_pair(pz, zero))));
   }
 }
 
@@ -308,20 +334,24 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
 
 // The stage input as primitives, own points and halo points in one launch (as k_view).  EULER: the
 // inviscid fluxes, which need no more than the point itself, instead of the primitives -- along
-// every axis at own points, along the axis of the face a halo point lies beyond.
+// every axis at own points, along the axis of the face a halo point lies beyond.  Both store the mass
+// fluxes that the state does not hold: beyond a face to the depth that is differenced, and on
+// curvilinear blocks.
 template <bool EULER>
-__global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
+__global__ void __launch_bounds__(256, EULER ? 3 : 4) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
                                                 const double* __restrict__ ring, int in_ring, const SubDev* __restrict__ subs,
                                                 const int2* __restrict__ halo, long long nhalo, const float4* __restrict__ H4,
-                                                const float2* __restrict__ H2, void* Wp, int stage, int s, int own_blocks, int rev) {
+                                                const float2* __restrict__ H2, void* Wp, void* Phi, int stage, int s, int own_blocks, int rev) {
   pdl_enter();
   sc = resolve(sc);
   const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
-  auto put = [&](const SubDev& d, const PrimsP& r, long long o, int ci, int cj, int as) {
+  // (m: the FP64 momentum; as 3: no flux)
+  auto put = [&](const SubDev& d, const PrimsP& r, auto m, long long o, int ci, int cj, int as) {
+    if (as < 3 && (as >= 0 || d.mbase >= 0)) store_mass_flux(g, d, Phi, o, m, ci, cj, as);
     if (EULER) {
       const float2* M = nullptr;
       if (d.mbase >= 0) M = g.metric_p + d.mbase + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
-      store_euler_flux(ph, Wp, g.Ptot, o, r, as, M, d.mpl);
+      store_euler_flux(ph, Phi, g.Ptot, o, r, as, M, d.mpl);
     } else {
       store_prims(w_view(Wp, g.Ptot), o, r);
     }
@@ -339,7 +369,7 @@ __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, Step
     double u[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) u[v] = Uin[d.bbase + v * d.bN + gi];
-    put(d, prims_of(ph, u), d.pbase + q, ci, cj, -1);
+    put(d, prims_of(ph, u), [&](int a) { return u[1 + a]; }, d.pbase + q, ci, cj, -1);
     return;
   }
   const long long e = (b - nown) * blockDim.x + threadIdx.x;
@@ -347,10 +377,12 @@ __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, Step
   const int2 hv = halo[e];
   const SubDev& d = subs[hv.x];
   const long long o = d.pbase + hv.y;
-  HaloPoint h{};
-  int as = -1;
-  if (EULER || sc.mode == 0 || d.ebase >= 0) h = halo_point(g, d, hv);
-  if (EULER) as = h.ci < 0 || h.ci >= d.sx ? 0 : (h.cj < 0 || h.cj >= d.sy ? 1 : 2);
+  const HaloPoint h = halo_point(g, d, hv);
+  // the axis along which the point's flux is differenced: that of the one face it lies beyond
+  const int dx = h.ci < 0 ? -h.ci : h.ci - d.sx + 1, dy = h.cj < 0 ? -h.cj : h.cj - d.sy + 1,
+            dz = h.ck < 0 ? -h.ck : h.ck - d.sz + 1;
+  int as = dx > 0 ? 0 : (dy > 0 ? 1 : 2);
+  if (max(dx, max(dy, dz)) > g.fs || (dx > 0) + (dy > 0) + (dz > 0) > 1) as = 3;
   if (sc.mode == 0 || (d.ebase >= 0 && h.beyond && any_own_source(h, d))) {
     double u[5];
     if (h.beyond) {
@@ -360,12 +392,13 @@ __global__ void __launch_bounds__(256) k_view_p(Geometry g, PairPhysics ph, Step
 #pragma unroll
       for (int v = 0; v < 5; ++v) u[v] = Uin[v * d.bN + h.gi];
     }
-    put(d, prims_of(ph, u), o, h.ci, h.cj, as);
+    put(d, prims_of(ph, u), [&](int a) { return u[1 + a]; }, o, h.ci, h.cj, as);
     return;
   }
   const int m = sc.mode == 2 ? 0 : stage;
   const P2 a = p_of(H4[(long long)(2 * m) * nhalo + e]), c = p_of(H4[(long long)(2 * m + 1) * nhalo + e]);
-  put(d, prims_p(ph, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e])), o, h.ci, h.cj, as);
+  put(d, prims_p(ph, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e])),
+      [&](int i) { return p_double(i == 0 ? p_y(a) : (i == 1 ? p_x(c) : p_y(c))); }, o, h.ci, h.cj, as);
 }
 
 // ------------------------------------------------------------------------------- k_flux_p
@@ -384,24 +417,14 @@ __device__ __forceinline__ Pr<W> diff2(const float4* __restrict__ f, long long q
   const W lo = v_add(v_fma(m8, y.l, x.l), v_fma(m8, v_sub(c.l, d.l), v_sub(a.l, b.l)));
   return p_norm(Pr<W>{s.h, v_add(s.l, lo)});
 }
-template <int R>
-__device__ __forceinline__ P1 diff1(const float2* __restrict__ f, long long q, long long st) {
-  const P1 c = p_of(f[q + st]), d = p_of(f[q - st]);
-  if (R == 1) return p_norm(p_sub(c, d));
-  const P1 a = p_of(f[q + 2 * st]), b = p_of(f[q - 2 * st]);
-  const P1 x = p_2diff(a.h, b.h), y = p_2diff(c.h, d.h);
-  const P1 s = p_2sum(x.h, v_mul(-8.f, y.h));
-  const float lo = v_add(v_fma(-8.f, y.l, x.l), v_fma(-8.f, v_sub(c.l, d.l), v_sub(a.l, b.l)));
-  return p_norm(P1{s.h, v_add(s.l, lo)});
-}
 
 }  // namespace
 
 __device__ float g_pow_pair[POW_PAIR_TAB];  // tables of p_pow
 
-// Combined fluxes at the owned points and the strips of r points beyond each face (the flux along
-// that face's axis only), thread by thread as in k_flux.  CURV: the context has curvilinear
-// blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.  Bound by instruction issue
+// Combined fluxes (but the mass flux, which is the momentum) at the owned points and the strips of r
+// points beyond each face (the flux along that face's axis only), thread by thread as in k_flux.
+// CURV: the context has curvilinear blocks.  R: stencil radius (CD4: 2).  LAW: the viscosity is the power law.  Bound by instruction issue
 // and memory about equally (128^3: half of each).  A Cartesian point forms most of its pairs of values from
 // components of others, and bringing those into register pairs for the packed instructions costs more than
 // they save: two plain instructions each are faster (121 -> 114 us at 128^3); on curvilinear blocks,
@@ -427,11 +450,10 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
   const float4* __restrict__ Cc = A + 2 * P;
   const float2* __restrict__ D = (const float2*)(A + 3 * P);
   float4* __restrict__ F4 = (float4*)Phi;
-  float2* __restrict__ F2 = (float2*)(F4 + 6 * P);
 
   const P2 uv = p_of<V2>(A[q]), wT = p_of<V2>(B[q]), rp = p_of<V2>(Cc[q]);
   const P1 w = p_x(wT), rho = p_x(rp), pr = p_y(rp);
-  const P1 netH = p_neg(p_norm(p_add(p_of(D[q]), cst(ph.H))));  // -(rho E + p)
+  const P1 rest = rest_enthalpy(ph, p_of(D[q]), rho);
   P1 iv = cst(ph.ivT);  // the factor of the viscous terms: 1/Re x (units of the differences) x mu
   // differences of (u, v) and (w, kappa T) along each axis
   P2 Gx = diff2<R, V2>(A, q, st[0]), Gy = diff2<R, V2>(A, q, st[1]), Gz = diff2<R, V2>(A, q, st[2]);
@@ -483,8 +505,7 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
     const P2 x = p_mul(uv, ra);
     return p_norm(p_fma(w, rc, p_add(p_add(p_x(x), p_y(x)), dT)));
   };
-  auto put = [&](int a, P1 n, P2 m, P2 e) {
-    F2[(long long)a * P + q] = p_store(n);
+  auto put = [&](int a, P2 m, P2 e) {
     F4[(long long)(2 * a) * P + q] = p_store(p_norm(m));
     F4[(long long)(2 * a + 1) * P + q] = p_store(p_norm(e));
   };
@@ -502,17 +523,17 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
       const P2 r0 = p_bc<V2>(p_x(row)), r1 = p_bc<V2>(p_y(row));
       P2 m = p_sub(p_mul(p_bc<V2>(n), uv), p_mul(p_bc<V2>(pr), row));
       m = p_fma(p_bc<V2>(iv), p_norm(p_fma(r0, p_pair<V2>(p_x(td), t01), p_mul(r1, p_pair<V2>(t01, p_y(td))))), m);
-      P2 e = p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, Uc));
+      P2 e = p_mul(p_pair<V2>(n, rest), p_pair<V2>(w, Uc));
       e = p_fma(p_bc<V2>(iv), p_norm(p_fma(r0, p_pair<V2>(p_x(t2), b0), p_mul(r1, p_pair<V2>(p_y(t2), b1)))), e);
-      put(a, n, m, e);
+      put(a, m, e);
     }
     if (as < 0 || as == 2) {
       const P1 Uc = p_norm(p_mul(zz, w)), n = p_norm(p_neg(p_mul(rho, Uc)));
       const P2 iz = p_bc<V2>(p_norm(p_mul(iv, zz)));
       const P2 m = p_fma(iz, t2, p_mul(p_bc<V2>(n), uv));
-      P2 e = p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, Uc));
+      P2 e = p_mul(p_pair<V2>(n, rest), p_pair<V2>(w, Uc));
       e = p_sub(e, p_pair<V2>(p_mul(zz, pr), zero));
-      put(2, n, m, p_fma(iz, p_pair<V2>(t22, b2), e));
+      put(2, m, p_fma(iz, p_pair<V2>(t22, b2), e));
     }
     return;
   }
@@ -520,36 +541,38 @@ __global__ void __launch_bounds__(256, CURV ? 3 : 4) k_flux_p(Geometry g, PairPh
   if (as < 0 || as == 0) {
     const P2 ra = p_pair<V2>(p_x(td), t01);
     P2 m = p_sub(p_mul(p_bc<V2>(p_x(nuv)), uv), p_pair<V2>(pr, zero));
-    P2 e = p_mul(p_pair<V2>(p_x(nuv), netH), p_pair<V2>(w, p_x(uv)));
-    put(0, p_x(nuv), p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_x(t2), heat(ra, p_x(t2), p_y(Hx))), e));
+    P2 e = p_mul(p_pair<V2>(p_x(nuv), rest), p_pair<V2>(w, p_x(uv)));
+    put(0, p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_x(t2), heat(ra, p_x(t2), p_y(Hx))), e));
   }
   if (as < 0 || as == 1) {
     const P2 ra = p_pair<V2>(t01, p_y(td));
     P2 m = p_sub(p_mul(p_bc<V2>(p_y(nuv)), uv), p_pair<V2>(zero, pr));
-    P2 e = p_mul(p_pair<V2>(p_y(nuv), netH), p_pair<V2>(w, p_y(uv)));
-    put(1, p_y(nuv), p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_y(t2), heat(ra, p_y(t2), p_y(Hy))), e));
+    P2 e = p_mul(p_pair<V2>(p_y(nuv), rest), p_pair<V2>(w, p_y(uv)));
+    put(1, p_fma(p_bc<V2>(iv), ra, m), p_fma(p_bc<V2>(iv), p_pair<V2>(p_y(t2), heat(ra, p_y(t2), p_y(Hy))), e));
   }
   if (as < 0 || as == 2) {
     const P1 n = p_norm(p_neg(p_mul(rho, w)));
     const P2 m = p_mul(p_bc<V2>(n), uv);
-    P2 e = p_sub(p_mul(p_pair<V2>(n, netH), p_pair<V2>(w, w)), p_pair<V2>(pr, zero));
-    put(2, n, p_fma(p_bc<V2>(iv), t2, m), p_fma(p_bc<V2>(iv), p_pair<V2>(t22, heat(t2, t22, p_y(Hz))), e));
+    P2 e = p_sub(p_mul(p_pair<V2>(n, rest), p_pair<V2>(w, w)), p_pair<V2>(pr, zero));
+    put(2, p_fma(p_bc<V2>(iv), t2, m), p_fma(p_bc<V2>(iv), p_pair<V2>(t22, heat(t2, t22, p_y(Hz))), e));
   }
 }
 
 // ------------------------------------------------------------------------------- k_rk_p
 
-// dt R = sum_a dt D_a Phi_a (times J on a curvilinear block) in pairs, then the low-storage update
-// Q = A Q + dt R, U^(m) = U^(m-1) + B Q in FP64.  Bound by memory latency (310 B of traffic per point
-// at half the DRAM rate, 64 registers): Q and the stage input, not read again before they
-// would be evicted anyway, pass by the caches as streaming accesses and leave the L2 to the fluxes that
-// neighbouring points share (128^3: 147 -> 122 us).
+// dt R = sum_a dt D_a Phi_a (times J on a curvilinear block), of the mass flux in FP64, of the others on
+// pairs, the energy taking H_ref times the mass's; then the low-storage update Q = A Q + dt R, U^(m) =
+// U^(m-1) + B Q in FP64.  Bound by memory latency (310 B of traffic per point at half the DRAM rate, 64
+// registers) and by the FP64 pipe, on which 24 operations per point take as long as 1,500 others: the
+// pairs are converted on the integer pipe (154 -> 135 us at 128^3).  Q, density and energy, not read again
+// before they would be evicted anyway, pass by the caches as streaming accesses and leave the L2
+// to what neighbouring points share.
 template <int R>
 __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
                                               const void* __restrict__ Phi, const double* __restrict__ Uin0,
                                               double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
-                                              int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
-                                              int last, int rev) {
+                                              int out_ring, double* __restrict__ Q, double A, double B, float2 dt, double dtd,
+                                              double H, int first, int last, int rev) {
   pdl_enter();
   sc = resolve(sc);
   const double* Uin = ring_or(Uin0, in_ring, ring, sc, 0);
@@ -565,31 +588,39 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
   const long long gi = d.bbase + (long long)(d.ox + ci) + (long long)d.bnx * ((long long)(d.oy + cj) + (long long)d.bny * (d.oz + ck));
   const long long P = g.Ptot;
   const float4* __restrict__ F4 = (const float4*)Phi;
-  const float2* __restrict__ F2 = (const float2*)(F4 + 6 * P);
+  const double* __restrict__ N = (const double*)(F4 + 6 * P);
   double qv[5], uv[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     qv[c] = first ? 0.0 : __ldcs(Q + c * d.bN + gi);
-    uv[c] = __ldcs(Uin + c * d.bN + gi);
+    uv[c] = c >= 1 && c <= 3 ? Uin[c * d.bN + gi] : __ldcs(Uin + c * d.bN + gi);
   }
   P2 m = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, e = m;
-  P1 n = {0.f, 0.f};
+  double n = 0.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const P1 k = p_norm(p_mul(cst(dt), cst(d.cg[a])));
     m = p_fma(p_bc(k), diff2<R>(F4 + (long long)(2 * a) * P, q, st[a]), m);
     e = p_fma(p_bc(k), diff2<R>(F4 + (long long)(2 * a + 1) * P, q, st[a]), e);
-    n = p_fma(k, diff1<R>(F2 + (long long)a * P, q, st[a]), n);
+    const int ca = a == 0 ? ci : (a == 1 ? cj : ck), sa = a == 0 ? d.sx : (a == 1 ? d.sy : d.sz);
+    const long long gst = a == 0 ? 1 : (a == 1 ? (long long)d.bnx : (long long)d.bnx * d.bny);
+    const double *pu = Uin + (1 + a) * d.bN + gi, *pn = N + a * P + q;
+    const bool cart = d.mbase < 0;
+    auto mass = [&](int o) { return cart && (unsigned)(ca + o) < (unsigned)sa ? __ldg(pu + o * gst) : __ldg(pn + o * st[a]); };
+    const double d1 = mass(1) - mass(-1);
+    n = R == 1 ? fma(d.c1[a], d1, n) : fma(d.c2[a], fma(-8.0, d1, mass(2) - mass(-2)), n);
   }
+  n *= -dtd;
   if (d.mbase >= 0) {
-    const P1 J = p_of(g.metric_p[d.mbase + 6 * d.mpl + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G)]);
+    const long long mq = d.mbase + 6 * d.mpl + (long long)(d.ox + ci + g.G) + (long long)d.mx * (d.oy + cj + g.G);
+    const P1 J = p_of(g.metric_p[mq]);
     m = p_mul(p_bc(J), p_norm(m));
     e = p_mul(p_bc(J), p_norm(e));
-    n = p_mul(J, p_norm(n));
+    n *= g.metric[mq];
   }
   m = p_norm(m);
   e = p_norm(e);
-  const double dtR[5] = {p_double(p_norm(n)), p_double(p_x(m)), p_double(p_y(m)), p_double(p_x(e)), p_double(p_y(e))};
+  const double dtR[5] = {n, p_double_int(p_x(m)), p_double_int(p_y(m)), p_double_int(p_x(e)), fma(H, n, p_double_int(p_y(e)))};
   const bool wallpt = d.wall && ((((d.wall >> 0) & 1) && ci == 0) || (((d.wall >> 1) & 1) && ci == d.sx - 1) ||
                                  (((d.wall >> 2) & 1) && cj == 0) || (((d.wall >> 3) & 1) && cj == d.sy - 1));
 #pragma unroll
@@ -605,92 +636,120 @@ __global__ void __launch_bounds__(256, 4) k_rk_p(Geometry g, StepSched sc, const
 // ------------------------------------------------------------------------------- compact scheme
 
 // Sixth-order compact derivative (Eq. 2, alpha = 1/3; closure as k_compact_div) of the fluxes along
-// `axis` on pairs, one thread per line and group of components: M (x, y momentum), E (z momentum,
-// energy), N (mass).  In units of b/(4h) the right side is (f_{i+2} - f_{i-2}) + 28 (f_{i+1} -
-// f_{i-1}); the sweeps z_i = rhs_i - c_{i-1} z_{i-1}, x_i = z_i / m_i - c_i x_{i+1} keep z_i in
-// shared memory ([n][CL], CL lines per CTA), where every line is staged first with all its loads in
-// flight (x: a warp along a line, y and z: a warp across 32 lines).  dt R gathers in the
-// pairs R over the x and y passes; the z pass adds its part and takes the low-storage update, so the
-// divergence is neither written nor read a third time.  In FP64 the three passes were bound by
-// their eight operations per value (190 us each at 128^3).
+// `axis`, one thread per line and group of components: M (x, y momentum) and E (z momentum, what the
+// energy flux carries beside H_ref times the mass flux) on pairs, N (mass) into FP64.  In units
+// of b/(4h) the right side is (f_{i+2} - f_{i-2}) + 28 (f_{i+1} - f_{i-1}); the sweeps z_i = rhs_i -
+// c_{i-1} z_{i-1}, x_i = z_i / m_i - c_i x_{i+1} keep z_i in shared memory ([n][CL], CL lines per CTA),
+// where every line is staged first with all its loads in flight (x: a warp along a line, y and z: a warp
+// across 32 lines).  dt R gathers in R over the x and y passes; the z pass adds its part and takes the
+// low-storage update, so the divergence is neither written nor read a third time.  The energy's dt R takes
+// H_ref times the whole of the mass's, so the y launch solves N along z as well (into the
+// scratch of its x flux, which the launch before consumed) and the z launch's E group updates the density
+// too.  In FP64 the three passes were bound by their eight operations per value (190 us each at 128^3).
 constexpr int CL = 64;  // lines per CTA
 
-__device__ __forceinline__ void cp_async_pair(float4* dst, const float4* src) { cp_async16(dst, src); }
-__device__ __forceinline__ void cp_async_pair(float2* dst, const float2* src) { cp_async8(dst, src); }
-
-template <class V>
-struct PairMem;
-template <>
-struct PairMem<float2> {
-  using T = float4;
-};
-template <>
-struct PairMem<float> {
-  using T = float2;
-};
-
-template <int axis, class V>
-__device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d, const typename PairMem<V>::T* __restrict__ F,
-                                              typename PairMem<V>::T* __restrict__ R, const float2* __restrict__ cth, int Lmax,
-                                              float2 dt, unsigned char* raw, int grp, const double* __restrict__ Uin,
-                                              double* __restrict__ Uout, double* __restrict__ Q, double A, double B, int first,
-                                              int last) {
-  using T = typename PairMem<V>::T;
-  T* sm = reinterpret_cast<T*>(raw);
-  constexpr int LD = axis == 0 ? CL + 1 : CL;
-  constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
-  const int sz[3] = {d.sx, d.sy, d.sz};
-  const int n = sz[axis], nl = sz[a1] * sz[a2], tid = threadIdx.x;
-  const int l0 = blockIdx.x * CL, nlines = min(CL, nl - l0);
-  const long long st[3] = {1, d.ex, (long long)d.ex * d.ey}, gst[3] = {1, d.bnx, (long long)d.bnx * d.bny};
-  const long long q0 = d.pbase + g.G + st[1] * g.G + st[2] * g.Gz;
-  const long long r0 = d.bbase / 5 + (long long)d.ox + gst[1] * d.oy + gst[2] * d.oz;
+// The lines of a CTA along `axis` of sub-domain d
+template <int axis>
+struct LineSet {
+  static constexpr int LD = axis == 0 ? CL + 1 : CL;
+  static constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  int n, nlines, l0, s1;
+  long long st[3], gst[3], q0, r0;
+  __device__ __forceinline__ LineSet(const Geometry& g, const SubDev& d) {
+    const int sz[3] = {d.sx, d.sy, d.sz};
+    n = sz[axis];
+    s1 = sz[a1];
+    l0 = blockIdx.x * CL;
+    nlines = min(CL, s1 * sz[a2] - l0);
+    st[0] = gst[0] = 1;
+    st[1] = d.ex;
+    st[2] = (long long)d.ex * d.ey;
+    gst[1] = d.bnx;
+    gst[2] = (long long)d.bnx * d.bny;
+    q0 = d.pbase + g.G + st[1] * g.G + st[2] * g.Gz;
+    r0 = d.bbase / 5 + (long long)d.ox + gst[1] * d.oy + gst[2] * d.oz;
+  }
   // line l of the CTA: its first point in the padded box and in the state's point order
-  auto line_at = [&](int l, long long& q, long long& r) {
-    const int t = l0 + l, t1 = t % sz[a1], t2 = t / sz[a1];
+  __device__ __forceinline__ void at(int l, long long& q, long long& r) const {
+    const int t = l0 + l, t1 = t % s1, t2 = t / s1;
     q = q0 + t1 * st[a1] + t2 * st[a2];
     r = r0 + t1 * gst[a1] + t2 * gst[a2];
-  };
-  const bool act = tid < nlines;
-  long long q = 0, r = 0;
-  if (act) line_at(tid, q, r);
-  if (axis == 0) {
-    const int lane = tid & 31;
-    for (int l = tid >> 5; l < nlines; l += CL / 32) {
-      long long ql, rl;
-      line_at(l, ql, rl);
-      for (int i = lane; i < n + 8; i += 32) cp_async_pair(sm + i * LD + l, F + ql + i - 4);
-    }
-  } else if (act) {
-    for (int i = 0; i < n + 8; ++i) cp_async_pair(sm + i * LD + tid, F + q + (i - 4) * st[axis]);
   }
-  cp_async_commit();
-  cp_async_wait_all();
-  __syncthreads();
-  if (act) {
+  // the lines and 4 points beyond each end to shared memory
+  __device__ __forceinline__ void stage(float4* sm, const float4* __restrict__ F) const {
+    const int tid = threadIdx.x;
+    long long q, r;
+    if (axis == 0) {
+      const int lane = tid & 31;
+      for (int l = tid >> 5; l < nlines; l += CL / 32) {
+        at(l, q, r);
+        for (int i = lane; i < n + 8; i += 32) cp_async16(sm + i * LD + l, F + q + i - 4);
+      }
+    } else if (tid < nlines) {
+      at(tid, q, r);
+      for (int i = 0; i < n + 8; ++i) cp_async16(sm + i * LD + tid, F + q + (i - 4) * st[axis]);
+    }
+    cp_async_commit();
+    cp_async_wait_all();
+    __syncthreads();
+  }
+  // the solved lines along x from shared memory to R
+  __device__ __forceinline__ void unstage(const float4* sm, float4* __restrict__ R) const {
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < nlines; l += CL / 32) {
+      long long q, r;
+      at(l, q, r);
+      for (int i = lane; i < n; i += 32) R[r + i] = sm[i * LD + l];
+    }
+  }
+};
+
+// What the z launch's update takes beside the group's own dt R
+struct CompactUpdate {
+  const double* Uin;
+  double *Uout, *Q;
+  const double *RN, *NZ;  // the mass's dt R: of the x and y passes in point order, of the z pass in scratch order
+  double A, B, H;
+  int first, last;
+};
+
+// grp 0: M, 1: E
+template <int axis, int grp>
+__device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d, const float4* __restrict__ F,
+                                              float4* __restrict__ R, const float2* __restrict__ cth, int Lmax, float2 dt,
+                                              unsigned char* raw, const CompactUpdate& up) {
+  float4* sm = reinterpret_cast<float4*>(raw);
+  const LineSet<axis> ls(g, d);
+  constexpr int LD = LineSet<axis>::LD;
+  const int n = ls.n, tid = threadIdx.x;
+  ls.stage(sm, F);
+  if (tid < ls.nlines) {
+    long long q, r;
+    ls.at(tid, q, r);
     const float2* __restrict__ cp = cth;
     const float2* __restrict__ im = cp + Lmax;
-    auto f = [&](int i) -> Pr<V> { return p_of(sm[(i + 4) * LD + tid]); };
+    auto f = [&](int i) -> P2 { return p_of(sm[(i + 4) * LD + tid]); };
     // closures at the first halo points, 0.6 (45 (f_1 - f_-1) - 9 (f_2 - f_-2) + (f_3 - f_-3)), times alpha
-    auto cst1 = [](float h, float l) { return Pr<V>{v_bc<V>(h), v_bc<V>(l)}; };
-    auto closure = [&](Pr<V> d1, Pr<V> d2, Pr<V> d3) {
-      Pr<V> x = p_fma(cst1(45.f, 0.f), d1, d3);
+    auto cst1 = [](float h, float l) { return P2{v_bc<float2>(h), v_bc<float2>(l)}; };
+    auto closure = [&](P2 d1, P2 d2, P2 d3) {
+      P2 x = p_fma(cst1(45.f, 0.f), d1, d3);
       x = p_norm(p_fma(cst1(-9.f, 0.f), d2, x));
       return p_norm(p_mul(cst1(0.2f, -2.9802323e-09f), x));  // 0.6 / 3
     };
-    Pr<V> w[5];  // f(i - 2) .. f(i + 2)
-    const Pr<V> m4 = f(-4), m3 = f(-3);
+    P2 w[5];  // f(i - 2) .. f(i + 2)
+    const P2 m4 = f(-4), m3 = f(-3);
     w[0] = f(-2);
     w[1] = f(-1);
     w[2] = f(0);
     w[3] = f(1);
     w[4] = f(2);
-    const Pr<V> dl = closure(p_norm(p_sub(w[2], w[0])), p_norm(p_sub(w[3], m3)), p_sub(w[4], m4));
-    Pr<V> z = {v_bc<V>(0.f), v_bc<V>(0.f)};
+    const P2 dl = closure(p_norm(p_sub(w[2], w[0])), p_norm(p_sub(w[3], m3)), p_sub(w[4], m4));
+    P2 z = {v_bc<float2>(0.f), v_bc<float2>(0.f)};
     float2 cm = make_float2(0.f, 0.f);
 #pragma unroll 4
     for (int i = 0; i < n; ++i) {
-      Pr<V> rhs = p_fma(cst1(28.f, 0.f), p_norm(p_sub(w[3], w[1])), p_sub(w[4], w[0]));
+      P2 rhs = p_fma(cst1(28.f, 0.f), p_norm(p_sub(w[3], w[1])), p_sub(w[4], w[0]));
       if (i == 0) rhs = p_sub(rhs, dl);
       if (i == n - 1)
         rhs = p_sub(rhs, closure(p_norm(p_sub(w[4], w[2])), p_norm(p_sub(f(n + 2), w[1])), p_sub(f(n + 3), w[0])));
@@ -704,26 +763,28 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
     }
     // k = dt b / (4h): the difference coefficient of the block is -1 / (12 h)
     const P1 k1 = p_norm(p_mul(p_norm(p_mul(P1{dt.x, dt.y}, cst(d.cg[axis]))), P1{-0.33333334f, 9.934108e-09f}));
-    const Pr<V> kk = cst1(k1.h, k1.l);
-    Pr<V> x = {v_bc<V>(0.f), v_bc<V>(0.f)};
-    constexpr bool two = sizeof(V) == 8;
+    const P2 kk = cst1(k1.h, k1.l);
+    P2 x = {v_bc<float2>(0.f), v_bc<float2>(0.f)};
+    constexpr int NU = grp == 0 ? 2 : 3;  // variables that the z launch updates: 1, 2 or 3, 4, 0
+    auto comp = [](int v) { return grp == 0 ? 1 + v : (v < 2 ? 3 + v : 0); };
     // four points at a time, what they read from memory in flight before the first is solved
     for (int i0 = n - 1; i0 >= 0; i0 -= 4) {
-      T rv[4];
-      double qv[4][2], uv[4][2];
+      float4 rv[4];
+      double qv[4][NU], uv[4][NU], nv[4];
       if (axis > 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (i0 - k >= 0) {
-            const long long ri = r + (long long)(i0 - k) * gst[axis], pt = ri - d.bbase / 5;
+            const long long ri = r + (long long)(i0 - k) * ls.gst[axis], pt = ri - d.bbase / 5;
             rv[k] = R[ri];
             if (axis == 2) {
 #pragma unroll
-              for (int v = 0; v < (two ? 2 : 1); ++v) {
-                const long long gi = d.bbase + (long long)(two ? 1 + 2 * grp + v : 0) * d.bN + pt;
-                qv[k][v] = first ? 0.0 : __ldcs(Q + gi);
-                uv[k][v] = __ldcs(Uin + gi);
+              for (int v = 0; v < NU; ++v) {
+                const long long gi = d.bbase + (long long)comp(v) * d.bN + pt;
+                qv[k][v] = up.first ? 0.0 : __ldcs(up.Q + gi);
+                uv[k][v] = __ldcs(up.Uin + gi);
               }
+              if (grp == 1) nv[k] = up.RN[ri] + up.NZ[q + (i0 - k) * ls.st[2]];
             }
           }
       }
@@ -733,71 +794,161 @@ __device__ __forceinline__ void compact_group(const Geometry& g, const SubDev& d
         if (i < 0) break;
         const float2 c = __ldg(cp + i), m = __ldg(im + i);
         x = p_norm(p_fma(cst1(-c.x, -c.y), x, p_mul(cst1(m.x, m.y), p_of(sm[i * LD + tid]))));
-        const Pr<V> kx = p_mul(kk, x);
+        const P2 kx = p_mul(kk, x);
         if (axis == 0) {
           sm[i * LD + tid] = p_store(p_norm(kx));
           continue;
         }
-        const long long ri = r + (long long)i * gst[axis];
-        const Pr<V> sum = p_norm(p_add(kx, p_of(rv[k])));
+        const long long ri = r + (long long)i * ls.gst[axis];
+        const P2 sum = p_norm(p_add(kx, p_of(rv[k])));
         if (axis == 1) {
           R[ri] = p_store(sum);
           continue;
         }
         const long long pt = ri - d.bbase / 5;
-        auto update = [&](int v, int comp, P1 dtR) {
-          const long long gi = d.bbase + (long long)comp * d.bN + pt;
-          const double t = p_double(dtR);
-          const double qn = first ? t : fma(A, qv[k][v], t);
-          if (!last) __stcs(Q + gi, qn);
-          Uout[gi] = fma(B, qn, uv[k][v]);
-        };
-        if constexpr (two) {
-          update(0, 1 + 2 * grp, p_x(sum));
-          update(1, 2 + 2 * grp, p_y(sum));
-        } else {
-          update(0, 0, sum);
+        double dtR[3] = {p_double(p_x(sum)), p_double(p_y(sum)), 0.0};
+        if (grp == 1) {
+          dtR[1] = fma(up.H, nv[k], dtR[1]);
+          dtR[2] = nv[k];
         }
+#pragma unroll
+        for (int v = 0; v < NU; ++v) {
+          const long long gi = d.bbase + (long long)comp(v) * d.bN + pt;
+          const double qn = up.first ? dtR[v] : fma(up.A, qv[k][v], dtR[v]);
+          if (!up.last) __stcs(up.Q + gi, qn);
+          up.Uout[gi] = fma(up.B, qn, uv[k][v]);
+        }
+      }
+    }
+  }
+  if (axis == 0) ls.unstage(sm, R);
+}
+
+// N along one axis: x into R, y added to it, z into the scratch array NZ, in FP64.  The line's right side is
+// differenced in FP64; the system is solved on pairs for what the solution x has beside 3/5 of it (the
+// system's row sum is 5/3), (1/3, 1, 1/3) y = -1/5 delta^2 rhs, which is small for smooth fluxes, so
+// that the sweeps' rounding is small against that of x.
+template <int axis>
+__device__ __forceinline__ void compact_mass(const Geometry& g, const SubDev& d, const double* __restrict__ Uin,
+                                             const double* __restrict__ F, double* __restrict__ R, double* __restrict__ NZ,
+                                             const float2* __restrict__ cth, int Lmax, double dt, unsigned char* raw) {
+  const LineSet<axis> ls(g, d);
+  constexpr int LD = LineSet<axis>::LD;
+  const int n = ls.n, tid = threadIdx.x;
+  float4* sm = reinterpret_cast<float4*>(raw);  // a slot: the FP64 flux in its first half, later the pairs z and rhs
+  auto val = [&](int i, int l) -> double& { return *reinterpret_cast<double*>(sm + i * LD + l); };
+  // the lines and 4 points beyond each end: inside the sub-domain from the momentum (indexed as R is, in point
+  // order over all blocks), beyond its faces from the scratch array
+  const double* __restrict__ U = Uin + d.bbase + (1 + axis) * d.bN - d.bbase / 5;
+  auto copy = [&](int l, int i, long long q, long long r) {
+    const int k = i - 4;
+    cp_async8(&val(i, l), (unsigned)k < (unsigned)n ? U + r + k * ls.gst[axis] : F + q + k * ls.st[axis]);
+  };
+  long long q, r;
+  if (axis == 0) {
+    for (int l = tid >> 5; l < ls.nlines; l += CL / 32) {
+      ls.at(l, q, r);
+      for (int i = tid & 31; i < n + 8; i += 32) copy(l, i, q, r);
+    }
+  } else if (tid < ls.nlines) {
+    ls.at(tid, q, r);
+    for (int i = 0; i < n + 8; ++i) copy(tid, i, q, r);
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  if (tid < ls.nlines) {
+    ls.at(tid, q, r);
+    auto f = [&](int i) { return val(i + 4, tid); };
+    const P1 fifth = {0.2f, -2.9802323e-09f};
+    // 1/3 of the closure at the first halo point, 0.6 (45 (f_1 - f_-1) - 9 (f_2 - f_-2) + (f_3 - f_-3))
+    auto closure = [&](double d1, double d2, double d3) { return p_mul(fifth, p_split(fma(45.0, d1, fma(-9.0, d2, d3)))); };
+    auto right = [](const double* w) { return p_split(fma(28.0, w[3] - w[1], w[4] - w[0])); };
+    double w[5] = {f(-3), f(-2), f(-1), f(0), f(1)};  // f(i - 2) .. f(i + 2)
+    auto next = [&](double v) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k] = w[k + 1];
+      w[4] = v;
+    };
+    P1 rm = right(w);  // right sides of points i - 1, i, i + 1
+    next(f(2));
+    P1 rc = right(w);
+    const P1 yl = p_norm(p_sub(closure(w[2] - w[0], w[3] - f(-3), w[4] - f(-4)), p_mul(fifth, rm)));
+    P1 z = {0.f, 0.f};
+    float2 cm = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      next(f(i + 3));
+      const P1 rn = right(w);
+      P1 h = p_norm(p_mul(fifth, p_norm(p_sub(p_sub(rc, rm), p_sub(rn, rc)))));
+      if (i == 0) h = p_sub(h, yl);
+      if (i == n - 1)
+        h = p_sub(h, p_norm(p_sub(closure(w[3] - w[1], w[4] - w[0], f(n + 3) - f(n - 3)), p_mul(fifth, rn))));
+      z = p_norm(p_fma(P1{-cm.x, -cm.y}, z, h));
+      // (slot i held f(i - 4), no longer read)
+      sm[i * LD + tid] = make_float4(z.h, z.l, rc.h, rc.l);
+      cm = __ldg(cth + i);
+      rm = rc;
+      rc = rn;
+    }
+    const double kk = dt * d.c2[axis] / 3.0;  // -dt b / (4h)
+    P1 y = {0.f, 0.f};
+    for (int i0 = n - 1; i0 >= 0; i0 -= 4) {
+      double rv[4];
+      if (axis == 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (i0 - k >= 0) rv[k] = R[r + (long long)(i0 - k) * ls.gst[1]];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 - k;
+        if (i < 0) break;
+        const float2 c = __ldg(cth + i), m = __ldg(cth + Lmax + i);
+        const float4 v = sm[i * LD + tid];
+        y = p_norm(p_fma(P1{-c.x, -c.y}, y, p_mul(P1{m.x, m.y}, P1{v.x, v.y})));
+        const double x = p_double_int(p_norm(p_fma(P1{0.6f, -2.3841858e-08f}, P1{v.z, v.w}, y)));
+        if (axis == 0) val(i, tid) = kk * x;
+        else if (axis == 1) R[r + (long long)i * ls.gst[1]] = fma(kk, x, rv[k]);
+        else NZ[q + i * ls.st[2]] = kk * x;
       }
     }
   }
   if (axis == 0) {
     __syncthreads();
-    const int lane = tid & 31;
-    for (int l = tid >> 5; l < nlines; l += CL / 32) {
-      long long ql, rl;
-      line_at(l, ql, rl);
-      for (int i = lane; i < n; i += 32) R[rl + i] = sm[i * LD + l];
+    for (int l = tid >> 5; l < ls.nlines; l += CL / 32) {
+      ls.at(l, q, r);
+      for (int i = tid & 31; i < n; i += 32) R[r + i] = val(i, l);
     }
   }
 }
 
+// blockIdx.y: M, E and, in the x and y launches, N along that axis, in the y launch N along z
 template <int axis>
-__global__ void __launch_bounds__(CL) k_compact_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs,
-                                                  const void* __restrict__ Phi, void* __restrict__ Rv,
-                                                  const float2* __restrict__ cth, int Lmax, const double* __restrict__ Uin0,
-                                                  double* __restrict__ Uout0, const double* __restrict__ ring, int in_ring,
-                                                  int out_ring, double* __restrict__ Q, double A, double B, float2 dt, int first,
-                                                  int last, int rev) {
+__global__ void __launch_bounds__(CL) k_compact_p(Geometry g, StepSched sc, const SubDev* __restrict__ subs, void* Phi,
+                                                  void* __restrict__ Rv, const float2* __restrict__ cth, int Lmax,
+                                                  const double* __restrict__ Uin0, double* __restrict__ Uout0,
+                                                  const double* __restrict__ ring, int in_ring, int out_ring,
+                                                  double* __restrict__ Q, double A, double B, double H, float2 dt, double dtd,
+                                                  int first, int last, int rev) {
   extern __shared__ __align__(16) unsigned char craw[];
   pdl_enter();
   const SubDev& d = subs[rev ? gridDim.z - 1 - blockIdx.z : blockIdx.z];
-  constexpr int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
-  const int sz[3] = {d.sx, d.sy, d.sz};
-  if (!d.own || (int)blockIdx.x * CL >= sz[a1] * sz[a2]) return;
-  sc = resolve(sc);
-  const double* Uin = axis == 2 ? ring_or(Uin0, in_ring, ring, sc, 0) : nullptr;
-  double* Uout = axis == 2 ? const_cast<double*>(ring_or(Uout0, out_ring, ring, sc, 1)) : nullptr;
-  const int grp = blockIdx.y;  // 0: M, 1: E, 2: N
+  const int grp = blockIdx.y;
+  const int lines = grp == 3 || axis == 2 ? d.sx * d.sy : (axis == 0 ? d.sy * d.sz : d.sx * d.sz);
+  if (!d.own || (int)blockIdx.x * CL >= lines) return;
   const long long P = g.Ptot, N = g.N;
   const float4* F4 = (const float4*)Phi;
+  double* FN = (double*)((float4*)Phi + 6 * P);
   float4* R4 = (float4*)Rv;
-  if (grp < 2)
-    compact_group<axis, float2>(g, d, F4 + (2 * axis + grp) * P, R4 + grp * N, cth, Lmax, dt, craw, grp, Uin, Uout, Q, A, B,
-                                first, last);
-  else
-    compact_group<axis, float>(g, d, (const float2*)(F4 + 6 * P) + axis * P, (float2*)(R4 + 2 * N), cth, Lmax, dt, craw, grp, Uin,
-                               Uout, Q, A, B, first, last);
+  double* RN = (double*)(R4 + 2 * N);
+  sc = resolve(sc);
+  const double* Uin = ring_or(Uin0, in_ring, ring, sc, 0);
+  CompactUpdate up{};
+  if (axis == 2) up = {Uin, const_cast<double*>(ring_or(Uout0, out_ring, ring, sc, 1)), Q, RN, FN, A, B, H, first, last};
+  if (grp == 0) compact_group<axis, 0>(g, d, F4 + 2 * axis * P, R4, cth, Lmax, dt, craw, up);
+  else if (grp == 1) compact_group<axis, 1>(g, d, F4 + (2 * axis + 1) * P, R4 + N, cth, Lmax, dt, craw, up);
+  else if (axis < 2 && grp == 2) compact_mass<axis>(g, d, Uin, FN + axis * P, RN, nullptr, cth, Lmax, dtd, craw);
+  else if (axis == 1) compact_mass<2>(g, d, Uin, FN + 2 * P, nullptr, FN, cth, Lmax, dtd, craw);
 }
 
 // ------------------------------------------------------------------------------- launchers
@@ -850,22 +1001,21 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   const int per_stage = a.compact ? 4 : (g.viscous ? 3 : 2);
   auto rev = [&](int k) { return (a.stage * per_stage + k) & 1; };
   // (inviscid: the fluxes come straight from the view)
-  TIMED(tm, 0, (launch_pdl(g.viscous ? k_view_p<false> : k_view_p<true>, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring,
-                           a.in_ring, a.subs, (const int2*)a.halo, a.nhalo, H4, H2, g.viscous ? a.Wp : a.Phi, a.stage, a.s,
-                           (int)own_blocks, rev(0))));
+  TIMED(tm, 0, (launch_pdl(g.viscous ? k_view_p<false> : k_view_p<true>, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring, a.in_ring, a.subs, (const int2*)a.halo,
+                           a.nhalo, H4, H2, a.Wp, a.Phi, a.stage, a.s, (int)own_blocks, rev(0))));
   if (launches) *launches += 1;
   if (a.compact) {
     // x and y passes gather dt R, the z pass takes the update
     const size_t slots = (size_t)(a.Lmax + 8) * CL, staged = (size_t)(a.Lmax + 8) * (CL + 1);
-    const dim3 gc(nblk((long long)a.Lmax * a.Lmax, CL), 3, g.nsub);
     const float2* cth = (const float2*)a.cthomas;
-    auto run = [&](auto kernel, size_t smem, int k) {
-      TIMED(tm, 2, (launch_pdl(kernel, gc, dim3(CL), smem * sizeof(float4), st, g, sc, a.subs, (const void*)a.Phi, (void*)a.R, cth,
-                               a.Lmax, a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last, rev(k))));
+    auto run = [&](auto kernel, size_t smem, unsigned groups, int k) {
+      const dim3 gc(nblk((long long)a.Lmax * a.Lmax, CL), groups, g.nsub);
+      TIMED(tm, 2, (launch_pdl(kernel, gc, dim3(CL), smem * sizeof(float4), st, g, sc, a.subs, a.Phi, (void*)a.R, cth, a.Lmax,
+                               a.Uin, a.Uout, a.ring, a.in_ring, a.out_ring, a.Q, a.A, a.B, ph.Hd, dt, a.dt, a.first, a.last, rev(k))));
     };
-    run(k_compact_p<0>, staged, 1);
-    run(k_compact_p<1>, slots, 2);
-    run(k_compact_p<2>, slots, 3);
+    run(k_compact_p<0>, staged, 3, 1);
+    run(k_compact_p<1>, slots, 4, 2);
+    run(k_compact_p<2>, slots, 2, 3);
     if (launches) *launches += 3;
     return (int)cudaGetLastError();
   }
@@ -881,7 +1031,7 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   }
   auto rk = g.r == 2 ? k_rk_p<2> : k_rk_p<1>;
   TIMED(tm, 2, (launch_pdl(rk, gr, dim3(B), 0, st, g, sc, a.subs, (const void*)a.Phi, a.Uin, a.Uout, a.ring, a.in_ring,
-                           a.out_ring, a.Q, a.A, a.B, dt, a.first, a.last, rev(g.viscous ? 2 : 1))));
+                           a.out_ring, a.Q, a.A, a.B, dt, a.dt, ph.Hd, a.first, a.last, rev(g.viscous ? 2 : 1))));
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
 }

@@ -80,3 +80,14 @@ def test_momentum_of_one_step(form, mach):
     tol = 2 * np.sqrt(3) * c.dt / c.dx * flux
     for v in (1, 2, 3):
         assert rms(e[v]) <= rounding(c, U, v) + tol, (v, rms(e[v]), rounding(c, U, v), tol)
+
+
+# the mass flux is the momentum, the energy flux 250 times it at M = 0.1
+@pytest.mark.parametrize("mach", [0.1, 0.01])
+@pytest.mark.parametrize("form", list(FORMS))
+def test_density_and_energy_of_one_step(form, mach):
+    c, U, e = one_step(form, mach)
+    # the rounding of the sums U + B Q, and what else there is, independent of it, below half of that:
+    # sqrt(1 + 1/4)
+    for v in (0, 4):
+        assert rms(e[v]) <= 1.12 * rounding(c, U, v), (v, rms(e[v]), rounding(c, U, v))
