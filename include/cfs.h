@@ -68,8 +68,10 @@ typedef struct {
                         blocks periodic on every face, FP64 (precision 0) only; 0: explicit CD */
 } cfs_params;
 
-/* Device allocator used by cfs_finalize and cfs_set_schedule.  alloc returns a device pointer
- * aligned to at least 256 bytes or NULL; free releases it. */
+/* Device allocator used by cfs_finalize, cfs_set_schedule and cfs_set_halo_model.  alloc returns a
+ * device pointer aligned to at least 256 bytes or NULL; free releases it.  Asynchronous 3-D runs keep the
+ * halo values of all stages of a step; where that allocation, or a later one beside it, returns NULL, they
+ * keep those of one stage, with the same results in more time. */
 typedef void* (*cfs_alloc_fn)(size_t bytes, void* user);
 typedef void (*cfs_free_fn)(void* ptr, void* user);
 

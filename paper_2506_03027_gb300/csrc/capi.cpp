@@ -126,7 +126,11 @@ struct cfs_ctx {
   // FP64 form on pairs of floats (3-D Navier-Stokes)
   bool pairs = false;
   cfs::PairPhysics pphys{};
-  void* d_hpair = nullptr;       // AT halo states of every stage, [2 s][nhalo] float4 then [s][nhalo] float2
+  // AT halo states of every stage, [2 s][nhalo] float4 then [s][nhalo] float2, from the first asynchronous
+  // schedule on; where there is no memory for them, of one stage (hpair_one), formed before it
+  void* d_hpair = nullptr;
+  bool hpair_one = false;
+  bool wh_one = false;           // FP32 form: the halo store Wh likewise
   float2* d_metric_p = nullptr;  // metric planes as pairs
 
   Geometry geo{};
@@ -230,9 +234,12 @@ static void* default_alloc(size_t bytes, void*) {
 }
 static void default_free(void* p, void*) { cudaFree(p); }
 
+static bool halo_store_gives_way(cfs_ctx* c);
+
 static void* dev_alloc(cfs_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 256;
   void* p = c->alloc(bytes, c->user);
+  if (!p && halo_store_gives_way(c)) p = c->alloc(bytes, c->user);
   if (p) c->owned.push_back(p);
   return p;
 }
@@ -245,6 +252,40 @@ static void dev_free(cfs_ctx* c, void* p) {
       c->freef(p, c->user);
       return;
     }
+}
+
+// Memory for the AT halo states of the FP64 form on pairs: of all stages, or (`all` false, or refused)
+// of one.  That one lies in the flux scratch, free until the view has read it, or, where the
+// view fills the flux scratch itself (inviscid runs), in 40 B per halo point of its own.  Both give the same
+// values; one reads the delayed levels once per stage instead of once per step.
+static cfs_status halo_states(cfs_ctx* c, bool all) {
+  const size_t one = (2 * sizeof(float4) + sizeof(float2)) * (size_t)c->nhalo;
+  c->hpair_one = true;
+  if (all && (c->d_hpair = dev_alloc(c, one * (size_t)c->s))) {
+    c->hpair_one = false;
+    return CFS_OK;
+  }
+  (void)cudaGetLastError();
+  c->d_hpair = c->p.viscous ? c->Phi : dev_alloc(c, one);
+  return c->d_hpair ? CFS_OK : fail(c, CFS_ENOMEM, "device allocation failed");
+}
+
+// An allocation was refused: the store of all stages' halo values, if there is one, shrinks to one stage's.
+static bool halo_store_gives_way(cfs_ctx* c) {
+  (void)cudaGetLastError();
+  const bool pairs = c->d_hpair && !c->hpair_one, fused = c->Wh && !c->wh_one;
+  if (!pairs && !fused) return false;
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+  c->graph_dirty = true;
+  if (pairs) {
+    dev_free(c, c->d_hpair);
+    c->d_hpair = nullptr;
+    return halo_states(c, false) == CFS_OK;
+  }
+  dev_free(c, c->Wh);
+  c->wh_one = true;
+  c->Wh = (float*)dev_alloc(c, sizeof(float) * 8 * (size_t)c->geo.Ptot);
+  return c->Wh != nullptr;
 }
 
 static void split_axis(int n, int p, int idx, int* off, int* len) {
@@ -757,6 +798,11 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     c->nwork = (int)(work.size() / 4);
     c->d_work = (int*)dev_alloc(c, sizeof(int) * work.size());
     c->Wh = (float*)dev_alloc(c, sizeof(float) * 8 * c->s * (size_t)pbase);
+    c->wh_one = !c->Wh;
+    if (c->wh_one) {
+      (void)cudaGetLastError();
+      c->Wh = (float*)dev_alloc(c, sizeof(float) * 8 * (size_t)pbase);
+    }
     if (!c->d_work || !c->Wh) return fail(c, CFS_ENOMEM, "device allocation failed");
     CUDA_TRY(c, cudaMemcpy(c->d_work, work.data(), sizeof(int) * work.size(), cudaMemcpyHostToDevice), "upload work list");
     int dev = 0, sms = 0;
@@ -845,24 +891,6 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       c->d_halo = (int*)dev_alloc(c, sizeof(int) * hl.size());
       if (!c->d_halo) return fail(c, CFS_ENOMEM, "device allocation failed");
       CUDA_TRY(c, cudaMemcpy(c->d_halo, hl.data(), sizeof(int) * hl.size(), cudaMemcpyHostToDevice), "upload halo list");
-    }
-  }
-  if (c->pairs && c->nhalo > 0) {
-    c->d_hpair = dev_alloc(c, (2 * sizeof(float4) + sizeof(float2)) * (size_t)c->s * (size_t)c->nhalo);
-    if (!c->d_hpair) {
-      // no room for the halo values of all stages: the FP64 kernels, which need none
-      (void)cudaGetLastError();
-      c->pairs = false;
-      if (!c->Wp) c->Wp = dev_alloc(c, tsz * 7 * (size_t)pbase);
-      if (!c->Wp) return fail(c, CFS_ENOMEM, "device allocation failed");
-      if (c->p.viscous && c->p.visc_law == 1) {
-        const int rc = cfs::pow_tables_init();
-        if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "power tables");
-      }
-      if (c->p.compact) {
-        const cfs_status rc = upload_compact_factors(c);
-        if (rc != CFS_OK) return rc;
-      }
     }
   }
   // exchange plan of a partitioned context: state offsets and block sizes of the strips sent to /
@@ -1055,6 +1083,10 @@ cfs_status cfs_set_schedule(cfs_ctx* c, int algo, int at, int L, long long nstep
     CUDA_TRY(c, cudaStreamSynchronize(c->stream), "upload schedule");
     c->sched_steps = nsteps;
   }
+  if (algo != 0 && c->pairs && c->nhalo > 0 && !c->d_hpair) {
+    const cfs_status rc = halo_states(c, true);
+    if (rc != CFS_OK) return rc;
+  }
   c->algo = algo;
   c->at = at ? 1 : 0;
   c->L = algo == 1 ? L : 1;
@@ -1209,17 +1241,24 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
     sc.LH = c->LH;
   }
-  if (c->fused && (graph || sc.mode != 0)) {
-    const int rc = c->fblock_n
-                       ? cfs::launch_halo_block(g, c->phys, sc, c->ring, c->d_subs, c->fblock_n, c->Wh, c->d_fbhalo, c->stream,
-                                                &c->launches, tm)
-                       : cfs::launch_halo_prims(g, c->phys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->Wh, c->s, c->stream,
-                                                &c->launches, tm);
-    if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
-  }
-  if (c->pairs && (graph || sc.mode != 0)) {
-    const int rc = cfs::launch_at_halo(g, c->pphys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->d_hpair, c->s, c->stream,
-                                       &c->launches, tm);
+  if (c->fused ? !c->Wh : c->pairs && c->algo != 0 && c->nhalo > 0 && !c->d_hpair)
+    return fail(c, CFS_ENOMEM, "no memory for the halo values");
+  // the AT halo values: of all stages before the first (only < 0), or of one before it
+  const bool halos = c->algo != 0 && (graph || sc.mode != 0), halo_one = c->fused ? c->wh_one : c->hpair_one;
+  auto halo_values = [&](int only) {
+    if (c->fused && c->fblock_n)
+      return cfs::launch_halo_block(g, c->phys, sc, c->ring, c->d_subs, c->fblock_n, c->Wh, c->d_fbhalo, only, c->stream,
+                                    &c->launches, tm);
+    if (c->fused)
+      return cfs::launch_halo_prims(g, c->phys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->Wh, c->s, only, c->stream,
+                                    &c->launches, tm);
+    if (c->pairs)
+      return cfs::launch_at_halo(g, c->pphys, sc, c->ring, c->d_subs, c->d_halo, c->nhalo, c->d_hpair, c->s, only, c->stream,
+                                 &c->launches, tm);
+    return 0;
+  };
+  if (halos && !halo_one) {
+    const int rc = halo_values(-1);
     if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
   }
   for (int op = 0; op < nops; ++op) {
@@ -1233,10 +1272,14 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       const cfs_status xs = exchange_strips(c, const_cast<double*>(src));
       if (xs != CFS_OK) return xs;
     }
+    if (op < c->s && halos && halo_one) {
+      rc = halo_values(op);
+      if (rc != 0) return cuda_fail(c, (cudaError_t)rc, "kernel launch");
+    }
     if (op < c->s && c->fused) {
       cfs::FusedLaunch a{};
       a.Uin = src; a.Uout = dst; a.Q = c->Q; a.subs = c->d_subs; a.work = c->d_work; a.nwork = c->nwork;
-      a.grid = c->fused_grid; a.fy = c->fused_fy; a.Wh = c->Wh; a.stage = op;
+      a.grid = c->fused_grid; a.fy = c->fused_fy; a.Wh = c->Wh; a.stage = c->wh_one ? 0 : op;
       a.A = c->A[op]; a.B = c->B[op]; a.dt = c->dt; a.first = op == 0; a.last = op == c->s - 1;
       a.ring = c->ring; a.in_ring = in_ring; a.out_ring = out_ring;
       a.curv = c->fused_curv ? 1 : 0;
@@ -1250,7 +1293,7 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       a.in_ring = in_ring; a.out_ring = out_ring;
       a.threads = c->threads;
       a.max_pad = c->max_pad; a.max_own = c->max_own; a.max_flux = c->max_flux;
-      a.halo = c->d_halo; a.nhalo = c->nhalo;
+      a.halo = c->d_halo; a.nhalo = c->nhalo; a.one_stage = c->hpair_one;
       a.compact = c->p.compact; a.R = c->Rbuf; a.cthomas = c->d_cthomas; a.Lmax = c->Lmax;
       rc = c->pairs ? cfs::launch_stage_pairs(g, c->pphys, sc, a, c->d_hpair, c->stream, &c->launches, tm)
            : c->euler2d.tiles ? cfs::launch_euler2d(g, c->phys, sc, a, c->euler2d, c->stream, &c->launches, tm)
@@ -1591,12 +1634,16 @@ cfs_status cfs_set_halo_model(cfs_ctx* c, const float* params, const double* sca
     }
     c->ncol = (long long)(cols.size() / 4);
     c->d_cols = (int*)dev_alloc(c, sizeof(int) * cols.size());
-    c->d_mlp = (float*)dev_alloc(c, sizeof(float) * MLP_NPARAM);
+    float* const mlp = (float*)dev_alloc(c, sizeof(float) * MLP_NPARAM);
     c->LH = (double*)dev_alloc(c, sizeof(double) * 5 * (size_t)c->geo.Ptot);
     const size_t ntile = (size_t)((c->ncol + MLP_TILE - 1) / MLP_TILE);
     c->d_mlpx = (float*)dev_alloc(c, sizeof(float) * ntile * MLP_TILE * MLP_K1);
     c->d_mlpa = (double*)dev_alloc(c, sizeof(double) * ntile * MLP_TILE * MLP_NOUT);
-    if (!c->d_cols || !c->d_mlp || !c->LH || !c->d_mlpx || !c->d_mlpa) return fail(c, CFS_ENOMEM, "device allocation failed");
+    if (!c->d_cols || !mlp || !c->LH || !c->d_mlpx || !c->d_mlpa) {
+      for (void* q : {(void*)c->d_cols, (void*)mlp, (void*)c->LH, (void*)c->d_mlpx, (void*)c->d_mlpa}) dev_free(c, q);
+      return fail(c, CFS_ENOMEM, "device allocation failed");
+    }
+    c->d_mlp = mlp;
     CUDA_TRY(c, cudaMemcpyAsync(c->d_cols, cols.data(), sizeof(int) * cols.size(), cudaMemcpyHostToDevice, c->stream), "upload columns");
     CUDA_TRY(c, cudaStreamSynchronize(c->stream), "upload columns");
   }

@@ -228,6 +228,7 @@ struct StageLaunch {
   // compact scheme (Eq. 2, alpha = 1/3): the flux divergence by line solves into R ([5][N], FP64),
   // then the stage update from R; cthomas = [2][Lmax] Thomas factors (forward factor
   // c'_i, reciprocal pivot 1 / m_i)
+  int one_stage;        // FP64 form on pairs: H holds this stage alone
   int compact;
   double* R;
   const void* cthomas;   // double, or float2 on pairs
@@ -245,13 +246,15 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
                  int precision, void* stream, long long* launches, const Timer* tm);
 
 // The stage of the FP64 form for 3-D Navier-Stokes on pairs of floats (stage_pairs.cu), and the AT
-// halo states of all s stages once per asynchronous step: H [2 s][nhalo] float4, [s][nhalo] float2.
+// halo states of all s stages once per asynchronous step: H [2 s][nhalo] float4, [s][nhalo] float2; or
+// (only >= 0) of that stage alone, before it: H [2][nhalo], [nhalo].
 int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const StageLaunch& a, const void* H,
                        void* stream, long long* launches, const Timer* tm);
 // (compact scheme: StageLaunch::R holds N float4, N float4, N doubles)
 int compact_pairs_prepare(int Lmax);
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
-                   const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm);
+                   const int* halo, long long nhalo, void* H, int s, int only, void* stream, long long* launches,
+                   const Timer* tm);
 
 // The stage of 2-D inviscid runs on periodic Cartesian blocks in one launch (euler2d.cu): small or
 // large tiles, and the most tiles a sub-domain has.
@@ -348,7 +351,7 @@ struct FusedLaunch {
   int grid;             // persistent grid size
   int fy;               // tile height: 4, 8 or 16 (tile width 32)
   const float* Wh;      // per-step AT/AS halo primitives [s][Ptot][8]
-  int stage;
+  int stage;            // which of them (0 where the store holds one stage)
   double A, B, dt;
   int first, last;
   const double* ring;
@@ -357,12 +360,13 @@ struct FusedLaunch {
 };
 int fused_smem_bytes(int fy, int curv);
 int fused_blocks_per_sm(int fy, int curv, int* blocks);  // sets the shared-memory attribute, then asks the occupancy API
+// The halo store Wh of all s stages, or (only >= 0) of that stage alone
 int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
-                      const int* halo, long long nhalo, float* Wh, int s, void* stream, long long* launches,
+                      const int* halo, long long nhalo, float* Wh, int s, int only, void* stream, long long* launches,
                       const Timer* tm);
 // The halo store together with the sub-domain filter's halos (cubic sub-domains of n points)
 int launch_halo_block(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs, int n,
-                      float* Wh, float* fh, void* stream, long long* launches, const Timer* tm);
+                      float* Wh, float* fh, int only, void* stream, long long* launches, const Timer* tm);
 int launch_stage_fused(const Geometry& g, const Physics& ph, const StepSched& sc, const FusedLaunch& a, void* stream,
                        long long* launches, const Timer* tm);
 

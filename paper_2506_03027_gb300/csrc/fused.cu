@@ -106,7 +106,8 @@ __device__ __forceinline__ void prims32(const double* u, const Phys32& k, float*
 
 namespace {
 
-// The halo store: per stage and padded point eight floats {u, v, w, T, rho, p - p_ref, rho E + p -
+// `only` (>= 0) of the halo kernels: form the values of that stage alone, where there is memory for the store of
+// one stage.  The halo store: per stage and padded point eight floats {u, v, w, T, rho, p - p_ref, rho E + p -
 // H_ref, -}: one 32-byte sector per point, whatever the shape of the strip
 // (arrays of one primitive each leave half of the sectors of a 4-wide x strip unused, and take seven
 // 4-byte copies per point in the stage where this takes four of 8 bytes).
@@ -130,7 +131,8 @@ __device__ __forceinline__ void store_halo(float4* __restrict__ Wh, long long P,
 // sums with W^(m) - W^(0) (table W32d).
 template <int S>
 __device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc, const Phys32& k32, const double (*r)[5],
-                                         const LevelDiffs& d, int kd, bool learned, long long o, float4* __restrict__ Wh) {
+                                         const LevelDiffs& d, int kd, bool learned, long long o, int only,
+                                         float4* __restrict__ Wh) {
   const int C = sc.C;
   // the value the sums are added to: U_0, or the network's stage-0 value (rho, momenta as pairs
   // of floats, rho E as its deviation from E_ref)
@@ -154,6 +156,7 @@ __device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc,
   const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * C;
 #pragma unroll
   for (int m = 0; m < S; ++m) {
+    if (only >= 0 && m != only) continue;
     float2 c[CFS_MAX_LEVELS];
 #pragma unroll
     for (int l = 0; l < CFS_MAX_LEVELS; ++l) c[l] = l < C ? __ldg(wt + m * C + l) : make_float2(0.f, 0.f);
@@ -162,7 +165,7 @@ __device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc,
     float w[7];
     prims32f(bh[0] + (bl[0] + dl[0]), bh[1] + (bl[1] + dl[1]), bh[2] + (bl[2] + dl[2]), bh[3] + (bl[3] + dl[3]),
              be + dl[4], k32, w);
-    store_halo(Wh, g.Ptot, m, o, w);
+    store_halo(Wh, g.Ptot, only < 0 ? m : 0, o, w);
   }
 }
 
@@ -171,7 +174,7 @@ __device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc,
 template <int S>
 __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
                                                     const SubDev* __restrict__ subs, const int2* __restrict__ halo,
-                                                    long long nhalo, float4* __restrict__ Wh) {
+                                                    long long nhalo, int only, float4* __restrict__ Wh) {
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: no halo store is read
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,9 +235,10 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
     }
 #pragma unroll
     for (int m = 0; m < (sc.mode == 2 ? 1 : S); ++m) {
+      if (sc.mode != 2 && only >= 0 && m != only) continue;
       float w[7];
       prims32(acc[m], k32, w);
-      store_halo(Wh, P, m, o, w);
+      store_halo(Wh, P, only < 0 ? m : 0, o, w);
     }
     return;
   }
@@ -256,7 +260,7 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
   const bool learned = sc.LH && ((int)(ci < 0 || ci >= d.sx) + (int)(cj < 0 || cj >= d.sy) + (int)(ck < 0 || ck >= d.sz) == 1);
   LevelDiffs ld;
   level_diffs(r, C, ld);
-  at_prims<S>(g, sc, k32, r, ld, kd, learned, o, Wh);
+  at_prims<S>(g, sc, k32, r, ld, kd, learned, o, only, Wh);
 }
 
 // The halo store and the sub-domain filter's halos from one read of the delayed levels, for contexts
@@ -268,8 +272,8 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
 // sub-domains: 1.83 ms, against 1.76 for the halo store alone and 0.43 for the filter's halos.
 template <int N>
 __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
-                                                    const SubDev* __restrict__ subs, float4* __restrict__ Wh,
-                                                    float* __restrict__ fh) {
+                                                    const SubDev* __restrict__ subs, int only,
+                                                    float4* __restrict__ Wh, float* __restrict__ fh) {
   constexpr int S = 5, NN = N * N, NF = 5 * NN;
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: neither is read
@@ -323,7 +327,7 @@ __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, Step
     }
   LevelDiffs ld;
   level_diffs(r, C, ld);
-  if (face >= 0) {
+  if (face >= 0 && only <= 0) {
     // the filter's halo: deviation of U_0 from the reference, plus the weighted differences
     const double* ref = ring + (long long)nR * lvN + d.bbase + (long long)d.ox + (long long)d.bnx * (d.oy + (long long)d.bny * d.oz);
     const float2* __restrict__ wf = (const float2*)sc.Wf32 + (long long)kd * sc.C;
@@ -340,6 +344,8 @@ __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, Step
       const float dv = dev_fast(r[0][v], rh, rl);
       out[(long long)v * 30 * NN] = sc.mode == 2 ? dv : __fadd_rn(dv, sum[v]);
     }
+  }
+  if (face >= 0) {
     const int depth = c[face >> 1] < 0 ? -c[face >> 1] : c[face >> 1] - N + 1;
     if (depth > HB) return;  // the stage reads to depth 4
   }
@@ -350,7 +356,7 @@ __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, Step
     store_halo(Wh, g.Ptot, 0, o, w);
     return;
   }
-  at_prims<S>(g, sc, k32, r, ld, kd, sc.LH && face >= 0, o, Wh);
+  at_prims<S>(g, sc, k32, r, ld, kd, sc.LH && face >= 0, o, only, Wh);
 }
 
 // ------------------------------------------------------------------------------- k_stage_fused
@@ -923,26 +929,26 @@ int fused_smem_bytes(int fy, int curv) {
 }
 
 int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
-                      const int* halo, long long nhalo, float* Wh, int s, void* stream, long long* launches,
+                      const int* halo, long long nhalo, float* Wh, int s, int only, void* stream, long long* launches,
                       const Timer* tm) {
   cudaStream_t st = (cudaStream_t)stream;
   if (nhalo <= 0) return 0;
   const unsigned nb = (unsigned)((nhalo + 255) / 256);
   if (tm) tm->rec(tm->self, 0, 1);
-  if (s == 2) k_halo_prims<2><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, (float4*)Wh);
-  else k_halo_prims<5><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, (float4*)Wh);
+  if (s == 2) k_halo_prims<2><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, only, (float4*)Wh);
+  else k_halo_prims<5><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, only, (float4*)Wh);
   if (tm) tm->rec(tm->self, 0, 0);
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
 }
 
 int launch_halo_block(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs, int n,
-                      float* Wh, float* fh, void* stream, long long* launches, const Timer* tm) {
+                      float* Wh, float* fh, int only, void* stream, long long* launches, const Timer* tm) {
   cudaStream_t st = (cudaStream_t)stream;
   const dim3 grid((30 * n * n + 48 * n + 255) / 256, g.nsub);
   if (tm) tm->rec(tm->self, 0, 1);
-  if (n == 32) k_halo_block<32><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, (float4*)Wh, fh);
-  else k_halo_block<16><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, (float4*)Wh, fh);
+  if (n == 32) k_halo_block<32><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, only, (float4*)Wh, fh);
+  else k_halo_block<16><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, only, (float4*)Wh, fh);
   if (tm) tm->rec(tm->self, 0, 0);
   if (launches) *launches += 1;
   return (int)cudaGetLastError();

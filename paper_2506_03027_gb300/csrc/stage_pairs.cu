@@ -229,11 +229,12 @@ __device__ __forceinline__ void gather_value(const Geometry& g, const StepSched&
 // sum of the weights: the levels differ by a step's change, so the products of pairs keep the sum
 // at the accuracy of the FP64 one.  With the learned halo, face points start from the network's
 // stage-0 value and add the sums with W^(m) - W^(0).  Stored [stage][entry]: (rho, rho u), (rho v,
-// rho w) and rho E - E_ref.  Bound by its reads: C x 40 bytes per entry at the sub-domains' faces.
+// rho w) and rho E - E_ref; or (only >= 0) of that stage alone.  Bound by its reads: C x 40 bytes per entry at the sub-domains' faces.
 template <int S>
 __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ ring,
                                                  const SubDev* __restrict__ subs, const int2* __restrict__ halo,
-                                                 long long nhalo, float4* __restrict__ H4, float2* __restrict__ H2) {
+                                                 long long nhalo, int only, float4* __restrict__ H4,
+                                                 float2* __restrict__ H2) {
   pdl_enter();
   sc = resolve(sc);
   if (sc.mode == 0) return;
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
   for (int l = 0; l < CFS_MAX_LEVELS; ++l) lev[l] = l < C ? slot(l) : 0;
   const bool learned = sc.LH && sc.mode == 1 && ((int)(h.ci < 0 || h.ci >= d.sx) + (int)(h.cj < 0 || h.cj >= d.sy) + (int)(h.ck < 0 || h.ck >= d.sz) == 1);
   // (AS, mode 2: the latest visible level, the same for every stage -- stage 0 alone is stored)
-  const int ns = sc.mode == 2 ? 1 : S;
+  const int one = sc.mode == 2 ? 0 : only;
   const float2* __restrict__ wt = (const float2*)(learned ? sc.W32d : sc.W32) + (long long)kd * S * sc.C;
   const long long lh = d.pbase + h.q;
   // two components at a time (rho and rho u, rho v and rho w, rho E alone): few registers, so that
@@ -322,10 +323,11 @@ __global__ void __launch_bounds__(256, 3) k_at_halo(Geometry g, PairPhysics ph, 
       }
 #pragma unroll
     for (int m = 0; m < S; ++m) {
-      if (m >= ns) break;
+      if (one >= 0 && m != one) continue;
       const P2 a = p_norm(acc[m]);
-      if (grp < 2) H4[(long long)(2 * m + grp) * nhalo + e] = p_store(a);
-      else H2[(long long)m * nhalo + e] = p_store(p_x(a));
+      const int row = one >= 0 ? 0 : m;
+      if (grp < 2) H4[(long long)(2 * row + grp) * nhalo + e] = p_store(a);
+      else H2[(long long)row * nhalo + e] = p_store(p_x(a));
     }
   }
 }
@@ -341,7 +343,7 @@ template <bool EULER>
 __global__ void __launch_bounds__(256, EULER ? 3 : 4) k_view_p(Geometry g, PairPhysics ph, StepSched sc, const double* __restrict__ Uin0,
                                                 const double* __restrict__ ring, int in_ring, const SubDev* __restrict__ subs,
                                                 const int2* __restrict__ halo, long long nhalo, const float4* __restrict__ H4,
-                                                const float2* __restrict__ H2, void* Wp, void* Phi, int stage, int s, int own_blocks, int rev) {
+                                                const float2* __restrict__ H2, void* Wp, void* Phi, int stage, int s, int one_stage, int own_blocks, int rev) {
   pdl_enter();
   sc = resolve(sc);
   const double* __restrict__ Uin = ring_or(Uin0, in_ring, ring, sc, 0);
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(256, EULER ? 3 : 4) k_view_p(Geometry g, PairP
     put(d, prims_of(ph, u), [&](int a) { return u[1 + a]; }, o, h.ci, h.cj, as);
     return;
   }
-  const int m = sc.mode == 2 ? 0 : stage;
+  const int m = sc.mode == 2 || one_stage ? 0 : stage;
   const P2 a = p_of(H4[(long long)(2 * m) * nhalo + e]), c = p_of(H4[(long long)(2 * m + 1) * nhalo + e]);
   put(d, prims_p(ph, p_x(a), p_pair(p_y(a), p_x(c)), p_y(c), p_of(H2[(long long)m * nhalo + e])),
       [&](int i) { return p_double(i == 0 ? p_y(a) : (i == 1 ? p_x(c) : p_y(c))); }, o, h.ci, h.cj, as);
@@ -974,12 +976,13 @@ int pow_pair_tables_init() {
 }
 
 int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc, const double* ring, const SubDev* subs,
-                   const int* halo, long long nhalo, void* H, int s, void* stream, long long* launches, const Timer* tm) {
+                   const int* halo, long long nhalo, void* H, int s, int only, void* stream, long long* launches,
+                   const Timer* tm) {
   if (nhalo <= 0) return 0;
   float4* H4 = (float4*)H;
-  float2* H2 = (float2*)(H4 + 2LL * s * nhalo);
+  float2* H2 = (float2*)(H4 + 2LL * (only >= 0 ? 1 : s) * nhalo);
   TIMED(tm, 0, (launch_pdl(s == 2 ? k_at_halo<2> : k_at_halo<5>, dim3(nblk(nhalo, 256)), dim3(256), 0, (cudaStream_t)stream, g,
-                           ph, sc, ring, subs, (const int2*)halo, nhalo, H4, H2)));
+                           ph, sc, ring, subs, (const int2*)halo, nhalo, only, H4, H2)));
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
 }
@@ -989,7 +992,7 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   const cudaStream_t st = (cudaStream_t)stream;
   const int B = a.threads == 128 ? 128 : 256;
   const float4* H4 = (const float4*)H;
-  const float2* H2 = (const float2*)(H4 + 2LL * a.s * a.nhalo);
+  const float2* H2 = (const float2*)(H4 + 2LL * (a.one_stage ? 1 : a.s) * a.nhalo);
   const unsigned own_blocks = nblk(a.max_own, B);
   const unsigned nb = own_blocks * (unsigned)g.nsub + nblk(a.nhalo, B);
   const dim3 gf(nblk(a.max_flux, B), g.nsub), gr(nblk(a.max_own, B), g.nsub);
@@ -1002,7 +1005,7 @@ int launch_stage_pairs(const Geometry& g, const PairPhysics& ph, const StepSched
   auto rev = [&](int k) { return (a.stage * per_stage + k) & 1; };
   // (inviscid: the fluxes come straight from the view)
   TIMED(tm, 0, (launch_pdl(g.viscous ? k_view_p<false> : k_view_p<true>, dim3(nb), dim3(B), 0, st, g, ph, sc, a.Uin, a.ring, a.in_ring, a.subs, (const int2*)a.halo,
-                           a.nhalo, H4, H2, a.Wp, a.Phi, a.stage, a.s, (int)own_blocks, rev(0))));
+                           a.nhalo, H4, H2, a.Wp, a.Phi, a.stage, a.s, a.one_stage, (int)own_blocks, rev(0))));
   if (launches) *launches += 1;
   if (a.compact) {
     // x and y passes gather dt R, the z pass takes the update

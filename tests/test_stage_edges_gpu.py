@@ -128,3 +128,86 @@ def test_run_without_room_for_the_halo_values(kind, monkeypatch):
     assert len(refused) == 1
     e = rel_l2(Ug, orc.run(c, U0, 10))
     assert np.all(np.isfinite(Ug)) and np.all(e <= PARITY_TOL), e
+
+
+def limited(monkeypatch, allowed):
+    """The allocator refuses what `allowed(bytes, bytes in use)` does not grant; the refused sizes."""
+    refused = []
+    alloc, free = cfs.TorchAllocator._alloc, cfs.TorchAllocator._free
+    held = {}
+
+    def get(self, nbytes, user):
+        if not allowed(nbytes, sum(held.values())):
+            refused.append(nbytes)
+            return None
+        p = alloc(self, nbytes, user)
+        held[p] = nbytes
+        return p
+
+    def put(self, ptr, user):
+        held.pop(ptr, None)
+        free(self, ptr, user)
+    monkeypatch.setattr(cfs.TorchAllocator, "_alloc", get)
+    monkeypatch.setattr(cfs.TorchAllocator, "_free", put)
+    return refused
+
+
+def advance(c, precision=0, graph=False, learned=False, steps=9):
+    import torch
+    U0 = I.tgv_state(c)
+    s = cfs.Solver(c, precision=precision, graph=graph, stream=torch.cuda.Stream())
+    s.set_schedule(delays=I.saa_delays(c, steps) if c.algo == "SAA" else None)
+    if learned:
+        cfs.cfs_set_halo_model(s.ctx, L.init_params(4),
+                               np.array([3e3, 2e3, 2e3, 2e3, 1e3, 4e2, 3e2, 3e2, 3e2, 2e2, 1e7, 1e6, 1e6, 1e6, 5e5]))
+    s.set_state(U0)
+    s.step(steps)
+    U = s.get_state()
+    s.close()
+    return U
+
+
+FORMS = {"viscous": (26, {}, {}), "power_law_graph": (26, {"visc_law": 1}, {"graph": True}), "euler": (26, {"viscous": False}, {}),
+         "compact": (26, {"viscous": False, "compact": 1}, {}), "latest_level": (26, {"at": False}, {}), "order2": (26, {"order": 2}, {}),
+         "fp32": (26, {}, {"precision": 1}), "fp32_cubes": (32, {}, {"precision": 1}), "fp32_cubes_graph": (32, {}, {"precision": 1, "graph": True}),
+         "fp32_latest_level": (32, {"at": False}, {"precision": 1})}
+
+
+# where there is no memory for the halo values of all stages, those of one at a time give the same bits
+@pytest.mark.parametrize("form", list(FORMS))
+def test_same_values_without_room_for_all_stages(form, monkeypatch):
+    n, kw, run = FORMS[form]
+    c = I.tgv_case(n, 2, "SAA", kmax=2, **kw)
+    c = c.replace(dt=I.cfl_dt(c, I.tgv_state(c), 0.1))
+    sizes = []
+    with monkeypatch.context() as m:
+        limited(m, lambda b, used: sizes.append(b) or True)
+        full = advance(c, **run)
+    w = n // 2
+    if run.get("precision"):
+        store = 4 * 8 * c.stages * c.nsub * (w + 8) ** 3
+    else:
+        G, r = (4, 2) if c.compact else ((2 * (c.order // 2), c.order // 2) if c.viscous else (2, 2))
+        store = 40 * c.stages * (c.nsub * 6 * w * w * G + (c.nsub * 12 * r * r * w if c.viscous else 0))
+    assert sizes.count(store) == 1
+    with monkeypatch.context() as m:
+        refused = limited(m, lambda b, used: b != store)
+        one = advance(c, **run)
+    assert refused == [store]
+    assert np.all(np.isfinite(full)) and np.array_equal(full, one)
+
+
+# the store gives way to what is allocated after it, here the halo network's buffers
+@pytest.mark.parametrize("precision", [0, 1])
+def test_store_of_all_stages_gives_way(precision, monkeypatch):
+    c = I.tgv_case(32, 2, "SAA", kmax=2)
+    c = c.replace(dt=I.cfl_dt(c, I.tgv_state(c), 0.1))
+    peak = []
+    with monkeypatch.context() as m:
+        limited(m, lambda b, used: peak.append(used + b) or True)
+        full = advance(c, precision=precision, learned=True)
+    with monkeypatch.context() as m:
+        refused = limited(m, lambda b, used: used + b < max(peak))
+        one = advance(c, precision=precision, learned=True)
+    assert len(refused) == 1
+    assert np.all(np.isfinite(full)) and np.array_equal(full, one)
