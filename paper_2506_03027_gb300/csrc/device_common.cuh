@@ -86,26 +86,6 @@ __device__ __forceinline__ float dev_fast(double x, float rh, float rl) {
   return (h - rh) + (r - rl);
 }
 
-// x in units of 2^(E-52-guard), rounded down, E + 1023 = ex the exponent field of a number no smaller
-__device__ __forceinline__ long long fixed_point(double x, int ex, int guard = 0) {
-  const int hi = __double2hiint(x);
-  const int sh = min(ex - ((hi >> 20) & 0x7ff), 63);
-  const long long m = (long long)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x));
-  const long long sg = hi >> 31;
-  return (((m ^ sg) - sg) << guard) >> sh;
-}
-
-// g 2^(q20 >> 20) in FP64 (|g| < 2^63), truncated to 53 bits, on the integer pipe
-__device__ __forceinline__ double from_fixed_point(long long g, int q20) {
-  const long long sg = g >> 63;
-  const unsigned long long m = (unsigned long long)((g ^ sg) - sg);
-  const int lz = __clzll((long long)m);
-  const unsigned long long t = (m << lz) >> 11;  // the leading one at bit 52
-  // (adding the leading one to the exponent field raises it by one)
-  const int hi = (int)(t >> 32) + ((1023 + 62 - lz) << 20) + q20;
-  return m ? __hiloint2double(hi | ((int)sg & (int)0x80000000), (int)t) : 0.0;
-}
-
 // Asynchronous global -> shared copies (cp.async; completion by cp_async_wait_all + a barrier).
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(dst);

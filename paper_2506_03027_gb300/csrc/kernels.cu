@@ -753,11 +753,11 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 //   (alpha, 1, alpha) d = (1 - 2 alpha)/1024 delta^10 f.
 // It is bound by the FP64 pipe when it differences in FP64 (2 FMA per clock and SM), so the
 // differences are 64-bit integers instead: every value of the line's window as a fixed-point number
-// with the last place of its largest value as the quantum (2^(E-52), smaller values rounded down;
-// the mean of that rounding drops out of the differences), ten integer subtractions give delta^10
-// exactly, and the two sweeps and the final sum f + d are four FP64 operations per point.  What the
-// rounding leaves passes through 1 - T <= 1, which is small everywhere but next to the shortest
-// wave, so it adds less than the rounding of the final sum.
+// with the last place of its largest value as the quantum (2^(E-52), smaller values rounded to
+// nearest), ten integer subtractions give delta^10 exactly, and the two sweeps and the final sum f + d are
+// four FP64 operations per point.  What the rounding leaves passes through 1 - T <= 1, which is small
+// everywhere but next to the shortest wave: it adds less than the rounding of the final sum of the line's
+// largest values.
 struct FilterTile {
   int LN;  // lines per CTA
   int TW;  // row stride in doubles (odd: 64-bit accesses of a warp's rows hit distinct banks)
@@ -786,6 +786,28 @@ __host__ __device__ inline size_t filter_tile_doubles(const FilterTile& t, int p
 __host__ __device__ inline size_t filter_smem_bytes(int Lmax, int precision, int sync) {
   const FilterTile t = filter_tile(Lmax, precision, sync);
   return (filter_tile_doubles(t, precision) + t.TW) * 8;
+}
+
+// x in units of 2^(E-52), rounded to nearest (the magnitude, so that -x gives the opposite number and
+// zeros of both signs and values below half a unit give 0), E + 1023 = ex >= 200 the exponent field of a
+// number no smaller
+__device__ __forceinline__ long long fixed_point(double x, int ex) {
+  const int hi = __double2hiint(x);
+  const int sh = min(ex - ((hi >> 20) & 0x7ff), 63);
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
+  const long long r = (long long)((m + ((1ull << sh) >> 1)) >> sh), sg = hi >> 31;
+  return (r ^ sg) - sg;
+}
+
+// g 2^(q20 >> 20) in FP64 (|g| < 2^63), truncated to 53 bits, on the integer pipe
+__device__ __forceinline__ double from_fixed_point(long long g, int q20) {
+  const long long sg = g >> 63;
+  const unsigned long long m = (unsigned long long)((g ^ sg) - sg);
+  const int lz = __clzll((long long)m);
+  const unsigned long long t = (m << lz) >> 11;  // the leading one at bit 52
+  // (adding the leading one to the exponent field raises it by one)
+  const int hi = (int)(t >> 32) + ((1023 + 62 - lz) << 20) + q20;
+  return m ? __hiloint2double(hi | ((int)sg & (int)0x80000000), (int)t) : 0.0;
 }
 
 template <typename T, int axis>

@@ -116,3 +116,45 @@ def test_memory_grows_with_the_line_not_its_square(filt, monkeypatch):
         return sum(sizes)
     a, b = total(340), total(680)
     assert b <= 2.0 * a, (a, b)
+
+
+def one_pass(c, U0):
+    s = cfs.Solver(c)
+    s.set_schedule()
+    s.set_state(U0)
+    s.step(1)
+    U = s.get_state()
+    s.close()
+    return U
+
+
+def tailed_state(c, tail, seed):
+    """Momenta of about 1 on the first third of every line along x and `tail` beyond it."""
+    U = rough_state(c, 1.0, seed)
+    U[1:4, :, :, c.nx // 3:] = tail(c.nx - c.nx // 3)
+    return U
+
+
+def reference(c, U0):
+    ref = U0.astype(np.longdouble)
+    for axis, p in ((-1, c.px), (-2, c.py), (-3, c.pz)):
+        ref = filter_axis(ref, axis, p, c.alpha_f)
+    return ref
+
+
+# lines along x of 200 points in one piece and in two
+@pytest.mark.parametrize("p", [1, 2])
+def test_filter_of_opposite_and_vanishing_values(p):
+    """-f filters to the opposite of f, and values far below the line's largest (of both signs, both
+    zeros) take no rounding of the size of that one's."""
+    c = I.tgv_case(16, 1, "SA").replace(nx=200, ny=12, nz=11, px=p, alpha_f=0.45, dt=1e-300)
+    U0 = tailed_state(c, lambda n: 1e-30 * np.where(np.arange(n) % 3, -1.0, 1.0) * (np.arange(n) % 5 > 0), 9)
+    U0[1:4][U0[1:4] == 0.0] *= -1.0
+    V0 = U0.copy()
+    V0[1:4] *= -1.0
+    U, V = one_pass(c, U0), one_pass(c, V0)
+    assert np.array_equal(U[1:4], -V[1:4])
+    # the large values, and their rounding, reach into the rest of their line with (1 - sqrt(1 - 4
+    # alpha^2)) / (2 alpha) = 0.63 per point: 1e-11 of their 2^-53 fifty-five points away
+    e = np.abs(U - reference(c, U0))[1:4, :, :, 122:143].max()
+    assert e <= 1e-24, e
