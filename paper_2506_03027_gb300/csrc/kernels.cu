@@ -757,7 +757,8 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 // nearest), ten integer subtractions give delta^10 exactly, and the two sweeps and the final sum f + d are
 // four FP64 operations per point.  What the rounding leaves passes through 1 - T <= 1, which is small
 // everywhere but next to the shortest wave: it adds less than the rounding of the final sum of the line's
-// largest values.
+// largest values.  Lines whose values differ by more than seven binades from place to place (a vortex in
+// still fluid) take the largest value of the surroundings instead, group of 8 points by group.
 struct FilterTile {
   int LN;  // lines per CTA
   int TW;  // row stride in doubles (odd: 64-bit accesses of a warp's rows hit distinct banks)
@@ -810,8 +811,10 @@ __device__ __forceinline__ double from_fixed_point(long long g, int q20) {
   return m ? __hiloint2double(hi | ((int)sg & (int)0x80000000), (int)t) : 0.0;
 }
 
+// (registers: seven CTAs per SM in the FP64 form; its y pass takes 162 us at 90 registers, 140 at 72, its x pass
+// 186 when held to the bound, 170 with the compiler's own 72)
 template <typename T, int axis>
-__global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
+__global__ void __launch_bounds__(128, std::is_same<T, float>::value || axis == 0 ? 0 : 7) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
   if (f.chain == 0) {
     pdl_enter();
   } else {  // (see FilterLaunch)
@@ -1069,9 +1072,22 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       // c_i d_{i+1}, the filter's scale in the 1 / m_i.  The forward sweep parks z_i in slot i
       // (position i - 5, no longer read); back substitution leaves d_i there.
       double* row = tile + line * TW;
-      int top = 0;
+      // The largest value of the line, and the smallest of the largest values of 16 neighbouring slots (8 and
+      // the next 8): where that is more than seven binades below, every group of 8 points takes the unit
+      // of its own window of 18 slots.
+      auto largest = [&](int i0, int i1) {
+        int t = 0;
 #pragma unroll 8
-      for (int i = 0; i < W; ++i) top = max(top, __double2hiint(row[i]) & 0x7fffffff);
+        for (int i = i0; i < i1; ++i) t = max(t, __double2hiint(row[i]) & 0x7fffffff);
+        return t;
+      };
+      int top = 0, low = 0x7fffffff, prev = 0x7fffffff;
+      for (int i0 = 0; i0 < W; i0 += 8) {
+        const int t = largest(i0, min(i0 + 8, W));
+        top = max(top, t);
+        low = min(low, max(prev, t));
+        prev = t;
+      }
       int ex = top >> 20;
       // a NaN or an infinity anywhere in the window (or a value of 2^1009 and more) reaches every
       // point of the line: d = NaN
@@ -1079,7 +1095,8 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       // a line of nothing but values below 2^-822 stays as it is: d = 0
       const bool tiny = ex < 200;
       ex = max(ex, 200);
-      const int q20 = (ex - 1023 - 52) * (1 << 20);
+      const int exline = ex, group = max(low >> 20, 200) >= ex - 7 ? len : 8;
+      int q20 = (ex - 1023 - 52) * (1 << 20);
       const double* __restrict__ cp = f.thomas_k;
       const double* __restrict__ im = cp + f.Lmax;
       long long s[10];
@@ -1095,14 +1112,26 @@ __global__ void __launch_bounds__(128) k_filter(Geometry g, StepSched sc, Filter
       };
 #pragma unroll
       for (int j = 0; j < 10; ++j) s[j] = 0;
-#pragma unroll
-      for (int i = 0; i < 10; ++i) diff10(i);
       double z = 0.0, c = 0.0;
+      for (int i0 = 0; i0 < len; i0 += group) {
+        bool prime = i0 == 0;
+        if (group < len) {
+          int e = max(largest(i0, min(i0 + 18, W)) >> 20, 200);
+          if (e >= exline - 7) e = exline;
+          prime = prime || e != ex;
+          ex = e;
+          q20 = (ex - 1023 - 52) * (1 << 20);
+        }
+        if (prime)
+#pragma unroll
+          for (int j = 0; j < 10; ++j) diff10(i0 + j);
+        const int i1 = min(i0 + group, len);
 #pragma unroll 4
-      for (int i = 0; i < len; ++i) {
-        z = fma(-c, z, from_fixed_point(diff10(i + 10), q20));
-        row[i] = z;
-        c = __ldg(cp + i);
+        for (int i = i0; i < i1; ++i) {
+          z = fma(-c, z, from_fixed_point(diff10(i + 10), q20));
+          row[i] = z;
+          c = __ldg(cp + i);
+        }
       }
       double x = bad ? __longlong_as_double(0x7ff8000000000000LL) : 0.0;
 #pragma unroll 4
