@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "cfs_internal.h"
 #include "device_common.cuh"
@@ -121,8 +122,10 @@ __device__ __forceinline__ Pr<V> diff_pts(Pr<V> m2, Pr<V> m1, Pr<V> p1, Pr<V> p2
 // Cartesian 3-D block: a CTA marches its tile of columns through planes [z0, z1).  Per plane the
 // velocities of the tile and of R points beyond it in x and y go to one of four shared-memory planes
 // (one barrier per plane), the column's own (u, v) stay in registers for the z differences; plane
-// L - R is finished when plane L has arrived.  A CTA that meets a value outside the pairs' range
-// (a density, a momentum; also NaN and infinity) takes its points in FP64 instead.
+// L - R is finished when plane L has arrived.  A CTA takes its points in FP64 instead when it meets a value
+// outside the pairs' range (a density, a momentum; also NaN and infinity), when what it forms from
+// them leaves that range (a sum of squares of 2^100 and more), and when the largest sum of squares of its
+// columns is below 2^-60 but not zero, so that the squares' low words may be lost.
 template <int R>
 __global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial,
                                                          int tiles_x, int tiles, int zc, int rows) {
@@ -171,6 +174,7 @@ __global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const d
 #pragma unroll
   for (int k = 0; k <= R; ++k) rh[k] = {0.f, 0.f};
   int nens = 0;
+  unsigned moving = 0;  // bits of the column's momenta, without the sign
   for (int L = z0 - R; L < z1 + R; ++L) {
     const bool inner = L >= z0 && L < z1;
     const double* __restrict__ pl = base + plane * wrapc(L, b.nz);
@@ -207,6 +211,8 @@ __global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const d
 #pragma unroll
         for (int v = 0; v < 5; ++v) acc[2 + v] += u[v];
         bad = bad || outside(u[4], 0);
+#pragma unroll
+        for (int v = 1; v < 4; ++v) moving |= (unsigned)(__double2hiint(u[v]) << 1) | (unsigned)__double2loint(u[v]);
         const P2 k2 = p_mul(mxy, uv[2 * R]);
         kin = p_norm(p_add(kin, p_norm(p_fma(mz, w, p_add(p_x(k2), p_y(k2))))));
       }
@@ -237,7 +243,10 @@ __global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const d
     const P1 w2 = p_norm(p_fma(c, c, p_add(p_x(a2), p_y(a2))));
     ens = p_norm(p_add(ens, p_norm(p_mul(rh[0], w2))));
   }
-  if (__syncthreads_or(bad)) {
+  bad = bad || !(kin.h < 0x1p100f) || !(ens.h < 0x1p100f);
+  const bool lost = (!__syncthreads_or(kin.h >= 0x1p-60f) && __syncthreads_or(moving != 0)) ||
+                    (!__syncthreads_or(ens.h >= 0x1p-60f) && __syncthreads_or(ens.h != 0.f));
+  if (__syncthreads_or(bad) || lost) {
     for (int c = 0; c < DIAG_NQ; ++c) acc[c] = 0.0;
     if (own)
       for (int z = z0; z < z1; ++z) diag_point(b, U, x, y, z, acc);
@@ -307,8 +316,13 @@ TileShape tile_shape(int nx, int ny, int nz) {
 
 constexpr int kGeneralRows = 2 * 152;
 
-// the marching kernel: 3-D Cartesian blocks computed here as a whole
-bool tiled(const DiagBlock& b) { return b.nz > 1 && !b.M && !b.subs; }
+// the marching kernel: 3-D Cartesian blocks computed here as a whole, of spacings within the pairs' range
+bool tiled(const DiagBlock& b) {
+  if (b.nz == 1 || b.M || b.subs) return false;
+  for (int a = 0; a < 3; ++a)
+    if (!(std::fabs(b.c1[a]) > 1e-12 && std::fabs(b.c1[a]) < 1e12)) return false;
+  return true;
+}
 
 }  // namespace
 

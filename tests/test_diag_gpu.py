@@ -75,3 +75,29 @@ def test_nonfinite_value_is_flagged(value):
         s.diagnostics()
     s.close()
     assert e.value.status == cfs.CFS_ENAN
+
+
+# products of values inside the pairs' range that leave it, above (velocities of 2^65) and below (of 1e-25
+# and 1e-15), and a spacing that leaves it
+@pytest.mark.parametrize("rho,vel,box", [(2.0 ** -30, 2.0 ** 65, 1.0), (2.0 ** 20, 2.0 ** -85, 1.0), (1.0, 1e-25, 1.0), (1.0, 1e-15, 1.0),
+                                         (1.0, 1.0, 1e25), (1.0, 1.0, 1e-25)])
+def test_products_outside_the_pairs_range(rho, vel, box):
+    c = I.tgv_case(16, 1, "SA").replace(nx=70, ny=60, nz=64, lx=1.3 * box, ly=2.0 * box, lz=0.7 * box)
+    U = state(c, 3)
+    U[0] *= rho
+    U[1:4] *= rho * vel
+    ref = reference(c, U)
+    got = static(c, U)
+    # (pairs: 2^-48 of the velocities, whose differences are of their size)
+    assert np.all(np.abs(got[:2] - ref[:2]) <= 1e-13 * np.abs(ref[:2])), (got[:2], ref[:2])
+    assert got[7] == 0.0
+
+
+def test_mixed_scales():
+    """Slabs of slow fluid beside fast ones, and fluid at rest, keep the totals."""
+    c = I.tgv_case(16, 1, "SA").replace(nx=70, ny=60, nz=64)
+    U = state(c, 3)
+    U[1:4, 10:50] *= 1e-20
+    U[1:4, 55:] = 0.0
+    ref, got = reference(c, U), static(c, U)
+    assert np.all(np.abs(got[:2] - ref[:2]) <= 1e-13 * np.abs(ref[:2])) and got[7] == 0.0
