@@ -412,7 +412,7 @@ struct DiagBlock {
   int P[3], sid0;
 };
 #define DIAG_NQ 9   // per block row: K, enstrophy, 5 totals, non-finite flag, enstrophy volume
-// Rows of partial sums a block takes (at most `most` unless the fixed general grid needs more), for
+// Rows of partial sums a block takes (at most `most`, and 1216 of the kernel by points), for
 // launch_diagnostics_block's `rows`.
 int diag_rows(int nx, int ny, int nz, int most);
 int launch_diagnostics_block(const DiagBlock& b, const double* U, double* partial, int row0, int rows, void* stream);

@@ -1,7 +1,7 @@
 // diag.cu -- diagnostics of a state: kinetic energy, enstrophy, totals and the non-finite flag.
 //
-// Per block of points one CTA (a tile of 32 x 8 columns marching through a chunk of z planes) writes
-// one row of partial sums; a last CTA adds the rows in a fixed order.  In FP64 the sums are bound by
+// Per block of points one CTA (256 points at a time, or, where that is faster, a tile of 32 x 8 columns marching
+// through a chunk of z planes) writes one row of partial sums; a last CTA adds the rows in a fixed order.  In FP64 the sums are bound by
 // the FP64 pipe: a reciprocal of the density and six differences per point are about 110 FP64
 // operations at 2 per clock and SM.  Only the five totals need FP64 accumulation point by point; the
 // velocities, their differences and the two squares are formed on pairs of floats (pairs.cuh), a
@@ -26,18 +26,19 @@ constexpr int DTX = 32, DTY = 8;
 // The five totals, the kinetic energy (x 2) and the enstrophy (x 2, and the volume it covers) of one
 // point in FP64: any block (curvilinear, two-dimensional, not periodic, partitioned), any finite or
 // non-finite value.
-__device__ __noinline__ void diag_point(const DiagBlock& b, const double* __restrict__ U, int x, int y, int z, double* acc) {
+template <bool CURV>
+__device__ __forceinline__ void diag_point(const DiagBlock& b, const double* __restrict__ U, int x, int y, int z, double* acc) {
   const int ndim = b.nz > 1 ? 3 : 2;
   const long long i = (long long)x + (long long)b.nx * ((long long)y + (long long)b.ny * z);
   const long long mq = (long long)(x + b.G) + (long long)b.mx * (y + b.G);  // metric plane index
-  const double dV = b.M ? b.M[5 * b.mpl + mq] : b.dV;  // cell volume (J^-1 on a curvilinear grid)
+  const double dV = CURV ? b.M[5 * b.mpl + mq] : b.dV;  // cell volume (J^-1 on a curvilinear grid)
   double u[5];
   for (int v = 0; v < 5; ++v) {
     u[v] = U[b.bbase + v * b.bN + i];
     if (!isfinite(u[v])) acc[7] = 1.0;
     acc[2 + v] += u[v] * dV;
   }
-  const double rho = u[0], ir = 1.0 / rho;
+  const double rho = u[0], ir = recip(rho);
   acc[0] += 0.5 * ir * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * dV;
   // enstrophy only where the CD stencils stay in the block or cross periodic faces
   if (b.nonper) {
@@ -50,16 +51,33 @@ __device__ __noinline__ void diag_point(const DiagBlock& b, const double* __rest
   acc[8] += dV;
   // velocity differences by the CD scheme, one reciprocal of the density per stencil point
   double dv[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-  for (int a = 0; a < ndim; ++a)
-    for (int o = 1; o <= (b.c2[a] != 0.0 ? 2 : 1); ++o)
-      for (int sd = -1; sd <= 1; sd += 2) {
-        const int xs = x + (a == 0 ? sd * o : 0), ys = y + (a == 1 ? sd * o : 0), zs = z + (a == 2 ? sd * o : 0);
-        const long long gi = b.bbase + (long long)wrapc(xs, b.nx) +
-                             (long long)b.nx * ((long long)wrapc(ys, b.ny) + (long long)b.ny * wrapc(zs, b.nz));
-        const double w = sd * (o == 1 ? b.c1[a] : b.c2[a]) / U[gi];
-        for (int c = 0; c < 3; ++c) dv[c][a] = fma(w, U[(1 + c) * b.bN + gi], dv[c][a]);
-      }
-  if (b.M) {  // index-space derivatives -> physical: d/dx_j = J sum_k (metric row k)_j d/dxi_k
+  const bool far = b.c2[0] != 0.0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (a >= ndim) continue;
+    // the axis's four (CD2: two) stencil points, all loads before the first division
+    const int n = a == 0 ? b.nx : (a == 1 ? b.ny : b.nz), c0 = a == 0 ? x : (a == 1 ? y : z);
+    const long long st = a == 0 ? 1 : (a == 1 ? (long long)b.nx : (long long)b.nx * b.ny);
+    double q[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int o = k < 2 ? 2 * k - 1 : 4 * k - 10;  // -1, 1, -2, 2
+      if (k >= 2 && !far) continue;
+      const double* src = U + b.bbase + i + (long long)(wrapc(c0 + o, n) - c0) * st;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (CURV || c != 1 + a) q[k][c] = src[c * b.bN];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k >= 2 && !far) continue;
+      const double w = ((k & 1) ? recip(q[k][0]) : -recip(q[k][0])) * (k < 2 ? b.c1[a] : b.c2[a]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (CURV || c != a) dv[c][a] = fma(w, q[k][1 + c], dv[c][a]);  // (the vorticity takes c != a)
+    }
+  }
+  if (CURV) {  // index-space derivatives -> physical: d/dx_j = J sum_k (metric row k)_j d/dxi_k
     const double J = b.M[6 * b.mpl + mq];
     const double m[3][3] = {{b.M[mq], b.M[b.mpl + mq], 0.0}, {b.M[2 * b.mpl + mq], b.M[3 * b.mpl + mq], 0.0},
                             {0.0, 0.0, b.M[4 * b.mpl + mq]}};
@@ -71,6 +89,11 @@ __device__ __noinline__ void diag_point(const DiagBlock& b, const double* __rest
   }
   const double wx = dv[2][1] - dv[1][2], wy = dv[0][2] - dv[2][0], wz = dv[1][0] - dv[0][1];
   acc[1] += 0.5 * rho * (wx * wx + wy * wy + wz * wz) * dV;
+}
+
+// The column of a marching CTA that cannot use the pairs (rare: out of line, so that the march keeps its registers)
+__device__ __noinline__ void diag_column(const DiagBlock& b, const double* __restrict__ U, int x, int y, int z0, int z1, double* acc) {
+  for (int z = z0; z < z1; ++z) diag_point<false>(b, U, x, y, z, acc);
 }
 
 // acc of 256 threads -> one row: through shared memory, a warp per quantity (each lane eight threads'
@@ -97,12 +120,13 @@ __device__ __forceinline__ void diag_row(const double* acc, double* __restrict__
   }
 }
 
+template <bool CURV>
 __global__ void __launch_bounds__(256) k_diag(DiagBlock b, const double* __restrict__ U, double* __restrict__ partial) {
   double acc[DIAG_NQ] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < b.bN; i += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(i % b.nx), y = (int)((i / b.nx) % b.ny), z = (int)(i / ((long long)b.nx * b.ny));
     if (b.subs && !b.subs[b.sid0 + b.owner[0][x] + b.P[0] * (b.owner[1][y] + b.P[1] * b.owner[2][z])].own) continue;
-    diag_point(b, U, x, y, z, acc);
+    diag_point<CURV>(b, U, x, y, z, acc);
   }
   __shared__ double buf[DIAG_NQ * 256];
   diag_row(acc, partial + (long long)blockIdx.x * DIAG_NQ, buf);
@@ -248,8 +272,7 @@ __global__ void __launch_bounds__(DTX * DTY, 3) k_diag_tile(DiagBlock b, const d
                     (!__syncthreads_or(ens.h >= 0x1p-60f) && __syncthreads_or(ens.h != 0.f));
   if (__syncthreads_or(bad) || lost) {
     for (int c = 0; c < DIAG_NQ; ++c) acc[c] = 0.0;
-    if (own)
-      for (int z = z0; z < z1; ++z) diag_point(b, U, x, y, z, acc);
+    if (own) diag_column(b, U, x, y, z0, z1, acc);
   } else {
 #pragma unroll
     for (int v = 0; v < 5; ++v) acc[2 + v] *= b.dV;
@@ -314,11 +337,24 @@ TileShape tile_shape(int nx, int ny, int nz) {
   return s;
 }
 
-constexpr int kGeneralRows = 2 * 152;
+// CTAs of the kernel by points: one per 256 points up to eight per SM.  (No more than have work: the first CTAs of
+// a larger grid share SMs.  32^3 points in 304 CTAs: 41 us, in 128: 21.)
+int point_rows(int nx, int ny, int nz) { return (int)std::min<long long>(((long long)nx * ny * nz + 255) / 256, 8 * 152); }
+
+// Whether a block's shape suits the marching kernel.  us it takes: per wave of 456 CTAs and plane 1.4 (the
+// latency of a plane) and up to 3.5 more as the SMs fill; the kernel by points 7.7 per 152 CTAs of 256 points.
+// Slender blocks leave most of a tile's columns or of the SMs without work, small ones are one
+// wave of either.  us per call, marching / by points: 4 x 4 x 16384 364 / 83, 8 x 8 x 4096 130 / 83,
+// 2 x 1024^2 952 / 421, 32^3 25 / 21, 12^2 x 2000 97 / 73, 20^2 x 800 54 / 80, 64^3 35 / 66, 256^3 800 / 3300.
+bool march(int nx, int ny, int nz, const TileShape& s) {
+  const double waves = (double)((s.rows + 455) / 456), fill = std::min(1.0, s.rows / 456.0);
+  const long long ctas = ((long long)nx * ny * nz + 255) / 256;
+  return nz > 1 && waves * (s.zc + 4) * (1.4 + 3.5 * fill) < 7.7 * (double)((ctas + 151) / 152);
+}
 
 // the marching kernel: 3-D Cartesian blocks computed here as a whole, of spacings within the pairs' range
-bool tiled(const DiagBlock& b) {
-  if (b.nz == 1 || b.M || b.subs) return false;
+bool tiled(const DiagBlock& b, const TileShape& s) {
+  if (b.M || b.subs || !march(b.nx, b.ny, b.nz, s)) return false;
   for (int a = 0; a < 3; ++a)
     if (!(std::fabs(b.c1[a]) > 1e-12 && std::fabs(b.c1[a]) < 1e12)) return false;
   return true;
@@ -328,18 +364,18 @@ bool tiled(const DiagBlock& b) {
 
 int diag_rows(int nx, int ny, int nz, int most) {
   const TileShape s = tile_shape(nx, ny, nz);
-  return (int)std::max<long long>(kGeneralRows, s.rows <= most ? s.rows : kGeneralRows);
+  return march(nx, ny, nz, s) && s.rows <= most ? (int)s.rows : point_rows(nx, ny, nz);
 }
 
 int launch_diagnostics_block(const DiagBlock& b, const double* U, double* partial, int row0, int rows, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   double* p = partial + (long long)row0 * DIAG_NQ;
   const TileShape s = tile_shape(b.nx, b.ny, b.nz);
-  if (tiled(b) && s.rows <= rows) {
+  if (tiled(b, s) && s.rows <= rows) {
     if (b.rs == 2) k_diag_tile<2><<<rows, dim3(DTX, DTY), 0, st>>>(b, U, p, s.tiles_x, s.tiles, s.zc, (int)s.rows);
     else k_diag_tile<1><<<rows, dim3(DTX, DTY), 0, st>>>(b, U, p, s.tiles_x, s.tiles, s.zc, (int)s.rows);
   } else {
-    k_diag<<<rows, 256, 0, st>>>(b, U, p);
+    (b.M ? k_diag<true> : k_diag<false>)<<<rows, 256, 0, st>>>(b, U, p);
   }
   return (int)cudaGetLastError();
 }

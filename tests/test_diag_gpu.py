@@ -101,3 +101,11 @@ def test_mixed_scales():
     U[1:4, 55:] = 0.0
     ref, got = reference(c, U), static(c, U)
     assert np.all(np.abs(got[:2] - ref[:2]) <= 1e-13 * np.abs(ref[:2])) and got[7] == 0.0
+
+
+# shapes that the marching kernel takes (a column and a row more than its tiles, a last chunk of fewer planes),
+# and slender and small ones that the kernel by points does
+@pytest.mark.parametrize("n", [(65, 57, 66), (64, 64, 64), (96, 65, 53), (129, 41, 50), (3, 5, 4000), (2, 300, 40), (33, 32, 32)])
+@pytest.mark.parametrize("order,scale", [(4, 1.0), (2, 1.0), (4, 1e25)])
+def test_shapes(n, order, scale):
+    test_tiles(n, order, scale)
