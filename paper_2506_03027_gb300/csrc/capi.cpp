@@ -665,7 +665,7 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
     pp.visc_law = ph.visc_law;
     pp.visc_exp = cfs::pair_of(ph.visc_exp);
   }
-  // 2-D inviscid FP64 runs on periodic Cartesian blocks: one launch per stage
+  // 2-D inviscid FP64 runs on periodic Cartesian blocks: one launch per stage, where that is faster
   c->euler2d = {0, 0};
   if (c->p.precision == 0 && c->ndim == 2 && !c->p.viscous && !c->p.compact && c->all_periodic && mtot == 0)
     c->euler2d = cfs::euler2d_shape(c->subs.data(), nsub, c->r);

@@ -257,7 +257,7 @@ int launch_at_halo(const Geometry& g, const PairPhysics& ph, const StepSched& sc
                    const Timer* tm);
 
 // The stage of 2-D inviscid runs on periodic Cartesian blocks in one launch (euler2d.cu): small or
-// large tiles, and the most tiles a sub-domain has.
+// large tiles, and the most tiles a sub-domain has (0: the kernels of kernels.cu are faster).
 struct Euler2dShape {
   int small, tiles;
 };

@@ -234,7 +234,16 @@ namespace {
 //   R = 1  24.7 / 12.4  24.7 / 14.4  25.8 / 18.5  26.7 / 30.8  41.0 / 45.1   49.2 / 57.4  75.6 / 96.3
 // so the line lies between 384^2 and 512^2 (2304 and 4096 small tiles), and between 192^2 and 240^2
 // (576 and 1024).
-constexpr long long small_tiles(int r) { return r == 1 ? 152 * 4 : 152 * 18; }
+//
+// A row of a large tile is a warp, so sub-domains whose width is not near a multiple of 32 leave lanes idle, and
+// the kernels of kernels.cu, three launches over the points of a sub-domain in a row, are faster.  A step,
+// us, three launches / large tiles, by the part of the lanes that have a point:
+//          33 wide: 0.52      40: 0.63    48: 0.75      60: 0.94   64: 1
+//   R = 2  1097 / 1724        293 / 382   1310 / 1411              881 / 758
+//   R = 1  361 / 576          99 / 129    439 / 459                348 / 303
+// (1056^2, 520^2, 1200^2, 1024^2 points).  The line is 0.8; below it small tiles are compared with the three
+// launches: 330^2 in 100 sub-domains (2500 tiles) 168 against 200 and 62 against 60.
+constexpr long long small_tiles(int r, bool full) { return r == 1 ? 152 * (full ? 4 : 16) : 152 * 18; }
 
 template <int R, int TX, int TY, int NT>
 int launch_tile(const Geometry& g, const Physics& ph, const StepSched& sc, const StageLaunch& a, int tiles, cudaStream_t st) {
@@ -265,16 +274,19 @@ int tiles_of(int sx, int sy, int tx, int ty) { return ((sx + tx - 1) / tx) * ((s
 
 Euler2dShape euler2d_shape(const SubDev* subs, int nsub, int r) {
   Euler2dShape e{0, 0};
-  long long small = 0;
+  long long small = 0, points = 0, lanes = 0;
   int most_small = 0, most_large = 0;
   for (int i = 0; i < nsub; ++i) {
     const int t = tiles_of(subs[i].sx, subs[i].sy, 8, 8);
     small += t;
+    points += (long long)subs[i].sx * subs[i].sy;
+    lanes += (long long)((subs[i].sx + 31) / 32) * 32 * subs[i].sy;
     most_small = std::max(most_small, t);
     most_large = std::max(most_large, tiles_of(subs[i].sx, subs[i].sy, 32, 16));
   }
-  e.small = small <= small_tiles(r);
-  e.tiles = e.small ? most_small : most_large;
+  const bool full = 10 * points >= 8 * lanes;
+  e.small = small <= small_tiles(r, full);
+  e.tiles = e.small ? most_small : (full ? most_large : 0);
   return e;
 }
 

@@ -211,3 +211,22 @@ def test_store_of_all_stages_gives_way(precision, monkeypatch):
         one = advance(c, precision=precision, learned=True)
     assert len(refused) == 1
     assert np.all(np.isfinite(full)) and np.array_equal(full, one)
+
+
+# the launches of a step: large tiles where the sub-domains' rows fill them (the second size ragged), three kernels
+# per stage where they do not, small tiles on small grids of either
+@pytest.mark.parametrize("n,p,order,launches", [((512, 448), (8, 7), 4, 5), ((510, 443), (8, 7), 4, 5), ((512, 448), (8, 7), 2, 2),
+                                                ((528, 528), (16, 16), 4, 15), ((528, 528), (16, 16), 2, 6), ((99, 99), (3, 3), 4, 5),
+                                                ((99, 99), (3, 3), 2, 2)])
+def test_two_dimensional_inviscid_route(n, p, order, launches):
+    c = I.vortex_case(32, 1, order=order).replace(nx=n[0], ny=n[1], px=p[0], py=p[1], lx=10.0, ly=7.0)
+    U0 = smooth_2d(c, 5)
+    c = c.replace(dt=I.cfl_dt(c, U0, 0.2))
+    s = cfs.Solver(c)
+    s.set_schedule()
+    s.set_state(U0)
+    s.step(1)
+    assert s.launches() == launches
+    U = s.get_state()
+    s.close()
+    assert np.all(rel_l2(U, orc.run(c, U0, 1)) <= PARITY_TOL)
