@@ -171,10 +171,11 @@ __device__ __forceinline__ void at_prims(const Geometry& g, const StepSched& sc,
 
 }  // namespace
 
-template <int S>
+template <int S, bool ONE>
 __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
                                                     const SubDev* __restrict__ subs, const int2* __restrict__ halo,
-                                                    long long nhalo, int only, float4* __restrict__ Wh) {
+                                                    long long nhalo, int only_, float4* __restrict__ Wh) {
+  const int only = ONE ? only_ : -1;
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: no halo store is read
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -269,16 +270,19 @@ __global__ void __launch_bounds__(256) k_halo_prims(Geometry g, Physics ph, Step
 // thread per point: the six faces to depth 5 (x faces: the five points of a row fastest), then the
 // twelve r x r edges.  The filter halo is the extrapolation to t_{n+1} (weights c(k+1)) as the FP32
 // deviation from the sub-domain's reference value, [(sub-domain, variable)][axis][10][N^2].  256^3 in 512
-// sub-domains: 1.83 ms, against 1.76 for the halo store alone and 0.43 for the filter's halos.
-template <int N>
+// sub-domains: 1.88 ms, against 1.76 for the halo store alone and 0.43 for the filter's halos.
+template <int N, bool ONE>
 __global__ void __launch_bounds__(256) k_halo_block(Geometry g, Physics ph, StepSched sc, const double* __restrict__ ring,
-                                                    const SubDev* __restrict__ subs, int only,
+                                                    const SubDev* __restrict__ subs, int only_,
                                                     float4* __restrict__ Wh, float* __restrict__ fh) {
+  const int only = ONE ? only_ : -1;
   constexpr int S = 5, NN = N * N, NF = 5 * NN;
   sc = resolve(sc);
   if (sc.mode == 0) return;  // synchronous step: neither is read
-  const int sid = blockIdx.y;
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  // (the sub-domains in blockIdx.x, which counts further than 65,535)
+  constexpr int per_sub = (6 * NF + 48 * N + 255) / 256;
+  const int sid = blockIdx.x / per_sub;
+  int t = (int)(blockIdx.x - sid * per_sub) * 256 + threadIdx.x;
   if (t >= 6 * NF + 48 * N) return;
   const Phys32 k32 = phys32(ph);
   const SubDev d = subs[sid];
@@ -935,8 +939,9 @@ int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc,
   if (nhalo <= 0) return 0;
   const unsigned nb = (unsigned)((nhalo + 255) / 256);
   if (tm) tm->rec(tm->self, 0, 1);
-  if (s == 2) k_halo_prims<2><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, only, (float4*)Wh);
-  else k_halo_prims<5><<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, only, (float4*)Wh);
+  const auto kernel = s == 2 ? (only < 0 ? k_halo_prims<2, false> : k_halo_prims<2, true>)
+                             : (only < 0 ? k_halo_prims<5, false> : k_halo_prims<5, true>);
+  kernel<<<nb, 256, 0, st>>>(g, ph, sc, ring, subs, (const int2*)halo, nhalo, only, (float4*)Wh);
   if (tm) tm->rec(tm->self, 0, 0);
   if (launches) *launches += 1;
   return (int)cudaGetLastError();
@@ -945,10 +950,11 @@ int launch_halo_prims(const Geometry& g, const Physics& ph, const StepSched& sc,
 int launch_halo_block(const Geometry& g, const Physics& ph, const StepSched& sc, const double* ring, const SubDev* subs, int n,
                       float* Wh, float* fh, int only, void* stream, long long* launches, const Timer* tm) {
   cudaStream_t st = (cudaStream_t)stream;
-  const dim3 grid((30 * n * n + 48 * n + 255) / 256, g.nsub);
+  const unsigned grid = (unsigned)((30 * n * n + 48 * n + 255) / 256) * (unsigned)g.nsub;
   if (tm) tm->rec(tm->self, 0, 1);
-  if (n == 32) k_halo_block<32><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, only, (float4*)Wh, fh);
-  else k_halo_block<16><<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, only, (float4*)Wh, fh);
+  const auto kernel = n == 32 ? (only < 0 ? k_halo_block<32, false> : k_halo_block<32, true>)
+                              : (only < 0 ? k_halo_block<16, false> : k_halo_block<16, true>);
+  kernel<<<grid, 256, 0, st>>>(g, ph, sc, ring, subs, only, (float4*)Wh, fh);
   if (tm) tm->rec(tm->self, 0, 0);
   if (launches) *launches += 1;
   return (int)cudaGetLastError();

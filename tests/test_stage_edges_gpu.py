@@ -230,3 +230,17 @@ def test_two_dimensional_inviscid_route(n, p, order, launches):
     U = s.get_state()
     s.close()
     assert np.all(rel_l2(U, orc.run(c, U0, 1)) <= PARITY_TOL)
+
+
+# more sub-domains than the second dimension of a grid counts
+@pytest.mark.parametrize("n", [16, 32])
+def test_halo_store_of_many_subdomains(n, tmp_path):
+    import ctypes
+    import os
+    import subprocess
+    from paper_2506_03027_gb300 import build as B
+    here = os.path.dirname(os.path.abspath(__file__))
+    out = str(tmp_path / "liblaunch.so")
+    subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", B.CSRC,
+                    os.path.join(here, "cuda", "launch_check.cu"), B.LIB, "-Xlinker", "-rpath=" + os.path.dirname(B.LIB), "-o", out], check=True)
+    assert ctypes.CDLL(out).halo_block_launch(70000, n) == 0
