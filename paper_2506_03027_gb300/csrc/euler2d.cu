@@ -8,7 +8,7 @@
 // beyond it, halo points by the schedule), the fluxes go through shared memory, and each thread
 // updates its points.  The mass flux is the momentum itself, the off-diagonal momentum flux is
 // shared by the axes, the differences are taken without their factor where the spacings are equal,
-// and a tile without z momentum leaves that component out (it stays zero).  Five fourth-order steps of
+// and a tile without z momentum and with finite velocities leaves that component out (it stays zero).  Five fourth-order steps of
 // 64^2: 359 -> 171 us; a second-order step of 1024^2: 348 -> 303 us (131 us per stage, 81 of them at
 // the FP64 rate).
 #include <cuda_runtime.h>
@@ -140,8 +140,9 @@ __global__ void __launch_bounds__(NT, NT >= 256 ? 3 : 1) k_euler2d(Geometry g, P
     }
     zm = zm || (kind && nonzero(u[k][3]));
   }
-  // whether the z momentum vanishes on the tile and its rim
+  // whether the z momentum is anything but zero on the tile and its rim
   const bool zmom = __syncthreads_or(zm);
+  bool bad = false;  // a velocity that is not finite: its product with zero is not zero
 
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(NT, NT >= 256 ? 3 : 1) k_euler2d(Geometry g, P
     const double* w = u[k];
     double vx, vy, p, et;
     prims(w, vx, vy, p, et);
+    bad = bad || max(__double2hiint(vx) & 0x7fffffff, __double2hiint(vy) & 0x7fffffff) >= 0x7ff00000;
     const int ox = pj * FW + pi + R, oy = (pj + R) * TX + pi;
     const double uv = w[1] * vy;
     if (kind & 1) {  // fluxes along x: the tile and its columns
@@ -178,7 +180,21 @@ __global__ void __launch_bounds__(NT, NT >= 256 ? 3 : 1) k_euler2d(Geometry g, P
     for (int v = 0; v < 5; ++v) q[v] = own ? Q[g0 + pi + (long long)d.bnx * pj + v * N] : 0.0;
   };
   load_q(0);
-  __syncthreads();
+  bool zflux = zmom;
+  if (__syncthreads_or(bad) && !zmom) {
+    zflux = true;
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+      int pi, pj;
+      const int kind = point(tid + k * NT, pi, pj);
+      if (!kind) continue;
+      double vx, vy, p, et;
+      prims(u[k], vx, vy, p, et);
+      if (kind & 1) sm.x[2][pj * FW + pi + R] = u[k][3] * vx;
+      if (kind & 2) sm.y[2][(pj + R) * TX + pi] = u[k][3] * vy;
+    }
+    __syncthreads();
+  }
 
   // ---- - dt (D_x F + D_y G) in units of the difference factor, and the low-storage update
   const double cx = R == 2 ? d.c2[0] : d.c1[0], cy = R == 2 ? d.c2[1] : d.c1[1];
@@ -206,8 +222,8 @@ __global__ void __launch_bounds__(NT, NT >= 256 ? 3 : 1) k_euler2d(Geometry g, P
     update(0, 4);
     update(1, 0);
     update(2, 1);
-    if (zmom || nonzero(q[3])) {
-      if (!zmom) {
+    if (zflux || nonzero(q[3])) {
+      if (!zflux) {
         const double qn = A * q[3];
         if (!last) Q[gi + 3 * N] = qn;
         Uout[gi + 3 * N] = fma(B, qn, u[k][3]);

@@ -244,3 +244,18 @@ def test_halo_store_of_many_subdomains(n, tmp_path):
     subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", B.CSRC,
                     os.path.join(here, "cuda", "launch_check.cu"), B.LIB, "-Xlinker", "-rpath=" + os.path.dirname(B.LIB), "-o", out], check=True)
     assert ctypes.CDLL(out).halo_block_launch(70000, n) == 0
+
+
+# a NaN or an infinity in another component reaches the z momentum though that is zero
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("component", [0, 1, 2])
+@pytest.mark.parametrize("n", [(35, 22), (510, 443)])
+def test_nonfinite_value_reaches_the_zero_z_momentum(n, component, value):
+    c = I.vortex_case(32, 1).replace(nx=n[0], ny=n[1], px=max(1, n[0] // 60), py=max(1, n[1] // 60), lx=10.0, ly=7.0, dt=1e-4)
+    U0 = smooth_2d(c, 5)
+    U0[3] = 0.0
+    U0[component, 0, 9, 17] = value
+    Ug, _ = gpu_run(c, U0, 1)
+    ref = orc.run(c, U0, 1)
+    assert not np.all(np.isfinite(ref[3]))
+    assert np.array_equal(np.isfinite(Ug[3]), np.isfinite(ref[3]))
