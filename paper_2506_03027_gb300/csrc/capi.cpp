@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -36,20 +37,18 @@ struct Block {
   long long ebase = -1;   // offset of its gather map in d_emap (blocks with a non-periodic face)
 };
 
-// A line-filter launch of one pass axis: the blocks whose shared-memory tiles (sized by their longest line) are at
-// least half as large as the largest of them, so that few CTAs are kept from an SM by memory they do
-// not use.  (The 12 blocks of an airfoil grid take one launch per axis.)
-struct FilterPass {
-  int nblk = 0;
+// The blocks that one line-filter launch covers: along the pass axis they have the same number of
+// sub-domains and equally long longest lines (the length sizes the shared-memory tiles).
+struct FilterGroup {
+  int Lt = 0, nblk = 0;
   unsigned ctas = 0;
-  size_t smem = 0;
   cfs::FilterBlk* d_blks = nullptr;
 };
 
 struct cfs_ctx {
   cfs_params p{};
   std::vector<Block> blocks;
-  std::vector<FilterPass> fpass[3];  // per pass axis
+  std::vector<FilterGroup> fgroups[3];  // per pass axis
   cudaStream_t stream = nullptr;
   cfs_alloc_fn alloc = nullptr;
   cfs_free_fn freef = nullptr;
@@ -1005,52 +1004,53 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
       CUDA_TRY(c, cudaMemcpyAsync(b.d_axis_len[a], keep[k0 + 2].data(), sizeof(int) * b.P[a], cudaMemcpyHostToDevice, st), "upload tables");
     }
   }
-  // line filter: per pass axis the blocks of one launch, those of the largest tiles first
-  std::vector<std::vector<cfs::FilterBlk>> fkeep(3);  // (alive until the stream is synchronised below)
+  // line filter: per pass axis the blocks by the length of their longest line and their split
+  std::vector<std::vector<cfs::FilterBlk>> fkeep;  // (alive until the stream is synchronised below)
   if (c->p.filter) {
     for (int ax = 0; ax < c->ndim; ++ax) {
-      std::vector<cfs::FilterBlk>& v = fkeep[ax];
+      std::map<std::pair<int, int>, std::vector<const Block*>> by_len;
       for (const Block& b : c->blocks) {
-        cfs::FilterBlk e{};
-        e.ebase = b.ebase;
-        e.gmx = b.nx + 2 * c->geo.GE;
-        e.gmy = b.ny + 2 * c->geo.GE;
-        for (int q = 0; q < 6; ++q) {
-          if (b.face[q].type >= cfs::FACE_WALL) e.phys |= 1 << q;
-          if (b.face[q].type == cfs::FACE_WALL) e.wall |= 1 << q;
-        }
-        e.n[0] = b.nx; e.n[1] = b.ny; e.n[2] = b.nz;
-        e.bN = b.N;
-        e.bbase = b.base;
-        e.sid0 = b.sid0;
-        for (int a = 0; a < 3; ++a) {
-          e.P[a] = b.P[a];
-          e.owner[a] = b.d_owner[a];
-          e.axis_off[a] = b.d_axis_off[a];
-          e.axis_len[a] = b.d_axis_len[a];
-        }
-        e.Lt = (e.n[ax] + e.P[ax] - 1) / e.P[ax];
-        v.push_back(e);
+        const int n3[3] = {b.nx, b.ny, b.nz};
+        by_len[{(n3[ax] + b.P[ax] - 1) / b.P[ax], b.P[ax]}].push_back(&b);
       }
-      const int sync = c->max_delay == 0;
-      auto smem = [&](const cfs::FilterBlk& e) { return cfs::filter_smem(e.Lt, c->p.precision, sync); };
-      std::stable_sort(v.begin(), v.end(), [&](const cfs::FilterBlk& a, const cfs::FilterBlk& b) { return smem(a) > smem(b); });
-      cfs::FilterBlk* blks = (cfs::FilterBlk*)dev_alloc(c, sizeof(cfs::FilterBlk) * v.size());
-      if (!blks) return fail(c, CFS_ENOMEM, "device allocation failed");
-      for (size_t i = 0; i < v.size(); ++i) {
-        std::vector<FilterPass>& passes = c->fpass[ax];
-        if (passes.empty() || 2 * smem(v[i]) < passes.back().smem) {
-          passes.emplace_back();
-          passes.back().smem = smem(v[i]);
-          passes.back().d_blks = blks + i;
+      for (const auto& kv : by_len) {
+        FilterGroup fg;
+        fg.Lt = kv.first.first;
+        std::vector<cfs::FilterBlk> v;
+        for (const Block* b : kv.second) {
+          cfs::FilterBlk e{};
+          e.ebase = b->ebase;
+          e.gmx = b->nx + 2 * c->geo.GE;
+          e.gmy = b->ny + 2 * c->geo.GE;
+          for (int q = 0; q < 6; ++q) {
+            if (b->face[q].type >= cfs::FACE_WALL) e.phys |= 1 << q;
+            if (b->face[q].type == cfs::FACE_WALL) e.wall |= 1 << q;
+          }
+          e.n[0] = b->nx; e.n[1] = b->ny; e.n[2] = b->nz;
+          e.bN = b->N;
+          e.bbase = b->base;
+          e.sid0 = b->sid0;
+          for (int a = 0; a < 3; ++a) {
+            e.P[a] = b->P[a];
+            e.owner[a] = b->d_owner[a];
+            e.axis_off[a] = b->d_axis_off[a];
+            e.axis_len[a] = b->d_axis_len[a];
+          }
+          e.cta0 = fg.ctas;
+          fg.ctas += cfs::filter_ctas(e.n, e.P, ax, fg.Lt, c->p.precision, c->max_delay == 0);
+          v.push_back(e);
         }
-        FilterPass& fp = passes.back();
-        v[i].cta0 = fp.ctas;
-        fp.ctas += cfs::filter_ctas(v[i].n, v[i].P, ax, v[i].Lt, c->p.precision, sync);
-        fp.nblk += 1;
+        fg.nblk = (int)v.size();
+        fg.d_blks = (cfs::FilterBlk*)dev_alloc(c, sizeof(cfs::FilterBlk) * v.size());
+        if (!fg.d_blks) return fail(c, CFS_ENOMEM, "device allocation failed");
+        fkeep.push_back(std::move(v));
+        CUDA_TRY(c, cudaMemcpyAsync(fg.d_blks, fkeep.back().data(), sizeof(cfs::FilterBlk) * fkeep.back().size(),
+                                    cudaMemcpyHostToDevice, st), "upload filter blocks");
+        c->fgroups[ax].push_back(fg);
       }
-      CUDA_TRY(c, cudaMemcpyAsync(blks, v.data(), sizeof(cfs::FilterBlk) * v.size(), cudaMemcpyHostToDevice, st),
-               "upload filter blocks");
+      // the largest launch first: the others run beside its last CTAs
+      std::stable_sort(c->fgroups[ax].begin(), c->fgroups[ax].end(),
+                       [](const FilterGroup& a, const FilterGroup& b) { return a.ctas > b.ctas; });
     }
   }
   CUDA_TRY(c, cudaMemsetAsync(c->ring, 0, sizeof(double) * 5 * N * c->R, st), "clear ring");
@@ -1308,17 +1308,19 @@ static cfs_status enqueue_step(cfs_ctx* c, long long n, bool graph) {
       // graph mode: the sub-domain filter (returns on synchronous steps) before the per-pass
       // kernels (which then return on asynchronous steps)
       if (op == c->s && c->fblock_n && graph) rc = launch_fblock(c, g, sc, src, nullptr, true);
-      for (const FilterPass& fp : c->fpass[op - c->s]) {
+      const std::vector<FilterGroup>& groups = c->fgroups[op - c->s];
+      for (const FilterGroup& fg : groups) {
         if (rc != 0) break;
         cfs::FilterLaunch f{};
         f.Uin = src; f.Uout = dst; f.ring = c->ring;
         f.in_ring = in_ring; f.out_ring = out_ring;
-        f.blks = fp.d_blks; f.nblk = fp.nblk; f.ctas = fp.ctas; f.smem = fp.smem;
+        f.blks = fg.d_blks; f.nblk = fg.nblk; f.ctas = fg.ctas; f.Lt = fg.Lt;
         f.thomas_k = c->d_thomas_k; f.thomas32 = c->d_thomas32; f.Lmax = c->Lmax; f.alpha = c->p.alpha_f;
         for (int m = 0; m < 6; ++m) f.h[m] = c->filt_h[m];
         f.b1 = c->filt_h[1] - c->p.alpha_f;
         f.sync = c->max_delay == 0;
         f.only_sync = graph && c->fblock_n;
+        f.chain = (&fg != &groups.back() ? 1 : 0) | (&fg != &groups.front() ? 2 : 0);
         f.subs = c->part_n > 1 ? c->d_subs : nullptr;
         rc = cfs::launch_filter(g, sc, f, op - c->s, c->p.precision, c->stream, &c->launches, tm);
       }

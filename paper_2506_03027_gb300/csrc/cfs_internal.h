@@ -275,7 +275,6 @@ struct FilterBlk {
   int P[3];                // sub-domains per axis
   long long bN, bbase;     // its points and the offset of its state in a state array
   int sid0;                // index of its first sub-domain
-  int Lt;                  // its longest sub-domain line along the pass axis (sizes its tiles)
   unsigned cta0;           // first CTA of the launch that works on it
   const int* owner[3];     // device: sub-domain index along each axis for every global coordinate
   const int* axis_off[3];  // device: per sub-domain index along the axis, its origin
@@ -287,14 +286,14 @@ struct FilterLaunch {
   double* Uout;
   const double* ring;
   int in_ring, out_ring;   // graph mode: input is ring level n / output is ring level n + 1
-  const FilterBlk* blks;   // device: the blocks of this launch
-  int nblk;
+  const FilterBlk* blks;   // device: the blocks of this launch (their longest lines along the pass
+  int nblk;                // axis are all Lt points, which sizes the tiles)
   unsigned ctas;
-  size_t smem;             // shared memory of the largest of their tiles
   const double* thomas_k;  // device: FP64 form: [2][Lmax]: c_i, and 1 / m_i times the filter's scale
                            // (1 - 2 alpha)/1024
   const float* thomas32;   // device: FP32 form: c_i and 1 / m_i rounded to FP32 (d2f_fast)
   int Lmax;
+  int Lt;                  // longest sub-domain line of these blocks along the pass axis
   double alpha;
   double h[6];             // filter right side: a_0, a_1/2, ..., a_5/2
   double b1;               // a_1/2 - alpha: weight of the first second difference (increment form)
@@ -302,10 +301,15 @@ struct FilterLaunch {
   int only_sync;           // graph mode beside the sub-domain filter: return unless the step is synchronous
   const SubDev* subs;      // partitioned context: the sub-domain table (lines of foreign sub-domains are
                            // skipped); null when every sub-domain is computed here
+  // The launches of one pass axis read the same input and write different blocks, so they overlap: bit 0
+  // when another launch of the axis follows, bit 1 when one went before.  The first waits for its
+  // predecessor and only then lets the second start; so the later ones, which start once every CTA of
+  // the one before has started, need not wait for that input.  They wait for the launch before them
+  // at their end instead, so that the next axis, which waits for the last launch, waits for all.
+  int chain;
 };
 // CTAs of a launch that one block of size n, split P, takes along `axis` with lines of Lt points
 unsigned filter_ctas(const int* n, const int* P, int axis, int Lt, int precision, int sync);
-size_t filter_smem(int Lt, int precision, int sync);  // shared memory of a CTA with lines of up to Lt points
 
 // FP32-intermediate filter of asynchronous steps, all three passes per (sub-domain, variable)
 // (filter_block.cu); cubic sub-domains of n points per axis, n in {16, 32}.

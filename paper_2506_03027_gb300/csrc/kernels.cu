@@ -735,9 +735,9 @@ int launch_stage(const Geometry& g, const Physics& ph, const StepSched& sc, cons
 // values by the schedule (SA: live neighbour; AT: extrapolation to t_{n+1} with the weights c(k+1)
 // in FP64; AS: the latest delayed level) -- in shared memory with coalesced loads (consecutive
 // threads along the line for the x pass, across lines for y and z), solves each line from there,
-// and stores the result with the same pattern.  Blocks share a launch, each with tiles of its own
-// length: the twelve blocks of an airfoil grid take three launches per step instead of 36 that each fill a
-// part of the chip.
+// and stores the result with the same pattern.  Blocks with the same split and line length
+// along the axis share a launch: the twelve blocks of an airfoil grid take seven launches per step
+// instead of 36 that each fill a part of the chip.
 //
 // Staging and storing waited for memory, one value of a thread after the other (10 to 15 cycles of
 // load latency per issue, DRAM at 8 to 39 %), so a thread now keeps eight of them in flight: own values in
@@ -815,9 +815,17 @@ __device__ __forceinline__ double from_fixed_point(long long g, int q20) {
 // 186 when held to the bound, 170 with the compiler's own 72)
 template <typename T, int axis>
 __global__ void __launch_bounds__(128, std::is_same<T, float>::value || axis == 0 ? 0 : 7) k_filter(Geometry g, StepSched sc, FilterLaunch f) {
-  pdl_enter();
+  if (f.chain == 0) {
+    pdl_enter();
+  } else {  // (see FilterLaunch)
+    if (!(f.chain & 2)) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  }
   sc = resolve(sc);
-  if (f.only_sync && sc.mode != 0) return;
+  if (f.only_sync && sc.mode != 0) {
+    if (f.chain & 2) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    return;
+  }
   constexpr bool F32 = std::is_same<T, float>::value;
   const double* __restrict__ Uin = ring_or(f.Uin, f.in_ring, f.ring, sc, 0);
   double* __restrict__ Uout = const_cast<double*>(ring_or(f.Uout, f.out_ring, f.ring, sc, 1));
@@ -833,7 +841,7 @@ __global__ void __launch_bounds__(128, std::is_same<T, float>::value || axis == 
   const FilterBlk& B = f.blks[bi];
   const int n[3] = {B.n[0], B.n[1], B.n[2]};
   const long long strides[3] = {1, n[0], (long long)n[0] * n[1]};
-  const FilterTile tl = filter_tile(B.Lt, F32 ? 1 : 0, f.sync);
+  const FilterTile tl = filter_tile(f.Lt, F32 ? 1 : 0, f.sync);
   const int LN = tl.LN, TW = tl.TW;
   extern __shared__ __align__(16) double fsm[];
   // [LN][TW] window slots (positions -5 .. len+4): FP64 values, or in the FP32 form FP32 offsets
@@ -1215,6 +1223,7 @@ __global__ void __launch_bounds__(128, std::is_same<T, float>::value || axis == 
       }
     }
   }
+  if (f.chain & 2) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 __global__ void k_round_table(const double* __restrict__ x, float* __restrict__ y, long long n) {
@@ -1258,8 +1267,6 @@ int filter_prepare(int Lmax, int precision) {
   return (int)e;
 }
 
-size_t filter_smem(int Lt, int precision, int sync) { return filter_smem_bytes(Lt, precision, sync); }
-
 unsigned filter_ctas(const int* n, const int* P, int axis, int Lt, int precision, int sync) {
   const int f1 = (axis == 0) ? 1 : 0;
   const int f2 = (axis == 2) ? 1 : 2;
@@ -1271,7 +1278,7 @@ unsigned filter_ctas(const int* n, const int* P, int axis, int Lt, int precision
 int launch_filter(const Geometry& g, const StepSched& sc, const FilterLaunch& f, int axis, int precision,
                   void* stream, long long* launches, const Timer* tm) {
   const unsigned nb = f.ctas;
-  const size_t sm = f.smem;
+  const size_t sm = filter_smem_bytes(f.Lt, precision, f.sync);
   cudaStream_t st = (cudaStream_t)stream;
   if (tm) tm->rec(tm->self, 3, 1);
   if (precision == 1) {
