@@ -303,9 +303,13 @@ struct FilterLaunch {
                            // skipped); null when every sub-domain is computed here
   // The launches of one pass axis read the same input and write different blocks, so they overlap: bit 0
   // when another launch of the axis follows, bit 1 when one went before.  The first waits for its
-  // predecessor and only then lets the second start; so the later ones, which start once every CTA of
-  // the one before has started, need not wait for that input.  They wait for the launch before them
-  // at their end instead, so that the next axis, which waits for the last launch, waits for all.
+  // predecessor and only then lets the second start; the later ones, which start once every CTA of the one
+  // before has started, do not wait for that input.  They wait for the launch before them at their end
+  // instead, so that the next axis, which waits for the last launch, waits for all.  That the later ones
+  // see the input does not follow from a griddepcontrol.wait of their own (PTX states visibility for the grid
+  // that waits); it rests on this order: the writer of the input has completed when the first launch's
+  // wait returns, each of its threads then passes a device-scope fence and triggers, and a later launch
+  // begins after all of them have, with a fence of its own before it reads.
   int chain;
 };
 // CTAs of a launch that one block of size n, split P, takes along `axis` with lines of Lt points

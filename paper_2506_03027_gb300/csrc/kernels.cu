@@ -819,6 +819,7 @@ __global__ void __launch_bounds__(128, std::is_same<T, float>::value || axis == 
     pdl_enter();
   } else {  // (see FilterLaunch)
     if (!(f.chain & 2)) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    __threadfence();
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   }
   sc = resolve(sc);

@@ -175,3 +175,21 @@ def test_filter_of_small_values_beside_large_ones(p, scale):
     # 0.63^33 = 2.1e-7 reaches fifty-one points away
     tol = (3 * 0.5 + 2 + 2.0 ** 7) * 2.0 ** -52 * scale + 2.1e-7 * 2.0 ** -52
     assert e.max() <= tol, (e.max(), tol)
+
+
+def test_blocks_of_unequal_lines():
+    """Blocks of long and short lines, whose launches overlap, in pieces and whole."""
+    base = I.tgv_case(16, 1, "SA").replace(alpha_f=0.45, dt=1e-300)
+    blocks = [base.replace(nx=n[0], ny=n[1], nz=n[2], px=p) for n, p in (((140, 10, 11), 1), ((12, 13, 10), 1), ((60, 11, 10), 2),
+                                                                        ((100, 12, 10), 1), ((33, 10, 12), 3))]
+    states = [rough_state(c, 1.0, 11 + k) for k, c in enumerate(blocks)]
+    s = cfs.Solver(blocks[0], blocks=blocks)
+    s.set_schedule()
+    s.set_states(states)
+    s.step(1)
+    got = s.get_states()
+    s.close()
+    for c, U0, U in zip(blocks, states, got):
+        ref = reference(c, U0)
+        for v in range(5):
+            assert np.abs(U[v] - ref[v]).max() <= 3 * 2 * 2.0 ** -53 * np.abs(U0[v]).max(), v
