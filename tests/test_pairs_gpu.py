@@ -96,3 +96,34 @@ def test_power_of_bad_values(lib):
     out = torch.empty((3, 2), dtype=torch.float32, device="cuda")
     assert lib.pairs_pow(t.data_ptr(), 0.76, out.data_ptr(), 3) == 0
     assert bool(torch.isnan(out.sum(dim=-1)).all())
+
+
+@pytest.mark.gpu
+def test_pair_to_double_on_the_integer_pipe(tmp_path):
+    """The FP64 sum h + l of normalised pairs over the range of a stage's dt R, powers of two with a negative
+    and a positive low part among them; the high part alone below 2^-66, NaN and infinity as NaN."""
+    import torch
+    out = str(tmp_path / "libpd.so")
+    subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", CSRC,
+                    os.path.join(HERE, "cuda", "pair_double_check.cu"), "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    lib.pair_double.argtypes = [ctypes.c_void_p] * 2 + [ctypes.c_int]
+    rng = np.random.default_rng(5)
+    n = 1 << 16
+    h = (rng.choice([-1.0, 1.0], n) * rng.uniform(1.0, 2.0, n) * 2.0 ** rng.integers(-65, 100, n)).astype(np.float32)
+    h[::4] = np.sign(h[::4]) * 2.0 ** np.floor(np.log2(np.abs(h[::4])))
+    l = (rng.uniform(-0.5, 0.5, n) * np.spacing(np.abs(h))).astype(np.float32)
+    l[::4] *= np.float32(0.5)  # (below a power of two the pair's low part is at most a quarter of its last place)
+    l[1::8] = 0.0
+    special = np.array([[0.0, 0.0], [-0.0, 0.0], [1e-25, 1e-33], [np.nan, 0.0], [np.inf, np.nan], [1.0, 2.0 ** -60]], dtype=np.float32)
+    a = np.concatenate([np.stack([h, l], 1), special])
+    t = torch.tensor(a, device="cuda")
+    y = torch.empty(len(a), dtype=torch.float64, device="cuda")
+    assert lib.pair_double(t.data_ptr(), y.data_ptr(), len(a)) == 0
+    got = y.cpu().numpy()
+    ref = h.astype(np.float64) + l.astype(np.float64)
+    # l rounds to a multiple of the sum's last place, as the sum does (ties may differ)
+    assert np.all(np.abs(got[:n] - ref) <= np.spacing(np.abs(ref)))
+    assert np.mean(got[:n] == ref) > 0.99
+    s = got[n:]
+    assert s[0] == 0.0 and s[1] == 0.0 and s[2] == np.float64(np.float32(1e-25)) and np.isnan(s[3]) and np.isnan(s[4]) and s[5] == 1.0
