@@ -15,10 +15,12 @@ Metric: point-RK-stage updates per second (Mpoint-stage/s) = 128^3 x 5 x steps /
   e2e       the same metric through the public API with host buffers: per step the state is
             copied in from pinned host memory, stepped, and copied back out; host_link gives the
             measured bandwidth of those copies and the floor they put under an e2e step.
-  roofline  the dominant kernel's algorithmic bytes per launch / average event-timed launch duration
-            against the measured copy bandwidth (the stage's right-hand side runs on pairs of
-            floats, so no stage kernel is bound by the FP64 pipe); fp64_probe: the FP64 rate, which
-            the line filter and the state update use.
+  roofline  the bytes the method has to move per step over the step's time, against the measured copy
+            bandwidth (the stage's right-hand side runs on pairs of floats, so no stage kernel is bound
+            by the FP64 pipe alone).  dominant_kernel: the kernel kind that takes most of the step, with
+            the bytes that this program's division into kernels moves through it (scratch arrays
+            included) over its event-timed launches; fp64_probe: the FP64 rate, which the line filter and
+            the state update use.
   cpu_baseline  the FP64 CPU oracle on the host cores on a bounded sample of the workload.
 
 forms (same metric, one GPU; each a dict in the JSON line):
@@ -62,11 +64,12 @@ HBM_GBS_FALLBACK = 6800.0
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of each kernel kind, with the sha1 of
 # the stage's source they were taken from (kernels_sha1; null once it changes); filled from profiles/.
-TRAFFIC = {"source_sha1": "136ec8a3bc35a787363802cd030a0add0b46a735",
-           # 128^3, 64 sub-domains, read + written: k_flux_p 209.4 + 239.9 MB, k_rk_p 491.8 + 120.9 (mean of
-           # the five stages), view (k_at_halo 617.5 + 322.3 once, k_view_p 164.7 + 171.6 five times),
-           # k_filter 327.3 + 57.1 (mean of the three passes)
-           "bytes_per_launch": {"flux": 449.3e6, "stage_update": 612.7e6, "view": 436.9e6, "filter": 384.4e6}}
+TRAFFIC = {"source_sha1": "9fc731a1e59ae7086fc4d069f9ac5351d493201b",
+           # 128^3, 64 sub-domains, read + written: k_flux_p 205.8 + 185.1 MB, k_rk_p 441.5 + 121.7 (mean of
+           # the five stages), view (k_at_halo 619.0 + 330.9 once, k_view_p 168.3 + 177.8 five times),
+           # k_filter 329.4 + 59.2 (mean of the three passes)
+           "bytes_per_launch": {"flux": 390.9e6, "stage_update": 563.2e6, "view": 446.7e6, "filter": 388.6e6},
+           "bytes_per_step": 8616.7e6}
 
 
 def kernels_sha1(root: str = ROOT) -> str:
@@ -229,22 +232,23 @@ def face_points(case, depth):
     return tot
 
 
-def algorithmic_bytes(case, kind):
-    """Bytes a launch of each kernel kind of the FP64 form has to move (scratch arrays of pairs: 56 B of
-    primitives and 40 B of fluxes per direction and point; FP64 state and Q: 40 B each per point),
-    averaged over a step's launches."""
+def kernel_bytes(case, kind):
+    """Bytes that the program's own division into kernels moves through a launch of each kernel kind of the
+    FP64 form (scratch arrays of pairs: 56 B of primitives, 32 B of fluxes per direction and point and 8 B of mass
+    flux in the strips beyond the faces; FP64 state and Q: 40 B each per point), averaged over a step's launches.
+    The method itself needs less: algorithmic_bytes_per_step."""
     N = case.npts
     r = 2 if case.order == 4 else 1
     halo, strips = face_points(case, 2 * r), face_points(case, r)
     if kind == "flux":
-        return N * (56 + 120) + halo * 56 + strips * 40
+        return N * (56 + 96) + halo * 56 + strips * 32
     if kind == "stage_update":
         # U in and out, Q in on every stage but the first and out on every one but the last
-        return N * (120 + 80 + 80 * (case.stages - 1) / case.stages) + strips * 40
+        return N * (96 + 80 + 80 * (case.stages - 1) / case.stages) + strips * (32 + 8)
     if kind == "view":
         # one launch for the AT halo values of all stages, one per stage for the primitives
         at = halo * 40 * (case.levels + case.stages)
-        return (at + case.stages * (N * (40 + 56) + halo * (40 + 56))) / (1 + case.stages)
+        return (at + case.stages * (N * (40 + 56) + halo * (40 + 56) + strips * 8)) / (1 + case.stages)
     if kind == "filter":
         return N * 80 + face_points(case, 5) / 3 * 40 * case.levels
     return 0
@@ -458,10 +462,14 @@ def run_ours(args, rank, world, local_rank):
     dom_ms, dom_n = kinds[dom]
     if args.precision == 0:
         peak = peaks.get("hbm_gbs", HBM_GBS_FALLBACK)
-        bytes_ = algorithmic_bytes(case, dom)
-        achieved = bytes_ / (dom_ms / dom_n * 1e-3) / 1e9
-        roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "kernel": dom,
-                "bytes_per_launch": bytes_,
+        step_gbs = algorithmic_bytes_per_step(case) * K / (ms * 1e-3) / 1e9
+        own = kernel_bytes(case, dom)
+        own_gbs = own / (dom_ms / dom_n * 1e-3) / 1e9
+        names = {"view": "k_at_halo once and k_view_p per stage", "flux": "k_flux_p", "stage_update": "k_rk_p", "filter": "k_filter"}
+        roof = {"bound": "hbm", "achieved": step_gbs, "peak": peak, "unit": "GB/s", "frac": step_gbs / peak, "kernel": "step",
+                "bytes_per_step": algorithmic_bytes_per_step(case),
+                "dominant_kernel": {"kind": dom, "kernels": names.get(dom), "own_bytes_per_launch": own, "own_gbs": own_gbs,
+                                    "own_frac": own_gbs / peak},
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback",
                 "fp64_probe": dict(fp64_peak(local_rank),
                                    nominal_tflops=SM_COUNT * FP64_FLOP_PER_CLK_SM * sm_max * 1e6 / 1e12)}
@@ -470,8 +478,11 @@ def run_ours(args, rank, world, local_rank):
         roof = fused_roofline(case, ktimes) or {"bound": "hbm", "achieved": None, "peak": None, "unit": "GB/s",
                                                 "frac": None}
         roof["kernel"] = dom
-    tr = TRAFFIC["bytes_per_launch"].get(dom) if TRAFFIC["source_sha1"] == kernels_sha1() else None
-    roof["traffic"] = tr
+    # (traffic: per step of the FP64 form, as its achieved bytes, and per launch of the dominant kernel)
+    known = TRAFFIC["source_sha1"] == kernels_sha1() and args.precision == 0
+    roof["traffic"] = TRAFFIC["bytes_per_step"] if known else None
+    if args.precision == 0:
+        roof["dominant_kernel"]["traffic"] = TRAFFIC["bytes_per_launch"].get(dom) if known else None
     roof["per_kernel_ms"] = {k: round(v[0] / max(v[1], 1), 4) for k, v in kinds.items()}
     hbm = peaks.get("hbm_gbs", HBM_GBS_FALLBACK)
     step_bytes = algorithmic_bytes_per_step(case)

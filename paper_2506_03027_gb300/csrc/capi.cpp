@@ -644,10 +644,11 @@ cfs_status cfs_finalize(cfs_ctx* c, int max_delay) {
   }
   // The FP64 form of filtered 3-D runs computes its right-hand side on pairs of floats (stage_pairs.cu)
   // when its constants, and with them a flow's nondimensional values (p about 1/(gamma M^2), rho and
-  // u about 1), lie well inside the FP32 range.  Runs without the filter keep the FP64 kernels: there
-  // a step's error against 64-bit arithmetic is the 5e-17 of the final rounding, which the pairs
-  // would raise to 2e-16 at CFL 0.5.  The compact passes hold their lines in shared memory as pairs
-  // of two components (210 points; the scheme itself takes 128).
+  // u about 1), lie well inside the FP32 range.  The error of a step is given at
+  // cfs_params.precision.  Runs without the filter keep the FP64 kernels.  The choice depends on the
+  // parameters alone, never on the memory that is free, so that every process of a partitioned run makes
+  // the same.  The compact passes hold their lines in shared memory as pairs of two components (210 points;
+  // the scheme itself takes 128).
   c->pairs = c->p.precision == 0 && c->ndim == 3 && c->p.filter;
   {
     auto in_range = [](double x) { const double a = std::fabs(x); return a == 0.0 || (a > 1e-12 && a < 1e12); };

@@ -3,7 +3,7 @@
 // one CTA.
 //
 // On an asynchronous step the halo of every pass comes from the ring of delayed levels
-// (AT: extrapolation to t_{n+1} with the weights c(k+1), in FP64; AS: the latest visible level),
+// (AT: extrapolation to t_{n+1} with the weights c(k+1); AS: the latest visible level),
 // not from the neighbours' previous pass, so a sub-domain can be filtered x -> y -> z on its own.
 // The CTA keeps the sub-domain's values as FP32 deviations from a reference value of the
 // sub-domain in shared memory (rows of odd stride: the lines of every pass are read without
@@ -12,10 +12,12 @@
 // the first halo point), adds the increments in FP32 between passes, and writes
 // U + (w_final - w_initial) in FP64 once.  The state is read and written once per step instead of
 // once per pass.  Synchronous steps keep the per-pass kernels (their halo is the neighbours'
-// previous pass).  The halo values -- 10 per line and pass, each a C-level FP64 sum over the
-// ring -- come from k_filter_block_halo, which runs just before with one thread per value (many
-// warps per SM hide the ring reads that a 512-thread, 176-KB CTA cannot) and stores them as FP32
-// deviations for coalesced loads.
+// previous pass).  The halo values -- 10 per line and pass, each a C-level sum over the ring --
+// are formed beforehand by kernels with many warps per SM, which hide the ring reads that a 512-thread,
+// 176-KB CTA cannot, and stored as FP32 deviations for coalesced loads: with the fused stage by
+// k_halo_block (fused.cu) at the start of the step, together with the stages' halo store and in
+// compensated FP32 sums; otherwise (inviscid or second-order runs) by k_filter_block_halo just before, in
+// FP64 sums.
 #include <cuda_runtime.h>
 
 #include <mutex>
