@@ -170,7 +170,12 @@ bool buffer_dudt_weights(int order, int e, int k, long double* d);
 int at_weight_table(int order, int kmax, double* W);
 int filter_extrap_table(int order, int kmax, double* Wf);
 bool pade10_coeffs(double alpha, double* a);
-// x as a pair of floats (hi, lo)
+// x as a pair of floats (hi, lo).  (For an FP64 value the rest is exact in FP64; long double is software on the
+// Arm hosts, which counts for the metric planes of a curvilinear grid.)
+inline float2 pair_of(double x) {
+  const float hi = (float)x;
+  return float2{hi, (float)(x - (double)hi)};
+}
 inline float2 pair_of(long double x) {
   const float hi = (float)x;
   return float2{hi, (float)(x - (long double)hi)};
